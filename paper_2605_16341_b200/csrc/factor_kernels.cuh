@@ -65,7 +65,7 @@ __device__ void group_tile(float* C, int64_t c_rs, int64_t c_cs, const float* A,
 
 struct CholArgs {
     Sel gram;        // r x r Gram matrix (input, left intact)
-    Sel work;        // r x r: receives L^{-1} (lower triangular, strict upper part zero)
+    Sel work;        // SIMT engine: r x r, receives L^{-1} (lower triangular, strict upper part zero)
     int32_t r;
     int32_t which;   // 0: left QR (P), 1: right QR (Q)
     int32_t pass;    // 1, 2 or 3
@@ -77,7 +77,12 @@ struct CholArgs {
     // no such bias.)
     Sel colsq;
     int32_t use_colsq, pad;
-    ImgRef img;      // img.off >= 0: also write L^{-1} as a split image (tensor-core operand)
+    // tensor engine: split image of L^{-T} (the result there, operand of the apply product), of L (same
+    // geometry, at limg_off), the Gram diagonal (fp32 [r]), the statistics of the diagonal blocks, and
+    // later passes: L^{-1}(j, j) over the value that its two image terms hold (fp32 [r], then one more
+    // float: not zero when these factors are to be used)
+    ImgRef img;
+    int64_t limg_off, diag_off, stat_off, scale_off;
     int64_t cnorm_off;   // >= 0: also leave the Gram diagonal (squared column norms) there, fp32 [r]
 };
 

@@ -75,7 +75,9 @@ Scratch scratch_layout(const orthdion_plan* p) {
     const size_t rr = align_up((size_t)p->r * p->r * 4, 256);
     size_t off = 0;
     s.gram = off; off += rr;
-    s.linv = off; off += rr;
+    // L^{-1} in fp32 (SIMT engine), or the split image of L (tensor engine)
+    s.linv = off;
+    off += p->engine == ORTHDION_ENGINE_TENSOR ? std::max(rr, (size_t)img_bytes(p->r, p->r)) : rr;
     if (p->engine == ORTHDION_ENGINE_TENSOR) {
         off = tensor_scratch_layout(p->m, p->n, p->r, fused_fp16(p), off, &s.ts);
         // (after everything whose offset must depend on r only)
@@ -180,25 +182,24 @@ int ensure_attributes() {
     if (state[dev]) return state[dev] > 0 ? 0 : ORTHDION_ERR_CUDA;
     cudaError_t e = cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)CH_SMEM_BYTES);
-    // the r x r factor kernel keeps 2 r floats in dynamic shared memory next to its static tables
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(chol_inv_tc_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kMaxRank * 4);
+        e = cudaFuncSetAttribute(factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(chol_inv_tc_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kMaxRank * 4);
+        e = cudaFuncSetAttribute(factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     // clusters of 16 CTAs are beyond the portable size: allowed per kernel, and used only where the
     // device says that it can place one
     g_factor_cluster_max[dev] = 8;
     if (e == cudaSuccess &&
-        cudaFuncSetAttribute(chol_inv_tc_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaFuncSetAttribute(factor_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(16, 1, 1); cfg.blockDim = dim3(CT_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = (size_t)2 * kMaxRank * 4;
+        cfg.dynamicSmemBytes = CT_SMEM_BYTES;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
         cfg.attrs = attr; cfg.numAttrs = 1;
         int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, chol_inv_tc_kernel<true>, &cfg) == cudaSuccess && clusters >= 1)
+        if (cudaOccupancyMaxActiveClusters(&clusters, factor_kernel<true>, &cfg) == cudaSuccess && clusters >= 1)
             g_factor_cluster_max[dev] = 16;
         else
             (void)cudaGetLastError();
@@ -291,6 +292,8 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
         ca.colsq = sel(W_SCRATCH, 0); ca.use_colsq = 0; ca.img = no_img(); ca.cnorm_off = -1;
         if (lead.tensor()) {
             ca.colsq = sel(W_SCRATCH, lead.sc.ts.colsq); ca.use_colsq = diag_from_gram ? 0 : 1; ca.img = lead.sc.ts.linv;
+            ca.limg_off = lead.sc.linv; ca.diag_off = lead.sc.ts.fdiag; ca.stat_off = lead.sc.ts.fstat;
+            ca.scale_off = lead.sc.ts.fscale;
             if (which == 1 && pass == 1) ca.cnorm_off = lead.sc.ts.cnorm;
         }
         merged->count = 0; merged->pad = 0; merged->scratch_stride = 0;
@@ -299,28 +302,27 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
             prof::Scope scope(prof::S_CHOL, st);
             if (lead.tensor()) {
                 // Fewer matrices than the device has room for CTAs (two per multiprocessor): share
-                // each matrix among the CTAs of a cluster (2, 4 or 8; 16 from rank 512 up, where the
-                // tile lists are long enough to feed them and the device can place such a cluster).
+                // each matrix among the CTAs of a cluster, up to one per 64-row tile (16 only
+                // where the device can place such a cluster).
                 // (counted over the whole grouped call: with more matrices than that, the other
                 // launch batches keep the rest of the device busy on their own streams.)
                 int csize = 1;
-                const int room = 2 * sm_count();
-                const int cmax = r >= 512 ? factor_cluster_max() : 8;
-                while (csize < cmax && std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
-                const size_t dyn = (size_t)2 * r * sizeof(float);
+                const int room = 2 * sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
+                while (csize < factor_cluster_max() && csize < tiles &&
+                       std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
                 if (csize == 1) {
-                    chol_inv_tc_kernel<false><<<merged->count, CT_THREADS, dyn, st>>>(*merged, ca, 1);
+                    factor_kernel<false><<<merged->count, CT_THREADS, CT_SMEM_BYTES, st>>>(*merged, ca, 1);
                 } else {
                     cudaLaunchConfig_t cfg{};
                     cfg.gridDim = dim3((unsigned)(merged->count * csize), 1, 1);
                     cfg.blockDim = dim3(CT_THREADS, 1, 1);
-                    cfg.dynamicSmemBytes = dyn;
+                    cfg.dynamicSmemBytes = CT_SMEM_BYTES;
                     cfg.stream = st;
                     cudaLaunchAttribute attr[1];
                     attr[0].id = cudaLaunchAttributeClusterDimension;
                     attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
                     cfg.attrs = attr; cfg.numAttrs = 1;
-                    if (cudaLaunchKernelEx(&cfg, chol_inv_tc_kernel<true>, *merged, ca, csize) != cudaSuccess)
+                    if (cudaLaunchKernelEx(&cfg, factor_kernel<true>, *merged, ca, csize) != cudaSuccess)
                         engine_error() = 4;
                 }
             } else {
@@ -390,7 +392,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, int
                 if (pass == 1) { out.normal = to_w1; out.shifted = to_w1; }
                 else if (pass == 2) { out.normal = to_fin; out.shifted = to_w0; out.shift_bit = shift_bit; }
                 else { out.normal = to_fin; out.shifted = to_fin; out.shift_bit = shift_bit; out.only_if_shifted = 1; }
-                tensor_apply(r, c.p->passes[1], *c.b, ts, src, rows, out, st);
+                tensor_apply(r, c.p->passes[1], *c.b, ts, src, rows, out, pass > 1, st);
             } else {
                 const Sel in = which ? sel(W_R) : sel(W_P);
                 const Sel tmpA = sel(W_SCRATCH, c.sc.tmpA), tmpB = sel(W_SCRATCH, c.sc.tmpB);
@@ -847,7 +849,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
         tc::Dest to_w1 = dest_none(); to_w1.img = img_view(ts.w1, p->n); to_w1.colsq = 1;
         tc::OutSpec out{};
         out.ld = r; out.normal = to_w1; out.shifted = to_w1;
-        tensor_apply(r, p->passes[1], sr->batch, ts, ts.r, p->n, out, st);
+        tensor_apply(r, p->passes[1], sr->batch, ts, ts.r, p->n, out, false, st);
         shard_gram(*sr, img_view(ts.w1, p->n), p->n, st);
     } else if (phase == 2) {
         {
@@ -862,7 +864,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
         to_fin.f32 = sel(W_Q); to_fin.has_f32 = 1; to_fin.img = ts.q;
         tc::OutSpec out{};
         out.ld = r; out.normal = to_fin; out.shifted = to_fin;
-        tensor_apply(r, p->passes[1], sr->batch, ts, img_view(ts.w1, p->n), p->n, out, st);
+        tensor_apply(r, p->passes[1], sr->batch, ts, img_view(ts.w1, p->n), p->n, out, true, st);
         shard_fused_pass(*sr, st);
     }
     delete merged;

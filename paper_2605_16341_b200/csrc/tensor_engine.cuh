@@ -23,6 +23,7 @@
 #include <cstdio>
 
 #include "common.cuh"
+#include "factor_tc.cuh"
 #include "profile.cuh"
 #include "simt_kernels.cuh"
 
@@ -90,6 +91,7 @@ struct GemmArgs {
     int64_t ld;                              // leading dimension of M, G, X
     ImgRef a, n1, n2;
     int64_t colsq_off;                       // scratch offset of the column-square partials
+    int64_t cscale_off;                      // apply: scratch offset of a factor per result column (fp32), or -1
     float ef_a, ef_b, wc, wd;
     OutSpec out;
     // tensor maps of the images a, n1, n2 over the whole launch batch; the box of each map is the
@@ -777,12 +779,22 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         bool ok = true;
         const int quarter = warp % 4;                    // tensor-memory lanes 32*quarter .. +31
         if (EPI == EPI_STORE) {
+            int scale_b = -1; bool scale_on = false;         // does matrix scale_b want its columns scaled
             for (int t = tile0; t < g.total_tiles && ok; t += tstride) {
                 const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
                 if (!c.active) continue;
+                const MatWork& w = batch.w[c.b];
+                const float* cscale = nullptr;
+                if constexpr (!A_BUF) {
+                    if (g.cscale_off >= 0) {
+                        // (rarely asked for: looked up once per matrix, while its first accumulator is formed)
+                        const float* f = reinterpret_cast<const float*>(w.scratch + g.cscale_off);
+                        if (c.b != scale_b) { scale_b = c.b; scale_on = f[g.Ncols] != 0.f; }
+                        if (scale_on) cscale = f;
+                    }
+                }
                 if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
                 tc_fence_after();
-                const MatWork& w = batch.w[c.b];
                 const int stw = scache.st;
                 const Dest& d = (g.out.shift_bit && (stw & g.out.shift_bit)) ? g.out.shifted : g.out.normal;
                 const uint32_t taddr = tmem_base + acc * acc_stride + ((uint32_t)(quarter * 32) << 16);
@@ -879,12 +891,20 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         }
 #pragma unroll
                         for (int i = 0; i < 16; ++i) f[q4 * 16 + i] = __uint_as_float(v[i]);
+                        if (cscale && q4 * 16 < valid) {
+#pragma unroll
+                            for (int i = 0; i < 16; i += 4) {
+                                const float4 cv = *reinterpret_cast<const float4*>(cscale + gj0 + q4 * 16 + i);
+                                f[q4 * 16 + i] *= cv.x; f[q4 * 16 + i + 1] *= cv.y;
+                                f[q4 * 16 + i + 2] *= cv.z; f[q4 * 16 + i + 3] *= cv.w;
+                            }
+                        }
                         if (csq && q4 * 16 < valid) {
                             // column sums of squares over the 32 rows of this warp: fold 16 values
                             // over the lane bits 4..1, then add the two lanes that hold the same column
                             float s[16];
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) { const float x = __uint_as_float(v[i]); s[i] = x * x; }
+                            for (int i = 0; i < 16; ++i) { const float x = f[q4 * 16 + i]; s[i] = x * x; }
 #pragma unroll
                             for (int half = 8, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
                                 const bool up = (lane & bit) != 0;
@@ -1385,6 +1405,8 @@ struct TensorScratch {      // where the images of one matrix live inside its sc
     int64_t colsq;          // fp32 [4 * ceil(max(m,n)/128)][r] column-square partials
     int64_t cnorm;          // fp32 [r] squared column norms of R
     int64_t rscale;         // fp32 inverse of the scale of R's fp16 plane
+    int64_t fdiag, fstat, fscale;   // factor kernel: fp32 [r] Gram diagonal, statistics of the diagonal blocks,
+                            // fp32 [r + 1] correction of the rounded diagonal of L^{-1}
 };
 
 inline bool tensor_engine_supports(int64_t m, int64_t n, int32_t r) {
@@ -1405,7 +1427,7 @@ inline int64_t img_bytes(int64_t rows, int64_t cols, int planes = 2) {
 }
 inline ImgRef no_img() { ImgRef im; im.off = -1; im.rows_pad = 0; im.panels = 0; im.planes = 0; im.pad = 0; return im; }
 
-// The offsets of linv, cnorm, rscale and colsq depend on r only (everything whose size depends on
+// The offsets of linv, cnorm, rscale, fdiag, fstat, fscale and colsq depend on r only (everything whose size depends on
 // the matrix shape comes after them), so that one Cholesky launch can serve matrices of
 // different shapes.
 // half_planes: P, R, Q carry the fp16 plane (fused pass in fp16).
@@ -1416,6 +1438,9 @@ inline size_t tensor_scratch_layout(int64_t m, int64_t n, int32_t r, bool half_p
     ts->linv = make_img(take(img_bytes(r, r)), r, r);
     ts->cnorm = take((int64_t)r * 4);
     ts->rscale = take(16);
+    ts->fdiag = take((int64_t)r * 4);
+    ts->fstat = take(CT_STAT_FLOATS * 4);
+    ts->fscale = take((int64_t)(r + 1) * 4);
     ts->colsq = take(4 * ((kmax + 127) / 128) * (int64_t)r * 4);
     const int pl = half_planes ? 3 : 2;
     ts->w0 = make_img(take(img_bytes(kmax, r)), kmax, r);
@@ -1760,6 +1785,7 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = src; g.n2 = no_img(); g.lower_only = 1;
     g.out.normal = dest_none(); g.out.normal.f32 = ksplit > 1 ? part : gram; g.out.normal.has_f32 = 1;
     g.out.shifted = g.out.normal; g.out.ld = r;
+    g.cscale_off = -1;
     g.out.shift_bit = only_shift_bit; g.out.only_if_shifted = only_shift_bit ? 1 : 0;
     g.ksplit = ksplit; g.split_stride = (int64_t)r * r;
     launch_gemm<tc::A_IMG_MN, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_GRAM, st);
@@ -1771,12 +1797,16 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
 }
 
 // dst = src * L^{-T}  (src: image of a rows x r matrix; image linv holds (L^{-1})^T, read MN-major)
+// unit: the columns of dst are unit vectors (second and third pass): the rounding of the diagonal of
+// L^{-1} to two bf16 terms, up to 2^-18 of a column's length and hence 2^-17 in its Gram diagonal, is
+// taken out again in the epilogue.
 inline void tensor_apply(int r, int passes, const Batch& b, const TensorScratch& ts, ImgRef src, int64_t rows,
-                         tc::OutSpec out, cudaStream_t st) {
+                         tc::OutSpec out, bool unit, cudaStream_t st) {
     tc::GemmArgs g{};
     g.Mrows = (int32_t)rows; g.Ncols = r; g.Kdim = r; g.BN = std::min(r, 256);
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = ts.linv; g.n2 = no_img(); g.tri = 1;
     g.colsq_off = ts.colsq;
+    g.cscale_off = unit ? ts.fscale : -1;
     g.out = out;
     launch_gemm<tc::A_IMG_K, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_APPLY, st);
 }

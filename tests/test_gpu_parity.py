@@ -127,6 +127,16 @@ def test_one_step_tensor_shapes(shape, mode, dt):
     one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_TENSOR)
 
 
+# ranks around the factor kernel's 64-wide blocks and their 32-wide halves: remainders of 16, 32 and 48, a
+# second, third and sixteenth block
+@pytest.mark.parametrize("shape", [(96, 128, 80), (160, 120, 96), (128, 136, 112), (264, 200, 144), (400, 368, 336),
+                                   (1100, 1040, 1008)])
+def test_factor_kernel_block_edges(shape):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, F32, BF16, seed=m + n + r)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR)
+
+
 @pytest.mark.parametrize("shape", [(384, 640, 64), (1000, 264, 128), (136, 2056, 32), (640, 384, 272)])
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("m_scale", [0.3, 3e-4, 300.0])
