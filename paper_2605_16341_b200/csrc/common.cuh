@@ -54,6 +54,23 @@ __device__ __forceinline__ float load_elem(const void* p, int64_t idx, int is_bf
     return reinterpret_cast<const float*>(p)[idx];
 }
 
+// ---- thread-block clusters ---------------------------------------------------------------------
+__device__ __forceinline__ void cluster_sync_all() {
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+// shared::cluster address of the location `addr` (a shared::cta address) in CTA `rank` of the cluster
+__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+
 // ---- bf16 splitting ---------------------------------------------------------------------------
 // An fp32 value v is carried through the tensor cores as v = t0 + t1 with t0 = bf16(v),
 // t1 = bf16(v - t0) (round to nearest even): the two terms together hold 16 significand bits.

@@ -60,10 +60,6 @@ constexpr int CT_STAT_FLOATS = 3 * CT_MAX_BLOCKS;   // per block: smallest and l
 constexpr float CT_THIRD_PASS_LIMIT = 0.02f; // bound on |Gram - I|_2 of the second pass above which a third follows
 constexpr float CT_SERIES_LIMIT = 1.4e-3f;   // bound on |Gram - I|_2 below which L^{-1} = I - Phi(E) is used
 
-__device__ __forceinline__ void ct_cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
 __device__ __forceinline__ void ct_bar_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -271,6 +267,21 @@ __device__ __forceinline__ void ct_diag_block(unsigned char* smem, int nbk, int 
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
 }
 
+// smallest and largest diagonal entry of the factor from the pivots of warp 0; smallest -1 after a breakdown
+__device__ __forceinline__ void ct_pivot_range(const float (&piv)[2], int nbk, int lane, float& mn, float& mx) {
+    mn = 3.0e38f; mx = 0.f;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        if (h * 32 + lane < nbk) {
+            if (!(piv[h] > 0.f) || !(piv[h] <= 3.0e38f)) mn = -1.f;
+            else { const float sq = sqrtf(piv[h]); mn = fminf(mn, sq); mx = fmaxf(mx, sq); }
+        }
+    }
+    for (int o = 16; o; o >>= 1) {
+        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    }
+}
 // v[e] over the value that its two bf16 terms hold
 __device__ __forceinline__ float ct_diag_scale(const float (&v)[8], const uint4& t0, const uint4& t1, int e) {
     const uint32_t h[4] = {t0.x, t0.y, t0.z, t0.w}, l[4] = {t1.x, t1.y, t1.z, t1.w};
@@ -308,12 +319,12 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     const int r = a.r;
     const int nb = (r + CT_NB - 1) / CT_NB;
     const int shift_bit = a.which ? ST_SHIFT_R : ST_SHIFT_L;
-    auto phase_sync = [&]() { if (MULTI) ct_cluster_sync(); else __syncthreads(); };
+    auto phase_sync = [&]() { if (MULTI) cluster_sync_all(); else __syncthreads(); };
 
     if (tid == 0) s_status = *w.status;
     __syncthreads();
     // every CTA of the cluster has read the status word before any of them may change it
-    if (MULTI) ct_cluster_sync();
+    if (MULTI) cluster_sync_all();
     const int st0 = s_status;
     if (st0 & ST_FAILED) return;
     if (a.pass == 3 && !(st0 & shift_bit)) return;
@@ -639,18 +650,8 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     float piv[2] = {1.f, 1.f};
                     ct_diag_block(smem, nbk, dw, lane, piv);
                     if (dw == 0) {
-                        float mn = 3.0e38f, mx = 0.f;
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            if (h * 32 + lane < nbk) {
-                                if (!(piv[h] > 0.f) || !(piv[h] <= 3.0e38f)) mn = -1.f;        // breakdown
-                                else { const float sq = sqrtf(piv[h]); mn = fminf(mn, sq); mx = fmaxf(mx, sq); }
-                            }
-                        }
-                        for (int o = 16; o; o >>= 1) {
-                            mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-                            mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                        }
+                        float mn, mx;
+                        ct_pivot_range(piv, nbk, lane, mn, mx);
                         if (lane == 0) { gstat[k] = mn; gstat[CT_MAX_BLOCKS + k] = mx; }
                     }
                     // X_k for the panels (in the unused diagonal tile of L's image) and X_k^T, the diagonal

@@ -14,6 +14,7 @@
 #include "profile.cuh"
 #include "factor_kernels.cuh"
 #include "factor_tc.cuh"
+#include "factor_simt.cuh"
 #include "diag_kernels.cuh"
 #include "rank_kernels.cuh"
 #include "simt_kernels.cuh"
@@ -180,8 +181,7 @@ int ensure_attributes() {
     if (dev < 0 || dev >= kMaxDevices) return ORTHDION_ERR_CUDA;
     std::lock_guard<std::mutex> lock(mu);
     if (state[dev]) return state[dev] > 0 ? 0 : ORTHDION_ERR_CUDA;
-    cudaError_t e = cudaFuncSetAttribute(chol_inv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)CH_SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     if (e == cudaSuccess)
@@ -257,12 +257,20 @@ DeviceLanes* device_lanes() {
     return d;
 }
 
-template <class RA, class RB, class EP>
-void launch_simt(const Batch& b, int64_t Md, int64_t Nd, int64_t Kd, RA ra, RB rb, EP ep, int stage,
-                 cudaStream_t st) {
-    dim3 grid((unsigned)((Nd + 63) / 64), (unsigned)((Md + 63) / 64), (unsigned)b.count);
+template <class RA, class RB>
+void launch_simt(const Batch& b, int64_t Md, int64_t Nd, int64_t Kd, RA ra, RB rb, SimtOut out, int stage, cudaStream_t st) {
+    const int parts = simt_parts(Kd);
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((Nd + 63) / 64 * parts), (unsigned)((Md + 63) / 64), (unsigned)b.count);
+    cfg.blockDim = dim3(256, 1, 1);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)parts; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
     prof::Scope scope(stage, st);
-    simt_gemm_kernel<RA, RB, EP><<<grid, 256, 0, st>>>(b, Md, Nd, Kd, ra, rb, ep);
+    if (cudaLaunchKernelEx(&cfg, simt_gemm_kernel<RA, RB>, b, Md, Nd, Kd, parts, ra, rb, out) != cudaSuccess)
+        engine_error() = 5;
 }
 
 Sel sel(int where, int64_t off = 0) { return Sel{where, 0, off}; }
@@ -326,7 +334,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                         engine_error() = 4;
                 }
             } else {
-                chol_inv_kernel<<<merged->count, CH_THREADS, CH_SMEM_BYTES, st>>>(*merged, ca);
+                factor_simt_kernel<<<merged->count, FS_THREADS, CT_SMEM_BYTES, st>>>(*merged, ca);
             }
             merged->count = 0;
         };
@@ -368,7 +376,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, int
             } else {
                 const Sel in = which ? sel(W_R) : sel(W_P);
                 const Sel src = pass == 1 ? in : (pass == 2 ? sel(W_SCRATCH, c.sc.tmpA) : sel(W_SCRATCH, c.sc.tmpB));
-                EpStore eg{gram, gram, only_shift ? shift_bit : 0, 1, r, only_shift};
+                SimtOut eg{gram, gram, only_shift ? shift_bit : 0, 1, r, only_shift, 1};
                 launch_simt(*c.b, r, r, rows, RdPlain{src, 1, r}, RdPlain{src, 1, r}, eg, prof::S_GRAM, st);
             }
         }
@@ -398,10 +406,10 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, int
                 const Sel tmpA = sel(W_SCRATCH, c.sc.tmpA), tmpB = sel(W_SCRATCH, c.sc.tmpB);
                 const Sel linv = sel(W_SCRATCH, c.sc.linv);
                 const Sel src = pass == 1 ? in : (pass == 2 ? tmpA : tmpB);
-                EpStore ea{};
-                if (pass == 1) ea = EpStore{tmpA, tmpA, 0, 1, r, 0};
-                else if (pass == 2) ea = EpStore{fin, tmpB, shift_bit, 1, r, 0};
-                else ea = EpStore{fin, fin, shift_bit, 1, r, 1};
+                SimtOut ea{};
+                if (pass == 1) ea = SimtOut{tmpA, tmpA, 0, 1, r, 0, 0};
+                else if (pass == 2) ea = SimtOut{fin, tmpB, shift_bit, 1, r, 0, 0};
+                else ea = SimtOut{fin, fin, shift_bit, 1, r, 1, 0};
                 launch_simt(*c.b, rows, r, r, RdPlain{src, r, 1}, RdPlain{linv, r, 1}, ea, prof::S_APPLY, st);
             }
         }
@@ -424,7 +432,7 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
         tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), 0, st);
     } else {
         const Sel sQ = sel(W_Q);
-        launch_simt(b, r, r, p->n, RdPlain{sQ, 1, r}, RdPlain{sQ, 1, r}, EpStore{gram, gram, 0, 1, r, 0},
+        launch_simt(b, r, r, p->n, RdPlain{sQ, 1, r}, RdPlain{sQ, 1, r}, SimtOut{gram, gram, 0, 1, r, 0, 0},
                     prof::S_GRAM, st);
     }
     {
@@ -469,7 +477,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
         if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st);
         else launch_simt(*c.b, p->m, p->r, p->n, RdBuffer{p->n, gb, 0}, RdPlain{sQ, 1, p->r},
-                         EpStore{sP, sP, 0, 0, p->r, 0}, prof::S_K1, st);
+                         SimtOut{sP, sP, 0, 0, p->r, 0, 0}, prof::S_K1, st);
     }
     qr_stage(cls, all, 0, merged, call_matrices, st);
     // Alg. 1, right-factor step:  R = (M + G)^T P
@@ -478,7 +486,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
         if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st);
         else launch_simt(*c.b, p->n, p->r, p->m, RdBuffer{p->n, gb, 1}, RdPlain{sP, 1, p->r},
-                         EpStore{sR, sR, 0, 0, p->r, 0}, prof::S_K3, st);
+                         SimtOut{sR, sR, 0, 0, p->r, 0, 0}, prof::S_K3, st);
     }
     // Alg. 1, normalisation step
     qr_stage(cls, orth, 1, merged, call_matrices, st);
@@ -503,10 +511,9 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
             tensor_k5(p->m, p->n, p->r, gb, xb, p->passes[2], p->passes[3], fp16, p->ef_a, p->ef_b, cc, dd, *c.b,
                       c.sc.ts, st);
         } else {
-            launch_simt(*c.b, p->m, p->n, p->r, RdPlain{sP, p->r, 1}, RdPlain{sR, p->r, 1},
-                        EpErrorFeedback{p->ef_a, p->ef_b, p->n, gb}, prof::S_K5, st);
-            launch_simt(*c.b, p->m, p->n, p->r, RdPlain{sP, p->r, 1}, RdPlain{sQ, p->r, 1},
-                        EpWeights{cc, dd, p->n, xb}, prof::S_K5, st);
+            dim3 grid((unsigned)((p->n + 63) / 64), (unsigned)((p->m + 63) / 64), (unsigned)c.b->count);
+            prof::Scope scope(prof::S_K5, st);
+            simt_update_kernel<<<grid, 256, 0, st>>>(*c.b, p->m, p->n, p->r, p->ef_a, p->ef_b, cc, dd, gb, xb);
         }
     }
     for (ClassRun& c : cls)

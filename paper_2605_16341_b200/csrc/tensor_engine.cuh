@@ -157,27 +157,12 @@ __device__ __forceinline__ void tma_load_box(uint32_t dst, const CUtensorMap* ma
 // leader's multicast commit.  All of them keep the default (CTA-scope) semantics of the single-CTA
 // barriers: with release/acquire at cluster scope on every arrive and wait the same kernels ran up
 // to twice as long (the producer thread then pays a cluster-wide fence per load).
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-// shared::cluster address of the location `addr` (a shared::cta address) in CTA `rank` of the cluster
-__device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
-    uint32_t r;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
-    return r;
-}
 __device__ __forceinline__ void mbar_arrive_remote(uint32_t cluster_addr) {
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 __device__ __forceinline__ void mbar_arrive_expect_tx_remote(uint32_t cluster_addr, uint32_t bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cluster.b64 _, [%0], %1;"
                  ::"r"(cluster_addr), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void cluster_sync_all() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Tiled TMA load of a CTA of a pair: the data lands in this CTA's shared memory, the bytes are
 // counted on the mbarrier at cluster address `bar` (the leader's).

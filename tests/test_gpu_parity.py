@@ -118,6 +118,15 @@ def test_one_step_simt_shapes(shape, mode, dt):
     one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_SIMT)
 
 
+# the fp32 engine's 64-wide factor blocks (one row into the second and the third, a full fourth) and the
+# depths at which its products are cut into one more chunk (128, 256, 512)
+@pytest.mark.parametrize("shape", [(127, 128, 65), (255, 256, 129), (511, 513, 200), (530, 300, 256)])
+def test_one_step_simt_block_and_chunk_edges(shape):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, F32, BF16, seed=m + n + r)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_SIMT)
+
+
 @pytest.mark.parametrize("shape", SHAPES_TENSOR)
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("dt", [(F32, F32), (BF16, BF16), (F32, BF16), (BF16, F32)])
