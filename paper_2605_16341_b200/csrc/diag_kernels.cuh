@@ -11,6 +11,7 @@
 // kernels around it.
 #pragma once
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace od {
 
@@ -28,6 +29,7 @@ __device__ __forceinline__ float* diag_record(const MatWork& w, const DiagBase& 
 }
 
 __global__ void diag_init_kernel(const __grid_constant__ Batch batch, DiagBase d) {
+    grid_dependency();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= batch.count * DIAG_STRIDE) return;
     diag_record(batch.w[i / DIAG_STRIDE], d)[i % DIAG_STRIDE] = 0.f;
@@ -38,6 +40,7 @@ __global__ void diag_init_kernel(const __grid_constant__ Batch batch, DiagBase d
 // along columns.
 __global__ void __launch_bounds__(1024)
 diag_colstats_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t stats_off) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     __shared__ float part[3][32][33];
     const int lane = threadIdx.x % 32, ry = threadIdx.x / 32;
@@ -64,6 +67,7 @@ diag_colstats_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int6
 // The same for r % 4 == 0: one CTA per 128 columns, a lane reads four adjacent columns.
 __global__ void __launch_bounds__(1024)
 diag_colstats4_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t stats_off) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     __shared__ __align__(16) float part[3][16][132];
     const int lane = threadIdx.x % 32, ry = threadIdx.x / 32;
@@ -105,6 +109,7 @@ diag_colstats4_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int
 // Sums of squares of M (fp32) and G over the whole matrix, accumulated in double.
 __global__ void __launch_bounds__(256)
 diag_frob_kernel(const __grid_constant__ Batch batch, int64_t elems, int g_bf16, DiagBase d) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     const int64_t quads = elems / 4;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -202,6 +207,7 @@ __device__ float diag_tridiag_max(const float* alpha, const float* beta, int k, 
 __global__ void __launch_bounds__(DIAG_THREADS)
 diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, int64_t stats_off, int mask,
                   float ef_a, float ef_b, DiagBase d) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.x];
     float* out = diag_record(w, d);
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;

@@ -1,6 +1,7 @@
 // Arguments of the r x r factor kernels; ColNorm; status initialisation.
 #pragma once
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace od {
 
@@ -34,6 +35,7 @@ struct CholArgs {
 // scaling, with the squared norms taken from cnorm_off.
 __global__ void __launch_bounds__(1024)
 colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t cnorm_off, int part_sel) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
     __shared__ float part[32][33];
@@ -70,6 +72,7 @@ colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t cn
 // (blocks beyond the matrix hold zeros).  One CTA per (32-row block, 256 columns).
 __global__ void __launch_bounds__(256)
 colsq_blocks_kernel(const __grid_constant__ Batch batch, Sel src, int64_t rows, int r, int64_t colsq_off) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
     const float* S = pick(w, src);
@@ -88,6 +91,7 @@ colsq_blocks_kernel(const __grid_constant__ Batch batch, Sel src, int64_t rows, 
 // over the shards carries the exact diagonal along.
 __global__ void __launch_bounds__(256)
 gram_diag_kernel(const __grid_constant__ Batch batch, Sel gram, int r, int64_t colsq_off, int blocks) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
     const int j = blockIdx.x * 256 + threadIdx.x;
@@ -99,6 +103,7 @@ gram_diag_kernel(const __grid_constant__ Batch batch, Sel gram, int r, int64_t c
 }
 
 __global__ void init_status_kernel(const __grid_constant__ Batch batch) {
+    grid_dependency();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < batch.count) *batch.w[i].status = 0;
 }

@@ -35,6 +35,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     const int tx = tid % 16, ty = tid / 16;
     const int r = a.r, nb = (r + CT_NB - 1) / CT_NB;
     const int shift_bit = a.which ? ST_SHIFT_R : ST_SHIFT_L;
+    grid_dependency();
     const int st0 = *w.status;
     if (st0 & ST_FAILED) return;
     if (a.pass == 3 && !(st0 & shift_bit)) return;

@@ -321,6 +321,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     const int shift_bit = a.which ? ST_SHIFT_R : ST_SHIFT_L;
     auto phase_sync = [&]() { if (MULTI) cluster_sync_all(); else __syncthreads(); };
 
+    grid_dependency();
     if (tid == 0) s_status = *w.status;
     __syncthreads();
     // every CTA of the cluster has read the status word before any of them may change it

@@ -260,17 +260,8 @@ DeviceLanes* device_lanes() {
 template <class RA, class RB>
 void launch_simt(const Batch& b, int64_t Md, int64_t Nd, int64_t Kd, RA ra, RB rb, SimtOut out, int stage, cudaStream_t st) {
     const int parts = simt_parts(Kd);
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)((Nd + 63) / 64 * parts), (unsigned)((Md + 63) / 64), (unsigned)b.count);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = (unsigned)parts; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr; cfg.numAttrs = 1;
-    prof::Scope scope(stage, st);
-    if (cudaLaunchKernelEx(&cfg, simt_gemm_kernel<RA, RB>, b, Md, Nd, Kd, parts, ra, rb, out) != cudaSuccess)
-        engine_error() = 5;
+    launch(simt_gemm_kernel<RA, RB>, dim3((unsigned)((Nd + 63) / 64 * parts), (unsigned)((Md + 63) / 64), (unsigned)b.count), 256, 0,
+           parts, stage, st, b, Md, Nd, Kd, parts, ra, rb, out);
 }
 
 Sel sel(int where, int64_t off = 0) { return Sel{where, 0, off}; }
@@ -307,7 +298,6 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
         merged->count = 0; merged->pad = 0; merged->scratch_stride = 0;
         auto flush = [&]() {
             if (!merged->count) return;
-            prof::Scope scope(prof::S_CHOL, st);
             if (lead.tensor()) {
                 // Fewer matrices than the device has room for CTAs (two per multiprocessor): share
                 // each matrix among the CTAs of a cluster, up to one per 64-row tile (16 only
@@ -318,23 +308,10 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 const int room = 2 * sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
                 while (csize < factor_cluster_max() && csize < tiles &&
                        std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
-                if (csize == 1) {
-                    factor_kernel<false><<<merged->count, CT_THREADS, CT_SMEM_BYTES, st>>>(*merged, ca, 1);
-                } else {
-                    cudaLaunchConfig_t cfg{};
-                    cfg.gridDim = dim3((unsigned)(merged->count * csize), 1, 1);
-                    cfg.blockDim = dim3(CT_THREADS, 1, 1);
-                    cfg.dynamicSmemBytes = CT_SMEM_BYTES;
-                    cfg.stream = st;
-                    cudaLaunchAttribute attr[1];
-                    attr[0].id = cudaLaunchAttributeClusterDimension;
-                    attr[0].val.clusterDim.x = (unsigned)csize; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-                    cfg.attrs = attr; cfg.numAttrs = 1;
-                    if (cudaLaunchKernelEx(&cfg, factor_kernel<true>, *merged, ca, csize) != cudaSuccess)
-                        engine_error() = 4;
-                }
+                launch(csize == 1 ? factor_kernel<false> : factor_kernel<true>, dim3((unsigned)(merged->count * csize)), CT_THREADS,
+                       CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
             } else {
-                factor_simt_kernel<<<merged->count, FS_THREADS, CT_SMEM_BYTES, st>>>(*merged, ca);
+                launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, CT_SMEM_BYTES, 1, prof::S_CHOL, st, *merged, ca);
             }
             merged->count = 0;
         };
@@ -424,10 +401,7 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
     const int r = p->r;
     const Sel gram = sel(W_SCRATCH, c.sc.gram);
     const int64_t stats_off = c.sc.linv;          // 3 r floats of the (now free) inverse slot
-    {
-        prof::Scope scope(prof::S_DIAG, st);
-        diag_init_kernel<<<(b.count * DIAG_STRIDE + 255) / 256, 256, 0, st>>>(b, db);
-    }
+    launch(diag_init_kernel, dim3((unsigned)((b.count * DIAG_STRIDE + 255) / 256)), 256, 0, 1, prof::S_DIAG, st, b, db);
     if (c.tensor()) {
         tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), 0, st);
     } else {
@@ -435,28 +409,21 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
         launch_simt(b, r, r, p->n, RdPlain{sQ, 1, r}, RdPlain{sQ, 1, r}, SimtOut{gram, gram, 0, 1, r, 0, 0},
                     prof::S_GRAM, st);
     }
-    {
-        prof::Scope scope(prof::S_DIAG, st);
-        if (r % 4 == 0) {
-            dim3 grid((unsigned)((r + 127) / 128), 1, (unsigned)b.count);
-            diag_colstats4_kernel<<<grid, 1024, 0, st>>>(b, p->n, r, stats_off);
-        } else {
-            dim3 grid((unsigned)((r + 31) / 32), 1, (unsigned)b.count);
-            diag_colstats_kernel<<<grid, 1024, 0, st>>>(b, p->n, r, stats_off);
-        }
-    }
+    if (r % 4 == 0)
+        launch(diag_colstats4_kernel, dim3((unsigned)((r + 127) / 128), 1, (unsigned)b.count), 1024, 0, 1, prof::S_DIAG, st, b, p->n, r,
+               stats_off);
+    else
+        launch(diag_colstats_kernel, dim3((unsigned)((r + 31) / 32), 1, (unsigned)b.count), 1024, 0, 1, prof::S_DIAG, st, b, p->n, r,
+               stats_off);
     if (p->diag & 2) {
         const int64_t elems = p->m * p->n;
         const int64_t want = (elems / 4 + 256 * 32 - 1) / (256 * 32);
         dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 1184 / std::max(1, b.count) + 1)), 1,
                   (unsigned)b.count);
-        prof::Scope scope(prof::S_DIAG, st);
-        diag_frob_kernel<<<grid, 256, 0, st>>>(b, elems, p->g_dtype == ORTHDION_DTYPE_BF16, db);
+        launch(diag_frob_kernel, grid, 256, 0, 1, prof::S_DIAG, st, b, elems, (int)(p->g_dtype == ORTHDION_DTYPE_BF16), db);
     }
-    {
-        prof::Scope scope(prof::S_DIAG, st);
-        diag_final_kernel<<<b.count, DIAG_THREADS, 0, st>>>(b, r, c.sc.gram, stats_off, p->diag, p->ef_a, p->ef_b, db);
-    }
+    launch(diag_final_kernel, dim3((unsigned)b.count), DIAG_THREADS, 0, 1, prof::S_DIAG, st, b, r, c.sc.gram, stats_off, p->diag, p->ef_a,
+           p->ef_b, db);
 }
 
 // One step of every class of a group, stage by stage.
@@ -467,10 +434,8 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         all.push_back((int)i);
         if (cls[i].p->mode == ORTHDION_MODE_ORTH) orth.push_back((int)i);
     }
-    for (ClassRun& c : cls) {
-        prof::Scope scope(prof::S_MISC, st);
-        init_status_kernel<<<(c.b->count + 255) / 256, 256, 0, st>>>(*c.b);
-    }
+    for (ClassRun& c : cls)
+        launch(init_status_kernel, dim3((unsigned)((c.b->count + 255) / 256)), 256, 0, 1, prof::S_MISC, st, *c.b);
     // Alg. 1, buffer and left-factor steps:  Y = (M + G) Q_prev
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
@@ -493,11 +458,8 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         if (p->mode == ORTHDION_MODE_ORTH) continue;
-        {
-            dim3 grid((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count);
-            prof::Scope scope(prof::S_COLNORM, st);
-            colnorm_kernel<<<grid, 1024, 0, st>>>(*c.b, p->n, p->r, c.tensor() ? c.sc.ts.cnorm : (int64_t)-1, 0);
-        }
+        launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b, p->n,
+               p->r, c.tensor() ? c.sc.ts.cnorm : (int64_t)-1, 0);
         if (c.tensor()) launch_pack(*c.b, sQ, p->n, p->r, c.sc.ts.q, st);
     }
     // Alg. 1, update and error-feedback steps:  M <- a B - b P R^T ;  X <- c X - d P Q^T
@@ -512,8 +474,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
                       c.sc.ts, st);
         } else {
             dim3 grid((unsigned)((p->n + 63) / 64), (unsigned)((p->m + 63) / 64), (unsigned)c.b->count);
-            prof::Scope scope(prof::S_K5, st);
-            simt_update_kernel<<<grid, 256, 0, st>>>(*c.b, p->m, p->n, p->r, p->ef_a, p->ef_b, cc, dd, gb, xb);
+            launch(simt_update_kernel, grid, 256, 0, 1, prof::S_K5, st, *c.b, p->m, p->n, p->r, p->ef_a, p->ef_b, cc, dd, gb, xb);
         }
     }
     for (ClassRun& c : cls)
@@ -696,6 +657,11 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
                           reinterpret_cast<float*>(ws + lay.diag_off)};
         const int lanes = std::min<int>({g_lanes.load(), kMaxLanes, (int)cls.size()});
         DeviceLanes* dl = lanes > 1 ? device_lanes() : nullptr;
+        // Launches of one chain overlap; with several chains they do not: the waiting CTAs of one chain
+        // would keep the others' kernels off the multiprocessors (measured, four streams: 320M model
+        // 2.50 -> 2.78 ms, 1.1B model 17.7 -> 18.2 ms; one chain: 256 x 512 r = 16 0.229 -> 0.198 ms,
+        // 520 x 384 r = 64 0.269 -> 0.235 ms, 4096 x 4096 r = 256 0.665 -> 0.633 ms).
+        overlap_launches() = dl == nullptr;
         if (dl) {
             // heaviest batch first, each batch a lane of its own (round robin beyond `lanes`)
             std::vector<int> order(cls.size());
@@ -795,9 +761,8 @@ void shard_gram(ShardRun& sr, const ImgRef& src, int64_t rows, cudaStream_t st) 
     const orthdion_plan* p = sr.c.p;
     const Sel gram = sel(W_SCRATCH, sr.c.sc.gram);
     tensor_gram(p->r, p->passes[1], sr.batch, src, rows, gram, sel(W_SCRATCH, sr.c.sc.gram_part), 0, st);
-    prof::Scope scope(prof::S_MISC, st);
-    gram_diag_kernel<<<dim3((unsigned)((p->r + 255) / 256), 1, 1), 256, 0, st>>>(
-        sr.batch, gram, p->r, sr.c.sc.ts.colsq, (int)(4 * ((rows + 127) / 128)));
+    launch(gram_diag_kernel, dim3((unsigned)((p->r + 255) / 256)), 256, 0, 1, prof::S_MISC, st, sr.batch, gram, p->r, sr.c.sc.ts.colsq,
+           (int)(4 * ((rows + 127) / 128)));
 }
 
 void shard_fused_pass(ShardRun& sr, cudaStream_t st) {
@@ -829,27 +794,21 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     const std::vector<int> only(1, 0);
     Batch* merged = new Batch();
     engine_error() = 0;
+    overlap_launches() = true;
     if (phase == 0) {
-        {
-            prof::Scope scope(prof::S_MISC, st);
-            init_status_kernel<<<1, 256, 0, st>>>(sr->batch);
-        }
+        launch(init_status_kernel, dim3(1), 256, 0, 1, prof::S_MISC, st, sr->batch);
         tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, true);
     } else if (phase == 1) {
         // the summed Y sits in the P slot: image and column squares, then the usual left QR
         launch_pack(sr->batch, sel(W_P), p->m, r, img_view(ts.w0, p->m), st);
-        {
-            prof::Scope scope(prof::S_MISC, st);
-            colsq_blocks_kernel<<<dim3((unsigned)(4 * ((p->m + 127) / 128)), (unsigned)((r + 255) / 256), 1), 256, 0, st>>>(
-                sr->batch, sel(W_P), p->m, r, ts.colsq);
-        }
+        launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((p->m + 127) / 128)), (unsigned)((r + 255) / 256)), 256, 0, 1, prof::S_MISC, st,
+               sr->batch, sel(W_P), p->m, r, ts.colsq);
         qr_stage(cls, only, 0, merged, 1, st);
         tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st);
         if (orth) {
             shard_gram(*sr, ts.r, p->n, st);
         } else {
-            prof::Scope scope(prof::S_COLNORM, st);
-            colnorm_kernel<<<dim3((unsigned)((r + 31) / 32), 1, 1), 1024, 0, st>>>(sr->batch, p->n, r, ts.cnorm, 1);
+            launch(colnorm_kernel, dim3((unsigned)((r + 31) / 32)), 1024, 0, 1, prof::S_COLNORM, st, sr->batch, p->n, r, ts.cnorm, 1);
         }
     } else if (phase == 2 && orth) {
         chol_stage(cls, only, 1, 1, merged, 1, st, true);
@@ -859,10 +818,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
         tensor_apply(r, p->passes[1], sr->batch, ts, ts.r, p->n, out, false, st);
         shard_gram(*sr, img_view(ts.w1, p->n), p->n, st);
     } else if (phase == 2) {
-        {
-            prof::Scope scope(prof::S_COLNORM, st);
-            colnorm_kernel<<<dim3((unsigned)((r + 31) / 32), 1, 1), 1024, 0, st>>>(sr->batch, p->n, r, ts.cnorm, 2);
-        }
+        launch(colnorm_kernel, dim3((unsigned)((r + 31) / 32)), 1024, 0, 1, prof::S_COLNORM, st, sr->batch, p->n, r, ts.cnorm, 2);
         launch_pack(sr->batch, sel(W_Q), p->n, r, ts.q, st);
         shard_fused_pass(*sr, st);
     } else {

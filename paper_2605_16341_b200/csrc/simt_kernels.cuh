@@ -11,6 +11,7 @@
 // 31, R = B^T P 217 -> 31, the two products of the update 19.5 + 19.0 -> 21.5 in one kernel.
 #pragma once
 #include "common.cuh"
+#include "launch.cuh"
 
 namespace od {
 
@@ -101,6 +102,7 @@ __device__ __forceinline__ void simt_fma(float (&acc)[4][4], const SimtStage& a,
 template <class RA, class RB>
 __global__ void __launch_bounds__(256)
 simt_gemm_kernel(const __grid_constant__ Batch batch, int64_t Md, int64_t Nd, int64_t Kd, int parts, RA ra, RB rb, SimtOut out) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     const int st = *w.status;
     if (!out.active(st)) return;
@@ -172,6 +174,7 @@ simt_gemm_kernel(const __grid_constant__ Batch batch, int64_t Md, int64_t Nd, in
 __global__ void __launch_bounds__(256)
 simt_update_kernel(const __grid_constant__ Batch batch, int64_t m, int64_t n, int r, float a, float b, float c, float d,
                    int g_bf16, int x_bf16) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
     __shared__ SimtStage Ps, Rs, Qs;

@@ -24,7 +24,7 @@
 
 #include "common.cuh"
 #include "factor_tc.cuh"
-#include "profile.cuh"
+#include "launch.cuh"
 #include "simt_kernels.cuh"
 
 namespace od {
@@ -196,6 +196,9 @@ __device__ __forceinline__ void umma_commit_pair(uint32_t bar) {
         ::"r"(bar), "h"((uint16_t)3) : "memory");
 }
 
+__device__ __forceinline__ void prefetch_tensor_map(const CUtensorMap* map) {
+    asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(map)) : "memory");
+}
 // Asynchronous 16-byte copy global -> shared (no register staging), grouped per thread.
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -298,6 +301,7 @@ struct PackArgs {
 
 __global__ void __launch_bounds__(256)
 pack_kernel(const __grid_constant__ Batch batch, PackArgs a) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
     const float* S = pick(w, a.src);
@@ -340,6 +344,7 @@ struct PackHalfArgs {
 
 __global__ void __launch_bounds__(256)
 pack_half_kernel(const __grid_constant__ Batch batch, PackHalfArgs a) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
     __shared__ float red[8];
@@ -502,11 +507,18 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async_smem();
     }
+    if (warp == 0 && lane == 0) {
+        if (!A_BUF) prefetch_tensor_map(&g.map_a);
+        prefetch_tensor_map(&g.map_n1);
+        if (EPI == EPI_K5) prefetch_tensor_map(&g.map_n2);
+    }
+    grid_dependency_launch();
     if (warp == 1) {
         if (PAIR) tmem_alloc_pair(smem_u32(tmem_slot), (uint32_t)g.tmem_cols);
         else tmem_alloc(smem_u32(tmem_slot), (uint32_t)g.tmem_cols);
     }
     tc_fence_before();
+    grid_dependency_wait();
     __syncthreads();
     if (PAIR) cluster_sync_all();       // the peer's barriers are initialised before anything reaches them
     tc_fence_after();
@@ -1462,10 +1474,6 @@ inline TensorMapEncodeFn tensor_map_encoder() {
     }
     return fn;
 }
-// First error met while preparing launches of the current step call (0 = none); one per host
-// thread, so that concurrent step calls do not see each other's.
-inline int& engine_error() { static thread_local int e = 0; return e; }
-
 // 5-d map over the images `img` of all matrices of a batch: (64 bf16, rows, panels, terms, matrix),
 // with the box (64, box_rows, box_panels, box_terms, 1).  The images are stored pre-swizzled, so
 // the copy itself does not swizzle; out-of-range parts of a box read as zeros.
@@ -1546,16 +1554,14 @@ inline void launch_pack_half(const Batch& b, int64_t rows, int64_t cols, const T
     tc::PackHalfArgs a{};
     a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.dst = ts.r; a.cnorm_off = ts.cnorm; a.rscale_off = ts.rscale;
     dim3 grid((unsigned)ts.r.panels, (unsigned)(ts.r.rows_pad / 128), (unsigned)b.count);
-    prof::Scope scope(prof::S_PACK, st);
-    tc::pack_half_kernel<<<grid, 256, 0, st>>>(b, a);
+    launch(tc::pack_half_kernel, grid, 256, 0, 1, prof::S_PACK, st, b, a);
 }
 
 inline void launch_pack(const Batch& b, Sel src, int64_t rows, int64_t cols, ImgRef dst, cudaStream_t st) {
     tc::PackArgs a{};
     a.src = src; a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.dst = dst;
     dim3 grid((unsigned)dst.panels, (unsigned)(dst.rows_pad / 128), (unsigned)b.count);
-    prof::Scope scope(prof::S_PACK, st);
-    tc::pack_kernel<<<grid, 256, 0, st>>>(b, a);
+    launch(tc::pack_kernel, grid, 256, 0, 1, prof::S_PACK, st, b, a);
 }
 
 // Fills in the tiling, ring and tensor-memory fields and launches.
@@ -1622,25 +1628,15 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     else encode_img_map(&g.map_n1, b, g.n1, 128, 1, n1_terms);
     if (EPI == tc::EPI_K5) encode_img_map(&g.map_n2, b, g.n2, 128, 1, n2_terms);
     if (engine_error()) return;
-    prof::Scope scope(stage, st);
     if constexpr (pair_capable(NMODE, EPI, XG)) {
         if (pair) {
-            cudaLaunchConfig_t cfg{};
-            cfg.gridDim = dim3((unsigned)(2 * std::min(g.total_tiles, sm_count() / 2)), 1, 1);
-            cfg.blockDim = dim3((unsigned)tc::gemm_threads(AMODE, EPI), 1, 1);
-            cfg.dynamicSmemBytes = smem;
-            cfg.stream = st;
-            cudaLaunchAttribute attr[1];
-            attr[0].id = cudaLaunchAttributeClusterDimension;
-            attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-            cfg.attrs = attr; cfg.numAttrs = 1;
-            if (cudaLaunchKernelEx(&cfg, tc::gemm_kernel<AMODE, NMODE, EPI, XG, true>, b, g) != cudaSuccess)
-                engine_error() = 3;
+            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true>, dim3((unsigned)(2 * std::min(g.total_tiles, sm_count() / 2))),
+                   tc::gemm_threads(AMODE, EPI), smem, 2, stage, st, b, g);
             return;
         }
     }
-    const int grid = std::min(g.total_tiles, sm_count());
-    tc::gemm_kernel<AMODE, NMODE, EPI, XG, false><<<grid, tc::gemm_threads(AMODE, EPI), smem, st>>>(b, g);
+    launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false>, dim3((unsigned)std::min(g.total_tiles, sm_count())),
+           tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
 }
 
 inline tc::Dest dest_none() {
@@ -1674,18 +1670,12 @@ __global__ void gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram
 // column squares per 32-row block
 inline void finish_split_product(const Batch& b, Sel dst, Sel part, int64_t rows, int r, int ksplit, ImgRef img,
                                  int64_t colsq_off, int stage, cudaStream_t st) {
-    {
-        prof::Scope scope(stage, st);
-        const int64_t total4 = rows * r / 4;
-        dim3 grid((unsigned)((total4 + 255) / 256), 1, (unsigned)b.count);
-        gram_reduce_kernel<<<grid, 256, 0, st>>>(b, dst, part, total4, ksplit, 0);
-    }
+    const int64_t total4 = rows * r / 4;
+    launch(gram_reduce_kernel, dim3((unsigned)((total4 + 255) / 256), 1, (unsigned)b.count), 256, 0, 1, stage, st, b, dst, part,
+           total4, ksplit, 0);
     launch_pack(b, dst, rows, r, img, st);
-    {
-        prof::Scope scope(stage, st);
-        dim3 grid((unsigned)(4 * ((rows + 127) / 128)), (unsigned)((r + 255) / 256), (unsigned)b.count);
-        colsq_blocks_kernel<<<grid, 256, 0, st>>>(b, dst, rows, r, colsq_off);
-    }
+    launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((rows + 127) / 128)), (unsigned)((r + 255) / 256), (unsigned)b.count), 256, 0, 1,
+           stage, st, b, dst, rows, r, colsq_off);
 }
 
 // Y = (M + G) Q_prev  -> image w0 (+ column squares)              (Alg. 1, buffer and left-factor steps)
@@ -1746,6 +1736,7 @@ inline int gram_ksplit(int r, int64_t rows) {
 // other), added in the order of the chunks
 __global__ void __launch_bounds__(256)
 gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit, int only_shift_bit) {
+    grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     const int st = *w.status;
     if ((st & ST_FAILED) || (only_shift_bit && !(st & only_shift_bit))) return;
@@ -1775,9 +1766,9 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
     g.ksplit = ksplit; g.split_stride = (int64_t)r * r;
     launch_gemm<tc::A_IMG_MN, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_GRAM, st);
     if (ksplit > 1) {
-        prof::Scope scope(prof::S_GRAM, st);
-        dim3 grid((unsigned)(((int64_t)r * r / 4 + 255) / 256), 1, (unsigned)b.count);
-        gram_reduce_kernel<<<grid, 256, 0, st>>>(b, gram, part, (int64_t)r * r / 4, ksplit, only_shift_bit);
+        const int64_t total4 = (int64_t)r * r / 4;
+        launch(gram_reduce_kernel, dim3((unsigned)((total4 + 255) / 256), 1, (unsigned)b.count), 256, 0, 1, prof::S_GRAM, st, b, gram,
+               part, total4, ksplit, only_shift_bit);
     }
 }
 
