@@ -44,15 +44,14 @@ constexpr int CT_NB = 64;                     // block width, tile rows
 constexpr int CT_TERM = CT_NB * 128;          // one bf16 term of a 64 x 64 tile: 64 image rows of 128 bytes
 constexpr int CT_TILE = 2 * CT_TERM;
 constexpr int CT_LDD = 68;                    // diagonal block, fp32 (rows 16-byte aligned, conflict-free by row)
-constexpr int CT_LDT = 68, CT_LDH = 36;       // transposed factor columns: 32 x 64, and 32 x 32 of the second half
+constexpr int CT_LDT = 68;                    // transposed factor columns: 32 x 64 (the second half's in place of L11's)
 constexpr int CT_LDS = 65;                    // transposing buffer of the first-order inverse
 // dynamic shared memory: two stages of an A tile and a B tile, then the diagonal block's work area
 constexpr int CT_OFF_D = 4 * CT_TILE;
-constexpr int CT_OFF_LT = CT_OFF_D + CT_NB * CT_LDD * 4;
-constexpr int CT_OFF_LT2 = CT_OFF_LT + 32 * CT_LDT * 4;
-constexpr int CT_OFF_T = CT_OFF_LT2 + 32 * CT_LDH * 4;
-constexpr int CT_OFF_RS = CT_OFF_T + 32 * CT_LDH * 4;
-constexpr int CT_SMEM_BYTES = CT_OFF_RS + 64 * 4 + 1024;       // + alignment of the tiles
+constexpr int CT_DG_LT = CT_NB * CT_LDD * 4;                   // work area of a diagonal block: the block itself first
+constexpr int CT_DG_RS = CT_DG_LT + 32 * CT_LDT * 4;
+constexpr int CT_DG_BYTES = CT_DG_RS + 64 * 4;
+constexpr int CT_SMEM_BYTES = CT_OFF_D + CT_DG_BYTES + 1024;   // + alignment of the tiles
 static_assert(2 * (CT_SMEM_BYTES + 2048) <= 228 * 1024, "two CTAs per multiprocessor");
 static_assert(3 * CT_NB * CT_LDS * 4 <= 4 * CT_TILE, "three transposing buffers fit the operand stages");
 constexpr int CT_MAX_BLOCKS = 64;             // r <= 4096
@@ -131,34 +130,35 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 }
 
 // ---- diagonal blocks (fp32, one warp) ------------------------------------------------------------
-// Cholesky of the 32 x 32 block at `blk` (ld CT_LDD).  Lane i holds row i in registers.  LT[j][i] <- L(i, j),
+// Cholesky of the leading NC columns of the 32 x 32 block at `blk` (ld CT_LDD).  Lane i holds row i in registers.  LT[j][i] <- L(i, j),
 // rs[j] <- 1 / L(j, j); the lane keeps its pivot in `piv`.  The pivot of column j + 1 is formed from two
 // values fetched before column j was scaled, so that the chain per column is one reciprocal square root
 // and two products; the next two columns get their multiplier by shuffle, the others from LT.
-__device__ __forceinline__ void ct_chol32(const float* blk, float* LT, int ldt, float* rs, float& piv, int lane) {
-    float a[32];
+template <int NC>
+__device__ __forceinline__ void ct_chol32(const float* blk, float* LT, float* rs, float& piv, int lane) {
+    float a[NC];
 #pragma unroll
-    for (int c = 0; c < 32; c += 4) {
+    for (int c = 0; c < NC; c += 4) {
         const float4 v = *reinterpret_cast<const float4*>(blk + lane * CT_LDD + c);
         a[c] = v.x; a[c + 1] = v.y; a[c + 2] = v.z; a[c + 3] = v.w;
     }
     float d = __shfl_sync(0xffffffffu, a[0], 0);
     float q = __shfl_sync(0xffffffffu, a[0], 1), p = __shfl_sync(0xffffffffu, a[1], 1);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) {
+    for (int j = 0; j < NC; ++j) {
         const float inv = rsqrtf(d);
         if (lane == j) { piv = d; rs[j] = inv; }
         const float la = a[j] * inv;
-        LT[j * ldt + lane] = la;
-        if (j + 1 < 32) { const float t = q * inv; d = fmaf(-t, t, p); }
+        LT[j * CT_LDT + lane] = la;
+        if (j + 1 < NC) { const float t = q * inv; d = fmaf(-t, t, p); }
 #pragma unroll
         for (int c = j + 1; c < j + 3; ++c)
-            if (c < 32) a[c] = fmaf(-la, __shfl_sync(0xffffffffu, la, c), a[c]);
-        if (j + 2 < 32) { q = __shfl_sync(0xffffffffu, a[j + 1], j + 2); p = __shfl_sync(0xffffffffu, a[j + 2], j + 2); }
+            if (c < NC) a[c] = fmaf(-la, __shfl_sync(0xffffffffu, la, c), a[c]);
+        if (j + 2 < NC) { q = __shfl_sync(0xffffffffu, a[j + 1], j + 2); p = __shfl_sync(0xffffffffu, a[j + 2], j + 2); }
         __syncwarp();
 #pragma unroll
-        for (int c4 = (j + 3) / 4; c4 < 8; ++c4) {
-            const float4 v = *reinterpret_cast<const float4*>(LT + j * ldt + 4 * c4);
+        for (int c4 = (j + 3) / 4; c4 < NC / 4; ++c4) {
+            const float4 v = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 4 * c4);
             const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -166,15 +166,16 @@ __device__ __forceinline__ void ct_chol32(const float* blk, float* LT, int ldt, 
         }
     }
 }
-// s <- L^{-1} s for the 32 x 32 factor held in LT, rs; each lane has a right-hand side of its own
-__device__ __forceinline__ void ct_solve32(float (&s)[32], const float* LT, int ldt, const float* rs) {
+// s <- L^{-1} s for the NC x NC factor held in LT, rs; each lane has a right-hand side of its own
+template <int NC>
+__device__ __forceinline__ void ct_solve32(float (&s)[NC], const float* LT, const float* rs) {
 #pragma unroll
-    for (int p = 0; p < 32; ++p) {
+    for (int p = 0; p < NC; ++p) {
         const float x = s[p] * rs[p];
         s[p] = x;
 #pragma unroll
-        for (int i4 = (p + 1) / 4; i4 < 8; ++i4) {
-            const float4 v = *reinterpret_cast<const float4*>(LT + p * ldt + 4 * i4);
+        for (int i4 = (p + 1) / 4; i4 < NC / 4; ++i4) {
+            const float4 v = *reinterpret_cast<const float4*>(LT + p * CT_LDT + 4 * i4);
             const float vv[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int e = 0; e < 4; ++e)
@@ -183,36 +184,39 @@ __device__ __forceinline__ void ct_solve32(float (&s)[32], const float* LT, int 
     }
 }
 // The four diagonal warps: sD (64 x 64, ld CT_LDD, identity beyond nbk) <- inverse of its Cholesky factor
-// (lower triangle; what lies above it is not defined).  piv[]: the lane's pivots of warp 0.
+// (lower triangle; what lies above it is not defined: the upper right quarter holds T).  piv[]: the lane's
+// pivots of warp 0.  `area`: CT_DG_BYTES of shared memory, sD first.  NC < 32: nbk <= NC, only the leading NC
+// columns are looked at.
 //   L11                                       warp 0
 //   L21 = D21 L11^{-T}  (warp 1)              X11 = L11^{-1}  (warp 2)
 //   D22 -= L21 L21^T                          all
 //   L22  (warp 0)                             T = L21 X11  (warps 1-3, by rows)
 //   X22 = L22^{-1}  (warp 0)                  X21 = -L22^{-1} T  (warp 1)
-__device__ __forceinline__ void ct_diag_block(unsigned char* smem, int nbk, int dw, int lane, float (&piv)[2]) {
-    float* sD = reinterpret_cast<float*>(smem + CT_OFF_D);
-    float* LT = reinterpret_cast<float*>(smem + CT_OFF_LT);
-    float* LT2 = reinterpret_cast<float*>(smem + CT_OFF_LT2);
-    float* sT = reinterpret_cast<float*>(smem + CT_OFF_T);
-    float* rs = reinterpret_cast<float*>(smem + CT_OFF_RS);
-    const bool two = nbk > 32;
-    if (dw == 0) ct_chol32(sD, LT, CT_LDT, rs, piv[0], lane);
+template <int NC>
+__device__ __forceinline__ void ct_diag_block(unsigned char* area, int nbk, int dw, int lane, float (&piv)[2]) {
+    float* sD = reinterpret_cast<float*>(area);
+    float* LT = reinterpret_cast<float*>(area + CT_DG_LT);
+    float* sT = sD + 32;
+    float* rs = reinterpret_cast<float*>(area + CT_DG_RS);
+    const bool two = NC == 32 && nbk > 32;
+    if (dw == 0) ct_chol32<NC>(sD, LT, rs, piv[0], lane);
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-    float s[32];
+    float s[NC];
     if (dw == 2 || (dw == 1 && two)) {
 #pragma unroll
-        for (int i = 0; i < 32; i += 4) {
+        for (int i = 0; i < NC; i += 4) {
             float4 v = make_float4(i == lane ? 1.f : 0.f, i + 1 == lane ? 1.f : 0.f, i + 2 == lane ? 1.f : 0.f, i + 3 == lane ? 1.f : 0.f);
             if (dw == 1) v = *reinterpret_cast<const float4*>(sD + (32 + lane) * CT_LDD + i);
             s[i] = v.x; s[i + 1] = v.y; s[i + 2] = v.z; s[i + 3] = v.w;
         }
-        ct_solve32(s, LT, CT_LDT, rs);
+        ct_solve32<NC>(s, LT, rs);
         float* dst = dw == 1 ? LT + 32 + lane : sD + lane;
         const int ld = dw == 1 ? CT_LDT : CT_LDD;
 #pragma unroll
-        for (int i = 0; i < 32; ++i) dst[i * ld] = s[i];
+        for (int i = 0; i < NC; ++i) dst[i * ld] = s[i];
     }
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+    if constexpr (NC == 32) {
     if (!two) return;
     {
         // D22(lane, 8 dw ..) -= sum_j L21(lane, j) L21(8 dw .., j)
@@ -233,7 +237,7 @@ __device__ __forceinline__ void ct_diag_block(unsigned char* smem, int nbk, int 
     }
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
     if (dw == 0) {
-        ct_chol32(sD + 32 * CT_LDD + 32, LT2, CT_LDH, rs + 32, piv[1], lane);
+        ct_chol32<32>(sD + 32 * CT_LDD + 32, LT, rs + 32, piv[1], lane);
     } else {
         // rows 12 (dw - 1) .. + 11 of T (the last warp: 8 rows), a column per lane
         const int i0 = 12 * (dw - 1);
@@ -254,17 +258,18 @@ __device__ __forceinline__ void ct_diag_block(unsigned char* smem, int nbk, int 
         }
 #pragma unroll
         for (int e = 0; e < 12; ++e)
-            if (e < 8 || dw < 3) sT[(i0 + e) * CT_LDH + lane] = t[e];
+            if (e < 8 || dw < 3) sT[(i0 + e) * CT_LDD + lane] = t[e];
     }
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
     if (dw < 2) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) s[i] = dw == 0 ? (i == lane ? 1.f : 0.f) : -sT[i * CT_LDH + lane];
-        ct_solve32(s, LT2, CT_LDH, rs + 32);
+        for (int i = 0; i < 32; ++i) s[i] = dw == 0 ? (i == lane ? 1.f : 0.f) : -sT[i * CT_LDD + lane];
+        ct_solve32<32>(s, LT, rs + 32);
 #pragma unroll
         for (int i = 0; i < 32; ++i) sD[(32 + i) * CT_LDD + (dw == 0 ? 32 : 0) + lane] = s[i];
     }
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+    }
 }
 
 // smallest and largest diagonal entry of the factor from the pivots of warp 0; smallest -1 after a breakdown
@@ -649,7 +654,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     const int nbk = min(CT_NB, r - k * CT_NB);
                     ct_bar_sync(CT_BAR_READY, CT_THREADS);
                     float piv[2] = {1.f, 1.f};
-                    ct_diag_block(smem, nbk, dw, lane, piv);
+                    ct_diag_block<32>(smem + CT_OFF_D, nbk, dw, lane, piv);
                     if (dw == 0) {
                         float mn, mx;
                         ct_pivot_range(piv, nbk, lane, mn, mx);

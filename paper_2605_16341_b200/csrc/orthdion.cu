@@ -83,7 +83,7 @@ Scratch scratch_layout(const orthdion_plan* p) {
         off = tensor_scratch_layout(p->m, p->n, p->r, fused_fp16(p), off, &s.ts);
         // (after everything whose offset must depend on r only)
         const int parts = std::max(gram_ksplit(p->r, p->m), gram_ksplit(p->r, p->n));
-        const int s1 = buffer_ksplit(p->r, p->m, p->n), s3 = buffer_ksplit(p->r, p->n, p->m);
+        const int s1 = buffer_chunks(p->r, p->m, p->n), s3 = buffer_chunks(p->r, p->n, p->m);
         size_t part_bytes = parts > 1 ? (size_t)parts * rr : 0;
         if (s1 > 1) part_bytes = std::max(part_bytes, align_up((size_t)s1 * p->m * p->r * 4, 256));
         if (s3 > 1) part_bytes = std::max(part_bytes, align_up((size_t)s3 * p->n * p->r * 4, 256));
@@ -171,7 +171,28 @@ Layout make_layout(const orthdion_t* hs, int32_t count, size_t scratch_bytes) {
 
 // Kernel attributes (dynamic shared-memory limits) belong to a device: they are set once per
 // device ordinal, on the first step call made with that device current.
-signed char g_factor_cluster_max[kMaxDevices] = {};   // written under ensure_attributes()'s lock
+// Largest clusters of the factor kernel and of the small-rank QR kernel (16 CTAs where the device can
+// place one, else 8); written under ensure_attributes()'s lock.
+signed char g_factor_cluster_max[kMaxDevices] = {}, g_qr_cluster_max[kMaxDevices] = {};
+
+// Clusters of 16 CTAs are beyond the portable size: allowed per kernel, and used only where the
+// device says that it can place one.
+template <class K>
+int largest_cluster(K* kernel, int threads, size_t smem) {
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(16, 1, 1); cfg.blockDim = dim3((unsigned)threads, 1, 1);
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr; cfg.numAttrs = 1;
+        int clusters = 0;
+        if (cudaOccupancyMaxActiveClusters(&clusters, kernel, &cfg) == cudaSuccess && clusters >= 1) return 16;
+    }
+    (void)cudaGetLastError();
+    return 8;
+}
 
 int ensure_attributes() {
     static std::mutex mu;
@@ -186,23 +207,17 @@ int ensure_attributes() {
         e = cudaFuncSetAttribute(factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
-    // clusters of 16 CTAs are beyond the portable size: allowed per kernel, and used only where the
-    // device says that it can place one
-    g_factor_cluster_max[dev] = 8;
-    if (e == cudaSuccess &&
-        cudaFuncSetAttribute(factor_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess) {
-        cudaLaunchConfig_t cfg{};
-        cfg.gridDim = dim3(16, 1, 1); cfg.blockDim = dim3(CT_THREADS, 1, 1);
-        cfg.dynamicSmemBytes = CT_SMEM_BYTES;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 16; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, factor_kernel<true>, &cfg) == cudaSuccess && clusters >= 1)
-            g_factor_cluster_max[dev] = 16;
-        else
-            (void)cudaGetLastError();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(qr_small_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(qr_small_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(qr_small_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
+    if (e == cudaSuccess) {
+        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<true>, CT_THREADS, CT_SMEM_BYTES);
+        g_qr_cluster_max[dev] = (signed char)std::min({largest_cluster(qr_small_kernel<16>, QS_THREADS, QS_SMEM_LIMIT),
+                                                       largest_cluster(qr_small_kernel<32>, QS_THREADS, QS_SMEM_LIMIT),
+                                                       largest_cluster(qr_small_kernel<64>, QS_THREADS, QS_SMEM_LIMIT)});
     }
     if (e == cudaSuccess) e = tensor_engine_set_attributes();
     if (e != cudaSuccess) {
@@ -214,10 +229,10 @@ int ensure_attributes() {
     return 0;
 }
 
-int factor_cluster_max() {
+int cluster_max(const signed char (&table)[kMaxDevices]) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 8;
-    return g_factor_cluster_max[dev] == 16 ? 16 : 8;
+    return table[dev] == 16 ? 16 : 8;
 }
 
 // ---- internal streams of the grouped step ---------------------------------------------------
@@ -306,7 +321,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 // launch batches keep the rest of the device busy on their own streams.)
                 int csize = 1;
                 const int room = 2 * sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
-                while (csize < factor_cluster_max() && csize < tiles &&
+                while (csize < cluster_max(g_factor_cluster_max) && csize < tiles &&
                        std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
                 launch(csize == 1 ? factor_kernel<false> : factor_kernel<true>, dim3((unsigned)(merged->count * csize)), CT_THREADS,
                        CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
@@ -331,12 +346,57 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
     }
 }
 
+// Whether the factor with `rows` rows is orthonormalised by the one-kernel QR (ranks up to 64).
+bool small_qr(const orthdion_plan* p, int64_t rows) {
+    return p->engine == ORTHDION_ENGINE_TENSOR && qs_fits(rows, p->r, cluster_max(g_qr_cluster_max));
+}
+
+// QR of one class's left (which = 0) or right factor in one kernel, or the column normalisation of the right
+// one; `splits` partial results in the depth-split scratch, or the fp32 slot.
+void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaStream_t st) {
+    const orthdion_plan* p = c.p;
+    const TensorScratch& ts = c.sc.ts;
+    const bool fp16 = fused_fp16(p);
+    QrSmallArgs a{};
+    a.rows = (int32_t)(which ? p->n : p->m); a.r = p->r; a.which = which;
+    const Sel slot = sel(which ? W_R : W_P);
+    a.src = splits > 1 ? sel(W_SCRATCH, c.sc.gram_part) : slot;
+    a.splits = splits; a.split_stride = (int64_t)a.rows * p->r;
+    const int cmax = cluster_max(g_qr_cluster_max), parts = qs_parts(a.rows, p->r, cmax);
+    a.csize = qs_ctas(a.rows, p->r, cmax, std::max(call_matrices, c.b->count), 2 * sm_count());
+    a.parts_per_cta = parts / a.csize;
+    a.rows_per_part = qs_rows_per_part(a.rows, parts);
+    a.colnorm = which && p->mode == ORTHDION_MODE_COLNORM;
+    a.shift_rel = kShiftRel; a.cond_limit = kCondLimit;      // fp32 arithmetic
+    a.dst = sel(which ? W_Q : W_P);
+    if (which) {
+        // the fused pass reads R and Q (the diagnostics Q's bf16 terms)
+        a.img = ts.q; a.img_planes = (fp16 ? 4 : 3) | (p->diag ? 3 : 0);
+        a.copy_r = splits > 1; a.r_dst = slot; a.r_img = ts.r; a.r_planes = fp16 ? 4 : 3; a.rscale_off = ts.rscale;
+    } else {
+        a.img = ts.p; a.img_planes = fp16 ? 7 : 3;
+    }
+    const size_t smem = (size_t)qs_smem((int64_t)a.rows_per_part * a.parts_per_cta, p->r);
+    const int width = qs_width(p->r);
+    launch(width == 16 ? qr_small_kernel<16> : (width == 32 ? qr_small_kernel<32> : qr_small_kernel<64>),
+           dim3((unsigned)(c.b->count * a.csize)), QS_THREADS, smem, a.csize, prof::S_QR, st, *c.b, a);
+}
+
 // ---- tall-skinny QR of every class in `which_cls` (CholeskyQR2; third pass when flagged) --------
 // which = 0: P = orth(Y) (Alg. 1, left-factor step), which = 1: Q = orth(R) (Alg. 1, normalisation step).
-// Tensor engine: the input is an image (w0 holds Y, image r holds R); SIMT engine: fp32 slots.
-void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, int which, Batch* merged,
-              int call_matrices, cudaStream_t st) {
+// Tensor engine: the input is an image (w0 holds Y, image r holds R), or what small_qr_stage reads; SIMT
+// engine: fp32 slots.  summed: the fp32 slot holds the input even where the product is split by depth.
+void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int which, Batch* merged,
+              int call_matrices, cudaStream_t st, bool summed = false) {
     const int shift_bit = which ? ST_SHIFT_R : ST_SHIFT_L;
+    std::vector<int> which_cls;
+    for (int ci : wanted) {
+        ClassRun& c = cls[ci];
+        const int64_t rows = which ? c.p->n : c.p->m, depth = which ? c.p->m : c.p->n;
+        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed ? 1 : buffer_ksplit(c.p->r, rows, depth, c.b->count), call_matrices, st);
+        else which_cls.push_back(ci);
+    }
+    if (which_cls.empty()) return;
     for (int pass = 1; pass <= 3; ++pass) {
         const int only_shift = pass == 3;
         for (int ci : which_cls) {
@@ -435,12 +495,13 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         if (cls[i].p->mode == ORTHDION_MODE_ORTH) orth.push_back((int)i);
     }
     for (ClassRun& c : cls)
-        launch(init_status_kernel, dim3((unsigned)((c.b->count + 255) / 256)), 256, 0, 1, prof::S_MISC, st, *c.b);
+        if (!c.tensor()) launch(init_status_kernel, dim3((unsigned)((c.b->count + 255) / 256)), 256, 0, 1, prof::S_MISC, st, *c.b);
     // Alg. 1, buffer and left-factor steps:  Y = (M + G) Q_prev
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
-        if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st);
+        if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
+                                  small_qr(p, p->m) ? OUT_F32 : OUT_IMAGE);
         else launch_simt(*c.b, p->m, p->r, p->n, RdBuffer{p->n, gb, 0}, RdPlain{sQ, 1, p->r},
                          SimtOut{sP, sP, 0, 0, p->r, 0, 0}, prof::S_K1, st);
     }
@@ -449,7 +510,8 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
-        if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st);
+        if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
+                                  small_qr(p, p->n) ? OUT_F32 : OUT_IMAGE);
         else launch_simt(*c.b, p->n, p->r, p->m, RdBuffer{p->n, gb, 1}, RdPlain{sP, 1, p->r},
                          SimtOut{sR, sR, 0, 0, p->r, 0, 0}, prof::S_K3, st);
     }
@@ -458,6 +520,10 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         if (p->mode == ORTHDION_MODE_ORTH) continue;
+        if (small_qr(p, p->n)) {
+            small_qr_stage(c, 1, buffer_ksplit(p->r, p->n, p->m, c.b->count), call_matrices, st);
+            continue;
+        }
         launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b, p->n,
                p->r, c.tensor() ? c.sc.ts.cnorm : (int64_t)-1, 0);
         if (c.tensor()) launch_pack(*c.b, sQ, p->n, p->r, c.sc.ts.q, st);
@@ -469,7 +535,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const float cc = 1.f - p->eta * p->wd, dd = p->eta * p->scale;
         if (c.tensor()) {
             const int fp16 = fused_fp16(p) ? 1 : 0;
-            if (fp16) launch_pack_half(*c.b, p->n, p->r, c.sc.ts, st);
+            if (fp16 && !small_qr(p, p->n)) launch_pack_half(*c.b, p->n, p->r, c.sc.ts, st);
             tensor_k5(p->m, p->n, p->r, gb, xb, p->passes[2], p->passes[3], fp16, p->ef_a, p->ef_b, cc, dd, *c.b,
                       c.sc.ts, st);
         } else {
@@ -796,15 +862,16 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     engine_error() = 0;
     overlap_launches() = true;
     if (phase == 0) {
-        launch(init_status_kernel, dim3(1), 256, 0, 1, prof::S_MISC, st, sr->batch);
-        tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, true);
+        tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_SUM);
     } else if (phase == 1) {
         // the summed Y sits in the P slot: image and column squares, then the usual left QR
-        launch_pack(sr->batch, sel(W_P), p->m, r, img_view(ts.w0, p->m), st);
-        launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((p->m + 127) / 128)), (unsigned)((r + 255) / 256)), 256, 0, 1, prof::S_MISC, st,
-               sr->batch, sel(W_P), p->m, r, ts.colsq);
-        qr_stage(cls, only, 0, merged, 1, st);
-        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st);
+        if (!small_qr(p, p->m)) {
+            launch_pack(sr->batch, sel(W_P), p->m, r, img_view(ts.w0, p->m), st);
+            launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((p->m + 127) / 128)), (unsigned)((r + 255) / 256)), 256, 0, 1, prof::S_MISC,
+                   st, sr->batch, sel(W_P), p->m, r, ts.colsq);
+        }
+        qr_stage(cls, only, 0, merged, 1, st, true);
+        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_IMAGE);
         if (orth) {
             shard_gram(*sr, ts.r, p->n, st);
         } else {

@@ -25,6 +25,7 @@
 #include "common.cuh"
 #include "factor_tc.cuh"
 #include "launch.cuh"
+#include "qr_small.cuh"
 #include "simt_kernels.cuh"
 
 namespace od {
@@ -87,6 +88,8 @@ struct GemmArgs {
     int32_t ksplit, kb_per_chunk;            // depth split: a tile is computed as `ksplit` partial products over
                                              // kb_per_chunk depth blocks each, stored split_stride floats apart
     int64_t split_stride;
+    int32_t acc_chunks, pad2;                // the same chunks within one tile: accumulators side by side in tensor memory,
+                                             // added up in chunk order by the epilogue (products with B)
     int64_t rscale_off;                      // fp16 fused pass: scratch offset of 1 / (scale of R's plane)
     int64_t ld;                              // leading dimension of M, G, X
     ImgRef a, n1, n2;
@@ -297,13 +300,18 @@ struct PackArgs {
     Sel src;
     int32_t rows, cols;
     ImgRef dst;
+    int32_t init, pad;      // first kernel of a step: clears the status word instead of reading it
 };
 
 __global__ void __launch_bounds__(256)
 pack_kernel(const __grid_constant__ Batch batch, PackArgs a) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
-    if (*w.status & ST_FAILED) return;
+    if (a.init) {
+        if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *w.status = 0;
+    } else if (*w.status & ST_FAILED) {
+        return;
+    }
     const float* S = pick(w, a.src);
     const int panel = blockIdx.x, rb = blockIdx.y;
     unsigned char* out0 = reinterpret_cast<unsigned char*>(w.scratch) + img_row_offset(a.dst, 0, panel, (int64_t)rb * 128);
@@ -666,6 +674,13 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
             for (int kb = c.kb_begin; kb < c.kb_end && ok; ++kb) {
                 if (!mbar_wait(a_full0 + 8 * as, aph, abort_flag)) { ok = false; break; }
                 const uint64_t a_kb = a_hi + (a_ring16 + as * a_slot16);
+                uint32_t dkb = dacc;
+                int kb0 = c.kb_begin;                    // first depth block of the chunk that kb belongs to
+                if (A_BUF && g.acc_chunks > 1) {
+                    const int v = kb / g.kb_per_chunk;
+                    kb0 = v * g.kb_per_chunk;
+                    dkb += (uint32_t)(v * g.BN);
+                }
                 if (NMODE == N_IMG_MN) {
                     const int pieces = mn_pieces(g, kb);
                     const int per_piece = g.ks / 16;
@@ -678,14 +693,14 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                             for (int j = 0; j < nsl; ++j) {
                                 const uint64_t a0 = a_kb + (uint32_t)(sub * per_piece + j) * a_slice16;
                                 const uint64_t a1 = a0 + a_term16;
-                                const uint32_t accum = (kb > c.kb_begin || sub > 0 || j > 0) ? 1u : 0u;
+                                const uint32_t accum = (kb > kb0 || sub > 0 || j > 0) ? 1u : 0u;
                                 uint64_t b0 = n_pc + (uint32_t)j * n_slice16;
                                 for (int cc = 0; cc < c.bn; cc += 256) {
                                     const uint32_t idesc = instr_desc((uint32_t)min(256, c.bn - cc), A_MN ? 1u : 0u, 1u, fmt, MROWS);
-                                    umma_any<PAIR>(dacc + cc, a0, b0, idesc, accum);
+                                    umma_any<PAIR>(dkb + cc, a0, b0, idesc, accum);
                                     if (three) {
-                                        umma_any<PAIR>(dacc + cc, a0, b0 + n_term16, idesc, 1u);
-                                        umma_any<PAIR>(dacc + cc, a1, b0, idesc, 1u);
+                                        umma_any<PAIR>(dkb + cc, a0, b0 + n_term16, idesc, 1u);
+                                        umma_any<PAIR>(dkb + cc, a1, b0, idesc, 1u);
                                     }
                                     b0 += n_block16;                        // next 256 columns
                                 }
@@ -812,6 +827,13 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     if (cc < c.bn) {
                         tmem_ld16(taddr + cc, v);
                         tmem_ld_wait();
+                        for (int ch = 1; ch < g.acc_chunks; ++ch) {
+                            uint32_t u[16];
+                            tmem_ld16(taddr + ch * g.BN + cc, u);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(u[i]));
+                        }
                     } else {
 #pragma unroll
                         for (int i = 0; i < 16; ++i) v[i] = 0u;
@@ -846,7 +868,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         // the lane bits 4..1, then add the two lanes that hold the same column
                         float s[16];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) { const float x = __uint_as_float(v[i]); s[i] = x * x; }
+                        for (int i = 0; i < 16; ++i) { const float x = __uint_as_float(v[i]); s[i] = __fmul_rn(x, x); }
 #pragma unroll
                         for (int half = 8, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
                             const bool up = (lane & bit) != 0;
@@ -1557,8 +1579,9 @@ inline void launch_pack_half(const Batch& b, int64_t rows, int64_t cols, const T
     launch(tc::pack_half_kernel, grid, 256, 0, 1, prof::S_PACK, st, b, a);
 }
 
-inline void launch_pack(const Batch& b, Sel src, int64_t rows, int64_t cols, ImgRef dst, cudaStream_t st) {
+inline void launch_pack(const Batch& b, Sel src, int64_t rows, int64_t cols, ImgRef dst, cudaStream_t st, bool init = false) {
     tc::PackArgs a{};
+    a.init = init ? 1 : 0;
     a.src = src; a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.dst = dst;
     dim3 grid((unsigned)dst.panels, (unsigned)(dst.rows_pad / 128), (unsigned)b.count);
     launch(tc::pack_kernel, grid, 256, 0, 1, prof::S_PACK, st, b, a);
@@ -1582,7 +1605,8 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     g.n_tiles = (g.Ncols + g.BN - 1) / g.BN;
     g.k_blocks = (g.Kdim + tc::BK - 1) / tc::BK;
     if (g.ksplit < 1) g.ksplit = 1;
-    if (g.ksplit > 1) g.kb_per_chunk = (g.k_blocks + g.ksplit - 1) / g.ksplit;
+    if (g.acc_chunks < 1) g.acc_chunks = 1;
+    if (g.ksplit * g.acc_chunks > 1) g.kb_per_chunk = (g.k_blocks + g.ksplit * g.acc_chunks - 1) / (g.ksplit * g.acc_chunks);
     g.total_tiles = b.count * g.m_tiles * g.n_tiles * g.ksplit;
     const int n1_terms = g.passes == 3 ? 2 : 1, n2_terms = g.passes2 == 3 ? 2 : 1;
     const int bn64 = (g.BN + 63) / 64 * 64;
@@ -1611,7 +1635,7 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
         g.n_piece_bytes = (n1_terms + (EPI == tc::EPI_K5 ? n2_terms : 0)) * tc::A_TERM_BYTES;
         if (pair) g.n_piece_bytes = tc::A_TERM_BYTES;    // the R piece (leader) or the Q piece (peer)
     }
-    const int accw = (EPI == tc::EPI_K5) ? 2 * g.BN : g.BN;
+    const int accw = (EPI == tc::EPI_K5) ? 2 * g.BN : g.acc_chunks * g.BN;
     g.acc_bufs = (2 * accw <= 512) ? 2 : 1;
     int cols = 32;
     while (cols < g.acc_bufs * accw) cols *= 2;
@@ -1646,76 +1670,156 @@ inline tc::Dest dest_none() {
 }
 
 // Depth split of the two products with the buffer.  With one matrix (or a few) in a call and a
-// small rank, the output has too few 256-row tile pairs for the device (16 for a 4096-wide
-// factor) and every one of them runs over the whole depth: the depth is cut into chunks that run
-// as separate tiles and leave fp32 partial results, which are then added in a fixed order, packed
-// into the operand image and given their column squares by small kernels.  Like the split of the
-// Gram product, the chunk count depends on the plan only (rank, rows of the result, depth), so a
-// matrix gets the same bits alone and in any group; ranks above 256 never split.
-inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth) {
+// small rank, the output has too few row tiles for the device (16 pairs for a 4096-wide factor)
+// and every one of them runs over the whole depth.  The depth is therefore cut into chunks whose
+// results are added in a fixed order.  Their number depends on the plan only (rank, rows of the result,
+// depth), so that a matrix gets the same bits alone and in any group; ranks above 256 have one.  Where
+// the row tiles of a launch leave the device idle the chunks run as tiles of their own and leave
+// fp32 partial results in memory; where they do not, one tile runs through all chunks with an
+// accumulator each, side by side in tensor memory (at most 512 columns: ranks up to 128), and the epilogue
+// adds them up.
+inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     if (r > 256) return 1;
     const int tiles = (int)((out_rows + 255) / 256);
     const int kb = (int)((depth + tc::BK - 1) / tc::BK);
-    if (tiles >= 37 || kb < 32) return 1;
-    const int want = std::min({8, 74 / tiles, kb / 8});
+    if (tiles >= 37) return 1;
+    int want;
+    if (r <= 128) {
+        want = std::min({r <= 64 ? 8 : 4, 74 / tiles, kb / 4});
+    } else {
+        if (kb < 32) return 1;
+        want = std::min({8, 74 / tiles, kb / 8});
+    }
     if (want < 2) return 1;
     const int per = (kb + want - 1) / want;
     return (kb + per - 1) / per;             // every chunk non-empty
+}
+// Partial results in memory of a launch of `count` matrices: the chunks, or 1 where they stay in tensor memory.
+// The line is where the unsplit row tiles fill half of the device.  Measured (before: always in memory, added
+// up, packed and squared by three kernels): 154 matrices of a 1.1B model at r = 128 9.7 -> 8.6 ms a step; one
+// 4096 x 4096 matrix at r = 256, three kernels in one, 0.633 -> 0.609 ms.
+inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int count) {
+    const int chunks = buffer_chunks(r, out_rows, depth);
+    if (r > 128) return chunks;
+    return (int64_t)count * ((out_rows + tc::BM - 1) / tc::BM) * 2 <= sm_count() ? chunks : 1;
 }
 
 __global__ void gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit,
                                    int only_shift_bit);
 
-// after a depth-split product: dst (rows x r fp32) <- sum of the partials, then its image and its
-// column squares per 32-row block
+// After a product whose chunks ran as tiles of their own: dst (rows x r fp32) <- sum of the partial results
+// in chunk order, its operand image and its column squares per 32-row block (added as the epilogue of
+// the unsplit form adds them).  One CTA per (64 columns, 32 rows): 256 threads, eight columns each.
+struct FinishArgs {
+    Sel dst, part;
+    int64_t rows;
+    int32_t r, ksplit;
+    ImgRef img;
+    int64_t colsq_off;
+};
+__global__ void __launch_bounds__(256)
+finish_split_kernel(const __grid_constant__ Batch batch, FinishArgs a) {
+    grid_dependency();
+    const MatWork& w = batch.w[blockIdx.z];
+    if (*w.status & ST_FAILED) return;
+    __shared__ float sq[32][65];
+    const int rho = threadIdx.x / 8, c = threadIdx.x % 8;
+    const int64_t row = (int64_t)blockIdx.y * 32 + rho;
+    const int panel = blockIdx.x, col = panel * 64 + c * 8;
+    float v[8] = {};
+    if (row < a.rows && col < a.r) {
+        const float* P = pick(w, a.part) + row * a.r + col;
+        const int64_t stride = a.rows * a.r;
+        tc::load8(P, 0, 0, v);
+#pragma unroll 4
+        for (int k = 1; k < a.ksplit; ++k) {
+            float u[8];
+            tc::load8(P + k * stride, 0, 0, u);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] += u[i];
+        }
+        float4* D = reinterpret_cast<float4*>(pick(w, a.dst) + row * a.r + col);
+        D[0] = make_float4(v[0], v[1], v[2], v[3]);
+        D[1] = make_float4(v[4], v[5], v[6], v[7]);
+    }
+    uint4 t0, t1;
+    split8(v, t0, t1);
+    unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
+    const int o = img_chunk_offset(rho, c);
+    *reinterpret_cast<uint4*>(scr + img_row_offset(a.img, 0, panel, row) + o) = t0;
+    *reinterpret_cast<uint4*>(scr + img_row_offset(a.img, 1, panel, row) + o) = t1;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) sq[rho][c * 8 + i] = __fmul_rn(v[i], v[i]);
+    __syncthreads();
+    if (threadIdx.x < 64 && panel * 64 + threadIdx.x < a.r) {
+        float s[32];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) s[i] = sq[i][threadIdx.x];
+#pragma unroll
+        for (int h = 16; h >= 1; h >>= 1)
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (i < h) s[i] += s[i + h];
+        reinterpret_cast<float*>(w.scratch + a.colsq_off)[(int64_t)blockIdx.y * a.r + panel * 64 + threadIdx.x] = s[0];
+    }
+}
 inline void finish_split_product(const Batch& b, Sel dst, Sel part, int64_t rows, int r, int ksplit, ImgRef img,
                                  int64_t colsq_off, int stage, cudaStream_t st) {
-    const int64_t total4 = rows * r / 4;
-    launch(gram_reduce_kernel, dim3((unsigned)((total4 + 255) / 256), 1, (unsigned)b.count), 256, 0, 1, stage, st, b, dst, part,
-           total4, ksplit, 0);
-    launch_pack(b, dst, rows, r, img, st);
-    launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((rows + 127) / 128)), (unsigned)((r + 255) / 256), (unsigned)b.count), 256, 0, 1,
-           stage, st, b, dst, rows, r, colsq_off);
+    FinishArgs a{};
+    a.dst = dst; a.part = part; a.rows = rows; a.r = r; a.ksplit = ksplit; a.img = img; a.colsq_off = colsq_off;
+    launch(finish_split_kernel, dim3((unsigned)img.panels, (unsigned)(img.rows_pad / 32), (unsigned)b.count), 256, 0, 1, stage, st, b, a);
 }
 
+// Where a product with B goes.
+enum ProductOut : int {
+    OUT_IMAGE = 0,     // operand image and column squares (and the fp32 R slot)
+    OUT_F32 = 1,       // fp32 slot, or partial results of a depth split, for the small-rank QR kernel
+    OUT_SUM = 2        // fp32 slot only: one shard of the columns, to be summed over the shards
+};
 // Y = (M + G) Q_prev  -> image w0 (+ column squares)              (Alg. 1, buffer and left-factor steps)
-// partial: the columns at hand are one shard of the matrix; the product goes to the fp32 P slot
-// only, to be summed over the shards before it is orthonormalised.
-// part: scratch for the partial results of a depth split (buffer_ksplit(r, m, n) > 1).
+// First kernel of a step: its packing of Q_prev also clears the status words.
+// part: scratch for the partial results of a depth split.
 inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const Batch& b, const TensorScratch& ts,
-                      Sel part, cudaStream_t st, bool partial = false) {
-    launch_pack(b, Sel{W_Q, 0, 0}, n, r, ts.qprev, st);
-    const int ksplit = partial ? 1 : buffer_ksplit(r, m, n);
+                      Sel part, cudaStream_t st, ProductOut kind) {
+    launch_pack(b, Sel{W_Q, 0, 0}, n, r, ts.qprev, st, true);
+    const int ksplit = kind == OUT_SUM ? 1 : buffer_ksplit(r, m, n, b.count);
     tc::GemmArgs g{};
+    if (kind != OUT_SUM && ksplit == 1) g.acc_chunks = buffer_chunks(r, m, n);
     g.Mrows = (int32_t)m; g.Ncols = r; g.Kdim = (int32_t)n; g.BN = std::min(r, 512);
     g.passes = passes; g.passes2 = 1; g.ld = n; g.n1 = ts.qprev; g.a = no_img(); g.n2 = no_img();
     g.colsq_off = ts.colsq;
     g.out.normal = dest_none();
     if (ksplit > 1) { g.out.normal.f32 = part; g.out.normal.has_f32 = 1; g.ksplit = ksplit; g.split_stride = m * r; }
-    else if (partial) { g.out.normal.f32 = Sel{W_P, 0, 0}; g.out.normal.has_f32 = 1; }
+    else if (kind != OUT_IMAGE) { g.out.normal.f32 = Sel{W_P, 0, 0}; g.out.normal.has_f32 = 1; }
     else { g.out.normal.img = img_view(ts.w0, m); g.out.normal.colsq = 1; }
     g.out.shifted = g.out.normal; g.out.ld = r;
     if (g_bf16) launch_gemm<tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 1>(b, g, prof::S_K1, st);
     else launch_gemm<tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_K1, st);
     // (the sum goes through the fp32 P slot, which holds nothing yet at this point of a step)
-    if (ksplit > 1) finish_split_product(b, Sel{W_P, 0, 0}, part, m, r, ksplit, img_view(ts.w0, m), ts.colsq, prof::S_K1, st);
+    if (ksplit > 1 && kind == OUT_IMAGE)
+        finish_split_product(b, Sel{W_P, 0, 0}, part, m, r, ksplit, img_view(ts.w0, m), ts.colsq, prof::S_K1, st);
 }
 
 // R = (M + G)^T P  -> fp32 R slot, image r (+ column squares)     (Alg. 1, right-factor step)
 inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const Batch& b, const TensorScratch& ts,
-                      Sel part, cudaStream_t st) {
-    const int ksplit = buffer_ksplit(r, n, m);
+                      Sel part, cudaStream_t st, ProductOut kind) {
+    const int ksplit = buffer_ksplit(r, n, m, b.count);
     tc::GemmArgs g{};
+    if (ksplit == 1) g.acc_chunks = buffer_chunks(r, n, m);
     g.Mrows = (int32_t)n; g.Ncols = r; g.Kdim = (int32_t)m; g.BN = std::min(r, 512);
     g.passes = passes; g.passes2 = 1; g.ld = n; g.n1 = ts.p; g.a = no_img(); g.n2 = no_img();
     g.colsq_off = ts.colsq;
     g.out.normal = dest_none(); g.out.normal.has_f32 = 1;
     if (ksplit > 1) { g.out.normal.f32 = part; g.ksplit = ksplit; g.split_stride = n * r; }
-    else { g.out.normal.f32 = Sel{W_R, 0, 0}; g.out.normal.img = ts.r; g.out.normal.colsq = 1; }
+    else {
+        g.out.normal.f32 = Sel{W_R, 0, 0};
+        if (kind == OUT_IMAGE) { g.out.normal.img = ts.r; g.out.normal.colsq = 1; }
+    }
     g.out.shifted = g.out.normal; g.out.ld = r;
     if (g_bf16) launch_gemm<tc::A_BUF_COL, tc::N_IMG_MN, tc::EPI_STORE, 1>(b, g, prof::S_K3, st);
     else launch_gemm<tc::A_BUF_COL, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_K3, st);
-    if (ksplit > 1) finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, ts.colsq, prof::S_K3, st);
+    if (ksplit > 1 && kind == OUT_IMAGE)
+        finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, ts.colsq, prof::S_K3, st);
 }
 
 // Depth split of the Gram product.  At small ranks the whole Gram matrix is one output tile whose

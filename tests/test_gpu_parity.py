@@ -146,6 +146,18 @@ def test_factor_kernel_block_edges(shape):
     one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR)
 
 
+# the one-kernel QR (ranks up to 64): one row past one, two and sixteen parts of a matrix, last parts without
+# rows, the tallest factors of its ranges and the first beyond them; r = 48 and 96 past a depth chunk of the products
+@pytest.mark.parametrize("shape", [(257, 264, 16), (129, 136, 32), (65, 72, 64), (300, 328, 48), (640, 200, 64), (648, 576, 64),
+                                   (2049, 264, 32), (4097, 136, 16), (520, 776, 96)])
+@pytest.mark.parametrize("mode", MODES)
+@pytest.mark.parametrize("dt", [(F32, F32), (BF16, BF16)])
+def test_small_rank_qr_edges(shape, mode, dt):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, dt[0], dt[1], seed=m + n + r)
+    one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_TENSOR)
+
+
 @pytest.mark.parametrize("shape", [(384, 640, 64), (1000, 264, 128), (136, 2056, 32), (640, 384, 272)])
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("m_scale", [0.3, 3e-4, 300.0])
@@ -342,6 +354,14 @@ def test_factor_kernel_forms_agree_bit_for_bit(shape, count):
         assert torch.equal(P, P1) and torch.equal(R, R1)
         gm.close()
     od.orthdion_destroy(h)
+
+
+# the one-kernel QR with sixteen, four and one parts of a factor per CTA, and the products' depth chunks as
+# tiles of their own (the matrix alone) and in one tile (the call of many), with the image and the fp32 result
+@pytest.mark.parametrize("shape,count", [((1152, 136, 32), 150), ((1152, 136, 32), 70), ((2000, 144, 16), 150), ((520, 264, 48), 150),
+                                         ((768, 1024, 128), 150), ((1100, 648, 80), 40)])
+def test_small_rank_qr_and_depth_chunks_agree_bit_for_bit(shape, count):
+    test_factor_kernel_forms_agree_bit_for_bit(shape, count)
 
 
 @pytest.mark.parametrize("engine", ENGINES, ids=ENGINE_IDS)
