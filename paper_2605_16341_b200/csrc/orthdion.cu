@@ -71,7 +71,8 @@ bool fused_fp16(const orthdion_plan* p) {
     return p->engine == ORTHDION_ENGINE_TENSOR && p->passes[2] == 1 && p->passes[3] == 1;
 }
 
-Scratch scratch_layout(const orthdion_plan* p) {
+// matrices: of the whole call.
+Scratch scratch_layout(const orthdion_plan* p, int matrices) {
     Scratch s{};
     const size_t rr = align_up((size_t)p->r * p->r * 4, 256);
     size_t off = 0;
@@ -82,8 +83,8 @@ Scratch scratch_layout(const orthdion_plan* p) {
     if (p->engine == ORTHDION_ENGINE_TENSOR) {
         off = tensor_scratch_layout(p->m, p->n, p->r, fused_fp16(p), off, &s.ts);
         // (after everything whose offset must depend on r only)
-        const int parts = std::max(gram_ksplit(p->r, p->m), gram_ksplit(p->r, p->n));
-        const int s1 = buffer_chunks(p->r, p->m, p->n), s3 = buffer_chunks(p->r, p->n, p->m);
+        const int parts = std::max(gram_ksplit(p->r, p->m, matrices), gram_ksplit(p->r, p->n, matrices));
+        const int s1 = buffer_ksplit(p->r, p->m, p->n, matrices), s3 = buffer_ksplit(p->r, p->n, p->m, matrices);
         size_t part_bytes = parts > 1 ? (size_t)parts * rr : 0;
         if (s1 > 1) part_bytes = std::max(part_bytes, align_up((size_t)s1 * p->m * p->r * 4, 256));
         if (s3 > 1) part_bytes = std::max(part_bytes, align_up((size_t)s3 * p->n * p->r * 4, 256));
@@ -116,7 +117,7 @@ Batching make_batches(const orthdion_t* hs, int32_t count) {
         std::vector<int> cls;
         for (int j = i; j < count; ++j)
             if (!done[j] && same_class(hs[i], hs[j])) { cls.push_back(j); done[j] = 1; }
-        const size_t per = scratch_layout(hs[i]).bytes;
+        const size_t per = scratch_layout(hs[i], count).bytes;
         size_t cap = std::max<size_t>(1, kScratchBudget / std::max<size_t>(per, 1));
         cap = std::min<size_t>(cap, MAXB);
         const size_t nb = (cls.size() + cap - 1) / cap;
@@ -363,7 +364,7 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
     a.src = splits > 1 ? sel(W_SCRATCH, c.sc.gram_part) : slot;
     a.splits = splits; a.split_stride = (int64_t)a.rows * p->r;
     const int cmax = cluster_max(g_qr_cluster_max), parts = qs_parts(a.rows, p->r, cmax);
-    a.csize = qs_ctas(a.rows, p->r, cmax, std::max(call_matrices, c.b->count), 2 * sm_count());
+    a.csize = qs_ctas(a.rows, p->r, cmax, call_matrices, 2 * sm_count());
     a.parts_per_cta = parts / a.csize;
     a.rows_per_part = qs_rows_per_part(a.rows, parts);
     a.colnorm = which && p->mode == ORTHDION_MODE_COLNORM;
@@ -393,7 +394,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
     for (int ci : wanted) {
         ClassRun& c = cls[ci];
         const int64_t rows = which ? c.p->n : c.p->m, depth = which ? c.p->m : c.p->n;
-        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed ? 1 : buffer_ksplit(c.p->r, rows, depth, c.b->count), call_matrices, st);
+        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed ? 1 : buffer_ksplit(c.p->r, rows, depth, call_matrices), call_matrices, st);
         else which_cls.push_back(ci);
     }
     if (which_cls.empty()) return;
@@ -409,7 +410,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
                 const ImgRef in = which ? ts.r : img_view(ts.w0, rows);
                 const ImgRef src = pass == 1 ? in : (pass == 2 ? img_view(ts.w1, rows) : img_view(ts.w0, rows));
                 tensor_gram(r, c.p->passes[1], *c.b, src, rows, gram, sel(W_SCRATCH, c.sc.gram_part),
-                            only_shift ? shift_bit : 0, st);
+                            only_shift ? shift_bit : 0, call_matrices, st);
             } else {
                 const Sel in = which ? sel(W_R) : sel(W_P);
                 const Sel src = pass == 1 ? in : (pass == 2 ? sel(W_SCRATCH, c.sc.tmpA) : sel(W_SCRATCH, c.sc.tmpB));
@@ -455,7 +456,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
 
 // Diagnostics of one class, after its step: Q^T Q from the engine's Gram product, column
 // statistics of R, optionally the norms of M' and G, then one CTA per matrix for the rest.
-void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
+void diag_stage(ClassRun& c, DiagBase db, int call_matrices, cudaStream_t st) {
     const orthdion_plan* p = c.p;
     const Batch& b = *c.b;
     const int r = p->r;
@@ -463,7 +464,7 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
     const int64_t stats_off = c.sc.linv;          // 3 r floats of the (now free) inverse slot
     launch(diag_init_kernel, dim3((unsigned)((b.count * DIAG_STRIDE + 255) / 256)), 256, 0, 1, prof::S_DIAG, st, b, db);
     if (c.tensor()) {
-        tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), 0, st);
+        tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), 0, call_matrices, st);
     } else {
         const Sel sQ = sel(W_Q);
         launch_simt(b, r, r, p->n, RdPlain{sQ, 1, r}, RdPlain{sQ, 1, r}, SimtOut{gram, gram, 0, 1, r, 0, 0},
@@ -500,7 +501,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
-        if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
+        if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), call_matrices, st,
                                   small_qr(p, p->m) ? OUT_F32 : OUT_IMAGE);
         else launch_simt(*c.b, p->m, p->r, p->n, RdBuffer{p->n, gb, 0}, RdPlain{sQ, 1, p->r},
                          SimtOut{sP, sP, 0, 0, p->r, 0, 0}, prof::S_K1, st);
@@ -510,7 +511,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
-        if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
+        if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), call_matrices, st,
                                   small_qr(p, p->n) ? OUT_F32 : OUT_IMAGE);
         else launch_simt(*c.b, p->n, p->r, p->m, RdBuffer{p->n, gb, 1}, RdPlain{sP, 1, p->r},
                          SimtOut{sR, sR, 0, 0, p->r, 0, 0}, prof::S_K3, st);
@@ -521,7 +522,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const orthdion_plan* p = c.p;
         if (p->mode == ORTHDION_MODE_ORTH) continue;
         if (small_qr(p, p->n)) {
-            small_qr_stage(c, 1, buffer_ksplit(p->r, p->n, p->m, c.b->count), call_matrices, st);
+            small_qr_stage(c, 1, buffer_ksplit(p->r, p->n, p->m, call_matrices), call_matrices, st);
             continue;
         }
         launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b, p->n,
@@ -544,7 +545,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         }
     }
     for (ClassRun& c : cls)
-        if (c.p->diag) diag_stage(c, db, st);
+        if (c.p->diag) diag_stage(c, db, call_matrices, st);
 }
 
 // Default pass counts of the fused feedback/update pass.  One fp16 pass carries P R^T with about
@@ -702,7 +703,7 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
         std::vector<ClassRun> cls;
         for (int bi : grp) {
             const auto& idx = bt.batches[bi];
-            ClassRun c{hs[idx[0]], &pool[bi], scratch_layout(hs[idx[0]])};
+            ClassRun c{hs[idx[0]], &pool[bi], scratch_layout(hs[idx[0]], count)};
             c.b->count = (int32_t)idx.size();
             c.b->pad = 0;
             c.b->scratch_stride = (int64_t)c.sc.bytes;
@@ -810,7 +811,7 @@ int shard_setup(orthdion_t h, void* X, float* M, const void* G, float* Q, void* 
     if (workspace_bytes < sr->lay.total) return ORTHDION_ERR_WORKSPACE;
     if ((e = ensure_attributes())) return e;
     char* ws = reinterpret_cast<char*>(workspace);
-    sr->c = ClassRun{h, &sr->batch, scratch_layout(h)};
+    sr->c = ClassRun{h, &sr->batch, scratch_layout(h, 1)};
     sr->batch.count = 1; sr->batch.pad = 0; sr->batch.scratch_stride = (int64_t)sr->c.sc.bytes;
     MatWork& w = sr->batch.w[0];
     w.X = X; w.M = M; w.G = G; w.Q = Q;
@@ -826,7 +827,7 @@ int shard_setup(orthdion_t h, void* X, float* M, const void* G, float* Q, void* 
 void shard_gram(ShardRun& sr, const ImgRef& src, int64_t rows, cudaStream_t st) {
     const orthdion_plan* p = sr.c.p;
     const Sel gram = sel(W_SCRATCH, sr.c.sc.gram);
-    tensor_gram(p->r, p->passes[1], sr.batch, src, rows, gram, sel(W_SCRATCH, sr.c.sc.gram_part), 0, st);
+    tensor_gram(p->r, p->passes[1], sr.batch, src, rows, gram, sel(W_SCRATCH, sr.c.sc.gram_part), 0, 1, st);
     launch(gram_diag_kernel, dim3((unsigned)((p->r + 255) / 256)), 256, 0, 1, prof::S_MISC, st, sr.batch, gram, p->r, sr.c.sc.ts.colsq,
            (int)(4 * ((rows + 127) / 128)));
 }
@@ -862,7 +863,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     engine_error() = 0;
     overlap_launches() = true;
     if (phase == 0) {
-        tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_SUM);
+        tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), 1, st, OUT_SUM);
     } else if (phase == 1) {
         // the summed Y sits in the P slot: image and column squares, then the usual left QR
         if (!small_qr(p, p->m)) {
@@ -871,7 +872,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
                    st, sr->batch, sel(W_P), p->m, r, ts.colsq);
         }
         qr_stage(cls, only, 0, merged, 1, st, true);
-        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_IMAGE);
+        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), 1, st, OUT_IMAGE);
         if (orth) {
             shard_gram(*sr, ts.r, p->n, st);
         } else {
@@ -915,7 +916,7 @@ int orthdion_shard_reduce_buffer(orthdion_t h, int32_t phase, void* workspace, f
     if (phase < 0 || phase > (orth ? 2 : 1)) return ORTHDION_ERR_INVALID_ARG;
     Batching bt = make_batches(&h, 1);
     Layout lay = make_layout(&h, 1, bt.scratch_bytes);
-    Scratch sc = scratch_layout(h);
+    Scratch sc = scratch_layout(h, 1);
     char* ws = reinterpret_cast<char*>(workspace);
     if (phase == 0) {
         *buffer = reinterpret_cast<float*>(ws + lay.p_off[0]);

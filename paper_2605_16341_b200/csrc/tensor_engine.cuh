@@ -88,7 +88,9 @@ struct GemmArgs {
     int32_t ksplit, kb_per_chunk;            // depth split: a tile is computed as `ksplit` partial products over
                                              // kb_per_chunk depth blocks each, stored split_stride floats apart
     int64_t split_stride;
-    int32_t acc_chunks, pad2;                // the same chunks within one tile: accumulators side by side in tensor memory,
+    int32_t run;                             // Gram product: this many consecutive tiles (the depth chunks of one result
+                                             // tile) go to the same CTA, which adds each to what it has stored
+    int32_t acc_chunks;                      // the same chunks within one tile: accumulators side by side in tensor memory,
                                              // added up in chunk order by the epilogue (products with B)
     int64_t rscale_off;                      // fp16 fused pass: scratch offset of 1 / (scale of R's plane)
     int64_t ld;                              // leading dimension of M, G, X
@@ -471,9 +473,14 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     constexpr int NE = epi_warps(AMODE, EPI);
     // PAIR: launched in clusters of two; rank 0 (the leader) issues every MMA for both CTAs
     const int crank = PAIR ? (int)cluster_ctarank() : 0;
-    const int tile0 = PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x;
+    const int tile0 = (PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * (AMODE == A_IMG_MN ? g.run : 1);
     const int tstride = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     constexpr bool A_BUF = a_is_buf(AMODE);
+    // the next tile of this CTA after tile t
+    auto next = [&](int t) {
+        if constexpr (AMODE == A_IMG_MN) return (t + 1) % g.run ? t + 1 : t + 1 + (tstride - 1) * g.run;
+        else return t + tstride;
+    };
     constexpr bool A_MN = (AMODE == A_IMG_MN || AMODE == A_BUF_COL);
     constexpr bool G_BF16 = (XG & 1) != 0;
     constexpr bool X_BF16 = (XG & 2) != 0;
@@ -562,7 +569,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     if (at >= g.total_tiles) { a_done = true; break; }
                     if (akb < 0) { ac = decode_tile<EPI>(batch, g, at, scache, crank); akb = ac.kb_begin; }
                     if (ac.active && akb < ac.kb_end) break;
-                    at += tstride; akb = -1;
+                    at = next(at); akb = -1;
                 }
             };
             auto n_pieces = [&](int kb) { return NMODE == N_IMG_MN ? mn_pieces(g, kb) : (nc.bn + 127) / 128; };
@@ -570,7 +577,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 while (!n_done) {
                     if (nt_ >= g.total_tiles) { n_done = true; break; }
                     if (nkb < 0) { nc = decode_tile<EPI>(batch, g, nt_, scache, crank); nkb = nc.kb_begin; npc = 0; }
-                    if (!nc.active || nkb >= nc.kb_end) { nt_ += tstride; nkb = -1; npc = 0; continue; }
+                    if (!nc.active || nkb >= nc.kb_end) { nt_ = next(nt_); nkb = -1; npc = 0; continue; }
                     if (npc >= n_pieces(nkb)) { ++nkb; npc = 0; continue; }
                     if (NMODE == N_IMG_K && !k_piece_active(g, nc, nkb, npc)) { ++npc; continue; }
                     break;
@@ -596,7 +603,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     }
                     if (++as == g.a_slots) { as = 0; aph ^= 1; }
                     ++akb;
-                    if (akb >= ac.kb_end) { at += tstride; akb = -1; }
+                    if (akb >= ac.kb_end) { at = next(at); akb = -1; }
                     a_seek();
                     progress = true;
                 }
@@ -662,7 +669,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         constexpr uint32_t MROWS = PAIR ? 256u : 128u;
         // pairs: a 256-column block of the N-side is this CTA's two 64-column groups, both terms
         const uint32_t n_block16 = (PAIR ? (uint32_t)n1_terms * 2u * group_stride : 4u * group_stride) >> 4;
-        for (int t = tile0; t < g.total_tiles && ok && crank == 0; t += tstride) {
+        for (int t = tile0; t < g.total_tiles && ok && crank == 0; t = next(t)) {
             const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
             if (!c.active) continue;
             if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1, abort_flag)) { ok = false; break; }
@@ -792,7 +799,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         const int quarter = warp % 4;                    // tensor-memory lanes 32*quarter .. +31
         if (EPI == EPI_STORE) {
             int scale_b = -1; bool scale_on = false;         // does matrix scale_b want its columns scaled
-            for (int t = tile0; t < g.total_tiles && ok; t += tstride) {
+            for (int t = tile0; t < g.total_tiles && ok; t = next(t)) {
                 const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
                 if (!c.active) continue;
                 const MatWork& w = batch.w[c.b];
@@ -943,17 +950,39 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     }
                     if (C) {
                         // fp32 block: 32 rows x 256 bytes, 16-byte chunks swizzled by (row & 7)
+                        const bool add = AMODE == A_IMG_MN && g.run > 1 && c.chunk > 0;
 #pragma unroll
                         for (int ch = 0; ch < 16; ++ch)
                             *reinterpret_cast<float4*>(stg + lane * 256 + ((ch ^ (lane & 7)) << 4)) =
                                 make_float4(f[4 * ch], f[4 * ch + 1], f[4 * ch + 2], f[4 * ch + 3]);
                         __syncwarp();
+                        if (add) {
+                            // the sum so far, stored by this very thread; all loads first (a load behind a store that
+                            // may alias it would wait for the store)
+                            float4 o[16];
+#pragma unroll
+                            for (int it = 0; it < 16; ++it) {
+                                const int r = it * 2 + lane / 16, ch = lane % 16;
+                                o[it] = make_float4(0.f, 0.f, 0.f, 0.f);
+                                if (gi0 + r < g.Mrows && ch * 4 < valid)
+                                    o[it] = *reinterpret_cast<const float4*>(C + (gi0 + r) * g.out.ld + gj0 + ch * 4);
+                            }
+#pragma unroll
+                            for (int it = 0; it < 16; ++it) {
+                                const int r = it * 2 + lane / 16, ch = lane % 16;
+                                const float4 x = *reinterpret_cast<const float4*>(stg + r * 256 + ((ch ^ (r & 7)) << 4));
+                                if (gi0 + r < g.Mrows && ch * 4 < valid)
+                                    *reinterpret_cast<float4*>(C + (gi0 + r) * g.out.ld + gj0 + ch * 4) =
+                                        make_float4(o[it].x + x.x, o[it].y + x.y, o[it].z + x.z, o[it].w + x.w);
+                            }
+                        } else {
 #pragma unroll
                         for (int it = 0; it < 16; ++it) {
                             const int r = it * 2 + lane / 16, ch = lane % 16;
                             const float4 x = *reinterpret_cast<const float4*>(stg + r * 256 + ((ch ^ (r & 7)) << 4));
                             if (gi0 + r < g.Mrows && ch * 4 < valid)
                                 *reinterpret_cast<float4*>(C + (gi0 + r) * g.out.ld + gj0 + ch * 4) = x;
+                        }
                         }
                         __syncwarp();
                     }
@@ -1605,6 +1634,7 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     g.n_tiles = (g.Ncols + g.BN - 1) / g.BN;
     g.k_blocks = (g.Kdim + tc::BK - 1) / tc::BK;
     if (g.ksplit < 1) g.ksplit = 1;
+    if (g.run < 1) g.run = 1;
     if (g.acc_chunks < 1) g.acc_chunks = 1;
     if (g.ksplit * g.acc_chunks > 1) g.kb_per_chunk = (g.k_blocks + g.ksplit * g.acc_chunks - 1) / (g.ksplit * g.acc_chunks);
     g.total_tiles = b.count * g.m_tiles * g.n_tiles * g.ksplit;
@@ -1654,12 +1684,12 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     if (engine_error()) return;
     if constexpr (pair_capable(NMODE, EPI, XG)) {
         if (pair) {
-            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true>, dim3((unsigned)(2 * std::min(g.total_tiles, sm_count() / 2))),
+            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true>, dim3((unsigned)(2 * std::min(g.total_tiles / g.run, sm_count() / 2))),
                    tc::gemm_threads(AMODE, EPI), smem, 2, stage, st, b, g);
             return;
         }
     }
-    launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false>, dim3((unsigned)std::min(g.total_tiles, sm_count())),
+    launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false>, dim3((unsigned)std::min(g.total_tiles / g.run, sm_count())),
            tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
 }
 
@@ -1668,6 +1698,9 @@ inline tc::Dest dest_none() {
     d.f32 = Sel{W_P, 0, 0}; d.img = no_img(); d.has_f32 = 0; d.colsq = 0;
     return d;
 }
+
+// Multiprocessors that the rules below count on: a constant, so that workspace sizes need no device.
+constexpr int SPLIT_SMS = 148;
 
 // Depth split of the two products with the buffer.  With one matrix (or a few) in a call and a
 // small rank, the output has too few row tiles for the device (16 pairs for a 4096-wide factor)
@@ -1694,14 +1727,14 @@ inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     const int per = (kb + want - 1) / want;
     return (kb + per - 1) / per;             // every chunk non-empty
 }
-// Partial results in memory of a launch of `count` matrices: the chunks, or 1 where they stay in tensor memory.
+// Partial results in memory of a product in a call of `matrices`: the chunks, or 1 where they stay in tensor memory.
 // The line is where the unsplit row tiles fill half of the device.  Measured (before: always in memory, added
 // up, packed and squared by three kernels): 154 matrices of a 1.1B model at r = 128 9.7 -> 8.6 ms a step; one
 // 4096 x 4096 matrix at r = 256, three kernels in one, 0.633 -> 0.609 ms.
-inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int count) {
+inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices) {
     const int chunks = buffer_chunks(r, out_rows, depth);
     if (r > 128) return chunks;
-    return (int64_t)count * ((out_rows + tc::BM - 1) / tc::BM) * 2 <= sm_count() ? chunks : 1;
+    return (int64_t)matrices * ((out_rows + tc::BM - 1) / tc::BM) * 2 <= SPLIT_SMS ? chunks : 1;
 }
 
 __global__ void gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit,
@@ -1778,11 +1811,11 @@ enum ProductOut : int {
 };
 // Y = (M + G) Q_prev  -> image w0 (+ column squares)              (Alg. 1, buffer and left-factor steps)
 // First kernel of a step: its packing of Q_prev also clears the status words.
-// part: scratch for the partial results of a depth split.
+// part: scratch for the partial results of a depth split.  matrices: of the whole call.
 inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const Batch& b, const TensorScratch& ts,
-                      Sel part, cudaStream_t st, ProductOut kind) {
+                      Sel part, int matrices, cudaStream_t st, ProductOut kind) {
     launch_pack(b, Sel{W_Q, 0, 0}, n, r, ts.qprev, st, true);
-    const int ksplit = kind == OUT_SUM ? 1 : buffer_ksplit(r, m, n, b.count);
+    const int ksplit = kind == OUT_SUM ? 1 : buffer_ksplit(r, m, n, matrices);
     tc::GemmArgs g{};
     if (kind != OUT_SUM && ksplit == 1) g.acc_chunks = buffer_chunks(r, m, n);
     g.Mrows = (int32_t)m; g.Ncols = r; g.Kdim = (int32_t)n; g.BN = std::min(r, 512);
@@ -1802,8 +1835,8 @@ inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const
 
 // R = (M + G)^T P  -> fp32 R slot, image r (+ column squares)     (Alg. 1, right-factor step)
 inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const Batch& b, const TensorScratch& ts,
-                      Sel part, cudaStream_t st, ProductOut kind) {
-    const int ksplit = buffer_ksplit(r, n, m, b.count);
+                      Sel part, int matrices, cudaStream_t st, ProductOut kind) {
+    const int ksplit = buffer_ksplit(r, n, m, matrices);
     tc::GemmArgs g{};
     if (ksplit == 1) g.acc_chunks = buffer_chunks(r, n, m);
     g.Mrows = (int32_t)n; g.Ncols = r; g.Kdim = (int32_t)m; g.BN = std::min(r, 512);
@@ -1822,18 +1855,38 @@ inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const
         finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, ts.colsq, prof::S_K3, st);
 }
 
-// Depth split of the Gram product.  At small ranks the whole Gram matrix is one output tile whose
-// main loop runs over all rows of the tall matrix on a single CTA (pair): the depth is cut into
-// chunks that run side by side and leave partial sums, which a small kernel adds up in a fixed
-// order.  The number of chunks depends on the rank and the row count only, never on how many
-// matrices a launch holds, so a matrix gets the same bits alone and in any group.
-inline int gram_ksplit(int r, int64_t rows) {
-    if (r > 256) return 1;
+// Depth split of the Gram product.  The Gram matrix is one output tile at small ranks and ten at r = 1024,
+// each with a main loop over all rows of the tall matrix: the depth is cut into chunks whose results are
+// added in a fixed order.  Their number depends on the rank and the row count only, so a matrix gets the same
+// bits alone and in any group.  The chunks run as tiles of their own and leave partial matrices that a small
+// kernel adds up; above r = 256, in calls with tiles enough for the device, one CTA takes the chunks of a tile
+// one after the other and adds each to the tile it has stored (the two accumulators alternate, so
+// the additions run beside the next chunk's products).
+inline int gram_tiles(int r) {               // tiles that touch the lower triangle
+    const int rows = r % 256 ? 128 : 256, cols = std::min(r, 256);
+    int n = 0;
+    for (int i = 0; i * rows < r; ++i)
+        for (int j = 0; j * cols < r; ++j)
+            if (j * cols <= i * rows + rows - 1) ++n;
+    return n;
+}
+inline int gram_chunks(int r, int64_t rows) {
     const int kb = (int)((rows + tc::BK - 1) / tc::BK);
-    const int want = std::min(16, kb / 8);
+    // At least 8 depth blocks per chunk at r <= 256; 24 above, where the additions cost calls with many matrices
+    // some of their Gram time (1.1B model at r = 512 3.03 -> 3.15 ms of an 18 ms step; with 16 blocks 3.31) and 16
+    // would give single matrices another 0.05 ms.
+    const int want = r <= 256 ? std::min(16, kb / 8) : std::min({16, kb / 24, 80 / gram_tiles(r)});
     if (want < 2) return 1;
     const int per = (kb + want - 1) / want;
     return (kb + per - 1) / per;             // every chunk non-empty
+}
+// Partial matrices in memory of a Gram product in a call of `matrices`.  Above r = 256 the line is where the
+// undivided tiles fill the device (there the partial matrices would be megabytes each).  Measured, the Gram
+// products of a step: one 11008 x 4096 matrix at r = 1024 0.64 -> 0.35 ms, one 4096 x 3584 matrix at r = 512 0.36 -> 0.26.
+inline int gram_ksplit(int r, int64_t rows, int matrices) {
+    if (r <= 256) return gram_chunks(r, rows);
+    const int room = r % 256 ? SPLIT_SMS : SPLIT_SMS / 2;
+    return (int64_t)matrices * gram_tiles(r) <= room ? gram_chunks(r, rows) : 1;
 }
 
 // dst <- sum of the `ksplit` partial results at `part` (4 * total4 floats each, one after the
@@ -1856,10 +1909,10 @@ gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int6
 }
 
 // Gram = src^T src (src: image of a rows x r matrix); only tiles that touch the lower triangle.
-// part: scratch for gram_ksplit(r, rows) partial matrices (used when that is more than one).
+// part: scratch for gram_ksplit(r, rows, matrices) partial matrices (used when that is more than one).
 inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t rows, Sel gram, Sel part,
-                        int only_shift_bit, cudaStream_t st) {
-    const int ksplit = gram_ksplit(r, rows);
+                        int only_shift_bit, int matrices, cudaStream_t st) {
+    const int ksplit = gram_ksplit(r, rows, matrices), chunks = gram_chunks(r, rows);
     tc::GemmArgs g{};
     g.Mrows = r; g.Ncols = r; g.Kdim = (int32_t)rows; g.BN = std::min(r, 256);
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = src; g.n2 = no_img(); g.lower_only = 1;
@@ -1867,7 +1920,9 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
     g.out.shifted = g.out.normal; g.out.ld = r;
     g.cscale_off = -1;
     g.out.shift_bit = only_shift_bit; g.out.only_if_shifted = only_shift_bit ? 1 : 0;
-    g.ksplit = ksplit; g.split_stride = (int64_t)r * r;
+    g.ksplit = chunks;
+    if (ksplit > 1) g.split_stride = (int64_t)r * r;
+    else g.run = chunks;
     launch_gemm<tc::A_IMG_MN, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_GRAM, st);
     if (ksplit > 1) {
         const int64_t total4 = (int64_t)r * r / 4;

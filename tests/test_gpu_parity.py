@@ -364,6 +364,13 @@ def test_small_rank_qr_and_depth_chunks_agree_bit_for_bit(shape, count):
     test_factor_kernel_forms_agree_bit_for_bit(shape, count)
 
 
+# the Gram product's depth chunks: tiles of their own (the matrix alone), added by one CTA (the call of many);
+# CTA pairs and single CTAs, a ragged last chunk
+@pytest.mark.parametrize("shape,count", [((3300, 520, 512), 30), ((3300, 600, 272), 40)])
+def test_gram_chunks_agree_bit_for_bit(shape, count):
+    test_factor_kernel_forms_agree_bit_for_bit(shape, count)
+
+
 @pytest.mark.parametrize("engine", ENGINES, ids=ENGINE_IDS)
 def test_state_is_only_m_and_q(engine):
     # 4 steps in one go == 2 steps, state copied out and back, 2 more steps (bitwise)
