@@ -352,6 +352,23 @@ bool small_qr(const orthdion_plan* p, int64_t rows) {
     return p->engine == ORTHDION_ENGINE_TENSOR && qs_fits(rows, p->r, cluster_max(g_qr_cluster_max));
 }
 
+// Whether the launches of a call's one chain overlap (programmatic dependent launch).  Not with several
+// chains, where the waiting CTAs of one keep the others' kernels off the multiprocessors (four streams: 320M model
+// 2.50 -> 2.78 ms, 1.1B model 17.7 -> 18.2 ms), and not in large calls: CTAs that start early crowd on the
+// multiprocessors that fall free first.  Six long kernels (one-kernel QR on both sides) lose from about 4 M
+// elements on (9113 x 2488, r = 32: 0.273 -> 0.319 ms; 2000 x 2000: equal; 1000 x 1000: 0.095 -> 0.084), the
+// thirty kernels of a larger rank gain up to 67 M elements (4096 x 4096, r = 256 0.650 -> 0.614, 8192 x 8192,
+// r = 128 0.885 -> 0.837, r = 512 equal).
+bool overlap_pays(const orthdion_t* hs, int32_t count) {
+    int64_t elements = 0;
+    bool small = true;
+    for (int i = 0; i < count; ++i) {
+        elements += hs[i]->m * hs[i]->n;
+        if (hs[i]->engine == ORTHDION_ENGINE_TENSOR && !(small_qr(hs[i], hs[i]->m) && small_qr(hs[i], hs[i]->n))) small = false;
+    }
+    return elements <= (small ? (int64_t)4 << 20 : (int64_t)64 << 20);
+}
+
 // QR of one class's left (which = 0) or right factor in one kernel, or the column normalisation of the right
 // one; `splits` partial results in the depth-split scratch, or the fp32 slot.
 void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaStream_t st) {
@@ -724,11 +741,7 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
                           reinterpret_cast<float*>(ws + lay.diag_off)};
         const int lanes = std::min<int>({g_lanes.load(), kMaxLanes, (int)cls.size()});
         DeviceLanes* dl = lanes > 1 ? device_lanes() : nullptr;
-        // Launches of one chain overlap; with several chains they do not: the waiting CTAs of one chain
-        // would keep the others' kernels off the multiprocessors (measured, four streams: 320M model
-        // 2.50 -> 2.78 ms, 1.1B model 17.7 -> 18.2 ms; one chain: 256 x 512 r = 16 0.229 -> 0.198 ms,
-        // 520 x 384 r = 64 0.269 -> 0.235 ms, 4096 x 4096 r = 256 0.665 -> 0.633 ms).
-        overlap_launches() = dl == nullptr;
+        overlap_launches() = dl == nullptr && overlap_pays(hs, count);
         if (dl) {
             // heaviest batch first, each batch a lane of its own (round robin beyond `lanes`)
             std::vector<int> order(cls.size());
@@ -861,7 +874,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     const std::vector<int> only(1, 0);
     Batch* merged = new Batch();
     engine_error() = 0;
-    overlap_launches() = true;
+    overlap_launches() = overlap_pays(&h, 1);
     if (phase == 0) {
         tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), 1, st, OUT_SUM);
     } else if (phase == 1) {
