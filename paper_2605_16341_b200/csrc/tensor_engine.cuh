@@ -1740,6 +1740,22 @@ inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices) {
 __global__ void gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit,
                                    int only_shift_bit);
 
+// Columns per tile of a product with B, out of r (count matrices in the launch).  A wide tile forms B's terms once
+// for all columns; narrow ones form them again for every tile (from L2), which pays only where all of
+// them run at once on multiprocessors that the wide ones leave idle.  The order in which an entry is summed does
+// not depend on the tile.  Measured, one matrix, 512 -> 256 columns: 4096 x 3584 at r = 512 K1 0.161 -> 0.112, K3
+// 0.194 -> 0.166 ms; 8192 x 8192 at r = 512 step 1.61 -> 1.44.  With several waves of tiles it loses: sixteen
+// 4096 x 4096 matrices at r = 512, four waves of wide tiles against seven narrow ones, K3 of the step 5.65 -> 7.07 ms.
+inline int buffer_bn(int r, int64_t out_rows, int count) {
+    const int wide = std::min(r, 512);
+    if (r <= 256) return wide;
+    if (r % 256 == 0) {
+        const int64_t tiles = (int64_t)count * ((out_rows + 255) / 256) * (r / 256);
+        return tiles <= SPLIT_SMS / 2 ? 256 : wide;
+    }
+    return (int64_t)count * ((out_rows + tc::BM - 1) / tc::BM) * ((r + 127) / 128) <= SPLIT_SMS ? 128 : wide;
+}
+
 // After a product whose chunks ran as tiles of their own: dst (rows x r fp32) <- sum of the partial results
 // in chunk order, its operand image and its column squares per 32-row block (added as the epilogue of
 // the unsplit form adds them).  One CTA per (64 columns, 32 rows): 256 threads, eight columns each.
@@ -1818,7 +1834,7 @@ inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const
     const int ksplit = kind == OUT_SUM ? 1 : buffer_ksplit(r, m, n, matrices);
     tc::GemmArgs g{};
     if (kind != OUT_SUM && ksplit == 1) g.acc_chunks = buffer_chunks(r, m, n);
-    g.Mrows = (int32_t)m; g.Ncols = r; g.Kdim = (int32_t)n; g.BN = std::min(r, 512);
+    g.Mrows = (int32_t)m; g.Ncols = r; g.Kdim = (int32_t)n; g.BN = buffer_bn(r, m, b.count);
     g.passes = passes; g.passes2 = 1; g.ld = n; g.n1 = ts.qprev; g.a = no_img(); g.n2 = no_img();
     g.colsq_off = ts.colsq;
     g.out.normal = dest_none();
@@ -1839,7 +1855,7 @@ inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const
     const int ksplit = buffer_ksplit(r, n, m, matrices);
     tc::GemmArgs g{};
     if (ksplit == 1) g.acc_chunks = buffer_chunks(r, n, m);
-    g.Mrows = (int32_t)n; g.Ncols = r; g.Kdim = (int32_t)m; g.BN = std::min(r, 512);
+    g.Mrows = (int32_t)n; g.Ncols = r; g.Kdim = (int32_t)m; g.BN = buffer_bn(r, n, b.count);
     g.passes = passes; g.passes2 = 1; g.ld = n; g.n1 = ts.p; g.a = no_img(); g.n2 = no_img();
     g.colsq_off = ts.colsq;
     g.out.normal = dest_none(); g.out.normal.has_f32 = 1;

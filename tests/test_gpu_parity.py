@@ -371,6 +371,13 @@ def test_gram_chunks_agree_bit_for_bit(shape, count):
     test_factor_kernel_forms_agree_bit_for_bit(shape, count)
 
 
+# the products with B in narrow column tiles (the matrix alone) and wide ones (the call of many): pairs at r = 512
+# and 768, single CTAs with a remainder of 16 and of 112 columns
+@pytest.mark.parametrize("shape,count", [((1300, 1032, 512), 30), ((900, 1104, 768), 40), ((600, 520, 272), 40), ((520, 648, 496), 60)])
+def test_column_tiles_agree_bit_for_bit(shape, count):
+    test_factor_kernel_forms_agree_bit_for_bit(shape, count)
+
+
 @pytest.mark.parametrize("engine", ENGINES, ids=ENGINE_IDS)
 def test_state_is_only_m_and_q(engine):
     # 4 steps in one go == 2 steps, state copied out and back, 2 more steps (bitwise)
