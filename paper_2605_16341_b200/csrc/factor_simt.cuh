@@ -112,7 +112,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             __syncthreads();
             if (warp < CT_DIAG_WARPS) {
                 float piv[2] = {1.f, 1.f};
-                ct_diag_block<32>(smem + CT_OFF_D, nbk, warp, lane, piv);
+                ct_diag_block<32>(sD, smem + CT_OFF_D, nbk, warp, lane, piv);
                 if (warp == 0) {
                     float mn, mx;
                     ct_pivot_range(piv, nbk, lane, mn, mx);

@@ -51,7 +51,8 @@ constexpr int CT_OFF_D = 4 * CT_TILE;
 constexpr int CT_DG_LT = CT_NB * CT_LDD * 4;                   // work area of a diagonal block: the block itself first
 constexpr int CT_DG_RS = CT_DG_LT + 32 * CT_LDT * 4;
 constexpr int CT_DG_BYTES = CT_DG_RS + 64 * 4;
-constexpr int CT_SMEM_BYTES = CT_OFF_D + CT_DG_BYTES + 1024;   // + alignment of the tiles
+constexpr int CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;              // the block of the odd columns (the even ones': CT_OFF_D)
+constexpr int CT_SMEM_BYTES = CT_OFF_D2 + CT_NB * CT_LDD * 4 + 1024;     // + alignment of the tiles
 static_assert(2 * (CT_SMEM_BYTES + 2048) <= 228 * 1024, "two CTAs per multiprocessor");
 static_assert(3 * CT_NB * CT_LDS * 4 <= 4 * CT_TILE, "three transposing buffers fit the operand stages");
 constexpr int CT_MAX_BLOCKS = 64;             // r <= 4096
@@ -65,7 +66,8 @@ __device__ __forceinline__ void ct_bar_sync(int id, int threads) {
 __device__ __forceinline__ void ct_bar_arrive(int id, int threads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3;    // named barriers (0: the whole CTA)
+// named barriers (0: the whole CTA); CT_BAR_XT: two, by the parity of the column
+constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_X = 4, CT_BAR_XT = 5;
 
 __device__ __forceinline__ void ct_cp16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -186,18 +188,17 @@ __device__ __forceinline__ void ct_solve32(float (&s)[NC], const float* LT, cons
 // The four diagonal warps: sD (64 x 64, ld CT_LDD, identity beyond nbk) <- inverse of its Cholesky factor
 // (lower triangle; what lies above it is not defined: the upper right quarter holds T).  piv[]: the lane's
 // pivots of warp 0.  `area`: CT_DG_BYTES of shared memory, sD first.  NC < 32: nbk <= NC, only the leading NC
-// columns are looked at.
+// columns are looked at.  (sD lies at the start of the area, or apart from its rest: `rest` is the area then.)
 //   L11                                       warp 0
 //   L21 = D21 L11^{-T}  (warp 1)              X11 = L11^{-1}  (warp 2)
 //   D22 -= L21 L21^T                          all
 //   L22  (warp 0)                             T = L21 X11  (warps 1-3, by rows)
 //   X22 = L22^{-1}  (warp 0)                  X21 = -L22^{-1} T  (warp 1)
 template <int NC>
-__device__ __forceinline__ void ct_diag_block(unsigned char* area, int nbk, int dw, int lane, float (&piv)[2]) {
-    float* sD = reinterpret_cast<float*>(area);
-    float* LT = reinterpret_cast<float*>(area + CT_DG_LT);
+__device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, int dw, int lane, float (&piv)[2]) {
+    float* LT = reinterpret_cast<float*>(rest + CT_DG_LT);
     float* sT = sD + 32;
-    float* rs = reinterpret_cast<float*>(area + CT_DG_RS);
+    float* rs = reinterpret_cast<float*>(rest + CT_DG_RS);
     const bool two = NC == 32 && nbk > 32;
     if (dw == 0) ct_chol32<NC>(sD, LT, rs, piv[0], lane);
     ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
@@ -313,7 +314,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         smem += ((raw + 1023u) & ~1023u) - raw;
     }
     const uint32_t smem0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
-    float* sD = reinterpret_cast<float*>(smem + CT_OFF_D);
+    auto diag_buf = [&](int k) { return reinterpret_cast<float*>(smem + ((k & 1) ? CT_OFF_D2 : CT_OFF_D)); };
     float* s_part = reinterpret_cast<float*>(smem);       // partial column sums, before the operand stages are in use
 
     // MULTI: the csize CTAs of a cluster (ranks 0 .. csize-1) share matrix blockIdx.x / csize
@@ -583,6 +584,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     };
     // sD <- diagonal block k: Gram - accd, the diagonal itself from gdiag (+ shift), identity beyond r
     auto write_diag = [&](const float (&accd)[4][4], int k, float shift) {
+        float* sD = diag_buf(k);
 #pragma unroll
         for (int nf = 0; nf < 4; ++nf)
 #pragma unroll
@@ -618,7 +620,9 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     sum_products(acc, accd, t, k, next);
                     finish_sum(acc, t, k);
                 }
-                phase_sync();                                                    // X_k is in memory
+                // X_k is in memory
+                if (MULTI) cluster_sync_all();
+                else ct_bar_sync(CT_BAR_X, CT_THREADS);
                 if (first) {
                     panel(acc, t, k);
                     if (next) {
@@ -645,65 +649,78 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                         seek();
                     }
                 }
-                phase_sync();                                                    // block column k is in memory
+                // block column k is in memory
+                if (MULTI) cluster_sync_all();
+                else ct_bar_sync(CT_BAR_XT + (k & 1), CT_THREADS);
             }
         } else {
+            // The four diagonal warps.  Block k + 1 is started as soon as the product warps have its sum, while they go
+            // on with block column k: what they owe the barriers of column k is an arrival, not a wait.
             const int dw = warp - CT_MMA_WARPS, dt = tid - CT_MMA_THREADS;
             for (int k = 0; k < nb; ++k) {
-                if (k % nshare == crank) {
-                    const int nbk = min(CT_NB, r - k * CT_NB);
+                const bool mine = k % nshare == crank;
+                const int nbk = min(CT_NB, r - k * CT_NB);
+                const float* sD = diag_buf(k);
+                if (mine) {
                     ct_bar_sync(CT_BAR_READY, CT_THREADS);
                     float piv[2] = {1.f, 1.f};
-                    ct_diag_block<32>(smem + CT_OFF_D, nbk, dw, lane, piv);
+                    ct_diag_block<32>(diag_buf(k), smem + CT_OFF_D, nbk, dw, lane, piv);
                     if (dw == 0) {
                         float mn, mx;
                         ct_pivot_range(piv, nbk, lane, mn, mx);
                         if (lane == 0) { gstat[k] = mn; gstat[CT_MAX_BLOCKS + k] = mx; }
                     }
-                    // X_k for the panels (in the unused diagonal tile of L's image) and X_k^T, the diagonal
-                    // tile of the L^{-T} image
+                    // X_k for the panels (in the unused diagonal tile of L's image)
                     unsigned char* xd = l_tile(k, k);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int q = dt + 128 * e, row = q / 8, ch = q % 8;
+                        const float4 u = *reinterpret_cast<const float4*>(sD + row * CT_LDD + ch * 8);
+                        const float4 w4 = *reinterpret_cast<const float4*>(sD + row * CT_LDD + ch * 8 + 4);
+                        float v[8] = {u.x, u.y, u.z, u.w, w4.x, w4.y, w4.z, w4.w};
+#pragma unroll
+                        for (int i = 0; i < 8; ++i)
+                            if (ch * 8 + i > row || row >= nbk) v[i] = 0.f;
+                        uint4 t0, t1;
+                        split8(v, t0, t1);
+                        const int o = row * 128 + img_chunk_offset(row, ch);
+                        *reinterpret_cast<uint4*>(xd + o) = t0;
+                        *reinterpret_cast<uint4*>(xd + term + o) = t1;
+                    }
+                }
+                if (MULTI) {
+                    if (k) cluster_wait();                  // (the arrival of the column before)
+                    cluster_sync_all();
+                } else {
+                    ct_bar_arrive(CT_BAR_X, CT_THREADS);
+                }
+                if (mine) {
+                    // and X_k^T, the diagonal tile of the L^{-T} image
                     unsigned char* xt = x_tile(k, k);
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
-                        const int q = dt + 128 * e;
-                        {
-                            const int row = q / 8, ch = q % 8;
-                            float v[8];
+                        const int q = dt + 128 * e, row = q % 64, ch = q / 64;
+                        float v[8];
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const int col = ch * 8 + i;
-                                v[i] = sD[row * CT_LDD + col];
-                                if (col > row || row >= nbk) v[i] = 0.f;
-                            }
-                            uint4 t0, t1;
-                            split8(v, t0, t1);
-                            const int o = row * 128 + img_chunk_offset(row, ch);
-                            *reinterpret_cast<uint4*>(xd + o) = t0;
-                            *reinterpret_cast<uint4*>(xd + term + o) = t1;
+                        for (int i = 0; i < 8; ++i) {
+                            const int col = ch * 8 + i;
+                            v[i] = sD[col * CT_LDD + row];
+                            if (row > col || col >= nbk) v[i] = 0.f;
                         }
-                        {
-                            const int row = q % 64, ch = q / 64;
-                            float v[8];
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) {
-                                const int col = ch * 8 + i;
-                                v[i] = sD[col * CT_LDD + row];
-                                if (row > col || col >= nbk) v[i] = 0.f;
-                            }
-                            uint4 t0, t1;
-                            split8(v, t0, t1);
-                            if (a.pass >= 2 && row / 8 == ch && row < nbk) gscale[k * CT_NB + row] = ct_diag_scale(v, t0, t1, row % 8);
-                            const int o = row * 128 + img_chunk_offset(row, ch);
-                            *reinterpret_cast<uint4*>(xt + o) = t0;
-                            *reinterpret_cast<uint4*>(xt + term + o) = t1;
-                        }
+                        uint4 t0, t1;
+                        split8(v, t0, t1);
+                        if (a.pass >= 2 && row / 8 == ch && row < nbk) gscale[k * CT_NB + row] = ct_diag_scale(v, t0, t1, row % 8);
+                        const int o = row * 128 + img_chunk_offset(row, ch);
+                        *reinterpret_cast<uint4*>(xt + o) = t0;
+                        *reinterpret_cast<uint4*>(xt + term + o) = t1;
                     }
                 }
-                phase_sync();
-                phase_sync();
+                if (MULTI) cluster_arrive();
+                else ct_bar_arrive(CT_BAR_XT + (k & 1), CT_THREADS);
             }
+            if (MULTI) cluster_wait();
         }
+        __syncthreads();
         // every CTA reads the same statistics and takes the same branch
         bool fail = false;
         float mn = 3.0e38f, mx = 0.f;

@@ -419,7 +419,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     __syncthreads();
                     if (warp < CT_DIAG_WARPS) {
                         float piv[2] = {1.f, 1.f};
-                        ct_diag_block<NC>(smem, r, warp, lane, piv);
+                        ct_diag_block<NC>(sD, smem, r, warp, lane, piv);
                         if (warp == 0) {
                             float mn, mx;
                             ct_pivot_range(piv, r, lane, mn, mx);
