@@ -28,7 +28,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     float* Xs = reinterpret_cast<float*>(smem + FS_OFF_X);
     float* sD = reinterpret_cast<float*>(smem + CT_OFF_D);
     __shared__ float red[FS_THREADS / 32];
-    __shared__ float s_min, s_max;
+    __shared__ float s_min[2], s_max[2];      // pivots, by the half of their diagonal block
 
     const MatWork& w = batch.w[blockIdx.x];
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
@@ -92,7 +92,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     const int max_attempts = (a.pass == 1) ? 2 : 1;
     for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
         const float shift = attempt ? a.shift_rel * trace : 0.f;
-        if (tid == 0) { s_min = 3.0e38f; s_max = 0.f; }
+        if (tid < 2) { s_min[tid] = 3.0e38f; s_max[tid] = 0.f; }
         for (int k = 0; k < nb; ++k) {
             const int k0 = k * CT_NB, nbk = min(CT_NB, r - k0);
             // diagonal block
@@ -111,12 +111,11 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             }
             __syncthreads();
             if (warp < CT_DIAG_WARPS) {
-                float piv[2] = {1.f, 1.f};
-                ct_diag_block<32>(sD, smem + CT_OFF_D, nbk, warp, lane, piv);
-                if (warp == 0) {
-                    float mn, mx;
-                    ct_pivot_range(piv, nbk, lane, mn, mx);
-                    if (lane == 0) { s_min = fminf(s_min, mn); s_max = fmaxf(s_max, mx); }
+                float mn, mx;
+                ct_diag_block(sD, smem + CT_OFF_D, nbk, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                if (lane == 0 && (warp == 0 || (warp == 3 && nbk > 32))) {
+                    s_min[warp / 3] = mx <= 3.0e38f ? fminf(s_min[warp / 3], mn) : -1.f;
+                    s_max[warp / 3] = fmaxf(s_max[warp / 3], mx);
                 }
             }
             __syncthreads();
@@ -159,8 +158,9 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             }
             __syncthreads();
         }
-        const bool fail = !(s_min > 0.f);
-        const bool ill = (a.pass == 1) && (s_max > a.cond_limit * s_min);
+        const float mn = fminf(s_min[0], s_min[1]), mx = fmaxf(s_max[0], s_max[1]);
+        const bool fail = !(mn > 0.f);
+        const bool ill = (a.pass == 1) && (sqrtf(mx) > a.cond_limit * sqrtf(mn));
         if (!fail && !(ill && attempt == 0)) {
             ok = true;
         } else if (attempt == 0 && a.pass == 1) {

@@ -13,14 +13,13 @@
 // 64 x 64 come in by cp.async one step ahead.
 //
 // What bounds it: the chain of r / 64 diagonal blocks.  Four extra warps per CTA factor and invert a
-// 64 x 64 block in fp32 (about 3 us: one warp eliminates 32 columns with the rows in registers and the
-// next pivot computed ahead of its column) while the eight product warps do the S sums of
+// 64 x 64 block in fp32 (below) while the eight product warps do the S sums of
 // the same block column, which do not depend on it; the tile below the diagonal goes first, together
 // with the next diagonal block's own sum, so that the chain never waits for the rest.  64-wide
-// blocks instead of 32: half the barriers, and a diagonal block still fits one warp pair's registers.
+// blocks instead of 32: half the barriers.
 // Measured, factor stage of a step (six launches, ms), before (32-wide blocks, fp32 tiles split at every
-// use, a pairwise inversion afterwards) -> now: one matrix r = 64 0.19 -> 0.09, r = 256 0.74 -> 0.26, r = 512
-// 1.47 -> 0.37, r = 1024 3.68 -> 0.70; 56 matrices at r = 512 2.7 -> 0.7, 154 of them 5.0 -> 1.5.
+// use, a pairwise inversion afterwards) -> now: one matrix r = 256 0.74 -> 0.21, r = 512
+// 1.47 -> 0.32, r = 1024 3.68 -> 0.68; 56 matrices at r = 512 2.7 -> 0.7, 154 of them 5.0 -> 1.5.
 //
 // The later passes of a CholeskyQR see a Gram matrix I + E with E tiny; when a rigorous bound on
 // |E|_2 is small enough, L^{-1} = I - Phi(E) (first order) replaces the factorisation.
@@ -49,14 +48,15 @@ constexpr int CT_LDS = 65;                    // transposing buffer of the first
 // dynamic shared memory: two stages of an A tile and a B tile, then the diagonal block's work area
 constexpr int CT_OFF_D = 4 * CT_TILE;
 constexpr int CT_DG_LT = CT_NB * CT_LDD * 4;                   // work area of a diagonal block: the block itself first
-constexpr int CT_DG_RS = CT_DG_LT + 32 * CT_LDT * 4;
-constexpr int CT_DG_BYTES = CT_DG_RS + 64 * 4;
+constexpr int CT_DG_BLK = CT_DG_LT + 32 * CT_LDT * 4;
+constexpr int CT_DG_S = CT_DG_BLK + 64 * 4;
+constexpr int CT_DG_BYTES = CT_DG_S + 8 * 32 * 4;
 constexpr int CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;              // the block of the odd columns (the even ones': CT_OFF_D)
 constexpr int CT_SMEM_BYTES = CT_OFF_D2 + CT_NB * CT_LDD * 4 + 1024;     // + alignment of the tiles
 static_assert(2 * (CT_SMEM_BYTES + 2048) <= 228 * 1024, "two CTAs per multiprocessor");
 static_assert(3 * CT_NB * CT_LDS * 4 <= 4 * CT_TILE, "three transposing buffers fit the operand stages");
 constexpr int CT_MAX_BLOCKS = 64;             // r <= 4096
-constexpr int CT_STAT_FLOATS = 3 * CT_MAX_BLOCKS;   // per block: smallest and largest diagonal entry, row-sum bound
+constexpr int CT_STAT_FLOATS = 5 * CT_MAX_BLOCKS;   // per block: smallest and largest pivot of its halves, row-sum bound
 constexpr float CT_THIRD_PASS_LIMIT = 0.02f; // bound on |Gram - I|_2 of the second pass above which a third follows
 constexpr float CT_SERIES_LIMIT = 1.4e-3f;   // bound on |Gram - I|_2 below which L^{-1} = I - Phi(E) is used
 
@@ -84,6 +84,10 @@ __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], const uint32_t (
 }
 __device__ __forceinline__ void ct_ldsm4(uint32_t (&v)[4], uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
+}
+__device__ __forceinline__ void ct_ldsm4t(uint32_t (&v)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(addr) : "memory");
 }
 
@@ -114,6 +118,33 @@ __device__ __forceinline__ void ct_tile_mma(float (&acc)[4][4], uint32_t a_tile,
         }
     }
 }
+// the same with B given transposed: acc += A B, B's rows (depth) in memory order
+__device__ __forceinline__ void ct_tile_mma_nt(float (&acc)[4][4], uint32_t a_tile, uint32_t b_tile, int warp, int lane) {
+    const int l8 = lane & 7;
+    const uint32_t a_row = a_tile + ((warp % 4) * 16 + l8 + ((lane >> 3) & 1) * 8) * 128;
+    const uint32_t b_row = b_tile + (l8 + ((lane >> 3) & 1) * 8) * 128;
+    const int a_ch = lane >> 4;
+#pragma unroll
+    for (int ks = 0; ks < 4; ++ks) {
+        const uint32_t ao = (uint32_t)(((2 * ks + a_ch) ^ l8) << 4);
+        uint32_t ah[4], al[4];
+        ct_ldsm4(ah, a_row + ao);
+        ct_ldsm4(al, a_row + CT_TERM + ao);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const uint32_t bo = (uint32_t)(ks * 2048 + ((((warp / 4) * 4 + 2 * h + (lane >> 4)) ^ l8) << 4));
+            uint32_t bh[4], bl[4];
+            ct_ldsm4t(bh, b_row + bo);
+            ct_ldsm4t(bl, b_row + CT_TERM + bo);
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                mma_bf16_16x8x16(acc[2 * h + u], ah, bh[2 * u], bh[2 * u + 1]);
+                mma_bf16_16x8x16(acc[2 * h + u], ah, bl[2 * u], bl[2 * u + 1]);
+                mma_bf16_16x8x16(acc[2 * h + u], al, bh[2 * u], bh[2 * u + 1]);
+            }
+        }
+    }
+}
 // this warp's part of a tile, v -> the two bf16 terms of a K-major tile in shared memory
 __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4][4], int warp, int lane) {
     const int row = (warp % 4) * 16 + lane / 4;             // row & 7 == lane / 4 for both halves
@@ -131,163 +162,210 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
     }
 }
 
-// ---- diagonal blocks (fp32, one warp) ------------------------------------------------------------
-// Cholesky of the leading NC columns of the 32 x 32 block at `blk` (ld CT_LDD).  Lane i holds row i in registers.  LT[j][i] <- L(i, j),
-// rs[j] <- 1 / L(j, j); the lane keeps its pivot in `piv`.  The pivot of column j + 1 is formed from two
-// values fetched before column j was scaled, so that the chain per column is one reciprocal square root
-// and two products; the next two columns get their multiplier by shuffle, the others from LT.
-template <int NC>
-__device__ __forceinline__ void ct_chol32(const float* blk, float* LT, float* rs, float& piv, int lane) {
-    float a[NC];
+// ---- diagonal blocks (fp32, four warps) ----------------------------------------------------------
+// sD (64 x 64 block, ld CT_LDD, identity beyond nbk; row by row the lower part counts) -> X, the inverse of its
+// Cholesky factor L, in the lower part of sD, and the rows of X^T = L^{-T} as they are found: out(row, chunk, z)
+// gets the entries 8 chunk .. + 7 of a row.
+//
+// As in the large, [D; I] L^{-T} = [L; L^{-T}]: rows of the block and of the identity go through the same
+// elimination, a row per lane.  The columns are taken in panels of eight, whose 8 x 8 diagonal block every
+// lane factors for itself from shared memory (a chain of eight reciprocal square roots and 16 products, no shuffle
+// in it); then the lane solves its own eight entries and the panel's columns of L go to the others through LT
+// (LT[j][i] = L(i, j)).  What bounds it is this chain, about 500 cycles per panel, so everything else runs beside it:
+//   first half (columns 0 .. 31)        second half
+//   warp 0  L11                         rows 0 .. 31 of L^{-T} beyond column 32
+//   warp 1  L21                         their sums  -X11^T L21^T, a panel ahead
+//   warp 2  rows 0 .. 31 of L^{-T}      rows 32 .. 63 of L^{-T}
+//   warp 3  D22 - L21 L21^T             L22
+// (Two 32-column factorisations by one warp with the columns passed by shuffle, triangular solves and the update
+// one after the other took 16 thousand cycles; fully unrolled they were also bound by instruction
+// fetch whenever another phase had evicted them.)
+__device__ __forceinline__ float ct_rsqrt(float x) {
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// the lane's row entries a[0 .. 7] -> its entries z of [L; L^{-T}]; blk: the panel's 8 x 8 diagonal block
+__device__ __forceinline__ void ct_panel8(const float* blk, const float* a, float (&z)[8], float& dmin, float& dmax) {
+    float b[8][8];
 #pragma unroll
-    for (int c = 0; c < NC; c += 4) {
-        const float4 v = *reinterpret_cast<const float4*>(blk + lane * CT_LDD + c);
-        a[c] = v.x; a[c + 1] = v.y; a[c + 2] = v.z; a[c + 3] = v.w;
+    for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int c = 0; c <= i; c += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(blk + i * 8 + c);
+            b[i][c] = v.x; b[i][c + 1] = v.y; b[i][c + 2] = v.z; b[i][c + 3] = v.w;
+        }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) z[j] = a[j];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        const float d = b[j][j], inv = ct_rsqrt(d);
+        dmin = d > 0.f ? fminf(dmin, d) : -1.f;              // (a breakdown stays: -1 is the smallest from then on)
+        dmax = fmaxf(dmax, d);
+        z[j] *= inv;
+#pragma unroll
+        for (int i = j + 1; i < 8; ++i) {
+            const float l = b[i][j] * inv;
+            b[i][j] = l;
+            z[i] = fmaf(-z[j], l, z[i]);
+        }
+#pragma unroll
+        for (int i = j + 1; i < 8; ++i)
+#pragma unroll
+            for (int c = j + 1; c <= i; ++c) b[i][c] = fmaf(-b[i][j], b[c][j], b[i][c]);
     }
-    float d = __shfl_sync(0xffffffffu, a[0], 0);
-    float q = __shfl_sync(0xffffffffu, a[0], 1), p = __shfl_sync(0xffffffffu, a[1], 1);
+}
+// a[0 .. 4 n4) -= sum_j z_j LT[j][c0 ..]
+template <int N4>
+__device__ __forceinline__ void ct_rank8(float* a, const float (&z)[8], const float* LT, int c0) {
 #pragma unroll
-    for (int j = 0; j < NC; ++j) {
-        const float inv = rsqrtf(d);
-        if (lane == j) { piv = d; rs[j] = inv; }
-        const float la = a[j] * inv;
-        LT[j * CT_LDT + lane] = la;
-        if (j + 1 < NC) { const float t = q * inv; d = fmaf(-t, t, p); }
+    for (int c = 0; c < 4 * N4; c += 4) {
 #pragma unroll
-        for (int c = j + 1; c < j + 3; ++c)
-            if (c < NC) a[c] = fmaf(-la, __shfl_sync(0xffffffffu, la, c), a[c]);
-        if (j + 2 < NC) { q = __shfl_sync(0xffffffffu, a[j + 1], j + 2); p = __shfl_sync(0xffffffffu, a[j + 2], j + 2); }
-        __syncwarp();
-#pragma unroll
-        for (int c4 = (j + 3) / 4; c4 < NC / 4; ++c4) {
-            const float4 v = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 4 * c4);
-            const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (4 * c4 + e >= j + 3) a[4 * c4 + e] = fmaf(-la, vv[e], a[4 * c4 + e]);
+        for (int j = 0; j < 8; ++j) {
+            const float4 l = *reinterpret_cast<const float4*>(LT + j * CT_LDT + c0 + c);
+            a[c] = fmaf(-z[j], l.x, a[c]); a[c + 1] = fmaf(-z[j], l.y, a[c + 1]);
+            a[c + 2] = fmaf(-z[j], l.z, a[c + 2]); a[c + 3] = fmaf(-z[j], l.w, a[c + 3]);
         }
     }
 }
-// s <- L^{-1} s for the NC x NC factor held in LT, rs; each lane has a right-hand side of its own
-template <int NC>
-__device__ __forceinline__ void ct_solve32(float (&s)[NC], const float* LT, const float* rs) {
-#pragma unroll
-    for (int p = 0; p < NC; ++p) {
-        const float x = s[p] * rs[p];
-        s[p] = x;
-#pragma unroll
-        for (int i4 = (p + 1) / 4; i4 < NC / 4; ++i4) {
-            const float4 v = *reinterpret_cast<const float4*>(LT + p * CT_LDT + 4 * i4);
-            const float vv[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int e = 0; e < 4; ++e)
-                if (4 * i4 + e > p) s[4 * i4 + e] = fmaf(-vv[e], x, s[4 * i4 + e]);
-        }
-    }
-}
-// The four diagonal warps: sD (64 x 64, ld CT_LDD, identity beyond nbk) <- inverse of its Cholesky factor
-// (lower triangle; what lies above it is not defined: the upper right quarter holds T).  piv[]: the lane's
-// pivots of warp 0.  `area`: CT_DG_BYTES of shared memory, sD first.  NC < 32: nbk <= NC, only the leading NC
-// columns are looked at.  (sD lies at the start of the area, or apart from its rest: `rest` is the area then.)
-//   L11                                       warp 0
-//   L21 = D21 L11^{-T}  (warp 1)              X11 = L11^{-1}  (warp 2)
-//   D22 -= L21 L21^T                          all
-//   L22  (warp 0)                             T = L21 X11  (warps 1-3, by rows)
-//   X22 = L22^{-1}  (warp 0)                  X21 = -L22^{-1} T  (warp 1)
-template <int NC>
-__device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, int dw, int lane, float (&piv)[2]) {
+// `rest`: CT_DG_BYTES of shared memory whose first part may be sD itself.  dmin, dmax: smallest (-1: breakdown)
+// and largest pivot, in the lanes of warp 0 (one half) or warp 3 (two).
+template <class Out>
+__device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, int dw, int lane, float& dmin, float& dmax, Out out) {
     float* LT = reinterpret_cast<float*>(rest + CT_DG_LT);
-    float* sT = sD + 32;
-    float* rs = reinterpret_cast<float*>(rest + CT_DG_RS);
-    const bool two = NC == 32 && nbk > 32;
-    if (dw == 0) ct_chol32<NC>(sD, LT, rs, piv[0], lane);
-    ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-    float s[NC];
-    if (dw == 2 || (dw == 1 && two)) {
-#pragma unroll
-        for (int i = 0; i < NC; i += 4) {
-            float4 v = make_float4(i == lane ? 1.f : 0.f, i + 1 == lane ? 1.f : 0.f, i + 2 == lane ? 1.f : 0.f, i + 3 == lane ? 1.f : 0.f);
-            if (dw == 1) v = *reinterpret_cast<const float4*>(sD + (32 + lane) * CT_LDD + i);
-            s[i] = v.x; s[i + 1] = v.y; s[i + 2] = v.z; s[i + 3] = v.w;
-        }
-        ct_solve32<NC>(s, LT, rs);
-        float* dst = dw == 1 ? LT + 32 + lane : sD + lane;
-        const int ld = dw == 1 ? CT_LDT : CT_LDD;
-#pragma unroll
-        for (int i = 0; i < NC; ++i) dst[i * ld] = s[i];
-    }
-    ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-    if constexpr (NC == 32) {
-    if (!two) return;
+    float* blk = reinterpret_cast<float*>(rest + CT_DG_BLK);
+    float* sS = reinterpret_cast<float*>(rest + CT_DG_S);
+    const bool two = nbk > 32;
+    float a[32], z[8];
+    dmin = 3.0e38f; dmax = 0.f;
     {
-        // D22(lane, 8 dw ..) -= sum_j L21(lane, j) L21(8 dw .., j)
-        float o[8];
+        // this lane's row: of D11, D21, the identity, D22
+        const float* src = sD + (lane + (dw == 1 || dw == 3 ? 32 : 0)) * CT_LDD + (dw == 3 ? 32 : 0);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) o[e] = sD[(32 + lane) * CT_LDD + 32 + 8 * dw + e];
-#pragma unroll 8
-        for (int j = 0; j < 32; ++j) {
-            const float l = LT[j * CT_LDT + 32 + lane];
-            const float4 u = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 32 + 8 * dw);
-            const float4 v = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 36 + 8 * dw);
-            o[0] = fmaf(-l, u.x, o[0]); o[1] = fmaf(-l, u.y, o[1]); o[2] = fmaf(-l, u.z, o[2]); o[3] = fmaf(-l, u.w, o[3]);
-            o[4] = fmaf(-l, v.x, o[4]); o[5] = fmaf(-l, v.y, o[5]); o[6] = fmaf(-l, v.z, o[6]); o[7] = fmaf(-l, v.w, o[7]);
+        for (int c = 0; c < 32; c += 4) {
+            float4 v = make_float4(lane == c ? 1.f : 0.f, lane == c + 1 ? 1.f : 0.f, lane == c + 2 ? 1.f : 0.f, lane == c + 3 ? 1.f : 0.f);
+            if (dw != 2 && (dw == 0 || two)) v = *reinterpret_cast<const float4*>(src + c);
+            a[c] = v.x; a[c + 1] = v.y; a[c + 2] = v.z; a[c + 3] = v.w;
         }
-#pragma unroll
-        for (int e = 0; e < 8; e += 4)
-            *reinterpret_cast<float4*>(sD + (32 + lane) * CT_LDD + 32 + 8 * dw + e) = make_float4(o[e], o[e + 1], o[e + 2], o[e + 3]);
     }
-    ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-    if (dw == 0) {
-        ct_chol32<32>(sD + 32 * CT_LDD + 32, LT, rs + 32, piv[1], lane);
-    } else {
-        // rows 12 (dw - 1) .. + 11 of T (the last warp: 8 rows), a column per lane
-        const int i0 = 12 * (dw - 1);
-        float t[12];
+    const int np = two ? 4 : (nbk + 7) / 8;
+    // first half; warps 0 to 2: the panel at hand is a[0 .. 7], the updates write eight registers down
+    for (int p = 0; p < np; ++p) {
+        if (dw == 0 && lane / 8 == p) {
+            *reinterpret_cast<float4*>(blk + (lane % 8) * 8) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4*>(blk + (lane % 8) * 8 + 4) = make_float4(a[4], a[5], a[6], a[7]);
+        }
+        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+        float* L = LT + p * 8 * CT_LDT;
+        if (dw < 3) {
+            ct_panel8(blk, a, z, dmin, dmax);
+            if (dw < 2) {
 #pragma unroll
-        for (int e = 0; e < 12; ++e) t[e] = 0.f;
-#pragma unroll 8
-        for (int q = 0; q < 32; ++q) {
-            const float x = sD[q * CT_LDD + lane];
+                for (int j = 0; j < 8; ++j) L[j * CT_LDT + 32 * dw + lane] = z[j];
+            } else {
 #pragma unroll
-            for (int e = 0; e < 12; e += 4) {
-                if (e < 8 || dw < 3) {
-                    const float4 v = *reinterpret_cast<const float4*>(LT + q * CT_LDT + 32 + i0 + e);
-                    t[e] = fmaf(v.x, x, t[e]); t[e + 1] = fmaf(v.y, x, t[e + 1]);
-                    t[e + 2] = fmaf(v.z, x, t[e + 2]); t[e + 3] = fmaf(v.w, x, t[e + 3]);
+                for (int j = 0; j < 8; ++j) sD[(8 * p + j) * CT_LDD + lane] = z[j];
+            }
+        }
+        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+        if (dw < 3) {
+            // (a group beyond the last column works on what is not used any more: branch-free but for whole groups)
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+                if (g < 3 - p) {
+                    float t[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) t[c] = a[8 * (g + 1) + c];
+                    ct_rank8<2>(t, z, L, 8 * (p + g + 1));
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) a[8 * g + c] = t[c];
+                }
+            }
+            if (dw == 2) out(lane, p, z);
+        } else if (two) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) z[j] = L[j * CT_LDT + 32 + lane];
+            ct_rank8<8>(a, z, L, 32);
+        }
+    }
+    if (!two) {
+        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+        return;
+    }
+    // second half; LT's first 32 columns hold L22 from here on.  Warp 0: z of the panels so far in a; warp 1: the
+    // lane's row of X11^T
+    if (dw == 2) {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) a[c] = lane == c ? 1.f : 0.f;
+    } else if (dw == 1) {
+#pragma unroll
+        for (int j = 0; j < 32; ++j) a[j] = sD[j * CT_LDD + lane];
+    }
+    for (int p = 0; p < 4; ++p) {
+        if (dw == 3 && lane / 8 == p) {
+            *reinterpret_cast<float4*>(blk + (lane % 8) * 8) = make_float4(a[0], a[1], a[2], a[3]);
+            *reinterpret_cast<float4*>(blk + (lane % 8) * 8 + 4) = make_float4(a[4], a[5], a[6], a[7]);
+        } else if (dw == 1) {
+            float t[8] = {};
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const float4 u = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 32 + 8 * p);
+                const float4 v = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 36 + 8 * p);
+                t[0] = fmaf(-a[j], u.x, t[0]); t[1] = fmaf(-a[j], u.y, t[1]); t[2] = fmaf(-a[j], u.z, t[2]); t[3] = fmaf(-a[j], u.w, t[3]);
+                t[4] = fmaf(-a[j], v.x, t[4]); t[5] = fmaf(-a[j], v.y, t[5]); t[6] = fmaf(-a[j], v.z, t[6]); t[7] = fmaf(-a[j], v.w, t[7]);
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) sS[c * 32 + lane] = t[c];
+        }
+        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+        float* L = LT + p * 8 * CT_LDT;
+        if (dw == 0) {
+            // (sums of the panels before: the z so far are in shared memory, X(32 + ., lane))
+            float t[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) t[c] = sS[c * 32 + lane];
+            for (int q = 0; q < 8 * p; ++q) {
+                const float x = sD[(32 + q) * CT_LDD + lane];
+                const float4 u = *reinterpret_cast<const float4*>(LT + q * CT_LDT + 8 * p);
+                const float4 v = *reinterpret_cast<const float4*>(LT + q * CT_LDT + 8 * p + 4);
+                t[0] = fmaf(-x, u.x, t[0]); t[1] = fmaf(-x, u.y, t[1]); t[2] = fmaf(-x, u.z, t[2]); t[3] = fmaf(-x, u.w, t[3]);
+                t[4] = fmaf(-x, v.x, t[4]); t[5] = fmaf(-x, v.y, t[5]); t[6] = fmaf(-x, v.z, t[6]); t[7] = fmaf(-x, v.w, t[7]);
+            }
+#pragma unroll
+            for (int c = 0; c < 8; ++c) a[c] = t[c];
+        }
+        if (dw != 1) {
+            float lo = 3.0e38f, hi = 0.f;
+            ct_panel8(blk, a, z, lo, hi);
+            if (dw == 3) { dmin = fminf(dmin, lo); dmax = fmaxf(dmax, hi); }
+            if (dw == 3) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) L[j * CT_LDT + lane] = z[j];
+            } else {
+                float* dst = sD + (32 + 8 * p) * CT_LDD + (dw == 2 ? 32 : 0) + lane;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) dst[j * CT_LDD] = z[j];
+            }
+        }
+        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+        if (dw >= 2) {
+#pragma unroll
+            for (int g = 0; g < 3; ++g) {
+                if (g < 3 - p) {
+                    float t[8];
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) t[c] = a[8 * (g + 1) + c];
+                    ct_rank8<2>(t, z, L, 8 * (p + g + 1));
+#pragma unroll
+                    for (int c = 0; c < 8; ++c) a[8 * g + c] = t[c];
                 }
             }
         }
-#pragma unroll
-        for (int e = 0; e < 12; ++e)
-            if (e < 8 || dw < 3) sT[(i0 + e) * CT_LDD + lane] = t[e];
-    }
-    ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-    if (dw < 2) {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) s[i] = dw == 0 ? (i == lane ? 1.f : 0.f) : -sT[i * CT_LDD + lane];
-        ct_solve32<32>(s, LT, rs + 32);
-#pragma unroll
-        for (int i = 0; i < 32; ++i) sD[(32 + i) * CT_LDD + (dw == 0 ? 32 : 0) + lane] = s[i];
-    }
-    ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
+        if (dw == 2) out(32 + lane, 4 + p, z);
+        else if (dw == 0) out(lane, 4 + p, z);
     }
 }
 
-// smallest and largest diagonal entry of the factor from the pivots of warp 0; smallest -1 after a breakdown
-__device__ __forceinline__ void ct_pivot_range(const float (&piv)[2], int nbk, int lane, float& mn, float& mx) {
-    mn = 3.0e38f; mx = 0.f;
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        if (h * 32 + lane < nbk) {
-            if (!(piv[h] > 0.f) || !(piv[h] <= 3.0e38f)) mn = -1.f;
-            else { const float sq = sqrtf(piv[h]); mn = fminf(mn, sq); mx = fmaxf(mx, sq); }
-        }
-    }
-    for (int o = 16; o; o >>= 1) {
-        mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, o));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    }
-}
 // v[e] over the value that its two bf16 terms hold
 __device__ __forceinline__ float ct_diag_scale(const float (&v)[8], const uint4& t0, const uint4& t1, int e) {
     const uint32_t h[4] = {t0.x, t0.y, t0.z, t0.w}, l[4] = {t1.x, t1.y, t1.z, t1.w};
@@ -400,9 +478,9 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     }
 
     // Tiles of the L^{-T} image below its diagonal that the apply product reads as zeros: those inside the
-    // same 256-column block
+    // same 256-column block; and a last diagonal tile that is written in part
     for (int t = crank; t < nb; t += nshare)
-        for (int c = t & ~3; c < t; ++c) {
+        for (int c = t & ~3; c < t + (t * CT_NB + CT_NB > r ? 1 : 0); ++c) {
             unsigned char* dst = x_tile(t, c);
             for (int q = tid; q < 1024; q += CT_THREADS)
                 *reinterpret_cast<uint4*>(dst + (q >= 512 ? term : 0) + (q & 511) * 16) = make_uint4(0u, 0u, 0u, 0u);
@@ -448,13 +526,13 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     mx = fmaxf(mx, s <= 3.0e38f ? s : 3.3e38f);
                 }
                 for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                if (lane == 0) gstat[2 * CT_MAX_BLOCKS + t] = mx;
+                if (lane == 0) gstat[4 * CT_MAX_BLOCKS + t] = mx;
             }
             __syncthreads();
         }
         phase_sync();
         float mx = 0.f;
-        for (int t = 0; t < nb; ++t) mx = fmaxf(mx, __ldcg(gstat + 2 * CT_MAX_BLOCKS + t));
+        for (int t = 0; t < nb; ++t) mx = fmaxf(mx, __ldcg(gstat + 4 * CT_MAX_BLOCKS + t));
         // Second pass with Q1 far from orthonormal (cond(Y)^2 u was not small): its result will
         // not be orthonormal to working accuracy either, so ask for the third pass.
         if (a.pass == 2 && !(mx <= CT_THIRD_PASS_LIMIT) && tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
@@ -564,13 +642,13 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     };
     // Z[t, k] = acc X_k^T -> its image; leaves the tile in the A slot of stage ^ 1
     auto panel = [&](float (&acc)[4][4], int t, int k) {
-        load_tile(b_slot(stage), l_tile(k, k));
+        load_tile(b_slot(stage), x_tile(k, k));
         ct_cp_commit();
         ct_store_tile(a_slot(stage), acc, warp, lane);
         ct_cp_wait_all();
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
         float o[4][4] = {};
-        ct_tile_mma(o, a_slot(stage), b_slot(stage), warp, lane);
+        ct_tile_mma_nt(o, a_slot(stage), b_slot(stage), warp, lane);
         ct_store_tile(a_slot(stage ^ 1), o, warp, lane);
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
         unsigned char* dst = t < k ? x_tile(t, k) : l_tile(t, k);
@@ -656,36 +734,37 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         } else {
             // The four diagonal warps.  Block k + 1 is started as soon as the product warps have its sum, while they go
             // on with block column k: what they owe the barriers of column k is an arrival, not a wait.
-            const int dw = warp - CT_MMA_WARPS, dt = tid - CT_MMA_THREADS;
+            const int dw = warp - CT_MMA_WARPS;
             for (int k = 0; k < nb; ++k) {
                 const bool mine = k % nshare == crank;
                 const int nbk = min(CT_NB, r - k * CT_NB);
-                const float* sD = diag_buf(k);
                 if (mine) {
                     ct_bar_sync(CT_BAR_READY, CT_THREADS);
-                    float piv[2] = {1.f, 1.f};
-                    ct_diag_block<32>(diag_buf(k), smem + CT_OFF_D, nbk, dw, lane, piv);
-                    if (dw == 0) {
-                        float mn, mx;
-                        ct_pivot_range(piv, nbk, lane, mn, mx);
-                        if (lane == 0) { gstat[k] = mn; gstat[CT_MAX_BLOCKS + k] = mx; }
-                    }
-                    // X_k for the panels (in the unused diagonal tile of L's image)
-                    unsigned char* xd = l_tile(k, k);
+                    // X_k^T goes to the diagonal tile of the L^{-T} image, chunk by chunk, while it is being found
+                    unsigned char* xt = x_tile(k, k);
+                    auto out = [&](int row, int ch, const float (&z)[8]) {
+                        float v[8];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int q = dt + 128 * e, row = q / 8, ch = q % 8;
-                        const float4 u = *reinterpret_cast<const float4*>(sD + row * CT_LDD + ch * 8);
-                        const float4 w4 = *reinterpret_cast<const float4*>(sD + row * CT_LDD + ch * 8 + 4);
-                        float v[8] = {u.x, u.y, u.z, u.w, w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            if (ch * 8 + i > row || row >= nbk) v[i] = 0.f;
+                        for (int i = 0; i < 8; ++i) v[i] = row < nbk && ch * 8 + i < nbk ? z[i] : 0.f;
                         uint4 t0, t1;
                         split8(v, t0, t1);
+                        if (a.pass >= 2 && row / 8 == ch && row < nbk) gscale[k * CT_NB + row] = ct_diag_scale(v, t0, t1, row % 8);
                         const int o = row * 128 + img_chunk_offset(row, ch);
-                        *reinterpret_cast<uint4*>(xd + o) = t0;
-                        *reinterpret_cast<uint4*>(xd + term + o) = t1;
+                        *reinterpret_cast<uint4*>(xt + o) = t0;
+                        *reinterpret_cast<uint4*>(xt + term + o) = t1;
+                    };
+                    if (dw == 1) {
+                        const float zero[8] = {};
+#pragma unroll
+                        for (int ch = 0; ch < 4; ++ch) out(32 + lane, ch, zero);
+                    }
+                    float mn, mx;
+                    ct_diag_block(diag_buf(k), smem + CT_OFF_D, nbk, dw, lane, mn, mx, out);
+                    // statistics: squared diagonal entries of L; two halves: warp 0's first, warp 3's second
+                    if (lane == 0 && (dw == 0 || (dw == 3 && nbk > 32))) {
+                        if (!(mx <= 3.0e38f)) mn = -1.f;
+                        gstat[(dw ? CT_MAX_BLOCKS : 0) + k] = mn;
+                        gstat[(dw ? 3 : 2) * CT_MAX_BLOCKS + k] = mx;
                     }
                 }
                 if (MULTI) {
@@ -693,27 +772,6 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     cluster_sync_all();
                 } else {
                     ct_bar_arrive(CT_BAR_X, CT_THREADS);
-                }
-                if (mine) {
-                    // and X_k^T, the diagonal tile of the L^{-T} image
-                    unsigned char* xt = x_tile(k, k);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int q = dt + 128 * e, row = q % 64, ch = q / 64;
-                        float v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const int col = ch * 8 + i;
-                            v[i] = sD[col * CT_LDD + row];
-                            if (row > col || col >= nbk) v[i] = 0.f;
-                        }
-                        uint4 t0, t1;
-                        split8(v, t0, t1);
-                        if (a.pass >= 2 && row / 8 == ch && row < nbk) gscale[k * CT_NB + row] = ct_diag_scale(v, t0, t1, row % 8);
-                        const int o = row * 128 + img_chunk_offset(row, ch);
-                        *reinterpret_cast<uint4*>(xt + o) = t0;
-                        *reinterpret_cast<uint4*>(xt + term + o) = t1;
-                    }
                 }
                 if (MULTI) cluster_arrive();
                 else ct_bar_arrive(CT_BAR_XT + (k & 1), CT_THREADS);
@@ -725,12 +783,15 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         bool fail = false;
         float mn = 3.0e38f, mx = 0.f;
         for (int k = 0; k < nb; ++k) {
-            const float lo = __ldcg(gstat + k);
-            if (!(lo > 0.f)) fail = true;
-            mn = fminf(mn, lo);
-            mx = fmaxf(mx, __ldcg(gstat + CT_MAX_BLOCKS + k));
+            const int halves = r - k * CT_NB > 32 ? 2 : 1;
+            for (int h = 0; h < halves; ++h) {
+                const float lo = __ldcg(gstat + h * CT_MAX_BLOCKS + k);
+                if (!(lo > 0.f)) fail = true;
+                mn = fminf(mn, lo);
+                mx = fmaxf(mx, __ldcg(gstat + (2 + h) * CT_MAX_BLOCKS + k));
+            }
         }
-        const bool ill = (a.pass == 1) && (mx > a.cond_limit * mn);
+        const bool ill = (a.pass == 1) && (sqrtf(mx) > a.cond_limit * sqrtf(mn));
         if (!fail && !(ill && attempt == 0)) {
             ok = true;
         } else if (attempt == 0 && a.pass == 1) {

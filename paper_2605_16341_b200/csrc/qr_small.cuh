@@ -92,7 +92,6 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
     constexpr int TX = R / 4;                        // threads along the columns of a 4 x 4-blocked product
     constexpr int GROUPS = QS_THREADS / (TX * TX);   // Gram product: thread groups that share the rows
     constexpr int RT = QS_THREADS / TX * 4;          // apply product: rows of a step
-    constexpr int NC = R < 32 ? R : 32;
     constexpr int ENT = R == 64 ? 4 : 1;             // Gram entries (in fours) per thread
     constexpr int LEVELS = R == 64 ? 3 : 5;
     extern __shared__ __align__(16) unsigned char smem[];
@@ -100,7 +99,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
     float* part = sD;
     float* G = reinterpret_cast<float*>(smem + CT_DG_BYTES);     // Gram matrix, then L^{-T}
     float* Y = G + R * R;                            // this CTA's rows
-    __shared__ float s_range[2], s_bound;
+    __shared__ float s_min[2], s_max[2], s_bound;
     static_assert(GROUPS * R * R * 4 <= CT_DG_BYTES, "partial Gram matrices fit the diagonal block's area");
 
     grid_dependency();
@@ -418,17 +417,17 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     }
                     __syncthreads();
                     if (warp < CT_DIAG_WARPS) {
-                        float piv[2] = {1.f, 1.f};
-                        ct_diag_block<NC>(sD, smem, r, warp, lane, piv);
-                        if (warp == 0) {
-                            float mn, mx;
-                            ct_pivot_range(piv, r, lane, mn, mx);
-                            if (lane == 0) { s_range[0] = mn; s_range[1] = mx; }
+                        float mn, mx;
+                        ct_diag_block(sD, smem, r, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                        if (lane == 0 && (warp == 0 || (warp == 3 && r > 32))) {
+                            s_min[warp / 3] = mx <= 3.0e38f ? mn : -1.f;
+                            s_max[warp / 3] = mx;
                         }
                     }
                     __syncthreads();
-                    const bool fail = !(s_range[0] > 0.f);
-                    const bool ill = pass == 1 && s_range[1] > a.cond_limit * s_range[0];
+                    const float mn = r > 32 ? fminf(s_min[0], s_min[1]) : s_min[0], mx = r > 32 ? fmaxf(s_max[0], s_max[1]) : s_max[0];
+                    const bool fail = !(mn > 0.f);
+                    const bool ill = pass == 1 && sqrtf(mx) > a.cond_limit * sqrtf(mn);
                     if (!fail && !(ill && attempt == 0)) ok = true;
                     else if (attempt == 0 && pass == 1) third = true;
                     __syncthreads();
