@@ -112,7 +112,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             __syncthreads();
             if (warp < CT_DIAG_WARPS) {
                 float mn, mx;
-                ct_diag_block(sD, smem + CT_OFF_D, nbk, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                ct_diag_block<64>(sD, smem + CT_OFF_D, nbk, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
                 if (lane == 0 && (warp == 0 || (warp == 3 && nbk > 32))) {
                     s_min[warp / 3] = mx <= 3.0e38f ? fminf(s_min[warp / 3], mn) : -1.f;
                     s_max[warp / 3] = fmaxf(s_max[warp / 3], mx);

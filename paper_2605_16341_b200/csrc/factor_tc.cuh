@@ -50,7 +50,7 @@ constexpr int CT_OFF_D = 4 * CT_TILE;
 constexpr int CT_DG_LT = CT_NB * CT_LDD * 4;                   // work area of a diagonal block: the block itself first
 constexpr int CT_DG_BLK = CT_DG_LT + 32 * CT_LDT * 4;
 constexpr int CT_DG_S = CT_DG_BLK + 64 * 4;
-constexpr int CT_DG_BYTES = CT_DG_S + 8 * 32 * 4;
+constexpr int CT_DG_BYTES = CT_DG_S + 32 * 32 * 4;
 constexpr int CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;              // the block of the odd columns (the even ones': CT_OFF_D)
 constexpr int CT_SMEM_BYTES = CT_OFF_D2 + CT_NB * CT_LDD * 4 + 1024;     // + alignment of the tiles
 static_assert(2 * (CT_SMEM_BYTES + 2048) <= 228 * 1024, "two CTAs per multiprocessor");
@@ -66,8 +66,8 @@ __device__ __forceinline__ void ct_bar_sync(int id, int threads) {
 __device__ __forceinline__ void ct_bar_arrive(int id, int threads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-// named barriers (0: the whole CTA); CT_BAR_XT: two, by the parity of the column
-constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_X = 4, CT_BAR_XT = 5;
+// named barriers (0: the whole CTA); CT_BAR_XT: two, by the parity of the column; CT_BAR_HAND: four, by the panel
+constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_X = 4, CT_BAR_XT = 5, CT_BAR_HAND = 7, CT_BAR_JOIN = 11;
 
 __device__ __forceinline__ void ct_cp16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -171,15 +171,17 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 // elimination, a row per lane.  The columns are taken in panels of eight, whose 8 x 8 diagonal block every
 // lane factors for itself from shared memory (a chain of eight reciprocal square roots and 16 products, no shuffle
 // in it); then the lane solves its own eight entries and the panel's columns of L go to the others through LT
-// (LT[j][i] = L(i, j)).  What bounds it is this chain, about 500 cycles per panel, so everything else runs beside it:
+// (LT[j][i] = L(i, j)).  What bounds it is this chain, so everything else runs beside it: only the next
+// panel's columns are updated at once, the others while the next panel is being factored, and what is not needed for the
+// next panel by a warp that follows behind:
 //   first half (columns 0 .. 31)        second half
 //   warp 0  L11                         rows 0 .. 31 of L^{-T} beyond column 32
-//   warp 1  L21                         their sums  -X11^T L21^T, a panel ahead
+//   warp 1  L21                         their sums  -X11^T L21^T, ahead
 //   warp 2  rows 0 .. 31 of L^{-T}      rows 32 .. 63 of L^{-T}
-//   warp 3  D22 - L21 L21^T             L22
-// (Two 32-column factorisations by one warp with the columns passed by shuffle, triangular solves and the update
-// one after the other took 16 thousand cycles; fully unrolled they were also bound by instruction
-// fetch whenever another phase had evicted them.)
+//   warp 3  D22 - L21 L21^T, behind     L22
+// Measured alone, cycles for 64 columns: 11200 with all updates in the chain, 9300 so.  (Two 32-column
+// factorisations by one warp with the columns passed by shuffle, then triangular solves and the update
+// one after the other: 16 thousand.)
 __device__ __forceinline__ float ct_rsqrt(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -230,139 +232,144 @@ __device__ __forceinline__ void ct_rank8(float* a, const float (&z)[8], const fl
 }
 // `rest`: CT_DG_BYTES of shared memory whose first part may be sD itself.  dmin, dmax: smallest (-1: breakdown)
 // and largest pivot, in the lanes of warp 0 (one half) or warp 3 (two).
-template <class Out>
+// COLS: at most so many columns (16, 32 or 64).
+template <int COLS, class Out>
 __device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, int dw, int lane, float& dmin, float& dmax, Out out) {
     float* LT = reinterpret_cast<float*>(rest + CT_DG_LT);
     float* blk = reinterpret_cast<float*>(rest + CT_DG_BLK);
     float* sS = reinterpret_cast<float*>(rest + CT_DG_S);
-    const bool two = nbk > 32;
-    float a[32], z[8];
+    constexpr int NA = COLS < 32 ? COLS : 32;
+    const bool two = COLS > 32 && nbk > 32;
+    // cur: the lane's entries of the panel at hand, a: of the columns behind it (the first ones)
+    float a[NA], cur[8], z[8];
     dmin = 3.0e38f; dmax = 0.f;
     {
         // this lane's row: of D11, D21, the identity, D22
         const float* src = sD + (lane + (dw == 1 || dw == 3 ? 32 : 0)) * CT_LDD + (dw == 3 ? 32 : 0);
 #pragma unroll
-        for (int c = 0; c < 32; c += 4) {
+        for (int c = 0; c < NA; c += 4) {
             float4 v = make_float4(lane == c ? 1.f : 0.f, lane == c + 1 ? 1.f : 0.f, lane == c + 2 ? 1.f : 0.f, lane == c + 3 ? 1.f : 0.f);
             if (dw != 2 && (dw == 0 || two)) v = *reinterpret_cast<const float4*>(src + c);
             a[c] = v.x; a[c + 1] = v.y; a[c + 2] = v.z; a[c + 3] = v.w;
         }
     }
+    auto shift = [&]() {            // the first eight of a become the panel at hand
+#pragma unroll
+        for (int c = 0; c < 8; ++c) cur[c] = a[c];
+#pragma unroll
+        for (int c = 0; c < NA - 8; ++c) a[c] = a[8 + c];
+    };
+    auto put_blk = [&](int p) {     // rows 8 p .. + 7 of the warp that factors
+        if (lane / 8 == p) {
+            *reinterpret_cast<float4*>(blk + (lane % 8) * 8) = make_float4(cur[0], cur[1], cur[2], cur[3]);
+            *reinterpret_cast<float4*>(blk + (lane % 8) * 8 + 4) = make_float4(cur[4], cur[5], cur[6], cur[7]);
+        }
+    };
+    // One panel of the warps in step (w: the one that factors): cur -> z, and the update of the panel before (zp) in
+    // the columns beyond this panel; then store(z), and the next panel's columns.
+    auto panel = [&](int p, int np, bool factors, auto store) {
+        float zp[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) zp[j] = z[j];
+        ct_panel8(blk, cur, z, dmin, dmax);
+        if (NA > 16 && (p == 1 || p == 2)) {
+            const float* Lp = LT + (p - 1) * 8 * CT_LDT;
+            ct_rank8<2>(a, zp, Lp, 8 * (p + 1));
+            if (p == 1) ct_rank8<2>(a + NA / 4, zp, Lp, 8 * (p + 2));
+        }
+        store();
+        ct_bar_sync(CT_BAR_DIAG, 96);
+        if (p + 1 < np) {
+            shift();
+            ct_rank8<2>(cur, z, LT + p * 8 * CT_LDT, 8 * (p + 1));
+            if (factors) put_blk(p + 1);
+        }
+    };
     const int np = two ? 4 : (nbk + 7) / 8;
-    // first half; warps 0 to 2: the panel at hand is a[0 .. 7], the updates write eight registers down
-    for (int p = 0; p < np; ++p) {
-        if (dw == 0 && lane / 8 == p) {
-            *reinterpret_cast<float4*>(blk + (lane % 8) * 8) = make_float4(a[0], a[1], a[2], a[3]);
-            *reinterpret_cast<float4*>(blk + (lane % 8) * 8 + 4) = make_float4(a[4], a[5], a[6], a[7]);
-        }
-        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-        float* L = LT + p * 8 * CT_LDT;
-        if (dw < 3) {
-            ct_panel8(blk, a, z, dmin, dmax);
-            if (dw < 2) {
+    if (dw < 3) {
+        shift();
+        if (dw == 0) put_blk(0);
+#pragma unroll 1
+        for (int p = 0; p < np; ++p) {
+            ct_bar_sync(CT_BAR_DIAG, 96);
+            panel(p, np, dw == 0, [&]() {
+                if (dw < 2) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) L[j * CT_LDT + 32 * dw + lane] = z[j];
-            } else {
+                    for (int j = 0; j < 8; ++j) LT[(8 * p + j) * CT_LDT + 32 * dw + lane] = z[j];
+                    if (dw == 1 && two) ct_bar_arrive(CT_BAR_HAND + p, 64);
+                } else {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) sD[(8 * p + j) * CT_LDD + lane] = z[j];
-            }
-        }
-        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-        if (dw < 3) {
-            // (a group beyond the last column works on what is not used any more: branch-free but for whole groups)
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                if (g < 3 - p) {
-                    float t[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) t[c] = a[8 * (g + 1) + c];
-                    ct_rank8<2>(t, z, L, 8 * (p + g + 1));
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) a[8 * g + c] = t[c];
+                    for (int j = 0; j < 8; ++j) sD[(8 * p + j) * CT_LDD + lane] = z[j];
                 }
-            }
+            });
             if (dw == 2) out(lane, p, z);
-        } else if (two) {
+        }
+    } else if constexpr (COLS > 32) {
+        if (two) {
+#pragma unroll 1
+        for (int p = 0; p < 4; ++p) {
+            const float* L = LT + p * 8 * CT_LDT;
+            ct_bar_sync(CT_BAR_HAND + p, 64);
 #pragma unroll
             for (int j = 0; j < 8; ++j) z[j] = L[j * CT_LDT + 32 + lane];
             ct_rank8<8>(a, z, L, 32);
         }
+        }
     }
-    if (!two) {
-        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-        return;
-    }
-    // second half; LT's first 32 columns hold L22 from here on.  Warp 0: z of the panels so far in a; warp 1: the
-    // lane's row of X11^T
-    if (dw == 2) {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) a[c] = lane == c ? 1.f : 0.f;
-    } else if (dw == 1) {
+    if constexpr (COLS > 32) {
+    if (!two) return;
+    ct_bar_sync(CT_BAR_JOIN, 128);
+    // second half; LT's first 32 columns hold L22 from here on
+    if (dw == 1) {
+        // the lane's row of X11^T times L21^T, eight columns after the other
 #pragma unroll
         for (int j = 0; j < 32; ++j) a[j] = sD[j * CT_LDD + lane];
-    }
-    for (int p = 0; p < 4; ++p) {
-        if (dw == 3 && lane / 8 == p) {
-            *reinterpret_cast<float4*>(blk + (lane % 8) * 8) = make_float4(a[0], a[1], a[2], a[3]);
-            *reinterpret_cast<float4*>(blk + (lane % 8) * 8 + 4) = make_float4(a[4], a[5], a[6], a[7]);
-        } else if (dw == 1) {
+#pragma unroll 1
+        for (int p = 0; p < 4; ++p) {
             float t[8] = {};
 #pragma unroll
             for (int j = 0; j < 32; ++j) {
                 const float4 u = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 32 + 8 * p);
                 const float4 v = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 36 + 8 * p);
-                t[0] = fmaf(-a[j], u.x, t[0]); t[1] = fmaf(-a[j], u.y, t[1]); t[2] = fmaf(-a[j], u.z, t[2]); t[3] = fmaf(-a[j], u.w, t[3]);
-                t[4] = fmaf(-a[j], v.x, t[4]); t[5] = fmaf(-a[j], v.y, t[5]); t[6] = fmaf(-a[j], v.z, t[6]); t[7] = fmaf(-a[j], v.w, t[7]);
+                t[0] = fmaf(a[j], u.x, t[0]); t[1] = fmaf(a[j], u.y, t[1]); t[2] = fmaf(a[j], u.z, t[2]); t[3] = fmaf(a[j], u.w, t[3]);
+                t[4] = fmaf(a[j], v.x, t[4]); t[5] = fmaf(a[j], v.y, t[5]); t[6] = fmaf(a[j], v.z, t[6]); t[7] = fmaf(a[j], v.w, t[7]);
             }
 #pragma unroll
-            for (int c = 0; c < 8; ++c) sS[c * 32 + lane] = t[c];
+            for (int c = 0; c < 8; ++c) sS[(8 * p + c) * 32 + lane] = t[c];
+            ct_bar_arrive(CT_BAR_HAND + p, 64);
         }
-        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-        float* L = LT + p * 8 * CT_LDT;
+        return;
+    }
+    if (dw == 3) { dmin = 3.0e38f; dmax = 0.f; }
+    else {
+#pragma unroll
+        for (int c = 0; c < 32; ++c) a[c] = dw == 2 && lane == c ? 1.f : 0.f;
+    }
+    shift();
+    if (dw == 3) put_blk(0);
+    const float mn0 = dmin, mx0 = dmax;
+#pragma unroll 1
+    for (int p = 0; p < 4; ++p) {
+        ct_bar_sync(CT_BAR_DIAG, 96);
         if (dw == 0) {
-            // (sums of the panels before: the z so far are in shared memory, X(32 + ., lane))
-            float t[8];
+            ct_bar_sync(CT_BAR_HAND + p, 64);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) t[c] = sS[c * 32 + lane];
-            for (int q = 0; q < 8 * p; ++q) {
-                const float x = sD[(32 + q) * CT_LDD + lane];
-                const float4 u = *reinterpret_cast<const float4*>(LT + q * CT_LDT + 8 * p);
-                const float4 v = *reinterpret_cast<const float4*>(LT + q * CT_LDT + 8 * p + 4);
-                t[0] = fmaf(-x, u.x, t[0]); t[1] = fmaf(-x, u.y, t[1]); t[2] = fmaf(-x, u.z, t[2]); t[3] = fmaf(-x, u.w, t[3]);
-                t[4] = fmaf(-x, v.x, t[4]); t[5] = fmaf(-x, v.y, t[5]); t[6] = fmaf(-x, v.z, t[6]); t[7] = fmaf(-x, v.w, t[7]);
-            }
-#pragma unroll
-            for (int c = 0; c < 8; ++c) a[c] = t[c];
+            for (int c = 0; c < 8; ++c) cur[c] -= sS[(8 * p + c) * 32 + lane];
         }
-        if (dw != 1) {
-            float lo = 3.0e38f, hi = 0.f;
-            ct_panel8(blk, a, z, lo, hi);
-            if (dw == 3) { dmin = fminf(dmin, lo); dmax = fmaxf(dmax, hi); }
+        panel(p, 4, dw == 3, [&]() {
             if (dw == 3) {
 #pragma unroll
-                for (int j = 0; j < 8; ++j) L[j * CT_LDT + lane] = z[j];
+                for (int j = 0; j < 8; ++j) LT[(8 * p + j) * CT_LDT + lane] = z[j];
             } else {
                 float* dst = sD + (32 + 8 * p) * CT_LDD + (dw == 2 ? 32 : 0) + lane;
 #pragma unroll
                 for (int j = 0; j < 8; ++j) dst[j * CT_LDD] = z[j];
             }
-        }
-        ct_bar_sync(CT_BAR_DIAG, 32 * CT_DIAG_WARPS);
-        if (dw >= 2) {
-#pragma unroll
-            for (int g = 0; g < 3; ++g) {
-                if (g < 3 - p) {
-                    float t[8];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) t[c] = a[8 * (g + 1) + c];
-                    ct_rank8<2>(t, z, L, 8 * (p + g + 1));
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) a[8 * g + c] = t[c];
-                }
-            }
-        }
+        });
         if (dw == 2) out(32 + lane, 4 + p, z);
         else if (dw == 0) out(lane, 4 + p, z);
+    }
+    if (dw == 0) { dmin = mn0; dmax = mx0; }        // (what it reports is the first half)
     }
 }
 
@@ -759,7 +766,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                         for (int ch = 0; ch < 4; ++ch) out(32 + lane, ch, zero);
                     }
                     float mn, mx;
-                    ct_diag_block(diag_buf(k), smem + CT_OFF_D, nbk, dw, lane, mn, mx, out);
+                    ct_diag_block<64>(diag_buf(k), smem + CT_OFF_D, nbk, dw, lane, mn, mx, out);
                     // statistics: squared diagonal entries of L; two halves: warp 0's first, warp 3's second
                     if (lane == 0 && (dw == 0 || (dw == 3 && nbk > 32))) {
                         if (!(mx <= 3.0e38f)) mn = -1.f;

@@ -418,7 +418,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     __syncthreads();
                     if (warp < CT_DIAG_WARPS) {
                         float mn, mx;
-                        ct_diag_block(sD, smem, r, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                        ct_diag_block<R>(sD, smem, r, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
                         if (lane == 0 && (warp == 0 || (warp == 3 && r > 32))) {
                             s_min[warp / 3] = mx <= 3.0e38f ? mn : -1.f;
                             s_max[warp / 3] = mx;
