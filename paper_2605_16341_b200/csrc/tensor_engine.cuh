@@ -273,6 +273,39 @@ __device__ __forceinline__ void umma_any(uint32_t d_tmem, uint64_t adesc, uint64
     if (PAIR) umma_bf16_pair(d_tmem, adesc, bdesc, idesc, accumulate);
     else umma_bf16(d_tmem, adesc, bdesc, idesc, accumulate);
 }
+// The same with the descriptors given as halves (the high one is constant), always adding to D.
+template <bool PAIR>
+__device__ __forceinline__ void umma_add(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                         uint32_t idesc) {
+    if (PAIR)
+        asm volatile("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+                     "tcgen05.mma.cta_group::2.kind::f16 [%0], a, b, %5, 1;\n\t}"
+                     ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
+    else
+        asm volatile("{\n\t.reg .b64 a, b;\n\tmov.b64 a, {%1, %2};\n\tmov.b64 b, {%3, %4};\n\t"
+                     "tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %5, 1;\n\t}"
+                     ::"r"(d_tmem), "r"(a_lo), "r"(a_hi), "r"(b_lo), "r"(b_hi), "r"(idesc) : "memory");
+}
+template <bool PAIR>
+__device__ __forceinline__ void umma_halves(uint32_t d_tmem, uint32_t a_lo, uint32_t a_hi, uint32_t b_lo, uint32_t b_hi,
+                                            uint32_t idesc, uint32_t accumulate) {
+    umma_any<PAIR>(d_tmem, ((uint64_t)a_hi << 32) | a_lo, ((uint64_t)b_hi << 32) | b_lo, idesc, accumulate);
+}
+// NS 16-deep slices in one straight line: descriptors by additions, nothing else between the instructions.
+template <bool PAIR, int NS, bool THREE>
+__device__ __forceinline__ void umma_slices(uint32_t d, uint32_t a, uint32_t a_hi, uint32_t b, uint32_t b_hi, uint32_t a_step,
+                                            uint32_t b_step, uint32_t a_term, uint32_t b_term, uint32_t idesc, uint32_t accum) {
+#pragma unroll
+    for (int j = 0; j < NS; ++j) {
+        const uint32_t aj = a + j * a_step, bj = b + j * b_step;
+        if (j == 0) umma_halves<PAIR>(d, aj, a_hi, bj, b_hi, idesc, accum);
+        else umma_add<PAIR>(d, aj, a_hi, bj, b_hi, idesc);
+        if (THREE) {
+            umma_add<PAIR>(d, aj, a_hi, bj + b_term, b_hi, idesc);
+            umma_add<PAIR>(d, aj + a_term, a_hi, bj, b_hi, idesc);
+        }
+    }
+}
 template <bool PAIR>
 __device__ __forceinline__ void commit_any(uint32_t bar) {
     if (PAIR) umma_commit_pair(bar);
@@ -648,8 +681,90 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 }
             }
         }
+    } else if (warp == 1 && NMODE == N_IMG_MN) {
+        // ---------------- MMA issuer, MN-major N-side (products with B, Gram, apply) ----------------
+        // One thread runs the whole loop.  Its scalar work bounds the products of small rank (a few warps of other
+        // roles share its scheduler, so every instruction costs several cycles): what an instruction of the tensor
+        // core needs is a pair of 32-bit additions, whole pieces have no inner loop, and nothing is recomputed
+        // per depth block.  One 11008 x 4096 matrix, r = 32 / 128: 2240 / 2160 -> 1500 / 1550 cycles a
+        // depth block beside the waits for operands.
+        if (lane == 0 && crank == 0) {
+            constexpr uint32_t MROWS = PAIR ? 256u : 128u;
+            constexpr uint32_t a_step = A_MN ? (2048u >> 4) : (32u >> 4), b_step = 2048u >> 4;     // one 16-deep slice
+            constexpr uint32_t a_term = A_TERM_BYTES >> 4;
+            const uint64_t a_desc = A_MN ? smem_desc(0, 8192, 1024) : smem_desc(0, 16, 1024);
+            const uint64_t b_desc = smem_desc(0, group_stride, 1024);
+            const uint32_t a_hi = (uint32_t)(a_desc >> 32), b_hi = (uint32_t)(b_desc >> 32);
+            const uint32_t a_base = (uint32_t)a_desc + (smem_u32(a_ring) >> 4), b_base = (uint32_t)b_desc + (smem_u32(n_ring) >> 4);
+            const uint32_t a_slot = (uint32_t)g.a_slot_bytes >> 4, b_slot = (uint32_t)g.n_piece_bytes >> 4;
+            const uint32_t b_term = mn_term_stride >> 4;
+            // 256 columns further on: four 64-column groups, or this CTA's two with both terms (pairs)
+            const uint32_t b_block = (PAIR ? (uint32_t)n1_terms * 2u * group_stride : 4u * group_stride) >> 4;
+            const bool three = g.passes == 3;
+            const int a_slots = g.a_slots, n_slots = g.n_slots, ks = g.ks, kdim = g.Kdim;
+            const uint32_t idesc_256 = instr_desc(256u, A_MN ? 1u : 0u, 1u, fmt, MROWS);
+            int as = 0, ns = 0; uint32_t aph = 0, nph = 0;
+            int acc = 0; uint32_t acc_phase = 0;
+            bool ok = true;
+            for (int t = tile0; t < g.total_tiles && ok; t = next(t)) {
+                const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
+                if (!c.active) continue;
+                if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1, abort_flag)) { ok = false; break; }
+                // orders this tile's MMAs after the epilogue's tensor-memory loads.  (The operand waits
+                // below need no tcgen05 fence: the operands arrive through the async proxy or behind
+                // a proxy fence, and a fence per piece stalled the issuer for hundreds of cycles.)
+                tc_fence_after();
+                uint32_t d = tmem_base + acc * acc_stride, accum = 0;
+                const uint32_t idesc_last = instr_desc((uint32_t)((c.bn - 1) % 256 + 1), A_MN ? 1u : 0u, 1u, fmt, MROWS);
+                // depth blocks left of the chunk that has the accumulator at d
+                int chunk_left = A_BUF && g.acc_chunks > 1 ? g.kb_per_chunk : c.kb_end - c.kb_begin;
+                for (int kb = c.kb_begin; kb < c.kb_end && ok; ++kb) {
+                    if (chunk_left-- == 0) { chunk_left = g.kb_per_chunk - 1; d += (uint32_t)g.BN; accum = 0; }
+                    if (!mbar_wait(a_full0 + 8 * as, aph, abort_flag)) { ok = false; break; }
+                    uint32_t a = a_base + as * a_slot;
+                    for (int left = min(BK, kdim - kb * BK); left > 0; left -= ks) {
+                        if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
+                        uint32_t b = b_base + ns * b_slot, dc = d;
+                        const int depth = min(ks, left);
+                        for (int cols = c.bn; cols > 0; cols -= 256) {
+                            const uint32_t idesc = cols < 256 ? idesc_last : idesc_256;
+                            if (three && depth == 64) {
+                                umma_slices<PAIR, 4, true>(dc, a, a_hi, b, b_hi, a_step, b_step, a_term, b_term, idesc, accum);
+                            } else if (three && depth == 32) {
+                                umma_slices<PAIR, 2, true>(dc, a, a_hi, b, b_hi, a_step, b_step, a_term, b_term, idesc, accum);
+                            } else if (three && depth <= 16) {
+                                umma_slices<PAIR, 1, true>(dc, a, a_hi, b, b_hi, a_step, b_step, a_term, b_term, idesc, accum);
+                            } else if (!three && depth == 64) {
+                                umma_slices<PAIR, 4, false>(dc, a, a_hi, b, b_hi, a_step, b_step, a_term, b_term, idesc, accum);
+                            } else {
+                                for (int j = 0; j * 16 < depth; ++j) {
+                                    const uint32_t acc_j = j > 0 ? 1u : accum, aj = a + j * a_step, bj = b + j * b_step;
+                                    umma_halves<PAIR>(dc, aj, a_hi, bj, b_hi, idesc, acc_j);
+                                    if (three) {
+                                        umma_add<PAIR>(dc, aj, a_hi, bj + b_term, b_hi, idesc);
+                                        umma_add<PAIR>(dc, aj + a_term, a_hi, bj, b_hi, idesc);
+                                    }
+                                }
+                            }
+                            b += b_block; dc += 256;
+                        }
+                        accum = 1;
+                        a += (ks / 16) * a_step;
+                        commit_any<PAIR>(n_empty0 + 8 * ns);
+                        if (++ns == n_slots) { ns = 0; nph ^= 1; }
+                    }
+                    if (!ok) break;
+                    commit_any<PAIR>(a_empty0 + 8 * as);
+                    if (++as == a_slots) { as = 0; aph ^= 1; }
+                }
+                if (!ok) break;
+                commit_any<PAIR>(tfull0 + 8 * acc);
+                if (++acc == g.acc_bufs) { acc = 0; acc_phase ^= 1; }
+            }
+        }
+        __syncwarp();
     } else if (warp == 1) {
-        // ---------------- MMA issuer ----------------
+        // ---------------- MMA issuer, K-major N-side (fused pass) ----------------
         // One thread issues.  A tcgen05.mma of N = 256 occupies the tensor core for 128 cycles, so the
         // scalar work per instruction has to stay at a handful of operations: every descriptor is a
         // constant high part plus (shared address >> 4), advanced by additions only.
@@ -658,129 +773,82 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         bool ok = true;
         // descriptor high parts (layout, strides) and address units of 16 bytes
         const uint64_t a_hi = A_MN ? smem_desc(0, 8192, 1024) : smem_desc(0, 16, 1024);
-        const uint64_t n_hi = (NMODE == N_IMG_MN) ? smem_desc(0, group_stride, 1024) : smem_desc(0, 16, 1024);
+        const uint64_t n_hi = smem_desc(0, 16, 1024);
         const uint32_t a_slice16 = A_MN ? (2048u >> 4) : (32u >> 4);        // one 16-deep slice of the A tile
-        const uint32_t n_slice16 = (NMODE == N_IMG_MN) ? (2048u >> 4) : (32u >> 4);
-        const uint32_t a_term16 = A_TERM_BYTES >> 4;
-        const uint32_t n_term16 = ((NMODE == N_IMG_MN) ? mn_term_stride : (uint32_t)A_TERM_BYTES) >> 4;
+        const uint32_t n_slice16 = 32u >> 4;
         const uint32_t a_ring16 = smem_u32(a_ring) >> 4, n_ring16 = smem_u32(n_ring) >> 4;
         const uint32_t a_slot16 = (uint32_t)g.a_slot_bytes >> 4, n_slot16 = (uint32_t)g.n_piece_bytes >> 4;
-        const bool three = g.passes == 3;
         constexpr uint32_t MROWS = PAIR ? 256u : 128u;
-        // pairs: a 256-column block of the N-side is this CTA's two 64-column groups, both terms
-        const uint32_t n_block16 = (PAIR ? (uint32_t)n1_terms * 2u * group_stride : 4u * group_stride) >> 4;
         for (int t = tile0; t < g.total_tiles && ok && crank == 0; t = next(t)) {
             const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
             if (!c.active) continue;
             if (!mbar_wait(tempty0 + 8 * acc, acc_phase ^ 1, abort_flag)) { ok = false; break; }
-            // orders this tile's MMAs after the epilogue's tensor-memory loads.  (The operand waits
-            // below need no tcgen05 fence: the operands arrive through the async proxy or behind
-            // a proxy fence, and a fence per piece stalled the issuer for hundreds of cycles.)
-            tc_fence_after();
+            tc_fence_after();        // as in the issuer above
             const uint32_t dacc = tmem_base + acc * acc_stride;
             for (int kb = c.kb_begin; kb < c.kb_end && ok; ++kb) {
                 if (!mbar_wait(a_full0 + 8 * as, aph, abort_flag)) { ok = false; break; }
-                const uint64_t a_kb = a_hi + (a_ring16 + as * a_slot16);
-                uint32_t dkb = dacc;
-                int kb0 = c.kb_begin;                    // first depth block of the chunk that kb belongs to
-                if (A_BUF && g.acc_chunks > 1) {
-                    const int v = kb / g.kb_per_chunk;
-                    kb0 = v * g.kb_per_chunk;
-                    dkb += (uint32_t)(v * g.BN);
-                }
-                if (NMODE == N_IMG_MN) {
-                    const int pieces = mn_pieces(g, kb);
-                    const int per_piece = g.ks / 16;
-                    for (int sub = 0; sub < pieces && ok; ++sub) {
-                        if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
-                        if (lane == 0) {
-                            const uint64_t n_pc = n_hi + (n_ring16 + ns * n_slot16);
-                            const int k0 = kb * BK + sub * g.ks;
-                            const int nsl = (min(g.ks, g.Kdim - k0) + 15) / 16;
-                            for (int j = 0; j < nsl; ++j) {
-                                const uint64_t a0 = a_kb + (uint32_t)(sub * per_piece + j) * a_slice16;
-                                const uint64_t a1 = a0 + a_term16;
-                                const uint32_t accum = (kb > kb0 || sub > 0 || j > 0) ? 1u : 0u;
-                                uint64_t b0 = n_pc + (uint32_t)j * n_slice16;
-                                for (int cc = 0; cc < c.bn; cc += 256) {
-                                    const uint32_t idesc = instr_desc((uint32_t)min(256, c.bn - cc), A_MN ? 1u : 0u, 1u, fmt, MROWS);
-                                    umma_any<PAIR>(dkb + cc, a0, b0, idesc, accum);
-                                    if (three) {
-                                        umma_any<PAIR>(dkb + cc, a0, b0 + n_term16, idesc, 1u);
-                                        umma_any<PAIR>(dkb + cc, a1, b0, idesc, 1u);
-                                    }
-                                    b0 += n_block16;                        // next 256 columns
-                                }
+                const int chunks = (c.bn + 127) / 128;
+                const int nsl = min(4, (g.Kdim - kb * BK + 15) / 16);
+                for (int ch = 0; ch < chunks && ok; ++ch) {
+                    if (!k_piece_active(g, c, kb, ch)) continue;
+                    if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
+                    if (lane == 0) {
+                        const uint32_t sa = smem_u32(a_ring + as * g.a_slot_bytes);
+                        const uint32_t sn = smem_u32(n_ring + (size_t)ns * g.n_piece_bytes);
+                        // N of the instruction must be a multiple of 16: round a ragged last chunk up
+                        // (rows beyond the matrix are zero in the images; those columns of D are never stored)
+                        const uint32_t ncols = (uint32_t)((min(128, c.bn - ch * 128) + 15) / 16 * 16);
+                        const uint32_t idesc = instr_desc(ncols, A_MN ? 1u : 0u, 0u, fmt, MROWS);
+                        // Fused pass with single-term operands: the R piece and the Q piece lie back
+                        // to back in the slot (256 rows of one K-major tile) and their accumulators in
+                        // adjacent columns, so one N = 256 instruction serves both products and reads
+                        // the P slice from shared memory once.
+                        const bool both = EPI == EPI_K5 && g.passes == 1 && g.passes2 == 1 && ncols == 128 && g.BN == 128;
+                        const uint32_t idesc2 = instr_desc(256u, A_MN ? 1u : 0u, 0u, fmt, MROWS);
+                        if (both) {
+                            // one instruction per 16-deep slice; descriptors advanced by additions so
+                            // that the issuing thread spends a handful of operations per instruction
+                            uint64_t a0 = a_hi + (a_ring16 + as * a_slot16);
+                            uint64_t b0 = n_hi + (n_ring16 + ns * n_slot16);
+                            const uint32_t d1 = dacc + ch * 128;
+                            umma_any<PAIR>(d1, a0, b0, idesc2, kb > c.kb_begin ? 1u : 0u);
+                            for (int j = 1; j < nsl; ++j) {
+                                a0 += a_slice16; b0 += n_slice16;
+                                umma_any<PAIR>(d1, a0, b0, idesc2, 1u);
                             }
-                            commit_any<PAIR>(n_empty0 + 8 * ns);
                         }
-                        __syncwarp();
-                        if (++ns == g.n_slots) { ns = 0; nph ^= 1; }
-                    }
-                } else {
-                    const int chunks = (c.bn + 127) / 128;
-                    const int nsl = min(4, (g.Kdim - kb * BK + 15) / 16);
-                    for (int ch = 0; ch < chunks && ok; ++ch) {
-                        if (!k_piece_active(g, c, kb, ch)) continue;
-                        if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
-                        if (lane == 0) {
-                            const uint32_t sa = smem_u32(a_ring + as * g.a_slot_bytes);
-                            const uint32_t sn = smem_u32(n_ring + (size_t)ns * g.n_piece_bytes);
-                            // N of the instruction must be a multiple of 16: round a ragged last chunk up
-                            // (rows beyond the matrix are zero in the images; those columns of D are never stored)
-                            const uint32_t ncols = (uint32_t)((min(128, c.bn - ch * 128) + 15) / 16 * 16);
-                            const uint32_t idesc = instr_desc(ncols, A_MN ? 1u : 0u, 0u, fmt, MROWS);
-                            // Fused pass with single-term operands: the R piece and the Q piece lie back
-                            // to back in the slot (256 rows of one K-major tile) and their accumulators in
-                            // adjacent columns, so one N = 256 instruction serves both products and reads
-                            // the P slice from shared memory once.
-                            const bool both = EPI == EPI_K5 && g.passes == 1 && g.passes2 == 1 && ncols == 128 && g.BN == 128;
-                            const uint32_t idesc2 = instr_desc(256u, A_MN ? 1u : 0u, 0u, fmt, MROWS);
-                            if (both) {
-                                // one instruction per 16-deep slice; descriptors advanced by additions so
-                                // that the issuing thread spends a handful of operations per instruction
-                                uint64_t a0 = a_hi + (a_ring16 + as * a_slot16);
-                                uint64_t b0 = n_hi + (n_ring16 + ns * n_slot16);
-                                const uint32_t d1 = dacc + ch * 128;
-                                umma_any<PAIR>(d1, a0, b0, idesc2, kb > c.kb_begin ? 1u : 0u);
-                                for (int j = 1; j < nsl; ++j) {
-                                    a0 += a_slice16; b0 += n_slice16;
-                                    umma_any<PAIR>(d1, a0, b0, idesc2, 1u);
+                        // (In the general form below the descriptors are rebuilt per instruction on
+                        // purpose: its N = 128 instructions ran best when not issued back to back.)
+                        for (int j = 0; j < nsl && !both; ++j) {
+                            const uint64_t a0 = A_MN ? smem_desc(sa + j * 2048, 8192, 1024)
+                                                     : smem_desc(sa + j * 32, 16, 1024);
+                            const uint64_t a1 = A_MN ? smem_desc(sa + A_TERM_BYTES + j * 2048, 8192, 1024)
+                                                     : smem_desc(sa + A_TERM_BYTES + j * 32, 16, 1024);
+                            const uint64_t b0 = smem_desc(sn + j * 32, 16, 1024);
+                            const uint64_t b1 = smem_desc(sn + A_TERM_BYTES + j * 32, 16, 1024);
+                            const uint32_t accum = (kb > c.kb_begin || j > 0) ? 1u : 0u;
+                            const uint32_t d1 = dacc + ch * 128;
+                            umma_any<PAIR>(d1, a0, b0, idesc, accum);
+                            if (g.passes == 3) {
+                                umma_any<PAIR>(d1, a0, b1, idesc, 1u);
+                                umma_any<PAIR>(d1, a1, b0, idesc, 1u);
+                            }
+                            if (EPI == EPI_K5) {
+                                const uint32_t s2 = sn + n1_terms * A_TERM_BYTES;
+                                const uint64_t c0 = smem_desc(s2 + j * 32, 16, 1024);
+                                const uint64_t c1 = smem_desc(s2 + A_TERM_BYTES + j * 32, 16, 1024);
+                                const uint32_t d2 = dacc + g.BN;
+                                umma_any<PAIR>(d2, a0, c0, idesc, accum);
+                                if (g.passes2 == 3) {
+                                    umma_any<PAIR>(d2, a0, c1, idesc, 1u);
+                                    umma_any<PAIR>(d2, a1, c0, idesc, 1u);
                                 }
                             }
-                            // (In the general form below the descriptors are rebuilt per instruction on
-                            // purpose: its N = 128 instructions ran best when not issued back to back.)
-                            for (int j = 0; j < nsl && !both; ++j) {
-                                const uint64_t a0 = A_MN ? smem_desc(sa + j * 2048, 8192, 1024)
-                                                         : smem_desc(sa + j * 32, 16, 1024);
-                                const uint64_t a1 = A_MN ? smem_desc(sa + A_TERM_BYTES + j * 2048, 8192, 1024)
-                                                         : smem_desc(sa + A_TERM_BYTES + j * 32, 16, 1024);
-                                const uint64_t b0 = smem_desc(sn + j * 32, 16, 1024);
-                                const uint64_t b1 = smem_desc(sn + A_TERM_BYTES + j * 32, 16, 1024);
-                                const uint32_t accum = (kb > c.kb_begin || j > 0) ? 1u : 0u;
-                                const uint32_t d1 = dacc + ch * 128;
-                                umma_any<PAIR>(d1, a0, b0, idesc, accum);
-                                if (g.passes == 3) {
-                                    umma_any<PAIR>(d1, a0, b1, idesc, 1u);
-                                    umma_any<PAIR>(d1, a1, b0, idesc, 1u);
-                                }
-                                if (EPI == EPI_K5) {
-                                    const uint32_t s2 = sn + n1_terms * A_TERM_BYTES;
-                                    const uint64_t c0 = smem_desc(s2 + j * 32, 16, 1024);
-                                    const uint64_t c1 = smem_desc(s2 + A_TERM_BYTES + j * 32, 16, 1024);
-                                    const uint32_t d2 = dacc + g.BN;
-                                    umma_any<PAIR>(d2, a0, c0, idesc, accum);
-                                    if (g.passes2 == 3) {
-                                        umma_any<PAIR>(d2, a0, c1, idesc, 1u);
-                                        umma_any<PAIR>(d2, a1, c0, idesc, 1u);
-                                    }
-                                }
-                            }
-                            commit_any<PAIR>(n_empty0 + 8 * ns);
                         }
-                        __syncwarp();
-                        if (++ns == g.n_slots) { ns = 0; nph ^= 1; }
+                        commit_any<PAIR>(n_empty0 + 8 * ns);
                     }
+                    __syncwarp();
+                    if (++ns == g.n_slots) { ns = 0; nph ^= 1; }
                 }
                 if (!ok) break;
                 if (lane == 0) commit_any<PAIR>(a_empty0 + 8 * as);
@@ -1309,90 +1377,85 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         }
     } else if (A_BUF) {
         // ---------------- transform warps: A tile of B = M + G (Alg. 1, buffer step) ----------------
-        // 512 threads, two 8-element chunks each per 128 x 64 tile; the loads of the next two
-        // tiles are in flight while the current one is split and stored.
+        // 512 threads, two 8-element chunks each per 128 x 64 tile; four chunks (two tiles) are in flight
+        // while a thread splits and stores, three of them (as many bytes) with fp32 gradients.  They are 48 of the
+        // 80 registers that 22 warps leave a thread, and a load whose register is spilled is waited for at
+        // once: what else lives in the loop is two pointers and one offset, and only one chunk is split
+        // at a time.  Before, with indexes per chunk, two tiles of either type and both chunks split
+        // together, 88 bytes were spilled with bf16 gradients and 292 with fp32.  With the issuer above, one 11008 x 4096
+        // matrix, first and second product: r = 32 0.111 -> 0.092 and 0.100 -> 0.063 ms, r = 128 0.134 -> 0.106 and
+        // 0.126 -> 0.088; fp32 gradients, r = 32 0.184 -> 0.097 and 0.102 -> 0.068; six layers of 2048-wide matrices,
+        // r = 512 0.979 -> 0.869 and 1.145 -> 1.047.
         const int xt = threadIdx.x - 32 * (2 + NE);     // 0 .. 511
         int as = 0; uint32_t aph = 0;
         bool ok = true;
-        struct Raw { float4 m[2][2]; uint32_t gq[2][G_BF16 ? 4 : 8]; };
+        struct Raw { float4 m[2]; uint32_t gq[G_BF16 ? 4 : 8]; };
+        constexpr int NR = G_BF16 ? 4 : 3;        // chunks in flight: 48 registers either way
+        constexpr int ROUND = G_BF16 ? 2 : 3;     // tiles after which the chunks are back in the same registers
+        // chunk e of a thread.  A_BUF_ROW: operand row = B row, depth = B column: row xt / 8 + 64 e,
+        // columns k0 + 8 (xt % 8) .. + 7.  A_BUF_COL: operand row = B column, depth = B row (MN-major tile):
+        // row k0 + xt / 16 + 32 e, columns 8 (xt % 16) .. + 7.
+        constexpr int E_STEP = AMODE == A_BUF_ROW ? 64 : 32;      // rows of B between a thread's two chunks
+        const int xr = AMODE == A_BUF_ROW ? xt / 8 : xt / 16, xc = AMODE == A_BUF_ROW ? xt % 8 : xt % 16;
+        const uint32_t dst_off = AMODE == A_BUF_ROW ? xr * 128 + img_chunk_offset(xr, xc)
+                                                    : (xc / 8) * 8192 + xr * 128 + img_chunk_offset(xr, xc % 8);
         for (int t = tile0; t < g.total_tiles && ok; t += tstride) {
             const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
             if (!c.active) continue;
             const MatWork& w = batch.w[c.b];
-            const int64_t ld = g.ld;
-            int64_t src_idx[2]; bool row_ok[2]; int kofs[2]; uint32_t dst_off[2];
+            const int64_t base = AMODE == A_BUF_ROW ? ((int64_t)c.mt * BM + xr) * g.ld + xc * 8
+                                                    : (int64_t)xr * g.ld + (int64_t)c.mt * BM + xc * 8;
+            const float* Mp = w.M + base;
+            const unsigned char* Gp = reinterpret_cast<const unsigned char*>(w.G) + base * (G_BF16 ? 2 : 4);
+            // rows left from this thread's first one on (columns of B in the other operand: a multiple of 8, all or none)
+            const int rleft = AMODE == A_BUF_ROW ? g.Mrows - c.mt * BM - xr : (c.mt * BM + xc * 8 < g.Mrows ? g.Kdim - xr : 0);
+            const int kend = c.kb_end;
+            auto fetch = [&](Raw& r, int kb, int e) {
+                const bool in = AMODE == A_BUF_ROW ? (e * E_STEP < rleft && kb * BK + xc * 8 < g.Kdim)
+                                                   : kb * BK + e * E_STEP < rleft;
+                if (in) {
+                    const int64_t idx = AMODE == A_BUF_ROW ? (int64_t)(e * E_STEP) * g.ld + kb * BK
+                                                           : (int64_t)(kb * BK + e * E_STEP) * g.ld;
+                    const float4* mp = reinterpret_cast<const float4*>(Mp + idx);
+                    r.m[0] = mp[0]; r.m[1] = mp[1];
+                    const uint4* gp = reinterpret_cast<const uint4*>(Gp + idx * (G_BF16 ? 2 : 4));
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const int q = xt + 512 * e;
-                if (AMODE == A_BUF_ROW) {
-                    // operand row = B row, depth = B column: chunk (rho, ch) = B[i0+rho][k0+8ch .. +7]
-                    const int rho = q / 8, ch = q % 8;
-                    const int64_t gr = (int64_t)c.mt * BM + rho;
-                    row_ok[e] = gr < g.Mrows;
-                    src_idx[e] = gr * ld + ch * 8;           // + k0
-                    kofs[e] = ch * 8;
-                    dst_off[e] = rho * 128 + img_chunk_offset(rho, ch);
+                    for (int i = 0; i < (G_BF16 ? 1 : 2); ++i) {
+                        const uint4 u = gp[i];
+                        r.gq[4 * i] = u.x; r.gq[4 * i + 1] = u.y; r.gq[4 * i + 2] = u.z; r.gq[4 * i + 3] = u.w;
+                    }
                 } else {
-                    // operand row = B column, depth = B row (MN-major tile):
-                    // chunk (k, cj) = B[k0+k][j0+8cj .. +7]
-                    const int k = q / 16, cj = q % 16;
-                    const int64_t gc = (int64_t)c.mt * BM + cj * 8;
-                    row_ok[e] = gc < g.Mrows;                // Mrows = number of B columns, a multiple of 8
-                    src_idx[e] = (int64_t)k * ld + gc;       // + k0 * ld
-                    kofs[e] = k;
-                    dst_off[e] = (cj / 8) * 8192 + k * 128 + img_chunk_offset(k, cj % 8);
-                }
-            }
-            auto fetch = [&](Raw& r, int kb) {
-                const int64_t k0 = (int64_t)kb * BK;
+                    r.m[0] = r.m[1] = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    const bool okk = row_ok[e] && (k0 + kofs[e] < g.Kdim);
-                    if (okk) {
-                        const int64_t idx = src_idx[e] + (AMODE == A_BUF_ROW ? k0 : k0 * ld);
-                        const float4* mp = reinterpret_cast<const float4*>(w.M + idx);
-                        r.m[e][0] = mp[0]; r.m[e][1] = mp[1];
-                        if constexpr (G_BF16) {
-                            const uint4 u = *reinterpret_cast<const uint4*>(reinterpret_cast<const __nv_bfloat16*>(w.G) + idx);
-                            r.gq[e][0] = u.x; r.gq[e][1] = u.y; r.gq[e][2] = u.z; r.gq[e][3] = u.w;
-                        } else {
-                            const uint4* gp = reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(w.G) + idx);
-                            const uint4 u0 = gp[0], u1 = gp[1];
-                            r.gq[e][0] = u0.x; r.gq[e][1] = u0.y; r.gq[e][2] = u0.z; r.gq[e][3] = u0.w;
-                            r.gq[e][4] = u1.x; r.gq[e][5] = u1.y; r.gq[e][6] = u1.z; r.gq[e][7] = u1.w;
-                        }
-                    } else {
-                        r.m[e][0] = r.m[e][1] = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-                        for (int i = 0; i < (G_BF16 ? 4 : 8); ++i) r.gq[e][i] = 0u;
-                    }
+                    for (int i = 0; i < (G_BF16 ? 4 : 8); ++i) r.gq[i] = 0u;
                 }
             };
-            // split the tile held in r into the two bf16 terms
-            auto split_raw = [&](const Raw& r, uint4 (&t0)[2], uint4 (&t1)[2]) {
+            // split a chunk into the two bf16 terms and store them
+            auto split_store = [&](const Raw& r, unsigned char* dst) {
+                float gv[8];
+                if constexpr (G_BF16) {
 #pragma unroll
-                for (int e = 0; e < 2; ++e) {
-                    float gv[8];
-                    if constexpr (G_BF16) {
+                    for (int i = 0; i < 4; ++i) { gv[2 * i] = bf16lo_to_f32(r.gq[i]); gv[2 * i + 1] = bf16hi_to_f32(r.gq[i]); }
+                } else {
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) { gv[2 * i] = bf16lo_to_f32(r.gq[e][i]); gv[2 * i + 1] = bf16hi_to_f32(r.gq[e][i]); }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) gv[i] = __uint_as_float(r.gq[e][i]);
-                    }
-                    const float v[8] = {r.m[e][0].x + gv[0], r.m[e][0].y + gv[1], r.m[e][0].z + gv[2], r.m[e][0].w + gv[3],
-                                        r.m[e][1].x + gv[4], r.m[e][1].y + gv[5], r.m[e][1].z + gv[6], r.m[e][1].w + gv[7]};
-                    split8(v, t0[e], t1[e]);
+                    for (int i = 0; i < 8; ++i) gv[i] = __uint_as_float(r.gq[i]);
                 }
+                const float v[8] = {r.m[0].x + gv[0], r.m[0].y + gv[1], r.m[0].z + gv[2], r.m[0].w + gv[3],
+                                    r.m[1].x + gv[4], r.m[1].y + gv[5], r.m[1].z + gv[6], r.m[1].w + gv[7]};
+                uint4 t0, t1;
+                split8(v, t0, t1);
+                *reinterpret_cast<uint4*>(dst) = t0;
+                *reinterpret_cast<uint4*>(dst + A_TERM_BYTES) = t1;
             };
-            // wait for the slot, store the tile, signal the MMA issuer
-            auto store = [&](const uint4 (&t0)[2], const uint4 (&t1)[2]) -> bool {
+            Raw r[NR];               // chunk i of the tile sequence (two per tile) is in r[i % NR]
+            // tile kb, the u-th of a round: wait for the slot, turn both chunks into terms, signal the MMA issuer
+            auto tile = [&](int u, int kb) -> bool {
                 if (!mbar_wait(a_empty0 + 8 * as, aph ^ 1, abort_flag)) return false;
-                unsigned char* sa = a_ring + as * g.a_slot_bytes;
+                unsigned char* dst = a_ring + as * g.a_slot_bytes + dst_off;
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
-                    *reinterpret_cast<uint4*>(sa + dst_off[e]) = t0[e];
-                    *reinterpret_cast<uint4*>(sa + A_TERM_BYTES + dst_off[e]) = t1[e];
+                    split_store(r[(2 * u + e) % NR], dst + e * E_STEP * 128);
+                    if (kb + (e + NR) / 2 < kend) fetch(r[(2 * u + e) % NR], kb + (e + NR) / 2, (e + NR) % 2);
                 }
                 fence_async_smem();
                 __syncwarp();
@@ -1400,19 +1463,13 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 if (++as == g.a_slots) { as = 0; aph ^= 1; }
                 return true;
             };
-            Raw r0, r1;
-            fetch(r0, c.kb_begin);
-            if (c.kb_begin + 1 < c.kb_end) fetch(r1, c.kb_begin + 1);
-            for (int kb = c.kb_begin; kb < c.kb_end && ok; kb += 2) {
-                uint4 t0[2], t1[2];
-                split_raw(r0, t0, t1);
-                if (kb + 2 < c.kb_end) fetch(r0, kb + 2);
-                if (!store(t0, t1)) { ok = false; break; }
-                if (kb + 1 < c.kb_end) {
-                    split_raw(r1, t0, t1);
-                    if (kb + 3 < c.kb_end) fetch(r1, kb + 3);
-                    if (!store(t0, t1)) { ok = false; break; }
-                }
+#pragma unroll
+            for (int i = 0; i < NR; ++i)
+                if (c.kb_begin + i / 2 < kend) fetch(r[i], c.kb_begin + i / 2, i % 2);
+            for (int kb = c.kb_begin; kb < kend && ok; kb += ROUND) {
+#pragma unroll
+                for (int u = 0; u < ROUND; ++u)
+                    if (ok && kb + u < kend) ok = tile(u, kb + u);
             }
         }
     }
