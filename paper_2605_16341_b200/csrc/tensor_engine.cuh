@@ -1107,15 +1107,6 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
             // accumulator slabs go through a swizzled staging block so that global accesses run
             // along rows (8 lanes x 16 bytes per row).
             const int half = (warp - 2) / 4;
-            auto next_tile = [&](int t) {
-                for (t += tstride; t < g.total_tiles; t += tstride)
-                    if (decode_tile<EPI>(batch, g, t, scache, crank).active) return t;
-                return g.total_tiles;
-            };
-            // the slabs of this warp in order: (tile, 0), (tile, 1), (next tile, 0), ...
-            auto advance = [&](int& t, int& slab) {
-                if (++slab == 2) { slab = 0; t = next_tile(t); }
-            };
             if constexpr (XG == 3) {
                 // bf16 G and X.  The 32 x 32 slabs of M, G, X come in by asynchronous copies
                 // (cp.async, no registers) into a per-warp buffer, one or two slabs ahead; each
@@ -1129,33 +1120,48 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 const int hrow = lane / 4, hch = lane % 4;      // G, X: 8 rows x 4 chunks per step
                 auto m_off = [](int r, int ch) { return r * 128 + ((ch ^ (r & 7)) << 4); };
                 auto h_off = [](int r, int ch) { return r * 64 + ((ch ^ ((r >> 1) & 3)) << 4); };
-                auto issue = [&](int t, int slab, unsigned char* buf) {
-                    const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
-                    const MatWork& w = batch.w[c.b];
-                    const int64_t gj0 = (int64_t)c.n0 + half * 64 + slab * 32;
-                    const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
+                // the same for this lane's chunk of step `it` (rows 4 it + mrow and 8 it + hrow)
+                const int m_off0 = m_off(mrow, mch), h_off0 = h_off(hrow, hch);
+                auto m_step = [&](int it) { return (m_off0 ^ ((it & 1) << 6)) + it * 512; };
+                auto h_step = [&](int it) { return h_off0 + it * 512; };
+                // The slabs of this warp in order: (tile, 0), (tile, 1), (next tile, 0), ...  A warp has little time
+                // per slab (14 KB, 8 warps: at the rate of the memory about 4800 cycles), and most of what it executed
+                // was addresses: a tile is decoded once now, rows are reached by additions.  11008 x 4096 at
+                // r = 32 / 256 0.123 / 0.132 -> 0.118 / 0.122 ms, six layers of 2048-wide matrices 0.840 / 0.866 -> 0.798 / 0.792.
+                struct Slab { int t, slab, b, i0, j0; };
+                auto advance = [&](Slab& s) {
+                    if (s.slab == 0) { s.slab = 1; s.j0 += 32; return; }
+                    for (s.t += tstride; s.t < g.total_tiles; s.t += tstride) {
+                        const TileCoord c = decode_tile<EPI>(batch, g, s.t, scache, crank);
+                        if (!c.active) continue;
+                        s.slab = 0; s.b = c.b; s.i0 = c.mt * BM + quarter * 32; s.j0 = c.n0 + half * 64;
+                        return;
+                    }
+                };
+                const int64_t ld = g.ld;
+                auto issue = [&](const Slab& s, unsigned char* buf) {
+                    const MatWork& w = batch.w[s.b];
                     const uint32_t sb = smem_u32(buf);
+                    const float* Mp = w.M + (s.i0 + mrow) * ld + s.j0 + mch * 4;
+                    const int mleft = s.j0 + mch * 4 < g.Ncols ? g.Mrows - s.i0 - mrow : 0;
 #pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const int r = it * 4 + mrow;
-                        const int64_t gi = gi0 + r, gj = gj0 + mch * 4;
-                        if (gi < g.Mrows && gj < g.Ncols) cp_async16(sb + m_off(r, mch), w.M + gi * g.ld + gj);
-                    }
+                    for (int it = 0; it < 8; ++it)
+                        if (it * 4 < mleft) cp_async16(sb + m_step(it), Mp + it * 4 * ld);
+                    const int64_t hidx = (s.i0 + hrow) * ld + s.j0 + hch * 8;
+                    const __nv_bfloat16* Gp = reinterpret_cast<const __nv_bfloat16*>(w.G) + hidx;
+                    const __nv_bfloat16* Xp = reinterpret_cast<const __nv_bfloat16*>(w.X) + hidx;
+                    const int hleft = s.j0 + hch * 8 < g.Ncols ? g.Mrows - s.i0 - hrow : 0;
 #pragma unroll
-                    for (int it = 0; it < 4; ++it) {
-                        const int r = it * 8 + hrow;
-                        const int64_t gi = gi0 + r, gj = gj0 + hch * 8;
-                        if (gi < g.Mrows && gj < g.Ncols) {
-                            const int64_t idx = gi * g.ld + gj;
-                            cp_async16(sb + 4096 + h_off(r, hch), reinterpret_cast<const __nv_bfloat16*>(w.G) + idx);
-                            cp_async16(sb + 6144 + h_off(r, hch), reinterpret_cast<const __nv_bfloat16*>(w.X) + idx);
+                    for (int it = 0; it < 4; ++it)
+                        if (it * 8 < hleft) {
+                            cp_async16(sb + 4096 + h_step(it), Gp + it * 8 * ld);
+                            cp_async16(sb + 6144 + h_step(it), Xp + it * 8 * ld);
                         }
-                    }
                     cp_async_commit();
                 };
-                auto process = [&](int t, int slab, unsigned char* buf) -> bool {
-                    const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
-                    const MatWork& w = batch.w[c.b];
+                auto process = [&](const Slab& s, unsigned char* buf) -> bool {
+                    const MatWork& w = batch.w[s.b];
+                    const int slab = s.slab;
                     const float efb = g.fp16 ? g.ef_b * *reinterpret_cast<const float*>(w.scratch + g.rscale_off) : g.ef_b;
                     if (slab == 0) {
                         if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) return false;
@@ -1211,46 +1217,52 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         if (++acc == g.acc_bufs) { acc = 0; acc_phase ^= 1; }
                     }
                     __syncwarp();
-                    const int64_t gj0 = (int64_t)c.n0 + half * 64 + slab * 32;
-                    const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
+                    float* Mp = w.M + (s.i0 + mrow) * ld + s.j0 + mch * 4;
+                    const int mleft = s.j0 + mch * 4 < g.Ncols ? g.Mrows - s.i0 - mrow : 0;
 #pragma unroll
-                    for (int it = 0; it < 8; ++it) {
-                        const int r = it * 4 + mrow;
-                        const int64_t gi = gi0 + r, gj = gj0 + mch * 4;
-                        if (gi < g.Mrows && gj < g.Ncols)
-                            *reinterpret_cast<float4*>(w.M + gi * g.ld + gj) = *reinterpret_cast<const float4*>(buf + m_off(r, mch));
-                    }
+                    for (int it = 0; it < 8; ++it)
+                        if (it * 4 < mleft)
+                            *reinterpret_cast<float4*>(Mp + it * 4 * ld) = *reinterpret_cast<const float4*>(buf + m_step(it));
+                    __nv_bfloat16* Xp = reinterpret_cast<__nv_bfloat16*>(w.X) + (s.i0 + hrow) * ld + s.j0 + hch * 8;
+                    const int hleft = s.j0 + hch * 8 < g.Ncols ? g.Mrows - s.i0 - hrow : 0;
 #pragma unroll
-                    for (int it = 0; it < 4; ++it) {
-                        const int r = it * 8 + hrow;
-                        const int64_t gi = gi0 + r, gj = gj0 + hch * 8;
-                        if (gi < g.Mrows && gj < g.Ncols)
-                            *reinterpret_cast<uint4*>(reinterpret_cast<__nv_bfloat16*>(w.X) + gi * g.ld + gj) =
-                                *reinterpret_cast<const uint4*>(buf + 6144 + h_off(r, hch));
-                    }
+                    for (int it = 0; it < 4; ++it)
+                        if (it * 8 < hleft)
+                            *reinterpret_cast<uint4*>(Xp + it * 8 * ld) = *reinterpret_cast<const uint4*>(buf + 6144 + h_step(it));
                     __syncwarp();
                     return true;
                 };
-                int t = next_tile(tile0 - tstride), slab = 0, ib = 0;
-                if (t < g.total_tiles) issue(t, slab, bufs);
-                while (t < g.total_tiles) {
-                    int t2 = t, slab2 = slab;
-                    advance(t2, slab2);
+                Slab cur{tile0 - tstride, 1, 0, 0, 0};
+                int ib = 0;
+                advance(cur);
+                if (cur.t < g.total_tiles) issue(cur, bufs);
+                while (cur.t < g.total_tiles) {
+                    Slab nxt = cur;
+                    advance(nxt);
                     if (nbuf == 2) {
-                        if (t2 < g.total_tiles) issue(t2, slab2, bufs + (ib ^ 1) * STAGING_BYTES_PER_WARP);
+                        if (nxt.t < g.total_tiles) issue(nxt, bufs + (ib ^ 1) * STAGING_BYTES_PER_WARP);
                         else cp_async_commit();
                         cp_async_wait<1>();
                     } else {
                         cp_async_wait<0>();
                     }
                     __syncwarp();
-                    if (!process(t, slab, bufs + ib * STAGING_BYTES_PER_WARP)) break;
+                    if (!process(cur, bufs + ib * STAGING_BYTES_PER_WARP)) break;
                     if (nbuf == 2) ib ^= 1;
-                    else if (t2 < g.total_tiles) issue(t2, slab2, bufs);
-                    t = t2; slab = slab2;
+                    else if (nxt.t < g.total_tiles) issue(nxt, bufs);
+                    cur = nxt;
                 }
                 cp_async_wait<0>();
             } else {
+            auto next_tile = [&](int t) {
+                for (t += tstride; t < g.total_tiles; t += tstride)
+                    if (decode_tile<EPI>(batch, g, t, scache, crank).active) return t;
+                return g.total_tiles;
+            };
+            // the slabs of this warp in order: (tile, 0), (tile, 1), (next tile, 0), ...
+            auto advance = [&](int& t, int& slab) {
+                if (++slab == 2) { slab = 0; t = next_tile(t); }
+            };
             unsigned char* S1 = staging + (warp - 2) * STAGING_BYTES_PER_WARP;
             unsigned char* S2 = S1 + 4096;
             const int rl = lane / 8, cq = lane % 8;      // row within a step, 4-column group
@@ -1705,8 +1717,12 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     g.epi_bufs = 1;
     if (EPI == tc::EPI_K5) {
         // the fused pass: 64 KB of A slots (four single-term ones or two two-term ones) and one
-        // epilogue buffer per warp (a second one, paid for with ring slots, measured slower)
+        // epilogue buffer per warp.  bf16 G and X in single terms, ranks below 512: a second buffer, paid for with an
+        // A slot and three N slots; the update is bound by bytes in flight until the products take as long.
+        // 11008 x 4096, one buffer -> two, before the leaner update: r = 32 0.141 -> 0.124 ms, 256 0.149 -> 0.131,
+        // 448 0.152 -> 0.148, 512 0.154 -> 0.160.
         g.a_slots = (a_terms == 1) ? 4 : 2;
+        if (XG == 3 && a_terms == 1 && g.k_blocks < 8) { g.a_slots = 3; g.epi_bufs = 2; }
     }
     if (NMODE == tc::N_IMG_MN) {
         if (pair) {

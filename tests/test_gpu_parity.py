@@ -158,6 +158,15 @@ def test_small_rank_qr_edges(shape, mode, dt):
     one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_TENSOR)
 
 
+# the fused pass with two epilogue buffers per warp and, from r = 512 on, one: several tiles per CTA pair, ragged last
+# tiles on either side, the last rank of the first form and the first of the second
+@pytest.mark.parametrize("shape", [(2200, 2056, 16), (600, 712, 448), (700, 520, 512)])
+def test_fused_pass_buffer_edges(shape):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, BF16, BF16, seed=m + n + r)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR, passes={2: 1, 3: 1})
+
+
 @pytest.mark.parametrize("shape", [(384, 640, 64), (1000, 264, 128), (136, 2056, 32), (640, 384, 272)])
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("m_scale", [0.3, 3e-4, 300.0])
