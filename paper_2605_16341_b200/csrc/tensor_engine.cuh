@@ -1775,25 +1775,42 @@ inline tc::Dest dest_none() {
 // Multiprocessors that the rules below count on: a constant, so that workspace sizes need no device.
 constexpr int SPLIT_SMS = 148;
 
+// Depth blocks that a launch takes one after the other when `tiles` row tiles run in `chunks` parts each: waves
+// times blocks per part, with two more for filling and emptying a part's pipeline.
+inline int64_t product_depth(int64_t tiles, int chunks, int kb) {
+    const int64_t waves = (tiles * chunks + SPLIT_SMS - 1) / SPLIT_SMS;
+    return waves * ((kb + chunks - 1) / chunks + 2);
+}
+// ... and what writing and adding up the partial results costs in the same unit (about a microsecond).
+inline int64_t partial_cost(int64_t tiles, int chunks, int r) { return 4 + tiles * chunks * r / 6000; }
+
 // Depth split of the two products with the buffer.  With one matrix (or a few) in a call and a
-// small rank, the output has too few row tiles for the device (16 pairs for a 4096-wide factor)
-// and every one of them runs over the whole depth.  The depth is therefore cut into chunks whose
+// small rank, the output has too few row tiles for the device, or one wave and a bit (a 4096-wide factor 32, an
+// 11008-wide one 86), and every one of them runs over the whole depth.  The depth is therefore cut into chunks whose
 // results are added in a fixed order.  Their number depends on the plan only (rank, rows of the result,
 // depth), so that a matrix gets the same bits alone and in any group; ranks above 256 have one.  Where
-// the row tiles of a launch leave the device idle the chunks run as tiles of their own and leave
-// fp32 partial results in memory; where they do not, one tile runs through all chunks with an
+// it shortens a launch the chunks run as tiles of their own and leave
+// fp32 partial results in memory; where it does not, one tile runs through all chunks with an
 // accumulator each, side by side in tensor memory (at most 512 columns: ranks up to 128), and the epilogue
 // adds them up.
+// Up to r = 128 the number is the one that makes the launch of one matrix shortest by the two counts above.  Measured
+// against as many chunks as fit 74 pairs of tiles, none from 37 on: 11008 x 4096, first product, r = 32 0.090 -> 0.074 ms,
+// r = 64 0.091 -> 0.086; 20480 x 4096 r = 32 0.170 -> 0.127, r = 128 0.198 -> 0.176.  Fewer chunks at r = 128, so that two
+// sets of accumulators fit, gain 2 % in a group of 2048-wide matrices and lose 50 % alone (4096 x 4096 0.051 -> 0.070).
 inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     if (r > 256) return 1;
-    const int tiles = (int)((out_rows + 255) / 256);
     const int kb = (int)((depth + tc::BK - 1) / tc::BK);
-    if (tiles >= 37) return 1;
-    int want;
+    int want = 1;
     if (r <= 128) {
-        want = std::min({r <= 64 ? 8 : 4, 74 / tiles, kb / 4});
+        const int64_t tiles = (out_rows + tc::BM - 1) / tc::BM;
+        int64_t best = product_depth(tiles, 1, kb);
+        for (int v = 2; v <= std::min(r <= 64 ? 8 : 4, kb / 4); ++v) {
+            const int64_t cost = product_depth(tiles, v, kb) + partial_cost(tiles, v, r);
+            if (cost < best) { best = cost; want = v; }
+        }
     } else {
-        if (kb < 32) return 1;
+        const int tiles = (int)((out_rows + 255) / 256);
+        if (tiles >= 37 || kb < 32) return 1;
         want = std::min({8, 74 / tiles, kb / 8});
     }
     if (want < 2) return 1;
@@ -1801,13 +1818,14 @@ inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     return (kb + per - 1) / per;             // every chunk non-empty
 }
 // Partial results in memory of a product in a call of `matrices`: the chunks, or 1 where they stay in tensor memory.
-// The line is where the unsplit row tiles fill half of the device.  Measured (before: always in memory, added
-// up, packed and squared by three kernels): 154 matrices of a 1.1B model at r = 128 9.7 -> 8.6 ms a step; one
-// 4096 x 4096 matrix at r = 256, three kernels in one, 0.633 -> 0.609 ms.
+// Measured (before: always in memory, added up, packed and squared by three kernels): 154 matrices of a 1.1B model
+// at r = 128 9.7 -> 8.6 ms a step; one 4096 x 4096 matrix at r = 256, three kernels in one, 0.633 -> 0.609 ms.
 inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices) {
     const int chunks = buffer_chunks(r, out_rows, depth);
-    if (r > 128) return chunks;
-    return (int64_t)matrices * ((out_rows + tc::BM - 1) / tc::BM) * 2 <= SPLIT_SMS ? chunks : 1;
+    if (r > 128 || chunks == 1) return chunks;
+    const int64_t tiles = matrices * ((out_rows + tc::BM - 1) / tc::BM);
+    const int kb = (int)((depth + tc::BK - 1) / tc::BK);
+    return product_depth(tiles, chunks, kb) + partial_cost(tiles, chunks, r) < product_depth(tiles, 1, kb) ? chunks : 1;
 }
 
 __global__ void gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit,

@@ -368,7 +368,7 @@ def test_factor_kernel_forms_agree_bit_for_bit(shape, count):
 # the one-kernel QR with sixteen, four and one parts of a factor per CTA, and the products' depth chunks as
 # tiles of their own (the matrix alone) and in one tile (the call of many), with the image and the fp32 result
 @pytest.mark.parametrize("shape,count", [((1152, 136, 32), 150), ((1152, 136, 32), 70), ((2000, 144, 16), 150), ((520, 264, 48), 150),
-                                         ((768, 1024, 128), 150), ((1100, 648, 80), 40)])
+                                         ((768, 1024, 128), 150), ((1100, 648, 80), 40), ((10000, 2048, 32), 3)])
 def test_small_rank_qr_and_depth_chunks_agree_bit_for_bit(shape, count):
     test_factor_kernel_forms_agree_bit_for_bit(shape, count)
 
