@@ -39,6 +39,7 @@ constexpr int MAX_A_SLOTS = 4;
 constexpr int MAX_N_SLOTS = 6;
 constexpr int NUM_XF_WARPS = 16;             // transform warps of the kernels that form B = M + G
 constexpr int STAGING_BYTES_PER_WARP = 8192; // epilogue staging: one 32 x 64 fp32 block (or M, G, X slabs) per warp
+constexpr int BUF_STAGING_BYTES = 4096;      // the same for the products with B: one 32 x 32 fp32 block per warp
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // about two seconds
 
@@ -524,7 +525,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     unsigned char* a_ring = smem;
     unsigned char* n_ring = smem + g.a_slots * g.a_slot_bytes;
     unsigned char* staging = n_ring + (size_t)g.n_slots * g.n_piece_bytes;
-    unsigned char* tail = staging + ((EPI == EPI_K5 || !A_BUF) ? NE * g.epi_bufs * STAGING_BYTES_PER_WARP : 0);
+    unsigned char* tail = staging + NE * (A_BUF ? BUF_STAGING_BYTES : g.epi_bufs * STAGING_BYTES_PER_WARP);
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
     const uint32_t a_full0 = smem_u32(bars), a_empty0 = a_full0 + 8 * MAX_A_SLOTS;
     const uint32_t n_full0 = a_empty0 + 8 * MAX_A_SLOTS, n_empty0 = n_full0 + 8 * MAX_N_SLOTS;
@@ -891,75 +892,95 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 float* csq = d.colsq ? reinterpret_cast<float*>(w.scratch + g.colsq_off) +
                                            (int64_t)(c.mt * 4 + quarter) * g.Ncols : nullptr;
                 if constexpr (A_BUF) {
-                // One wide tile per long main loop: the epilogue is a small share of the time, so
-                // it stores row per lane, 16 columns at a time, straight from the registers.
-                const int64_t gi = (int64_t)c.mt * BM + quarter * 32 + lane;
+                // 32 columns at a time: this warp's 32 x 32 block goes through a 4 KB staging buffer so that
+                // global stores run along rows: 8 lines per instruction where one row per lane took 32.  Tiles
+                // of 512 columns leave no second accumulator, and the tensor core waits for this (19 % of the first
+                // product and 33 % of the second at r = 512, before).  First and second product: six layers of
+                // 2048-wide matrices, r = 192 0.772 -> 0.699 and 0.768 -> 0.700 ms, r = 512 0.873 -> 0.870 and 1.044 -> 0.933 (one
+                // slot of the N ring pays for the buffers); 24 layers of 768-wide ones, r = 192 0.407 -> 0.385 and 0.472 -> 0.417.
+                unsigned char* stg = staging + (warp - 2) * BUF_STAGING_BYTES;
+                const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
                 // (pairs: the CTA whose rows lie beyond the matrix stores nothing)
                 const bool has_rows = !PAIR || (int64_t)c.mt * BM < g.Mrows;
                 const int bn64 = !has_rows ? 0 : (to_img ? (c.bn + 63) / 64 * 64 : c.bn);
-                for (int cc = 0; cc < bn64; cc += 16) {
-                    uint32_t v[16];
-                    if (cc < c.bn) {
-                        tmem_ld16(taddr + cc, v);
-                        tmem_ld_wait();
-                        for (int ch = 1; ch < g.acc_chunks; ++ch) {
-                            uint32_t u[16];
-                            tmem_ld16(taddr + ch * g.BN + cc, u);
-                            tmem_ld_wait();
+                const int srow = lane / 4, sch = lane % 4;      // stores: 8 rows x 4 chunks of 8 columns per step
+                for (int cc = 0; cc < bn64; cc += 32) {
+                    uint32_t v[2][16];
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(u[i]));
+                    for (int h = 0; h < 2; ++h) {
+                        if (cc + 16 * h < c.bn) {
+                            tmem_ld16(taddr + cc + 16 * h, v[h]);
+                        } else {
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) v[h][i] = 0u;
                         }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) v[i] = 0u;
                     }
-                    const int gj = c.n0 + cc;
-                    if (C && gi < g.Mrows && cc < c.bn) {
-#pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            *reinterpret_cast<uint4*>(C + gi * g.out.ld + gj + 4 * u) =
-                                make_uint4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
-                    }
-                    if (to_img) {
-                        const int panel = gj / 64, ch0 = (gj % 64) / 8;
-                        unsigned char* r0 = scr + img_row_offset(d.img, 0, panel, gi);
-                        unsigned char* r1 = scr + img_row_offset(d.img, 1, panel, gi);
+                    tmem_ld_wait();
+                    for (int ch = 1; ch < g.acc_chunks; ++ch) {
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
-                            float f[8];
+                            if (cc + 16 * h < c.bn) {
+                                uint32_t u[16];
+                                tmem_ld16(taddr + ch * g.BN + cc + 16 * h, u);
+                                tmem_ld_wait();
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) f[i] = __uint_as_float(v[8 * h + i]);
-                            uint4 t0, t1;
-                            split8(f, t0, t1);
-                            const int o = img_chunk_offset((int)(gi & 7), ch0 + h);
-                            *reinterpret_cast<uint4*>(r0 + o) = t0;
-                            *reinterpret_cast<uint4*>(r1 + o) = t1;
-                            if (d.img.planes == 3)
-                                *reinterpret_cast<uint4*>(scr + img_row_offset(d.img, 2, panel, gi) + o) = half8(f, 1.f);
+                                for (int i = 0; i < 16; ++i)
+                                    v[h][i] = __float_as_uint(__uint_as_float(v[h][i]) + __uint_as_float(u[i]));
+                            }
                         }
                     }
-                    if (csq && cc < c.bn) {
-                        // column sums of squares over the 32 rows of this warp: fold 16 values over
-                        // the lane bits 4..1, then add the two lanes that hold the same column
-                        float s[16];
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) { const float x = __uint_as_float(v[i]); s[i] = __fmul_rn(x, x); }
+                    for (int ch = 0; ch < 8; ++ch)
+                        *reinterpret_cast<uint4*>(stg + lane * 128 + img_chunk_offset(lane, ch)) =
+                            make_uint4(v[ch / 4][ch % 4 * 4], v[ch / 4][ch % 4 * 4 + 1], v[ch / 4][ch % 4 * 4 + 2], v[ch / 4][ch % 4 * 4 + 3]);
+                    __syncwarp();
+                    const int gj = c.n0 + cc;
+                    if (csq) {
+                        // column sums of squares over the 32 rows of this warp: fold 32 values over the five
+                        // lane bits, after which every lane has the sum of one column
+                        float s[32];
 #pragma unroll
-                        for (int half = 8, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
-                            const bool up = (lane & bit) != 0;
+                        for (int i = 0; i < 32; ++i) { const float x = __uint_as_float(v[i / 16][i % 16]); s[i] = __fmul_rn(x, x); }
 #pragma unroll
-                            for (int i = 0; i < 8; ++i) {
+                        for (int half = 16; half >= 1; half >>= 1) {
+                            const bool up = (lane & half) != 0;
+#pragma unroll
+                            for (int i = 0; i < 16; ++i) {
                                 if (i < half) {
                                     const float send = up ? s[i] : s[i + half];
                                     const float keep = up ? s[i + half] : s[i];
-                                    s[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
+                                    s[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
                                 }
                             }
                         }
-                        s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
-                        const int col = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-                        if (!(lane & 1)) csq[gj + col] = s[0];
+                        if (cc + lane < c.bn) csq[gj + lane] = s[0];
                     }
+                    // (the image has 128 rows per tile, the fp32 result only those of the matrix)
+                    const int rows = (int)min((int64_t)32, g.Mrows - gi0) - srow;
+                    const bool col_in = cc + sch * 8 < c.bn;
+                    float* Cp = C + (gi0 + srow) * g.out.ld + gj + sch * 8;
+                    unsigned char* ip = scr + (to_img ? img_row_offset(d.img, 0, gj / 64, gi0 + srow) : 0) +
+                                        img_chunk_offset(srow, gj % 64 / 8 + sch);
+                    const int64_t plane_bytes = (int64_t)d.img.panels * d.img.rows_pad * 128;
+#pragma unroll
+                    for (int it = 0; it < 4; ++it) {
+                        const unsigned char* sp = stg + (it * 8 + srow) * 128;
+                        const float4 x = *reinterpret_cast<const float4*>(sp + img_chunk_offset(srow, 2 * sch));
+                        const float4 y = *reinterpret_cast<const float4*>(sp + img_chunk_offset(srow, 2 * sch + 1));
+                        if (C && it * 8 < rows && col_in) {
+                            *reinterpret_cast<float4*>(Cp + it * 8 * g.out.ld) = x;
+                            *reinterpret_cast<float4*>(Cp + it * 8 * g.out.ld + 4) = y;
+                        }
+                        if (to_img) {
+                            const float f[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+                            uint4 t0, t1;
+                            split8(f, t0, t1);
+                            *reinterpret_cast<uint4*>(ip + it * 1024) = t0;
+                            *reinterpret_cast<uint4*>(ip + plane_bytes + it * 1024) = t1;
+                            if (d.img.planes == 3) *reinterpret_cast<uint4*>(ip + 2 * plane_bytes + it * 1024) = half8(f, 1.f);
+                        }
+                    }
+                    __syncwarp();
                 }
                 } else {
                 // 64 columns at a time: this warp's 32 x 64 block goes through an 8 KB staging
@@ -1744,7 +1765,7 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     while (cols < g.acc_bufs * accw) cols *= 2;
     g.tmem_cols = cols;
     const size_t fixed = (size_t)g.a_slots * g.a_slot_bytes +
-                         (tc::a_is_buf(AMODE) ? 0 : (size_t)tc::epi_warps(AMODE, EPI) * g.epi_bufs * tc::STAGING_BYTES_PER_WARP) +
+                         (size_t)tc::epi_warps(AMODE, EPI) * (tc::a_is_buf(AMODE) ? tc::BUF_STAGING_BYTES : g.epi_bufs * tc::STAGING_BYTES_PER_WARP) +
                          256 + 1024;
     g.n_slots = (int)std::min<size_t>(tc::MAX_N_SLOTS, (tc::SMEM_LIMIT - fixed) / (size_t)g.n_piece_bytes);
     // more than half of an SM's shared memory: one CTA per SM, whatever its tensor-memory share
