@@ -1983,6 +1983,20 @@ inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const
         finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, ts.colsq, prof::S_K3, st);
 }
 
+// Columns per tile of a product between images (`copies`: matrices times depth chunks; lower: tiles that touch the lower
+// triangle).  256 columns, in CTA pairs where the rank allows, do the least work; 128 where all such
+// tiles run at once on multiprocessors that the wide ones leave idle.  An entry is summed in the same order either way.
+// Measured, 256 -> 128 columns: one 4096 x 4096 matrix at r = 256, Gram products of a step 0.170 -> 0.152 ms, applies 0.110 ->
+// 0.090; 4096 x 3584 at r = 512 0.238 -> 0.203 and 0.118 -> 0.095; 28 matrices 1000 wide at r = 272 0.911 -> 0.727 and
+// 0.487 -> 0.469.  (64 columns: another 5 % at r = 256, but 0.304 -> 0.357 ms for the Gram products of 11008 x 4096 at r = 1024.)
+inline int image_bn(int r, int64_t out_rows, int64_t copies, bool lower) {
+    const int wide = std::min(r, 256);
+    if (wide <= 128) return wide;
+    const int64_t rows = (out_rows + tc::BM - 1) / tc::BM, cols = (r + 127) / 128;
+    const int64_t tiles = lower ? rows * (rows + 1) / 2 : rows * cols;
+    return tiles * copies <= SPLIT_SMS ? 128 : wide;
+}
+
 // Depth split of the Gram product.  The Gram matrix is one output tile at small ranks and ten at r = 1024,
 // each with a main loop over all rows of the tall matrix: the depth is cut into chunks whose results are
 // added in a fixed order.  Their number depends on the rank and the row count only, so a matrix gets the same
@@ -2042,7 +2056,7 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
                         int only_shift_bit, int matrices, cudaStream_t st) {
     const int ksplit = gram_ksplit(r, rows, matrices), chunks = gram_chunks(r, rows);
     tc::GemmArgs g{};
-    g.Mrows = r; g.Ncols = r; g.Kdim = (int32_t)rows; g.BN = std::min(r, 256);
+    g.Mrows = r; g.Ncols = r; g.Kdim = (int32_t)rows; g.BN = image_bn(r, r, (int64_t)b.count * (ksplit > 1 ? chunks : 1), true);
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = src; g.n2 = no_img(); g.lower_only = 1;
     g.out.normal = dest_none(); g.out.normal.f32 = ksplit > 1 ? part : gram; g.out.normal.has_f32 = 1;
     g.out.shifted = g.out.normal; g.out.ld = r;
@@ -2066,7 +2080,7 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
 inline void tensor_apply(int r, int passes, const Batch& b, const TensorScratch& ts, ImgRef src, int64_t rows,
                          tc::OutSpec out, bool unit, cudaStream_t st) {
     tc::GemmArgs g{};
-    g.Mrows = (int32_t)rows; g.Ncols = r; g.Kdim = r; g.BN = std::min(r, 256);
+    g.Mrows = (int32_t)rows; g.Ncols = r; g.Kdim = r; g.BN = image_bn(r, rows, b.count, false);
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = ts.linv; g.n2 = no_img(); g.tri = 1;
     g.colsq_off = ts.colsq;
     g.cscale_off = unit ? ts.fscale : -1;

@@ -380,6 +380,13 @@ def test_gram_chunks_agree_bit_for_bit(shape, count):
     test_factor_kernel_forms_agree_bit_for_bit(shape, count)
 
 
+# Gram products and applies in 128-column single-CTA tiles (the matrix alone) and in 256-column tiles, in pairs or
+# not (the call of many): several row tiles, ragged last ones
+@pytest.mark.parametrize("shape,count", [((1000, 520, 256), 60), ((700, 520, 272), 40), ((1100, 1000, 768), 30)])
+def test_image_product_tiles_agree_bit_for_bit(shape, count):
+    test_factor_kernel_forms_agree_bit_for_bit(shape, count)
+
+
 # the products with B in narrow column tiles (the matrix alone) and wide ones (the call of many): pairs at r = 512
 # and 768, single CTAs with a remainder of 16 and of 112 columns
 @pytest.mark.parametrize("shape,count", [((1300, 1032, 512), 30), ((900, 1104, 768), 40), ((600, 520, 272), 40), ((520, 648, 496), 60)])
