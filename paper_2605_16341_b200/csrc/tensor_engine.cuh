@@ -896,8 +896,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 // global stores run along rows: 8 lines per instruction where one row per lane took 32.  Tiles
                 // of 512 columns leave no second accumulator, and the tensor core waits for this (19 % of the first
                 // product and 33 % of the second at r = 512, before).  First and second product: six layers of
-                // 2048-wide matrices, r = 192 0.772 -> 0.699 and 0.768 -> 0.700 ms, r = 512 0.873 -> 0.870 and 1.044 -> 0.933 (one
-                // slot of the N ring pays for the buffers); 24 layers of 768-wide ones, r = 192 0.407 -> 0.385 and 0.472 -> 0.417.
+                // 2048-wide matrices, r = 192 0.772 -> 0.699 and 0.768 -> 0.700 ms, r = 512 0.873 -> 0.870 and 1.044 -> 0.933; 24 layers of 768-wide ones, r = 192 0.407 -> 0.385 and 0.472 -> 0.417.
                 unsigned char* stg = staging + (warp - 2) * BUF_STAGING_BYTES;
                 const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
                 // (pairs: the CTA whose rows lie beyond the matrix stores nothing)
@@ -1764,10 +1763,25 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     int cols = 32;
     while (cols < g.acc_bufs * accw) cols *= 2;
     g.tmem_cols = cols;
+    int max_n_slots = tc::MAX_N_SLOTS;
+    if (tc::a_is_buf(AMODE)) {
+        // The loads of M and G under way (96 KB a CTA) need room in the L1 cache, which is what shared memory leaves of
+        // 256 KB: up to 196 KB of it are used, where 228 would leave 28 KB of cache.  Three slots in either
+        // ring, two in the A ring where three do not fit.  First and second product, as many slots as fit -> this:
+        // 11008 x 4096 r = 128 0.102 -> 0.092 and 0.088 -> 0.080 ms, r = 256 0.116 -> 0.105 and 0.099 -> 0.090; six layers of
+        // 2048-wide matrices r = 128 0.532 -> 0.468 and 0.569 -> 0.496, r = 192 0.697 -> 0.617 and 0.695 -> 0.608.  (Two slots in the N
+        // ring: r = 512 0.858 -> 0.917.)
+        max_n_slots = 3;
+        g.a_slots = 3;
+        if (3 * (size_t)g.a_slot_bytes + 3 * (size_t)g.n_piece_bytes + 4 * tc::BUF_STAGING_BYTES + 2304 > 196 * 1024) g.a_slots = 2;
+    }
+    // (the fused pass on other types than bf16 loads M, G and X into registers: the same line.  bf16 X and fp32 G, 4096 x 4096
+    // r = 128 0.079 -> 0.066 ms, r = 512 0.088 -> 0.075; fp32 X fits one slot either way)
+    if (EPI == tc::EPI_K5 && XG != 3) max_n_slots = 2;
     const size_t fixed = (size_t)g.a_slots * g.a_slot_bytes +
                          (size_t)tc::epi_warps(AMODE, EPI) * (tc::a_is_buf(AMODE) ? tc::BUF_STAGING_BYTES : g.epi_bufs * tc::STAGING_BYTES_PER_WARP) +
                          256 + 1024;
-    g.n_slots = (int)std::min<size_t>(tc::MAX_N_SLOTS, (tc::SMEM_LIMIT - fixed) / (size_t)g.n_piece_bytes);
+    g.n_slots = (int)std::min<size_t>(max_n_slots, (tc::SMEM_LIMIT - fixed) / (size_t)g.n_piece_bytes);
     // more than half of an SM's shared memory: one CTA per SM, whatever its tensor-memory share
     const size_t smem = std::max<size_t>(fixed + (size_t)g.n_slots * g.n_piece_bytes, 120 * 1024);
     if (AMODE == tc::A_IMG_K) encode_img_map(&g.map_a, b, g.a, 128, 1, a_terms);
