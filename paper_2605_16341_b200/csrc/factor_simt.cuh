@@ -92,6 +92,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     const int max_attempts = (a.pass == 1) ? 2 : 1;
     for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
         const float shift = attempt ? a.shift_rel * trace : 0.f;
+        const float pad = A[0] + shift;         // diagonal of the padding: the first pivot (see factor_tc.cuh)
         if (tid < 2) { s_min[tid] = 3.0e38f; s_max[tid] = 0.f; }
         for (int k = 0; k < nb; ++k) {
             const int k0 = k * CT_NB, nbk = min(CT_NB, r - k0);
@@ -104,7 +105,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
 #pragma unroll
                     for (int f = 0; f < 4; ++f) {
                         const int i = ty * 4 + e, j = tx * 4 + f;
-                        float v = i == j ? 1.f : 0.f;
+                        float v = i == j ? pad : 0.f;
                         if (i < nbk && j < nbk) v = A[(int64_t)(k0 + max(i, j)) * r + k0 + min(i, j)] + (i == j ? shift : 0.f) - acc[e][f];
                         sD[i * CT_LDD + j] = v;
                     }

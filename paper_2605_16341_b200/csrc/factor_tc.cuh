@@ -163,7 +163,7 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 }
 
 // ---- diagonal blocks (fp32, four warps) ----------------------------------------------------------
-// sD (64 x 64 block, ld CT_LDD, identity beyond nbk; row by row the lower part counts) -> X, the inverse of its
+// sD (64 x 64 block, ld CT_LDD, beyond nbk a diagonal of the matrix's first pivot; row by row the lower part counts) -> X, the inverse of its
 // Cholesky factor L, in the lower part of sD, and the rows of X^T = L^{-T} as they are found: out(row, chunk, z)
 // gets the entries 8 chunk .. + 7 of a row.
 //
@@ -667,16 +667,18 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
             *reinterpret_cast<uint4*>(dst + term + q) = *reinterpret_cast<const uint4*>(src + CT_TERM + q);
         }
     };
-    // sD <- diagonal block k: Gram - accd, the diagonal itself from gdiag (+ shift), identity beyond r
+    // sD <- diagonal block k: Gram - accd, the diagonal itself from gdiag (+ shift); beyond r the matrix's first pivot on
+    // the diagonal, which changes neither the smallest nor the largest (a one would: it is not of the matrix's scale)
     auto write_diag = [&](const float (&accd)[4][4], int k, float shift) {
         float* sD = diag_buf(k);
+        const float pad = __ldcg(gdiag) + shift;
 #pragma unroll
         for (int nf = 0; nf < 4; ++nf)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const int il = mrow + 8 * (e / 2), jl = mcol + nf * 8 + (e % 2);
                 const int i = k * CT_NB + il, j = k * CT_NB + jl;
-                float v = il == jl ? 1.f : 0.f;
+                float v = il == jl ? pad : 0.f;
                 if (i < r && j < r) v = (il == jl ? __ldcg(gdiag + i) + shift : A[(int64_t)i * r + j]) - accd[nf][e];
                 sD[il * CT_LDD + jl] = v;
             }

@@ -409,10 +409,11 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                 bool ok = false;
                 for (int attempt = 0; attempt < (pass == 1 ? 2 : 1) && !ok; ++attempt) {
                     const float shift = attempt ? a.shift_rel * trace : 0.f;
+                    const float pad = G[0] + shift;      // diagonal of the padding: the first pivot (see factor_tc.cuh)
                     constexpr int DN = R <= 32 ? 32 : 64;
                     for (int q = tid; q < DN * DN; q += QS_THREADS) {
                         const int i = q / DN, j = q % DN;
-                        float v = i == j ? 1.f : 0.f;
+                        float v = i == j ? pad : 0.f;
                         if (i < r && j < r) v = G[i * R + j] + (i == j ? shift : 0.f);
                         sD[i * CT_LDD + j] = v;
                     }

@@ -256,6 +256,29 @@ def test_ill_conditioned_projection_takes_shifted_path(engine):
     gm.close()
 
 
+# ranks whose last diagonal block is padded (48, 112, 240: a last half of 16 columns; fp32 engine: no multiple of
+# eight either), the one-kernel QR on both sides and on neither
+@pytest.mark.parametrize("engine,shape", [(od.ENGINE_TENSOR, (512, 384, 48)), (od.ENGINE_TENSOR, (700, 800, 48)),
+                                          (od.ENGINE_TENSOR, (500, 600, 112)), (od.ENGINE_TENSOR, (520, 504, 240)),
+                                          (od.ENGINE_SIMT, (200, 328, 7)), (od.ENGINE_SIMT, (300, 277, 40)),
+                                          (od.ENGINE_SIMT, (600, 520, 200))])
+def test_scale_of_a_well_conditioned_buffer_changes_no_status_and_no_factor(engine, shape):
+    """Conditioning is a ratio: a well-conditioned buffer is no less so when it is small or large.  Scaled by a power
+    of two every product, sum and pivot scales exactly, so the status stays clear and P and Q keep their bits."""
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, F32, F32, seed=m + n + r)
+    first = None
+    for scale in (1.0, 2.0 ** -20, 2.0 ** 20):
+        gm = GpuMatrix(spec, X, M * scale, Q, mu=0.95, eta=0.01, engine=engine)
+        gm.step(G * scale)
+        assert gm.status() == 0, scale
+        P = gm.factors()[0].clone()
+        if first is None:
+            first = (P, gm.Q)
+        assert torch.equal(P, first[0]) and torch.equal(gm.Q, first[1]), scale
+        gm.close()
+
+
 # ------------------------------------------------------------------ grouped == single, resume
 @pytest.mark.parametrize("engine", ENGINES, ids=ENGINE_IDS)
 def test_grouped_matches_single_and_is_deterministic(engine):

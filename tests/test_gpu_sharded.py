@@ -66,6 +66,18 @@ def test_sharded_step_matches_the_oracle_on_the_whole_matrix(shape, k, mode):
         od.orthdion_destroy(s["h"])
 
 
+@pytest.mark.parametrize("scale", [2.0 ** -12, 2.0 ** 12])
+def test_status_does_not_depend_on_the_scale_of_the_buffer(scale):
+    # a rank whose last diagonal block is padded: the padding is not part of the conditioning test
+    spec, X, M, G, Q = make_problem(512, 640, 112, torch.float32, torch.float32, seed=7)
+    h = od.orthdion_create(512, 640, 112, 0.95, 0.01, 0.0, od.MODE_ORTH)
+    od.orthdion_set_dtypes(h, torch.float32, torch.float32)
+    ws = poisoned_workspace(od.orthdion_workspace_bytes(h))
+    sharding.sharded_step(od, h, True, X.cuda(), (M * scale).cuda(), (G * scale).cuda(), Q.cuda(), ws)
+    assert od.orthdion_last_status([h], ws) == [0]
+    od.orthdion_destroy(h)
+
+
 def test_one_shard_without_reduction_is_the_plain_step():
     spec, X, M, G, Q = make_problem(512, 640, 64, BF16, BF16, seed=5)
     h = od.orthdion_create(512, 640, 64, 0.95, 0.01, 0.0, od.MODE_ORTH)
