@@ -79,6 +79,8 @@ typedef struct orthdion_plan* orthdion_t;
 #define ORTHDION_STATUS_SHIFTED_RIGHT   2   /* or a second pass that met a poorly conditioned   */
                                             /* Q1); same for the right QR                       */
 #define ORTHDION_STATUS_RANK_DEFICIENT  4   /* factorisation failed: X, M, Q left unchanged     */
+                                            /* (also where squared column norms underflow:      */
+                                            /* columns of B Q_prev or R below about 1e-22)      */
 #define ORTHDION_STATUS_NONFINITE       8   /* a Gram matrix held Inf/NaN: treated as failure   */
 #define ORTHDION_STATUS_ZERO_COLUMN    16   /* COLNORM met a zero column of R (kept zero)       */
 #define ORTHDION_STATUS_WAIT_LIMIT     32   /* a bounded device-side wait expired (kernel bug): */

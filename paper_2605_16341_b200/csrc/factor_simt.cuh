@@ -28,6 +28,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     float* Xs = reinterpret_cast<float*>(smem + FS_OFF_X);
     float* sD = reinterpret_cast<float*>(smem + CT_OFF_D);
     __shared__ float red[FS_THREADS / 32];
+    __shared__ float s_up[2];                 // scales of a tiny matrix (see ct_rsqrt)
     __shared__ float s_min[2], s_max[2];      // pivots, by the half of their diagonal block
 
     const MatWork& w = batch.w[blockIdx.x];
@@ -88,6 +89,8 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
         __syncthreads();
     };
 
+    if (tid == 0) { s_up[0] = trace < CT_TINY_TRACE ? CT_TINY_UP : 1.f; s_up[1] = trace < CT_TINY_TRACE ? CT_TINY_UP_ROOT : 1.f; }
+
     bool ok = false;
     const int max_attempts = (a.pass == 1) ? 2 : 1;
     for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
@@ -107,13 +110,13 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
                         const int i = ty * 4 + e, j = tx * 4 + f;
                         float v = i == j ? pad : 0.f;
                         if (i < nbk && j < nbk) v = A[(int64_t)(k0 + max(i, j)) * r + k0 + min(i, j)] + (i == j ? shift : 0.f) - acc[e][f];
-                        sD[i * CT_LDD + j] = v;
+                        sD[i * CT_LDD + j] = v * s_up[0];
                     }
             }
             __syncthreads();
             if (warp < CT_DIAG_WARPS) {
                 float mn, mx;
-                ct_diag_block<64>(sD, smem + CT_OFF_D, nbk, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                ct_diag_block<64>(sD, smem + CT_OFF_D, nbk, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
                 if (lane == 0 && (warp == 0 || (warp == 3 && nbk > 32))) {
                     s_min[warp / 3] = mx <= 3.0e38f ? fminf(s_min[warp / 3], mn) : -1.f;
                     s_max[warp / 3] = fmaxf(s_max[warp / 3], mx);
@@ -122,7 +125,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             __syncthreads();
             for (int q = tid; q < CT_NB * CT_NB; q += FS_THREADS) {
                 const int i = q / CT_NB, j = q % CT_NB;
-                const float v = sD[max(i, j) * CT_LDD + min(i, j)];
+                const float v = sD[max(i, j) * CT_LDD + min(i, j)] * s_up[1];
                 if (i < nbk && j < nbk) W[(int64_t)(k0 + i) * r + k0 + j] = v;
                 Xs[i * SIMT_LD + j] = (i <= j && j < nbk) ? v : 0.f;         // X_k(j, i)
             }

@@ -163,9 +163,9 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 }
 
 // ---- diagonal blocks (fp32, four warps) ----------------------------------------------------------
-// sD (64 x 64 block, ld CT_LDD, beyond nbk a diagonal of the matrix's first pivot; row by row the lower part counts) -> X, the inverse of its
-// Cholesky factor L, in the lower part of sD, and the rows of X^T = L^{-T} as they are found: out(row, chunk, z)
-// gets the entries 8 chunk .. + 7 of a row.
+// sD (64 x 64 block, ld CT_LDD, beyond nbk a diagonal of the matrix's first pivot; row by row the lower part
+// counts) -> X, the inverse of its Cholesky factor L, in the lower part of sD, and the rows of X^T = L^{-T} as they
+// are found: out(row, chunk, z) gets the entries 8 chunk .. + 7 of a row.
 //
 // As in the large, [D; I] L^{-T} = [L; L^{-T}]: rows of the block and of the identity go through the same
 // elimination, a row per lane.  The columns are taken in panels of eight, whose 8 x 8 diagonal block every
@@ -182,6 +182,15 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 // Measured alone, cycles for 64 columns: 11200 with all updates in the chain, 9300 so.  (Two 32-column
 // factorisations by one warp with the columns passed by shuffle, then triangular solves and the update
 // one after the other: 16 thousand.)
+// Pivots are normal numbers here: the form of rsqrt that takes subnormal ones costs the chain three more
+// dependent instructions per column.  A Gram matrix so small that its pivots may be subnormal (squared column
+// norms of the factor below 2^-60) comes into sD times CT_TINY_UP, and `unit`, the root of that, in place of the
+// identity's ones takes it out of the inverse again.  (Free: multiplying the entries of X^T as they leave cost 4 of
+// 480 us at 4096 x 4096, r = 256.  A subnormal pivot in a Gram matrix of ordinary size means an
+// ill-conditioned one, and fails.)
+constexpr float CT_TINY_TRACE = 8.67361738e-19f;          // 2^-60
+constexpr float CT_TINY_UP = 1.20892582e24f;              // 2^80
+constexpr float CT_TINY_UP_ROOT = 1.09951163e12f;         // 2^40
 __device__ __forceinline__ float ct_rsqrt(float x) {
     float y;
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -231,10 +240,10 @@ __device__ __forceinline__ void ct_rank8(float* a, const float (&z)[8], const fl
     }
 }
 // `rest`: CT_DG_BYTES of shared memory whose first part may be sD itself.  dmin, dmax: smallest (-1: breakdown)
-// and largest pivot, in the lanes of warp 0 (one half) or warp 3 (two).
+// and largest pivot, in the lanes of warp 0 (one half) or warp 3 (two).  unit: 1, or what ct_rsqrt says.
 // COLS: at most so many columns (16, 32 or 64).
 template <int COLS, class Out>
-__device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, int dw, int lane, float& dmin, float& dmax, Out out) {
+__device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, float unit, int dw, int lane, float& dmin, float& dmax, Out out) {
     float* LT = reinterpret_cast<float*>(rest + CT_DG_LT);
     float* blk = reinterpret_cast<float*>(rest + CT_DG_BLK);
     float* sS = reinterpret_cast<float*>(rest + CT_DG_S);
@@ -248,7 +257,7 @@ __device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, in
         const float* src = sD + (lane + (dw == 1 || dw == 3 ? 32 : 0)) * CT_LDD + (dw == 3 ? 32 : 0);
 #pragma unroll
         for (int c = 0; c < NA; c += 4) {
-            float4 v = make_float4(lane == c ? 1.f : 0.f, lane == c + 1 ? 1.f : 0.f, lane == c + 2 ? 1.f : 0.f, lane == c + 3 ? 1.f : 0.f);
+            float4 v = make_float4(lane == c ? unit : 0.f, lane == c + 1 ? unit : 0.f, lane == c + 2 ? unit : 0.f, lane == c + 3 ? unit : 0.f);
             if (dw != 2 && (dw == 0 || two)) v = *reinterpret_cast<const float4*>(src + c);
             a[c] = v.x; a[c + 1] = v.y; a[c + 2] = v.z; a[c + 3] = v.w;
         }
@@ -343,7 +352,7 @@ __device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, in
     if (dw == 3) { dmin = 3.0e38f; dmax = 0.f; }
     else {
 #pragma unroll
-        for (int c = 0; c < 32; ++c) a[c] = dw == 2 && lane == c ? 1.f : 0.f;
+        for (int c = 0; c < 32; ++c) a[c] = dw == 2 && lane == c ? unit : 0.f;
     }
     shift();
     if (dw == 3) put_blk(0);
@@ -680,7 +689,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                 const int i = k * CT_NB + il, j = k * CT_NB + jl;
                 float v = il == jl ? pad : 0.f;
                 if (i < r && j < r) v = (il == jl ? __ldcg(gdiag + i) + shift : A[(int64_t)i * r + j]) - accd[nf][e];
-                sD[il * CT_LDD + jl] = v;
+                sD[il * CT_LDD + jl] = trace < CT_TINY_TRACE ? v * CT_TINY_UP : v;         // see ct_rsqrt
             }
     };
 
@@ -768,7 +777,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                         for (int ch = 0; ch < 4; ++ch) out(32 + lane, ch, zero);
                     }
                     float mn, mx;
-                    ct_diag_block<64>(diag_buf(k), smem + CT_OFF_D, nbk, dw, lane, mn, mx, out);
+                    ct_diag_block<64>(diag_buf(k), smem + CT_OFF_D, nbk, trace < CT_TINY_TRACE ? CT_TINY_UP_ROOT : 1.f, dw, lane, mn, mx, out);
                     // statistics: squared diagonal entries of L; two halves: warp 0's first, warp 3's second
                     if (lane == 0 && (dw == 0 || (dw == 3 && nbk > 32))) {
                         if (!(mx <= 3.0e38f)) mn = -1.f;

@@ -406,6 +406,11 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     G[q] = k < j ? -v : (k == j ? 0.5f * (3.f - v) : 0.f);
                 }
             } else {
+                const bool tiny = pass == 1 && trace < CT_TINY_TRACE;          // see ct_rsqrt
+                auto scale_block = [&](float f) {
+                    for (int q = tid; q < R * R; q += QS_THREADS) sD[q / R * CT_LDD + q % R] *= f;
+                    __syncthreads();
+                };
                 bool ok = false;
                 for (int attempt = 0; attempt < (pass == 1 ? 2 : 1) && !ok; ++attempt) {
                     const float shift = attempt ? a.shift_rel * trace : 0.f;
@@ -418,9 +423,10 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                         sD[i * CT_LDD + j] = v;
                     }
                     __syncthreads();
+                    if (tiny) scale_block(CT_TINY_UP);
                     if (warp < CT_DIAG_WARPS) {
                         float mn, mx;
-                        ct_diag_block<R>(sD, smem, r, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                        ct_diag_block<R>(sD, smem, r, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
                         if (lane == 0 && (warp == 0 || (warp == 3 && r > 32))) {
                             s_min[warp / 3] = mx <= 3.0e38f ? mn : -1.f;
                             s_max[warp / 3] = mx;
@@ -438,6 +444,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     if (tid == 0 && crank == 0) atomicOr(w.status, ST_RANKDEF | (third ? shift_bit : 0));
                     return;
                 }
+                if (tiny) scale_block(CT_TINY_UP_ROOT);
                 for (int q = tid; q < R * R; q += QS_THREADS) {
                     const int k = q / R, j = q % R;
                     G[q] = (k <= j && j < r) ? sD[j * CT_LDD + k] : 0.f;

@@ -279,6 +279,18 @@ def test_scale_of_a_well_conditioned_buffer_changes_no_status_and_no_factor(engi
         gm.close()
 
 
+@pytest.mark.parametrize("engine,shape", [(od.ENGINE_TENSOR, (512, 384, 16)), (od.ENGINE_TENSOR, (512, 384, 48)),
+                                          (od.ENGINE_TENSOR, (700, 800, 64)), (od.ENGINE_TENSOR, (520, 504, 240)),
+                                          (od.ENGINE_SIMT, (300, 277, 40)), (od.ENGINE_SIMT, (600, 520, 200))])
+@pytest.mark.parametrize("scale", [2.0 ** -58, 2.0 ** -66, 2.0 ** -72])
+def test_buffer_whose_squared_column_norms_are_subnormal(engine, shape, scale):
+    # columns of Y and R of length about 20 scale: squared 1e-32 (normal), 1e-37 (the smallest normal number is
+    # 1.2e-38, and pivots are smaller than squared norms), 2e-41 (subnormal)
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, F32, F32, seed=m + n + r)
+    one_step_compare(spec, X, M * scale, G * scale, Q, mode=od.MODE_ORTH, engine=engine)
+
+
 # ------------------------------------------------------------------ grouped == single, resume
 @pytest.mark.parametrize("engine", ENGINES, ids=ENGINE_IDS)
 def test_grouped_matches_single_and_is_deterministic(engine):
