@@ -113,7 +113,10 @@ int orthdion_set_engine(orthdion_t h, int32_t engine);
  * passes <= 0 hands it back to the default rule. */
 int orthdion_set_passes(orthdion_t h, int32_t which, int32_t passes);
 
-/* Workspace sizes in bytes (host computation, no CUDA call). */
+/* Workspace sizes in bytes (host computation, no CUDA call).  In calls of one or a few matrices they include
+ * partial results that shorten the products.  A step with less workspace does without those where the rest
+ * fits, to the same bits, so what was sized for a call serves any call of some of its matrices; and for a
+ * single plan they are left out where they alone would exceed ORTHDION_NOALLOC_SCRATCH_BYTES. */
 size_t orthdion_workspace_bytes(orthdion_t h);
 size_t orthdion_workspace_bytes_grouped(const orthdion_t* hs, int32_t count);
 

@@ -21,8 +21,8 @@ struct MatWork {
     float* R;           // n x r   (workspace slot)
     int32_t* status;    // one word
     char* scratch;      // per-matrix scratch area
-    int32_t aux0;       // launch-specific per-matrix integer (Cholesky: rows of column-square partials)
-    int32_t aux1;
+    int32_t aux0;       // launch-specific per-matrix integers (Cholesky: rows of column-square partials,
+    int32_t aux1;       // and the scratch offset of the image of L in KB)
 };
 
 constexpr int MAXB = 256;   // matrices per launch batch

@@ -19,12 +19,12 @@ struct CholArgs {
     // no such bias.)
     Sel colsq;
     int32_t use_colsq, pad;
-    // tensor engine: split image of L^{-T} (the result there, operand of the apply product), of L (same
-    // geometry, at limg_off), the Gram diagonal (fp32 [r]), the statistics of the diagonal blocks, and
-    // later passes: L^{-1}(j, j) over the value that its two image terms hold (fp32 [r], then one more
-    // float: not zero when these factors are to be used)
+    // tensor engine: split image of L^{-T} (the result there, operand of the apply product; the image of L has the
+    // same geometry and lies at MatWork::aux1), the Gram diagonal (fp32 [r]), the statistics of the
+    // diagonal blocks, and later passes: L^{-1}(j, j) over the value that its two image terms hold (fp32 [r], then
+    // one more float: not zero when these factors are to be used)
     ImgRef img;
-    int64_t limg_off, diag_off, stat_off, scale_off;
+    int64_t diag_off, stat_off, scale_off;
     int64_t cnorm_off;   // >= 0: also leave the Gram diagonal (squared column norms) there, fp32 [r]
 };
 

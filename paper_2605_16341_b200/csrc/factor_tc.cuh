@@ -436,7 +436,8 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     float* gstat = reinterpret_cast<float*>(w.scratch + a.stat_off);
     float* gscale = reinterpret_cast<float*>(w.scratch + a.scale_off);
     const int64_t term = (int64_t)a.img.panels * a.img.rows_pad * 128;    // bytes between the terms of an image
-    auto l_tile = [&](int t, int c) { return scr + a.limg_off + ((int64_t)c * a.img.rows_pad + (int64_t)t * CT_NB) * 128; };
+    unsigned char* limg = scr + (int64_t)w.aux1 * 1024;
+    auto l_tile = [&](int t, int c) { return limg + ((int64_t)c * a.img.rows_pad + (int64_t)t * CT_NB) * 128; };
     auto x_tile = [&](int t, int c) { return scr + a.img.off + ((int64_t)c * a.img.rows_pad + (int64_t)t * CT_NB) * 128; };
 
     // ---- Gram diagonal (from the fp32 column sums of squares), by row tile --------------------

@@ -57,8 +57,9 @@ bool same_class(const orthdion_plan* a, const orthdion_plan* b) {
            std::memcmp(a->passes, b->passes, sizeof(a->passes)) == 0;
 }
 
-// Per-matrix scratch carving (byte offsets).  gram, linv and the tensor engine's first entries
-// depend on r only, so one Cholesky launch can serve matrices of different shapes.
+// Per-matrix scratch carving (byte offsets).  gram, linv (the inverse factor: fp32, or the tensor engine's image)
+// and the tensor engine's first entries depend on r only, so one Cholesky launch can serve matrices of
+// different shapes.
 struct Scratch {
     int64_t gram, linv, tmpA, tmpB;
     int64_t gram_part;     // partial results of a depth-split product (tensor engine, small ranks)
@@ -71,26 +72,31 @@ bool fused_fp16(const orthdion_plan* p) {
     return p->engine == ORTHDION_ENGINE_TENSOR && p->passes[2] == 1 && p->passes[3] == 1;
 }
 
-// matrices: of the whole call.
-Scratch scratch_layout(const orthdion_plan* p, int matrices) {
+// matrices: of the whole call.  lean: no partial results in memory beyond those that a product cannot do without.
+// The same chunks are then added up in tensor memory or tile by tile: the same bits, longer launches for a few
+// matrices.  A lean layout never needs more than the plan's images and fixed slots.
+Scratch scratch_layout(const orthdion_plan* p, int matrices, bool lean) {
     Scratch s{};
     const size_t rr = align_up((size_t)p->r * p->r * 4, 256);
     size_t off = 0;
     s.gram = off; off += rr;
-    // L^{-1} in fp32 (SIMT engine), or the split image of L (tensor engine)
-    s.linv = off;
-    off += p->engine == ORTHDION_ENGINE_TENSOR ? std::max(rr, (size_t)img_bytes(p->r, p->r)) : rr;
     if (p->engine == ORTHDION_ENGINE_TENSOR) {
-        off = tensor_scratch_layout(p->m, p->n, p->r, fused_fp16(p), off, &s.ts);
+        TensorScratch& ts = s.ts;
+        off = tensor_scratch_layout(p->m, p->n, p->r, fused_fp16(p), off, &ts);
+        s.linv = ts.linv.off;
         // (after everything whose offset must depend on r only)
-        const int parts = std::max(gram_ksplit(p->r, p->m, matrices), gram_ksplit(p->r, p->n, matrices));
-        const int s1 = buffer_ksplit(p->r, p->m, p->n, matrices), s3 = buffer_ksplit(p->r, p->n, p->m, matrices);
+        ts.gram_parts_m = gram_ksplit(p->r, p->m, matrices, lean);
+        ts.gram_parts_n = gram_ksplit(p->r, p->n, matrices, lean);
+        ts.y_parts = buffer_ksplit(p->r, p->m, p->n, matrices, lean);
+        ts.r_parts = buffer_ksplit(p->r, p->n, p->m, matrices, lean);
+        const int parts = std::max(ts.gram_parts_m, ts.gram_parts_n);
         size_t part_bytes = parts > 1 ? (size_t)parts * rr : 0;
-        if (s1 > 1) part_bytes = std::max(part_bytes, align_up((size_t)s1 * p->m * p->r * 4, 256));
-        if (s3 > 1) part_bytes = std::max(part_bytes, align_up((size_t)s3 * p->n * p->r * 4, 256));
+        if (ts.y_parts > 1) part_bytes = std::max(part_bytes, align_up((size_t)ts.y_parts * p->m * p->r * 4, 256));
+        if (ts.r_parts > 1) part_bytes = std::max(part_bytes, align_up((size_t)ts.r_parts * p->n * p->r * 4, 256));
         s.gram_part = (int64_t)off;
         off += part_bytes;
     } else {
+        s.linv = off; off += rr;
         const size_t kr = align_up((size_t)std::max(p->m, p->n) * p->r * 4, 256);
         s.tmpA = off; off += kr;
         s.tmpB = off; off += kr;
@@ -106,10 +112,12 @@ struct Batching {
     std::vector<std::vector<int>> groups;    // batch indices per group
     std::vector<size_t> batch_off;           // scratch offset of each batch inside its group
     size_t scratch_bytes = 0;                // max over groups
+    bool lean = false;                       // scratch without optional partial results
 };
 
-Batching make_batches(const orthdion_t* hs, int32_t count) {
+Batching make_batches(const orthdion_t* hs, int32_t count, bool lean) {
     Batching out;
+    out.lean = lean;
     std::vector<char> done(count, 0);
     size_t group_bytes = 0;
     for (int i = 0; i < count; ++i) {
@@ -117,7 +125,7 @@ Batching make_batches(const orthdion_t* hs, int32_t count) {
         std::vector<int> cls;
         for (int j = i; j < count; ++j)
             if (!done[j] && same_class(hs[i], hs[j])) { cls.push_back(j); done[j] = 1; }
-        const size_t per = scratch_layout(hs[i], count).bytes;
+        const size_t per = scratch_layout(hs[i], count, lean).bytes;
         size_t cap = std::max<size_t>(1, kScratchBudget / std::max<size_t>(per, 1));
         cap = std::min<size_t>(cap, MAXB);
         const size_t nb = (cls.size() + cap - 1) / cap;
@@ -159,6 +167,17 @@ Layout make_layout(const orthdion_t* hs, int32_t count, size_t scratch_bytes) {
     l.scratch_off = align_up(off, 1024);
     l.total = l.scratch_off + scratch_bytes;
     return l;
+}
+
+// The batches and layout of a call with a workspace of `bytes`: with all partial results in memory where that
+// fits, else lean.  (So a workspace that was sized for more matrices, or for another rank, serves a smaller call although
+// partial results are kept for small calls only.)
+void plan_call(const orthdion_t* hs, int32_t count, size_t bytes, Batching* bt, Layout* lay) {
+    for (int lean = 0; lean < 2; ++lean) {
+        *bt = make_batches(hs, count, lean != 0);
+        *lay = make_layout(hs, count, bt->scratch_bytes);
+        if (lay->total <= bytes) return;
+    }
 }
 
 #define CU_CHECK(expr)                                                     \
@@ -307,7 +326,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
         ca.colsq = sel(W_SCRATCH, 0); ca.use_colsq = 0; ca.img = no_img(); ca.cnorm_off = -1;
         if (lead.tensor()) {
             ca.colsq = sel(W_SCRATCH, lead.sc.ts.colsq); ca.use_colsq = diag_from_gram ? 0 : 1; ca.img = lead.sc.ts.linv;
-            ca.limg_off = lead.sc.linv; ca.diag_off = lead.sc.ts.fdiag; ca.stat_off = lead.sc.ts.fstat;
+            ca.diag_off = lead.sc.ts.fdiag; ca.stat_off = lead.sc.ts.fstat;
             ca.scale_off = lead.sc.ts.fscale;
             if (which == 1 && pass == 1) ca.cnorm_off = lead.sc.ts.cnorm;
         }
@@ -340,6 +359,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 MatWork& w = merged->w[merged->count++];
                 w = c.b->w[k];
                 w.aux0 = (int32_t)(4 * ((rows + 127) / 128));
+                w.aux1 = c.tensor() ? (int32_t)(c.sc.ts.q.off / 1024) : 0;
                 if (merged->count == MAXB) flush();
             }
         }
@@ -410,8 +430,8 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
     std::vector<int> which_cls;
     for (int ci : wanted) {
         ClassRun& c = cls[ci];
-        const int64_t rows = which ? c.p->n : c.p->m, depth = which ? c.p->m : c.p->n;
-        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed ? 1 : buffer_ksplit(c.p->r, rows, depth, call_matrices), call_matrices, st);
+        const int64_t rows = which ? c.p->n : c.p->m;
+        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed ? 1 : (which ? c.sc.ts.r_parts : c.sc.ts.y_parts), call_matrices, st);
         else which_cls.push_back(ci);
     }
     if (which_cls.empty()) return;
@@ -427,7 +447,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
                 const ImgRef in = which ? ts.r : img_view(ts.w0, rows);
                 const ImgRef src = pass == 1 ? in : (pass == 2 ? img_view(ts.w1, rows) : img_view(ts.w0, rows));
                 tensor_gram(r, c.p->passes[1], *c.b, src, rows, gram, sel(W_SCRATCH, c.sc.gram_part),
-                            only_shift ? shift_bit : 0, call_matrices, st);
+                            which ? ts.gram_parts_n : ts.gram_parts_m, only_shift ? shift_bit : 0, st);
             } else {
                 const Sel in = which ? sel(W_R) : sel(W_P);
                 const Sel src = pass == 1 ? in : (pass == 2 ? sel(W_SCRATCH, c.sc.tmpA) : sel(W_SCRATCH, c.sc.tmpB));
@@ -473,7 +493,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
 
 // Diagnostics of one class, after its step: Q^T Q from the engine's Gram product, column
 // statistics of R, optionally the norms of M' and G, then one CTA per matrix for the rest.
-void diag_stage(ClassRun& c, DiagBase db, int call_matrices, cudaStream_t st) {
+void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
     const orthdion_plan* p = c.p;
     const Batch& b = *c.b;
     const int r = p->r;
@@ -481,7 +501,7 @@ void diag_stage(ClassRun& c, DiagBase db, int call_matrices, cudaStream_t st) {
     const int64_t stats_off = c.sc.linv;          // 3 r floats of the (now free) inverse slot
     launch(diag_init_kernel, dim3((unsigned)((b.count * DIAG_STRIDE + 255) / 256)), 256, 0, 1, prof::S_DIAG, st, b, db);
     if (c.tensor()) {
-        tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), 0, call_matrices, st);
+        tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), c.sc.ts.gram_parts_n, 0, st);
     } else {
         const Sel sQ = sel(W_Q);
         launch_simt(b, r, r, p->n, RdPlain{sQ, 1, r}, RdPlain{sQ, 1, r}, SimtOut{gram, gram, 0, 1, r, 0, 0},
@@ -518,7 +538,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
-        if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), call_matrices, st,
+        if (c.tensor()) tensor_k1(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
                                   small_qr(p, p->m) ? OUT_F32 : OUT_IMAGE);
         else launch_simt(*c.b, p->m, p->r, p->n, RdBuffer{p->n, gb, 0}, RdPlain{sQ, 1, p->r},
                          SimtOut{sP, sP, 0, 0, p->r, 0, 0}, prof::S_K1, st);
@@ -528,7 +548,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
-        if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), call_matrices, st,
+        if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
                                   small_qr(p, p->n) ? OUT_F32 : OUT_IMAGE);
         else launch_simt(*c.b, p->n, p->r, p->m, RdBuffer{p->n, gb, 1}, RdPlain{sP, 1, p->r},
                          SimtOut{sR, sR, 0, 0, p->r, 0, 0}, prof::S_K3, st);
@@ -539,7 +559,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const orthdion_plan* p = c.p;
         if (p->mode == ORTHDION_MODE_ORTH) continue;
         if (small_qr(p, p->n)) {
-            small_qr_stage(c, 1, buffer_ksplit(p->r, p->n, p->m, call_matrices), call_matrices, st);
+            small_qr_stage(c, 1, c.sc.ts.r_parts, call_matrices, st);
             continue;
         }
         launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b, p->n,
@@ -562,7 +582,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         }
     }
     for (ClassRun& c : cls)
-        if (c.p->diag) diag_stage(c, db, call_matrices, st);
+        if (c.p->diag) diag_stage(c, db, st);
 }
 
 // Default pass counts of the fused feedback/update pass.  One fp16 pass carries P R^T with about
@@ -687,8 +707,13 @@ size_t orthdion_workspace_bytes_grouped(const orthdion_t* hs, int32_t count) {
     if (!hs || count < 1) return 0;
     for (int i = 0; i < count; ++i)
         if (!valid(hs[i])) return 0;
-    Batching bt = make_batches(hs, count);
-    return make_layout(hs, count, bt.scratch_bytes).total;
+    size_t total = make_layout(hs, count, make_batches(hs, count, false).scratch_bytes).total;
+    // partial results do not take a plan out of orthdion_step_noalloc's reach
+    if (count == 1 && total > ORTHDION_NOALLOC_SCRATCH_BYTES) {
+        const size_t lean = make_layout(hs, count, make_batches(hs, count, true).scratch_bytes).total;
+        if (lean <= ORTHDION_NOALLOC_SCRATCH_BYTES) total = lean;
+    }
+    return total;
 }
 
 size_t orthdion_workspace_bytes(orthdion_t h) { return orthdion_workspace_bytes_grouped(&h, 1); }
@@ -705,8 +730,9 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
             return e;
     }
     if (reinterpret_cast<uintptr_t>(workspace) % 256) return ORTHDION_ERR_WORKSPACE;
-    Batching bt = make_batches(hs, count);
-    Layout lay = make_layout(hs, count, bt.scratch_bytes);
+    Batching bt;
+    Layout lay;
+    plan_call(hs, count, workspace_bytes, &bt, &lay);
     if (workspace_bytes < lay.total) return ORTHDION_ERR_WORKSPACE;
     int e = ensure_attributes();
     if (e) return e;
@@ -720,7 +746,7 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
         std::vector<ClassRun> cls;
         for (int bi : grp) {
             const auto& idx = bt.batches[bi];
-            ClassRun c{hs[idx[0]], &pool[bi], scratch_layout(hs[idx[0]], count)};
+            ClassRun c{hs[idx[0]], &pool[bi], scratch_layout(hs[idx[0]], count, bt.lean)};
             c.b->count = (int32_t)idx.size();
             c.b->pad = 0;
             c.b->scratch_stride = (int64_t)c.sc.bytes;
@@ -819,12 +845,12 @@ int shard_setup(orthdion_t h, void* X, float* M, const void* G, float* Q, void* 
     if ((e = check_ptr(X)) || (e = check_ptr(M)) || (e = check_ptr(G)) || (e = check_ptr(Q))) return e;
     if (!workspace) return ORTHDION_ERR_NULL;
     if (reinterpret_cast<uintptr_t>(workspace) % 256) return ORTHDION_ERR_WORKSPACE;
-    Batching bt = make_batches(&h, 1);
-    sr->lay = make_layout(&h, 1, bt.scratch_bytes);
+    Batching bt;
+    plan_call(&h, 1, workspace_bytes, &bt, &sr->lay);
     if (workspace_bytes < sr->lay.total) return ORTHDION_ERR_WORKSPACE;
     if ((e = ensure_attributes())) return e;
     char* ws = reinterpret_cast<char*>(workspace);
-    sr->c = ClassRun{h, &sr->batch, scratch_layout(h, 1)};
+    sr->c = ClassRun{h, &sr->batch, scratch_layout(h, 1, bt.lean)};
     sr->batch.count = 1; sr->batch.pad = 0; sr->batch.scratch_stride = (int64_t)sr->c.sc.bytes;
     MatWork& w = sr->batch.w[0];
     w.X = X; w.M = M; w.G = G; w.Q = Q;
@@ -840,7 +866,7 @@ int shard_setup(orthdion_t h, void* X, float* M, const void* G, float* Q, void* 
 void shard_gram(ShardRun& sr, const ImgRef& src, int64_t rows, cudaStream_t st) {
     const orthdion_plan* p = sr.c.p;
     const Sel gram = sel(W_SCRATCH, sr.c.sc.gram);
-    tensor_gram(p->r, p->passes[1], sr.batch, src, rows, gram, sel(W_SCRATCH, sr.c.sc.gram_part), 0, 1, st);
+    tensor_gram(p->r, p->passes[1], sr.batch, src, rows, gram, sel(W_SCRATCH, sr.c.sc.gram_part), sr.c.sc.ts.gram_parts_n, 0, st);
     launch(gram_diag_kernel, dim3((unsigned)((p->r + 255) / 256)), 256, 0, 1, prof::S_MISC, st, sr.batch, gram, p->r, sr.c.sc.ts.colsq,
            (int)(4 * ((rows + 127) / 128)));
 }
@@ -876,7 +902,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     engine_error() = 0;
     overlap_launches() = overlap_pays(&h, 1);
     if (phase == 0) {
-        tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), 1, st, OUT_SUM);
+        tensor_k1(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_SUM);
     } else if (phase == 1) {
         // the summed Y sits in the P slot: image and column squares, then the usual left QR
         if (!small_qr(p, p->m)) {
@@ -885,7 +911,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
                    st, sr->batch, sel(W_P), p->m, r, ts.colsq);
         }
         qr_stage(cls, only, 0, merged, 1, st, true);
-        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), 1, st, OUT_IMAGE);
+        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_IMAGE);
         if (orth) {
             shard_gram(*sr, ts.r, p->n, st);
         } else {
@@ -927,9 +953,9 @@ int orthdion_shard_reduce_buffer(orthdion_t h, int32_t phase, void* workspace, f
     if (h->engine != ORTHDION_ENGINE_TENSOR) return ORTHDION_ERR_INVALID_ARG;
     const bool orth = h->mode == ORTHDION_MODE_ORTH;
     if (phase < 0 || phase > (orth ? 2 : 1)) return ORTHDION_ERR_INVALID_ARG;
-    Batching bt = make_batches(&h, 1);
-    Layout lay = make_layout(&h, 1, bt.scratch_bytes);
-    Scratch sc = scratch_layout(h, 1);
+    // (none of these offsets depends on the partial results)
+    Layout lay = make_layout(&h, 1, 0);
+    Scratch sc = scratch_layout(h, 1, false);
     char* ws = reinterpret_cast<char*>(workspace);
     if (phase == 0) {
         *buffer = reinterpret_cast<float*>(ws + lay.p_off[0]);

@@ -1544,6 +1544,8 @@ struct TensorScratch {      // where the images of one matrix live inside its sc
     int64_t rscale;         // fp32 inverse of the scale of R's fp16 plane
     int64_t fdiag, fstat, fscale;   // factor kernel: fp32 [r] Gram diagonal, statistics of the diagonal blocks,
                             // fp32 [r + 1] correction of the rounded diagonal of L^{-1}
+    // partial results in memory (1: none) of Y = B Q_prev, of R = B^T P and of the Gram products over m and n rows
+    int32_t y_parts, r_parts, gram_parts_m, gram_parts_n;
 };
 
 inline bool tensor_engine_supports(int64_t m, int64_t n, int32_t r) {
@@ -1566,18 +1568,19 @@ inline ImgRef no_img() { ImgRef im; im.off = -1; im.rows_pad = 0; im.panels = 0;
 
 // The offsets of linv, cnorm, rscale, fdiag, fstat, fscale and colsq depend on r only (everything whose size depends on
 // the matrix shape comes after them), so that one Cholesky launch can serve matrices of
-// different shapes.
+// different shapes.  The image of L that the factor kernel works on lies where the image of Q does, which is written after the
+// last factorisation (and is as tall: n >= r).
 // half_planes: P, R, Q carry the fp16 plane (fused pass in fp16).
 inline size_t tensor_scratch_layout(int64_t m, int64_t n, int32_t r, bool half_planes, size_t off, TensorScratch* ts) {
     const int64_t kmax = std::max(m, n);
     off = (off + 1023) / 1024 * 1024;
     auto take = [&](int64_t bytes) { int64_t o = (int64_t)off; off += (size_t)((bytes + 1023) / 1024 * 1024); return o; };
     ts->linv = make_img(take(img_bytes(r, r)), r, r);
-    ts->cnorm = take((int64_t)r * 4);
-    ts->rscale = take(16);
-    ts->fdiag = take((int64_t)r * 4);
-    ts->fstat = take(CT_STAT_FLOATS * 4);
-    ts->fscale = take((int64_t)(r + 1) * 4);
+    ts->cnorm = take(3 * (int64_t)r * 4 + 32 + CT_STAT_FLOATS * 4);       // (r is a multiple of 16)
+    ts->fdiag = ts->cnorm + (int64_t)r * 4;
+    ts->fscale = ts->fdiag + (int64_t)r * 4;
+    ts->rscale = ts->fscale + (int64_t)r * 4 + 16;
+    ts->fstat = ts->rscale + 16;
     ts->colsq = take(4 * ((kmax + 127) / 128) * (int64_t)r * 4);
     const int pl = half_planes ? 3 : 2;
     ts->w0 = make_img(take(img_bytes(kmax, r)), kmax, r);
@@ -1852,12 +1855,14 @@ inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     const int per = (kb + want - 1) / want;
     return (kb + per - 1) / per;             // every chunk non-empty
 }
-// Partial results in memory of a product in a call of `matrices`: the chunks, or 1 where they stay in tensor memory.
+// Partial results in memory of a product in a call of `matrices`: the chunks, or 1 where they stay in tensor memory
+// (up to rank 128 always, when the workspace is to be `lean`).
 // Measured (before: always in memory, added up, packed and squared by three kernels): 154 matrices of a 1.1B model
 // at r = 128 9.7 -> 8.6 ms a step; one 4096 x 4096 matrix at r = 256, three kernels in one, 0.633 -> 0.609 ms.
-inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices) {
+inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices, bool lean) {
     const int chunks = buffer_chunks(r, out_rows, depth);
     if (r > 128 || chunks == 1) return chunks;
+    if (lean) return 1;
     const int64_t tiles = matrices * ((out_rows + tc::BM - 1) / tc::BM);
     const int kb = (int)((depth + tc::BK - 1) / tc::BK);
     return product_depth(tiles, chunks, kb) + partial_cost(tiles, chunks, r) < product_depth(tiles, 1, kb) ? chunks : 1;
@@ -1953,11 +1958,11 @@ enum ProductOut : int {
 };
 // Y = (M + G) Q_prev  -> image w0 (+ column squares)              (Alg. 1, buffer and left-factor steps)
 // First kernel of a step: its packing of Q_prev also clears the status words.
-// part: scratch for the partial results of a depth split.  matrices: of the whole call.
+// part: scratch for the partial results of a depth split (ts.y_parts of them).
 inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const Batch& b, const TensorScratch& ts,
-                      Sel part, int matrices, cudaStream_t st, ProductOut kind) {
+                      Sel part, cudaStream_t st, ProductOut kind) {
     launch_pack(b, Sel{W_Q, 0, 0}, n, r, ts.qprev, st, true);
-    const int ksplit = kind == OUT_SUM ? 1 : buffer_ksplit(r, m, n, matrices);
+    const int ksplit = kind == OUT_SUM ? 1 : ts.y_parts;
     tc::GemmArgs g{};
     if (kind != OUT_SUM && ksplit == 1) g.acc_chunks = buffer_chunks(r, m, n);
     g.Mrows = (int32_t)m; g.Ncols = r; g.Kdim = (int32_t)n; g.BN = buffer_bn(r, m, b.count);
@@ -1977,8 +1982,8 @@ inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const
 
 // R = (M + G)^T P  -> fp32 R slot, image r (+ column squares)     (Alg. 1, right-factor step)
 inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const Batch& b, const TensorScratch& ts,
-                      Sel part, int matrices, cudaStream_t st, ProductOut kind) {
-    const int ksplit = buffer_ksplit(r, n, m, matrices);
+                      Sel part, cudaStream_t st, ProductOut kind) {
+    const int ksplit = ts.r_parts;
     tc::GemmArgs g{};
     if (ksplit == 1) g.acc_chunks = buffer_chunks(r, n, m);
     g.Mrows = (int32_t)n; g.Ncols = r; g.Kdim = (int32_t)m; g.BN = buffer_bn(r, n, b.count);
@@ -2037,10 +2042,12 @@ inline int gram_chunks(int r, int64_t rows) {
     return (kb + per - 1) / per;             // every chunk non-empty
 }
 // Partial matrices in memory of a Gram product in a call of `matrices`.  Above r = 256 the line is where the
-// undivided tiles fill the device (there the partial matrices would be megabytes each).  Measured, the Gram
+// undivided tiles fill the device (there the partial matrices would be megabytes each), and there are none
+// when the workspace is to be `lean`.  Measured, the Gram
 // products of a step: one 11008 x 4096 matrix at r = 1024 0.64 -> 0.35 ms, one 4096 x 3584 matrix at r = 512 0.36 -> 0.26.
-inline int gram_ksplit(int r, int64_t rows, int matrices) {
+inline int gram_ksplit(int r, int64_t rows, int matrices, bool lean) {
     if (r <= 256) return gram_chunks(r, rows);
+    if (lean) return 1;
     const int room = r % 256 ? SPLIT_SMS : SPLIT_SMS / 2;
     return (int64_t)matrices * gram_tiles(r) <= room ? gram_chunks(r, rows) : 1;
 }
@@ -2065,10 +2072,10 @@ gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int6
 }
 
 // Gram = src^T src (src: image of a rows x r matrix); only tiles that touch the lower triangle.
-// part: scratch for gram_ksplit(r, rows, matrices) partial matrices (used when that is more than one).
-inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t rows, Sel gram, Sel part,
-                        int only_shift_bit, int matrices, cudaStream_t st) {
-    const int ksplit = gram_ksplit(r, rows, matrices), chunks = gram_chunks(r, rows);
+// part: scratch for the `ksplit` partial matrices (used when that is more than one).
+inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t rows, Sel gram, Sel part, int ksplit,
+                        int only_shift_bit, cudaStream_t st) {
+    const int chunks = gram_chunks(r, rows);
     tc::GemmArgs g{};
     g.Mrows = r; g.Ncols = r; g.Kdim = (int32_t)rows; g.BN = image_bn(r, r, (int64_t)b.count * (ksplit > 1 ? chunks : 1), true);
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = src; g.n2 = no_img(); g.lower_only = 1;

@@ -71,6 +71,17 @@ def test_grouped_workspace_is_at_least_the_sum_of_factors(L):
         b.orthdion_destroy(h)
 
 
+@pytest.mark.parametrize("shape", [(4096, 3072, 512), (2560, 4096, 512), (3072, 1024, 768), (5632, 4096, 384), (14336, 11008, 128),
+                                   (8192, 13824, 128), (10109, 37928, 32), (6256, 1456, 448)])
+def test_partial_results_keep_no_plan_out_of_the_built_in_scratch(L, shape):
+    # the images and fixed slots of these plans fit 64 MiB, with partial results of the products they do not:
+    # those are an option, and orthdion_step_noalloc takes the plans without them
+    from paper_2605_16341_b200 import binding as b
+    h = b.orthdion_create(*shape, 0.95, 0.01, 0.0, 0)
+    assert b.orthdion_workspace_bytes(h) <= b.NOALLOC_SCRATCH_BYTES
+    b.orthdion_destroy(h)
+
+
 def test_default_pass_counts_follow_dtypes_and_feedback_form(L):
     """The pass counts of the fused feedback/update product follow the plan until the caller fixes
     them: one fp16 pass each for bf16 weights in the momentum form (|b| <= 0.1 |a|), three bf16

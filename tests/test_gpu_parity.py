@@ -325,6 +325,26 @@ def test_grouped_matches_single_and_is_deterministic(engine):
         od.orthdion_destroy(h)
 
 
+def test_workspace_of_a_larger_group_serves_a_smaller_one():
+    """Calls of a few matrices keep partial results of the products in memory, so four of these matrices ask for more
+    workspace than five do.  In the workspace of the five they are stepped without them, to the same bits."""
+    m, n, r = 1040, 1056, 48
+    h = od.orthdion_create(m, n, r, 0.95, 0.01, 0.0, od.MODE_ORTH)
+    need = {k: od.orthdion_workspace_bytes_grouped([h] * k) for k in (4, 5)}
+    assert need[4] > need[5]
+    probs = [make_problem(m, n, r, BF16, BF16, seed=500 + i) for i in range(4)]
+    outs = []
+    for k in (4, 5):
+        X, M, G, Q = ([p[j].cuda() for p in probs] for j in (1, 2, 3, 4))
+        ws = poisoned_workspace(need[k])
+        od.orthdion_step_grouped(od.PointerTable([h] * 4, X, M, G, Q), ws)
+        torch.cuda.synchronize()
+        assert od.orthdion_last_status([h] * 4, ws) == [0] * 4
+        outs.append(X + M + Q)
+    assert all(torch.equal(a, b) for a, b in zip(*outs))
+    od.orthdion_destroy(h)
+
+
 def test_internal_streams_change_no_bit():
     """A grouped call runs its launch batches on 1 to 8 internal streams: two steps of five classes
     (twelve matrices) leave the same bits whatever the number of streams."""

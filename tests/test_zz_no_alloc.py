@@ -82,6 +82,28 @@ def test_noalloc_matches_step_on_two_calls_in_a_row(shape, dtype, mode):
     od.orthdion_destroy(h)
 
 
+# plans that fit the built-in scratch only without partial results (Gram chunks at r = 512 and 448, chunks of the products
+# with the buffer at r = 96 and 112): the bits of orthdion_step with a workspace that holds them
+@pytest.mark.parametrize("shape", [(2560, 4096, 512), (6256, 1456, 448), (1632, 19928, 96), (20240, 1624, 112)])
+def test_noalloc_takes_plans_whose_partial_results_do_not_fit(shape):
+    m, n, r = shape
+    dtype = torch.bfloat16
+    X, M, Gs, Q = _problem(m, n, r, dtype, seed=m + n + r)
+    h = od.orthdion_create(m, n, r, 0.95, 0.01, 0.0, od.MODE_ORTH)
+    assert od.orthdion_workspace_bytes(h) <= od.NOALLOC_SCRATCH_BYTES
+    ws = od.alloc_workspace(3 * od.NOALLOC_SCRATCH_BYTES)
+    G = Gs[0].cuda()
+    a = [t.cuda() for t in (X, M, Q)]
+    b = [t.cuda() for t in (X, M, Q)]
+    status = torch.full((1,), -1, dtype=torch.int32, device="cuda")
+    od.orthdion_step(h, a[0], a[1], G, a[2], ws)
+    od.orthdion_step_noalloc(h, b[0], b[1], G, b[2], status)
+    torch.cuda.synchronize()
+    assert status.item() == od.orthdion_last_status([h], ws)[0] == 0
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    od.orthdion_destroy(h)
+
+
 def test_noalloc_rejects_plans_beyond_the_built_in_scratch():
     h = od.orthdion_create(8192, 8192, 512, 0.95, 0.01, 0.0, od.MODE_ORTH)
     assert od.orthdion_workspace_bytes(h) > od.NOALLOC_SCRATCH_BYTES
