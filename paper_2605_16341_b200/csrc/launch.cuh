@@ -15,8 +15,9 @@ __device__ __forceinline__ void grid_dependency_launch() { asm volatile("griddep
 // both at once, for kernels without a prologue of their own
 __device__ __forceinline__ void grid_dependency() { grid_dependency_launch(); grid_dependency_wait(); }
 
-// First error met while preparing launches of the current step call (0 = none); one per host
+// First error met while preparing launches of the current step call (0 = none, 1 and 2: tensor maps); one per host
 // thread, so that concurrent step calls do not see each other's.
+constexpr int LAUNCH_FAILED = 3;       // the runtime's last error says why
 inline int& engine_error() { static thread_local int e = 0; return e; }
 
 // Whether the launches of the current call overlap as described above (one flag per host thread).
@@ -45,7 +46,7 @@ inline void launch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, 
     cfg.attrs = attr;
     cfg.numAttrs = (unsigned)n;
     prof::Scope scope(stage, st);
-    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess) engine_error() = 3;
+    if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess && !engine_error()) engine_error() = LAUNCH_FAILED;
 }
 
 }  // namespace od

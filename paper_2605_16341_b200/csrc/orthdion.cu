@@ -299,6 +299,17 @@ void launch_simt(const Batch& b, int64_t Md, int64_t Nd, int64_t Kd, RA ra, RB r
            parts, stage, st, b, Md, Nd, Kd, parts, ra, rb, out);
 }
 
+// What became of the launches since engine_error() was reset.  Clears the runtime's last error, so that a launch
+// that failed here does not turn up in a later call's check.
+int launch_result() {
+    const cudaError_t ce = cudaGetLastError();
+    const int ee = engine_error();
+    if (!ee && ce == cudaSuccess) return ORTHDION_OK;
+    if (ee && ee != LAUNCH_FAILED) std::fprintf(stderr, "orthdion: tensor map setup failed (%d)\n", ee);
+    else std::fprintf(stderr, "orthdion: launch failed: %s\n", cudaGetErrorString(ce));
+    return ORTHDION_ERR_CUDA;
+}
+
 Sel sel(int where, int64_t off = 0) { return Sel{where, 0, off}; }
 
 // One class of a group while it is being stepped.
@@ -791,17 +802,8 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
         } else {
             run_group(cls, merged, db, count, st);
         }
-        if (engine_error()) {
-            std::fprintf(stderr, "orthdion: tensor map setup failed (%d)\n", engine_error());
-            rc = ORTHDION_ERR_CUDA;
-            break;
-        }
-        cudaError_t ce = cudaGetLastError();
-        if (ce != cudaSuccess) {
-            std::fprintf(stderr, "orthdion: launch failed: %s\n", cudaGetErrorString(ce));
-            rc = ORTHDION_ERR_CUDA;
-            break;
-        }
+        rc = launch_result();
+        if (rc) break;
     }
     return rc;
 }
@@ -939,13 +941,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     }
     delete merged;
     delete sr;
-    if (engine_error()) return ORTHDION_ERR_CUDA;
-    cudaError_t ce = cudaGetLastError();
-    if (ce != cudaSuccess) {
-        std::fprintf(stderr, "orthdion: launch failed: %s\n", cudaGetErrorString(ce));
-        return ORTHDION_ERR_CUDA;
-    }
-    return ORTHDION_OK;
+    return launch_result();
 }
 
 int orthdion_shard_reduce_buffer(orthdion_t h, int32_t phase, void* workspace, float** buffer, int64_t* count) {

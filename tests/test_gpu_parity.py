@@ -291,6 +291,23 @@ def test_buffer_whose_squared_column_norms_are_subnormal(engine, shape, scale):
     one_step_compare(spec, X, M * scale, G * scale, Q, mode=od.MODE_ORTH, engine=engine)
 
 
+def test_rejected_launch_is_reported_and_leaves_no_error_behind(capfd):
+    # the fp32 engine's row tiles go along the grid's second dimension, which ends at 65535: the runtime refuses the
+    # launches of a taller matrix.  The call says so, and the next one does not find that error
+    tall = GpuMatrix(wl.MatrixSpec("t", 65536 * 64, 1, 1, F32, F32), torch.zeros(65536 * 64, 1), torch.zeros(65536 * 64, 1),
+                     torch.ones(1, 1), mu=0.95, eta=0.01, mode=od.MODE_ORTH)
+    tall.ws.zero_()
+    with pytest.raises(od.OrthDionError) as e:
+        tall.step(torch.zeros(65536 * 64, 1))
+    assert e.value.code == -5
+    err = capfd.readouterr().err
+    assert "launch failed: invalid" in err and "tensor map" not in err
+    torch.cuda.synchronize()
+    tall.close()
+    spec, X, M, G, Q = make_problem(256, 384, 32, F32, F32, seed=8)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR)
+
+
 # ------------------------------------------------------------------ grouped == single, resume
 @pytest.mark.parametrize("engine", ENGINES, ids=ENGINE_IDS)
 def test_grouped_matches_single_and_is_deterministic(engine):
