@@ -472,12 +472,6 @@ __device__ __forceinline__ int mn_pieces(const GemmArgs& g, int kb) {
     const int left = g.Kdim - kb * BK;
     return (min(left, BK) + g.ks - 1) / g.ks;
 }
-// N_IMG_K: the pieces of depth block kb are 128-row chunks of the tile's N range; with a lower
-// triangular N-side a chunk is skipped once the depth block lies beyond its last row.
-__device__ __forceinline__ bool k_piece_active(const GemmArgs& g, const TileCoord& c, int kb, int chunk) {
-    return !g.tri || kb * BK <= c.n0 + min(c.bn, (chunk + 1) * 128) - 1;
-}
-
 // ------------------------------------------------------------------------------------------
 // The GEMM kernel.  D (128 x bn, fp32 in tensor memory) = A (128 x K) * N^T (bn x K).
 //   warp 0        producer: bulk copies of image tiles into the A ring and the N ring
@@ -488,7 +482,7 @@ __device__ __forceinline__ bool k_piece_active(const GemmArgs& g, const TileCoor
 //          A_IMG_K / A_IMG_MN   image tile, K-major / MN-major
 //          A_BUF_ROW            rows of B = M + G      (K-major;  Y = B Q_prev, Alg. 1, left-factor step)
 //          A_BUF_COL            columns of B = M + G   (MN-major; R = B^T P,    Alg. 1, right-factor step)
-// NMODE  N_IMG_K   pieces = 128-row chunks of the N range, 64 deep (image K-major)
+// NMODE  N_IMG_K   pieces = 128-row chunks of the N range, 64 deep (image K-major; the fused pass)
 //        N_IMG_MN  pieces = ks-deep slices of the whole N range (image MN-major)
 // EPI    EPI_STORE  fp32 copy and/or split image (+ column-square partials) of D
 //        EPI_K5     M <- a (M+G) - b D1,  X <- c X - d D2     (Alg. 1, update and error-feedback steps), D1 = P R^T, D2 = P Q^T
@@ -613,7 +607,6 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     if (nkb < 0) { nc = decode_tile<EPI>(batch, g, nt_, scache, crank); nkb = nc.kb_begin; npc = 0; }
                     if (!nc.active || nkb >= nc.kb_end) { nt_ = next(nt_); nkb = -1; npc = 0; continue; }
                     if (npc >= n_pieces(nkb)) { ++nkb; npc = 0; continue; }
-                    if (NMODE == N_IMG_K && !k_piece_active(g, nc, nkb, npc)) { ++npc; continue; }
                     break;
                 }
             };
@@ -769,14 +762,13 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         // One thread issues.  A tcgen05.mma of N = 256 occupies the tensor core for 128 cycles, so the
         // scalar work per instruction has to stay at a handful of operations: every descriptor is a
         // constant high part plus (shared address >> 4), advanced by additions only.
+        static_assert(NMODE == N_IMG_MN || (EPI == EPI_K5 && AMODE == A_IMG_K), "only the fused pass has a K-major N-side");
         int as = 0, ns = 0; uint32_t aph = 0, nph = 0;
         int acc = 0; uint32_t acc_phase = 0;
         bool ok = true;
         // descriptor high parts (layout, strides) and address units of 16 bytes
-        const uint64_t a_hi = A_MN ? smem_desc(0, 8192, 1024) : smem_desc(0, 16, 1024);
-        const uint64_t n_hi = smem_desc(0, 16, 1024);
-        const uint32_t a_slice16 = A_MN ? (2048u >> 4) : (32u >> 4);        // one 16-deep slice of the A tile
-        const uint32_t n_slice16 = 32u >> 4;
+        const uint64_t op_hi = smem_desc(0, 16, 1024);
+        const uint32_t slice16 = 32u >> 4;               // one 16-deep slice of either operand
         const uint32_t a_ring16 = smem_u32(a_ring) >> 4, n_ring16 = smem_u32(n_ring) >> 4;
         const uint32_t a_slot16 = (uint32_t)g.a_slot_bytes >> 4, n_slot16 = (uint32_t)g.n_piece_bytes >> 4;
         constexpr uint32_t MROWS = PAIR ? 256u : 128u;
@@ -791,7 +783,6 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 const int chunks = (c.bn + 127) / 128;
                 const int nsl = min(4, (g.Kdim - kb * BK + 15) / 16);
                 for (int ch = 0; ch < chunks && ok; ++ch) {
-                    if (!k_piece_active(g, c, kb, ch)) continue;
                     if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
                     if (lane == 0) {
                         const uint32_t sa = smem_u32(a_ring + as * g.a_slot_bytes);
@@ -799,32 +790,30 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         // N of the instruction must be a multiple of 16: round a ragged last chunk up
                         // (rows beyond the matrix are zero in the images; those columns of D are never stored)
                         const uint32_t ncols = (uint32_t)((min(128, c.bn - ch * 128) + 15) / 16 * 16);
-                        const uint32_t idesc = instr_desc(ncols, A_MN ? 1u : 0u, 0u, fmt, MROWS);
+                        const uint32_t idesc = instr_desc(ncols, 0u, 0u, fmt, MROWS);
                         // Fused pass with single-term operands: the R piece and the Q piece lie back
                         // to back in the slot (256 rows of one K-major tile) and their accumulators in
                         // adjacent columns, so one N = 256 instruction serves both products and reads
                         // the P slice from shared memory once.
-                        const bool both = EPI == EPI_K5 && g.passes == 1 && g.passes2 == 1 && ncols == 128 && g.BN == 128;
-                        const uint32_t idesc2 = instr_desc(256u, A_MN ? 1u : 0u, 0u, fmt, MROWS);
+                        const bool both = g.passes == 1 && g.passes2 == 1 && ncols == 128 && g.BN == 128;
+                        const uint32_t idesc2 = instr_desc(256u, 0u, 0u, fmt, MROWS);
                         if (both) {
                             // one instruction per 16-deep slice; descriptors advanced by additions so
                             // that the issuing thread spends a handful of operations per instruction
-                            uint64_t a0 = a_hi + (a_ring16 + as * a_slot16);
-                            uint64_t b0 = n_hi + (n_ring16 + ns * n_slot16);
+                            uint64_t a0 = op_hi + (a_ring16 + as * a_slot16);
+                            uint64_t b0 = op_hi + (n_ring16 + ns * n_slot16);
                             const uint32_t d1 = dacc + ch * 128;
                             umma_any<PAIR>(d1, a0, b0, idesc2, kb > c.kb_begin ? 1u : 0u);
                             for (int j = 1; j < nsl; ++j) {
-                                a0 += a_slice16; b0 += n_slice16;
+                                a0 += slice16; b0 += slice16;
                                 umma_any<PAIR>(d1, a0, b0, idesc2, 1u);
                             }
                         }
                         // (In the general form below the descriptors are rebuilt per instruction on
                         // purpose: its N = 128 instructions ran best when not issued back to back.)
                         for (int j = 0; j < nsl && !both; ++j) {
-                            const uint64_t a0 = A_MN ? smem_desc(sa + j * 2048, 8192, 1024)
-                                                     : smem_desc(sa + j * 32, 16, 1024);
-                            const uint64_t a1 = A_MN ? smem_desc(sa + A_TERM_BYTES + j * 2048, 8192, 1024)
-                                                     : smem_desc(sa + A_TERM_BYTES + j * 32, 16, 1024);
+                            const uint64_t a0 = smem_desc(sa + j * 32, 16, 1024);
+                            const uint64_t a1 = smem_desc(sa + A_TERM_BYTES + j * 32, 16, 1024);
                             const uint64_t b0 = smem_desc(sn + j * 32, 16, 1024);
                             const uint64_t b1 = smem_desc(sn + A_TERM_BYTES + j * 32, 16, 1024);
                             const uint32_t accum = (kb > c.kb_begin || j > 0) ? 1u : 0u;
@@ -834,16 +823,14 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                                 umma_any<PAIR>(d1, a0, b1, idesc, 1u);
                                 umma_any<PAIR>(d1, a1, b0, idesc, 1u);
                             }
-                            if (EPI == EPI_K5) {
-                                const uint32_t s2 = sn + n1_terms * A_TERM_BYTES;
-                                const uint64_t c0 = smem_desc(s2 + j * 32, 16, 1024);
-                                const uint64_t c1 = smem_desc(s2 + A_TERM_BYTES + j * 32, 16, 1024);
-                                const uint32_t d2 = dacc + g.BN;
-                                umma_any<PAIR>(d2, a0, c0, idesc, accum);
-                                if (g.passes2 == 3) {
-                                    umma_any<PAIR>(d2, a0, c1, idesc, 1u);
-                                    umma_any<PAIR>(d2, a1, c0, idesc, 1u);
-                                }
+                            const uint32_t s2 = sn + n1_terms * A_TERM_BYTES;
+                            const uint64_t c0 = smem_desc(s2 + j * 32, 16, 1024);
+                            const uint64_t c1 = smem_desc(s2 + A_TERM_BYTES + j * 32, 16, 1024);
+                            const uint32_t d2 = dacc + g.BN;
+                            umma_any<PAIR>(d2, a0, c0, idesc, accum);
+                            if (g.passes2 == 3) {
+                                umma_any<PAIR>(d2, a0, c1, idesc, 1u);
+                                umma_any<PAIR>(d2, a1, c0, idesc, 1u);
                             }
                         }
                         commit_any<PAIR>(n_empty0 + 8 * ns);
