@@ -86,13 +86,13 @@ struct GemmArgs {
     int32_t a_slots, a_slot_bytes;           // A ring
     int32_t epi_bufs;                        // fused pass: 8 KB epilogue buffers per warp (1 or 2)
     int32_t pair;                            // launched as CTA pairs (clusters of two, M = 256 instructions)
-    int32_t ksplit, kb_per_chunk;            // depth split: a tile is computed as `ksplit` partial products over
-                                             // kb_per_chunk depth blocks each, stored split_stride floats apart
-    int64_t split_stride;
-    int32_t run;                             // Gram product: this many consecutive tiles (the depth chunks of one result
-                                             // tile) go to the same CTA, which adds each to what it has stored
-    int32_t acc_chunks;                      // the same chunks within one tile: accumulators side by side in tensor memory,
-                                             // added up in chunk order by the epilogue (products with B)
+    int32_t chunks, kb_per_chunk;            // depth chunks whose sums are added up in order, and their depth blocks
+    int32_t acc_chunks;                      // chunks within one tile: accumulators side by side in tensor memory,
+                                             // added up by the epilogue (products with B)
+    int32_t ksplit, kb_per_tile;             // tiles of such chunks that a result tile is computed as, their depth
+    int64_t split_stride;                    // blocks; stored split_stride floats apart
+    int32_t run;                             // ksplit or 1: so many consecutive tiles (those of one result tile) go to the
+                                             // same CTA, which adds each to what it has stored
     int64_t rscale_off;                      // fp16 fused pass: scratch offset of 1 / (scale of R's plane)
     int64_t ld;                              // leading dimension of M, G, X
     ImgRef a, n1, n2;
@@ -457,7 +457,7 @@ __device__ __forceinline__ TileCoord decode_tile(const Batch& batch, const GemmA
     c.kb_begin = 0;
     c.kb_end = g.k_blocks;
     if (g.tri) c.kb_end = min(g.k_blocks, (c.n0 + c.bn + BK - 1) / BK);
-    if (g.ksplit > 1) { c.kb_begin = c.chunk * g.kb_per_chunk; c.kb_end = min(g.k_blocks, c.kb_begin + g.kb_per_chunk); }
+    if (g.ksplit > 1) { c.kb_begin = c.chunk * g.kb_per_tile; c.kb_end = min(g.k_blocks, c.kb_begin + g.kb_per_tile); }
     if (c.b != sc.b) { sc.b = c.b; sc.st = *batch.w[c.b].status; }
     const int st = sc.st;
     c.active = !(st & ST_FAILED);
@@ -495,19 +495,22 @@ struct K5Pre {      // M, G, X of one 32 x 32 slab: 8 steps of (4 rows x 32 colu
     uint32_t x[8][(XG & 2) ? 2 : 4];
 };
 
-template <int AMODE, int NMODE, int EPI, int XG, bool PAIR>
+// RUN    the tiles come in runs (GemmArgs::run): the Gram product, and products with B that have more chunks than
+//        accumulators.  (Instantiations of their own for the latter: the test for a run alone cost the other
+//        products with B up to 1 % of a step, in registers that the transform warps then lack.)
+template <int AMODE, int NMODE, int EPI, int XG, bool PAIR, bool RUN>
 __global__ void __launch_bounds__(gemm_threads(AMODE, EPI), 1)
 gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArgs g) {
     constexpr int NE = epi_warps(AMODE, EPI);
     // PAIR: launched in clusters of two; rank 0 (the leader) issues every MMA for both CTAs
     const int crank = PAIR ? (int)cluster_ctarank() : 0;
-    const int tile0 = (PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * (AMODE == A_IMG_MN ? g.run : 1);
-    const int tstride = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     constexpr bool A_BUF = a_is_buf(AMODE);
+    const int tile0 = (PAIR ? (int)(blockIdx.x >> 1) : (int)blockIdx.x) * (RUN ? g.run : 1);
+    const int tstride = PAIR ? (int)(gridDim.x >> 1) : (int)gridDim.x;
     // the next tile of this CTA after tile t
     auto next = [&](int t) {
-        if constexpr (AMODE == A_IMG_MN) return (t + 1) % g.run ? t + 1 : t + 1 + (tstride - 1) * g.run;
-        else return t + tstride;
+        if constexpr (!RUN) return t + tstride;
+        else return (t + 1) % g.run ? t + 1 : t + 1 + (tstride - 1) * g.run;
     };
     constexpr bool A_MN = (AMODE == A_IMG_MN || AMODE == A_BUF_COL);
     constexpr bool G_BF16 = (XG & 1) != 0;
@@ -875,8 +878,10 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 const uint32_t taddr = tmem_base + acc * acc_stride + ((uint32_t)(quarter * 32) << 16);
                 float* C = d.has_f32 ? pick(w, d.f32) + (int64_t)c.chunk * g.split_stride : nullptr;
                 unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
-                const bool to_img = d.img.off >= 0;
-                float* csq = d.colsq ? reinterpret_cast<float*>(w.scratch + g.colsq_off) +
+                // (a run of tiles with chunks of their own: image and column squares when the sum is complete)
+                const bool whole = !(A_BUF && RUN) || c.chunk == g.run - 1;
+                const bool to_img = d.img.off >= 0 && whole;
+                float* csq = d.colsq && whole ? reinterpret_cast<float*>(w.scratch + g.colsq_off) +
                                            (int64_t)(c.mt * 4 + quarter) * g.Ncols : nullptr;
                 if constexpr (A_BUF) {
                 // 32 columns at a time: this warp's 32 x 32 block goes through a 4 KB staging buffer so that
@@ -889,6 +894,8 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 // (pairs: the CTA whose rows lie beyond the matrix stores nothing)
                 const bool has_rows = !PAIR || (int64_t)c.mt * BM < g.Mrows;
                 const int bn64 = !has_rows ? 0 : (to_img ? (c.bn + 63) / 64 * 64 : c.bn);
+                // (the last tile of a run may have fewer chunks than the others)
+                const int tile_chunks = RUN && c.chunk > 0 ? (c.kb_end - c.kb_begin + g.kb_per_chunk - 1) / g.kb_per_chunk : g.acc_chunks;
                 const int srow = lane / 4, sch = lane % 4;      // stores: 8 rows x 4 chunks of 8 columns per step
                 for (int cc = 0; cc < bn64; cc += 32) {
                     uint32_t v[2][16];
@@ -902,7 +909,24 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         }
                     }
                     tmem_ld_wait();
-                    for (int ch = 1; ch < g.acc_chunks; ++ch) {
+                    if (RUN && c.chunk > 0 && gi0 + lane < g.Mrows) {
+                        // the sum so far of this lane's row, stored by this warp
+                        const float* o = C + (gi0 + lane) * g.out.ld + c.n0 + cc;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            if (cc + 16 * h < c.bn) {
+#pragma unroll
+                                for (int i = 0; i < 16; i += 4) {
+                                    const float4 x = *reinterpret_cast<const float4*>(o + 16 * h + i);
+                                    v[h][i] = __float_as_uint(x.x + __uint_as_float(v[h][i]));
+                                    v[h][i + 1] = __float_as_uint(x.y + __uint_as_float(v[h][i + 1]));
+                                    v[h][i + 2] = __float_as_uint(x.z + __uint_as_float(v[h][i + 2]));
+                                    v[h][i + 3] = __float_as_uint(x.w + __uint_as_float(v[h][i + 3]));
+                                }
+                            }
+                        }
+                    }
+                    for (int ch = 1; ch < tile_chunks; ++ch) {
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             if (cc + 16 * h < c.bn) {
@@ -1025,7 +1049,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     }
                     if (C) {
                         // fp32 block: 32 rows x 256 bytes, 16-byte chunks swizzled by (row & 7)
-                        const bool add = AMODE == A_IMG_MN && g.run > 1 && c.chunk > 0;
+                        const bool add = RUN && g.run > 1 && c.chunk > 0;
 #pragma unroll
                         for (int ch = 0; ch < 16; ++ch)
                             *reinterpret_cast<float4*>(stg + lane * 256 + ((ch ^ (lane & 7)) << 4)) =
@@ -1418,7 +1442,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         const int xr = AMODE == A_BUF_ROW ? xt / 8 : xt / 16, xc = AMODE == A_BUF_ROW ? xt % 8 : xt % 16;
         const uint32_t dst_off = AMODE == A_BUF_ROW ? xr * 128 + img_chunk_offset(xr, xc)
                                                     : (xc / 8) * 8192 + xr * 128 + img_chunk_offset(xr, xc % 8);
-        for (int t = tile0; t < g.total_tiles && ok; t += tstride) {
+        for (int t = tile0; t < g.total_tiles && ok; t = next(t)) {
             const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
             if (!c.active) continue;
             const MatWork& w = batch.w[c.b];
@@ -1653,11 +1677,17 @@ constexpr bool pair_capable(int nmode, int epi, int xg) {
 
 template <int AMODE, int NMODE, int EPI, int XG>
 inline cudaError_t set_gemm_attr() {
-    cudaError_t e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false>,
+    constexpr bool GRAM = AMODE == tc::A_IMG_MN;
+    cudaError_t e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, GRAM>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
     if constexpr (pair_capable(NMODE, EPI, XG)) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true>,
+            e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true, GRAM>,
+                                     cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
+    }
+    if constexpr (tc::a_is_buf(AMODE)) {
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, true>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
     }
     return e;
@@ -1712,10 +1742,12 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     if (pair) g.m_tiles = (g.m_tiles + 1) / 2;      // scheduled row tiles of 256 rows
     g.n_tiles = (g.Ncols + g.BN - 1) / g.BN;
     g.k_blocks = (g.Kdim + tc::BK - 1) / tc::BK;
-    if (g.ksplit < 1) g.ksplit = 1;
-    if (g.run < 1) g.run = 1;
+    if (g.chunks < 1) g.chunks = 1;
     if (g.acc_chunks < 1) g.acc_chunks = 1;
-    if (g.ksplit * g.acc_chunks > 1) g.kb_per_chunk = (g.k_blocks + g.ksplit * g.acc_chunks - 1) / (g.ksplit * g.acc_chunks);
+    g.kb_per_chunk = (g.k_blocks + g.chunks - 1) / g.chunks;
+    g.kb_per_tile = g.acc_chunks * g.kb_per_chunk;
+    g.ksplit = (g.chunks + g.acc_chunks - 1) / g.acc_chunks;
+    g.run = g.run ? g.ksplit : 1;
     g.total_tiles = b.count * g.m_tiles * g.n_tiles * g.ksplit;
     const int n1_terms = g.passes == 3 ? 2 : 1, n2_terms = g.passes2 == 3 ? 2 : 1;
     const int bn64 = (g.BN + 63) / 64 * 64;
@@ -1780,15 +1812,22 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     else encode_img_map(&g.map_n1, b, g.n1, 128, 1, n1_terms);
     if (EPI == tc::EPI_K5) encode_img_map(&g.map_n2, b, g.n2, 128, 1, n2_terms);
     if (engine_error()) return;
+    constexpr bool GRAM = AMODE == tc::A_IMG_MN;
     if constexpr (pair_capable(NMODE, EPI, XG)) {
         if (pair) {
-            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true>, dim3((unsigned)(2 * std::min(g.total_tiles / g.run, sm_count() / 2))),
+            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true, GRAM>, dim3((unsigned)(2 * std::min(g.total_tiles / g.run, sm_count() / 2))),
                    tc::gemm_threads(AMODE, EPI), smem, 2, stage, st, b, g);
             return;
         }
     }
-    launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false>, dim3((unsigned)std::min(g.total_tiles / g.run, sm_count())),
-           tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
+    const dim3 grid((unsigned)std::min(g.total_tiles / g.run, sm_count()));
+    if constexpr (tc::a_is_buf(AMODE)) {
+        if (g.run > 1) {
+            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, true>, grid, tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
+            return;
+        }
+    }
+    launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, GRAM>, grid, tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
 }
 
 inline tc::Dest dest_none() {
@@ -1815,28 +1854,30 @@ inline int64_t partial_cost(int64_t tiles, int chunks, int r) { return 4 + tiles
 // results are added in a fixed order.  Their number depends on the plan only (rank, rows of the result,
 // depth), so that a matrix gets the same bits alone and in any group; ranks above 256 have one.  Where
 // it shortens a launch the chunks run as tiles of their own and leave
-// fp32 partial results in memory; where it does not, one tile runs through all chunks with an
-// accumulator each, side by side in tensor memory (at most 512 columns: ranks up to 128), and the epilogue
-// adds them up.
-// Up to r = 128 the number is the one that makes the launch of one matrix shortest by the two counts above.  Measured
-// against as many chunks as fit 74 pairs of tiles, none from 37 on: 11008 x 4096, first product, r = 32 0.090 -> 0.074 ms,
-// r = 64 0.091 -> 0.086; 20480 x 4096 r = 32 0.170 -> 0.127, r = 128 0.198 -> 0.176.  Fewer chunks at r = 128, so that two
-// sets of accumulators fit, gain 2 % in a group of 2048-wide matrices and lose 50 % alone (4096 x 4096 0.051 -> 0.070).
+// fp32 partial results in memory; where it does not, up to rank 128, one tile runs through as many chunks as have
+// an accumulator each in the 512 columns of tensor memory, the epilogue adds them up, and where they are not all (five
+// to eight chunks above rank 64) the next tile of the same CTA adds the others to what the first one stored.
+// The tensor core truncates when it adds into its accumulator, so a sum loses the more the longer its chunk: with 11 to 32
+// depth blocks a chunk R = B^T P of a 16384 x 1024 matrix at r = 96 is off by 7e-6, with 64 by 1.3e-5.  Hence at least as
+// many chunks, up to eight of at least eight blocks, as fit 74 pairs of tiles, at any rank.
+// Up to r = 128 it may be more: the number that makes the launch of one matrix shortest by the two counts above.  Measured
+// against the first rule alone: 11008 x 4096, first product, r = 32 0.090 -> 0.074 ms,
+// r = 64 0.091 -> 0.086; 20480 x 4096 r = 32 0.170 -> 0.127, r = 128 0.198 -> 0.176.  Against four chunks at most above
+// r = 64: one 16384 x 1024 matrix at r = 96 0.470 -> 0.426 ms a step, 2048 x 5632 r = 128 0.379 -> 0.368; in a group, where
+// the tiles of a run follow one another, six layers of a 1.1B model at r = 128 1.127 -> 1.155.
 inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     if (r > 256) return 1;
-    const int kb = (int)((depth + tc::BK - 1) / tc::BK);
-    int want = 1;
+    const int kb = (int)((depth + tc::BK - 1) / tc::BK), pairs = (int)((out_rows + 255) / 256);
+    int want = pairs < 37 && kb >= 32 ? std::min({8, 74 / pairs, kb / 8}) : 1;
     if (r <= 128) {
         const int64_t tiles = (out_rows + tc::BM - 1) / tc::BM;
         int64_t best = product_depth(tiles, 1, kb);
+        int fast = 1;
         for (int v = 2; v <= std::min(r <= 64 ? 8 : 4, kb / 4); ++v) {
             const int64_t cost = product_depth(tiles, v, kb) + partial_cost(tiles, v, r);
-            if (cost < best) { best = cost; want = v; }
+            if (cost < best) { best = cost; fast = v; }
         }
-    } else {
-        const int tiles = (int)((out_rows + 255) / 256);
-        if (tiles >= 37 || kb < 32) return 1;
-        want = std::min({8, 74 / tiles, kb / 8});
+        want = std::max(want, fast);
     }
     if (want < 2) return 1;
     const int per = (kb + want - 1) / want;
@@ -1855,8 +1896,14 @@ inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices, b
     return product_depth(tiles, chunks, kb) + partial_cost(tiles, chunks, r) < product_depth(tiles, 1, kb) ? chunks : 1;
 }
 
-__global__ void gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit,
-                                   int only_shift_bit);
+// The chunks of a product with B in `parts` tiles of their own, or in as few tiles as tensor memory allows.
+inline void set_chunks(tc::GemmArgs& g, int r, int chunks, int parts) {
+    g.chunks = chunks;
+    if (parts > 1 || chunks == 1) return;
+    const int fit = 512 / r, tiles = (chunks + fit - 1) / fit;
+    g.acc_chunks = (chunks + tiles - 1) / tiles;
+    g.run = tiles > 1 ? 1 : 0;
+}
 
 // Columns per tile of a product with B, out of r (count matrices in the launch).  A wide tile forms B's terms once
 // for all columns; narrow ones form them again for every tile (from L2), which pays only where all of
@@ -1951,18 +1998,18 @@ inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const
     launch_pack(b, Sel{W_Q, 0, 0}, n, r, ts.qprev, st, true);
     const int ksplit = kind == OUT_SUM ? 1 : ts.y_parts;
     tc::GemmArgs g{};
-    if (kind != OUT_SUM && ksplit == 1) g.acc_chunks = buffer_chunks(r, m, n);
+    if (kind != OUT_SUM) set_chunks(g, r, buffer_chunks(r, m, n), ksplit);
     g.Mrows = (int32_t)m; g.Ncols = r; g.Kdim = (int32_t)n; g.BN = buffer_bn(r, m, b.count);
     g.passes = passes; g.passes2 = 1; g.ld = n; g.n1 = ts.qprev; g.a = no_img(); g.n2 = no_img();
     g.colsq_off = ts.colsq;
     g.out.normal = dest_none();
-    if (ksplit > 1) { g.out.normal.f32 = part; g.out.normal.has_f32 = 1; g.ksplit = ksplit; g.split_stride = m * r; }
+    if (ksplit > 1) { g.out.normal.f32 = part; g.out.normal.has_f32 = 1; g.split_stride = m * r; }
     else if (kind != OUT_IMAGE) { g.out.normal.f32 = Sel{W_P, 0, 0}; g.out.normal.has_f32 = 1; }
-    else { g.out.normal.img = img_view(ts.w0, m); g.out.normal.colsq = 1; }
+    else { g.out.normal.img = img_view(ts.w0, m); g.out.normal.colsq = 1; g.out.normal.has_f32 = g.run; }
     g.out.shifted = g.out.normal; g.out.ld = r;
     if (g_bf16) launch_gemm<tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 1>(b, g, prof::S_K1, st);
     else launch_gemm<tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_K1, st);
-    // (the sum goes through the fp32 P slot, which holds nothing yet at this point of a step)
+    // (a sum in parts goes through the fp32 P slot, which holds nothing yet at this point of a step)
     if (ksplit > 1 && kind == OUT_IMAGE)
         finish_split_product(b, Sel{W_P, 0, 0}, part, m, r, ksplit, img_view(ts.w0, m), ts.colsq, prof::S_K1, st);
 }
@@ -1972,12 +2019,12 @@ inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const
                       Sel part, cudaStream_t st, ProductOut kind) {
     const int ksplit = ts.r_parts;
     tc::GemmArgs g{};
-    if (ksplit == 1) g.acc_chunks = buffer_chunks(r, n, m);
+    set_chunks(g, r, buffer_chunks(r, n, m), ksplit);
     g.Mrows = (int32_t)n; g.Ncols = r; g.Kdim = (int32_t)m; g.BN = buffer_bn(r, n, b.count);
     g.passes = passes; g.passes2 = 1; g.ld = n; g.n1 = ts.p; g.a = no_img(); g.n2 = no_img();
     g.colsq_off = ts.colsq;
     g.out.normal = dest_none(); g.out.normal.has_f32 = 1;
-    if (ksplit > 1) { g.out.normal.f32 = part; g.ksplit = ksplit; g.split_stride = n * r; }
+    if (ksplit > 1) { g.out.normal.f32 = part; g.split_stride = n * r; }
     else {
         g.out.normal.f32 = Sel{W_R, 0, 0};
         if (kind == OUT_IMAGE) { g.out.normal.img = ts.r; g.out.normal.colsq = 1; }
@@ -2070,9 +2117,9 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
     g.out.shifted = g.out.normal; g.out.ld = r;
     g.cscale_off = -1;
     g.out.shift_bit = only_shift_bit; g.out.only_if_shifted = only_shift_bit ? 1 : 0;
-    g.ksplit = chunks;
+    g.chunks = chunks;
     if (ksplit > 1) g.split_stride = (int64_t)r * r;
-    else g.run = chunks;
+    else g.run = 1;
     launch_gemm<tc::A_IMG_MN, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_GRAM, st);
     if (ksplit > 1) {
         const int64_t total4 = (int64_t)r * r / 4;

@@ -445,6 +445,45 @@ def test_small_rank_qr_and_depth_chunks_agree_bit_for_bit(shape, count):
     test_factor_kernel_forms_agree_bit_for_bit(shape, count)
 
 
+# more depth chunks than accumulators (five to eight above rank 64): tiles of their own (the matrix alone), runs of two
+# tiles whose sums one CTA adds up (the call of many), the last one with fewer chunks; both products, both gradient types
+@pytest.mark.parametrize("shape,count", [((264, 4200, 128), 40), ((2600, 264, 112), 40)])
+@pytest.mark.parametrize("dt", [(F32, F32), (BF16, BF16)])
+def test_runs_of_depth_chunks_agree_bit_for_bit(shape, count, dt):
+    m, n, r = shape
+    probs = [make_problem(m, n, r, *dt, seed=900 + i) for i in range(count)]
+    h = od.orthdion_create(m, n, r, 0.95, 0.01, 0.0, od.MODE_ORTH)
+    od.orthdion_set_dtypes(h, *dt)
+    X, M, G, Q = ([p[j].cuda() for p in probs] for j in (1, 2, 3, 4))
+    ws = poisoned_workspace(od.orthdion_workspace_bytes_grouped([h] * count))
+    od.orthdion_step_grouped(od.PointerTable([h] * count, X, M, G, Q), ws)
+    torch.cuda.synchronize()
+    assert od.orthdion_last_status([h] * count, ws) == [0] * count
+    for i in (0, count - 1):
+        spec, x, mm, g, q = probs[i]
+        gm = GpuMatrix(spec, x, mm, q, mu=0.95, eta=0.01, engine=od.ENGINE_TENSOR)
+        gm.step(g)
+        assert gm.status() == 0
+        assert torch.equal(gm.X, X[i]) and torch.equal(gm.M, M[i]) and torch.equal(gm.Q, Q[i])
+        gm.close()
+    od.orthdion_destroy(h)
+
+
+@pytest.mark.parametrize("r", [64, 96, 128, 256])
+def test_sums_over_a_long_depth_lose_no_more_than_short_chunks_do(r):
+    # The tensor core truncates when it adds into its accumulator, about half of 2^-23 of the running sum (half of the
+    # total on average) per addition: with eight chunks of 32 blocks, 12 additions each, 12 * 32 * 2^-25 = 1.1e-5 at
+    # most (measured 6.3e-6), with four chunks twice that (1.25e-5).  R is compared with B^T P from the device's own P.
+    m, n = 16384, 1024
+    spec, X, M, G, Q = make_problem(m, n, r, F32, F32, seed=3)
+    gm = GpuMatrix(spec, X, M, Q, mu=0.95, eta=0.01, engine=od.ENGINE_TENSOR)
+    gm.step(G)
+    P, R = gm.factors()
+    want = (M.cuda() + G.cuda()).double().T @ P.double()
+    assert float(1.0 - (R.double() * want).sum() / (want * want).sum()) <= 9e-6
+    gm.close()
+
+
 # the Gram product's depth chunks: tiles of their own (the matrix alone), added by one CTA (the call of many);
 # CTA pairs and single CTAs, a ragged last chunk
 @pytest.mark.parametrize("shape,count", [((3300, 520, 512), 30), ((3300, 600, 272), 40)])
