@@ -58,10 +58,12 @@ inline int qs_parts(int64_t rows, int r, int max_ctas) {
 }
 inline int qs_rows_per_part(int64_t rows, int parts) { return (int)((rows + parts * 32 - 1) / (parts * 32) * 32); }
 inline int64_t qs_smem(int64_t rows_per_cta, int r) { return rows_per_cta * qs_row_bytes(r) + qs_fixed(r); }
-// Whether the kernel takes a rows x r factor.  From r = 33 up only short ones: the fp32 products and the
-// repeated factorisations cost a call with many matrices more than the separate tensor-core kernels do
-// (24 layers of 768-wide matrices at r = 64: 1.80 ms a step with separate kernels, 1.95 with one for every
-// factor, 1.65 with this limit; one 4096 x 4096 matrix 0.347 against 0.412).
+// Whether the kernel takes a rows x r factor.  From r = 33 up only short ones: the fp32 products and the repeated
+// factorisations cost a call with many matrices more than the separate tensor-core kernels do, and the choice cannot
+// depend on the call (a matrix gets the same bits alone and in a group).  Step with separate kernels and with this one
+// at r = 64: 512 x 512 one 0.204 and 0.106 ms, 72 of them 0.383 and 0.321; 640 x 640 one 0.214 and 0.101, 24 0.285 and
+// 0.189, 72 0.491 and 0.547; 768 x 768 one 0.220 and 0.100, 24 0.331 and 0.207, 72 0.556 and 0.612; 24 layers of a
+// 768-wide model (168 matrices) 1.39 and 1.61; 4096 x 4096 one 0.336 and 0.263.
 inline bool qs_fits(int64_t rows, int r, int max_ctas) {
     if (r > QS_MAX_RANK || (r > 32 && rows > QS_MAX_ROWS_64)) return false;
     const int c = qs_parts(rows, r, max_ctas);
