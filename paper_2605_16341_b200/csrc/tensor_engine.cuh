@@ -1759,12 +1759,15 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     g.epi_bufs = 1;
     if (EPI == tc::EPI_K5) {
         // the fused pass: 64 KB of A slots (four single-term ones or two two-term ones) and one
-        // epilogue buffer per warp.  bf16 G and X in single terms, ranks below 512: a second buffer, paid for with an
-        // A slot and three N slots; the update is bound by bytes in flight until the products take as long.
-        // 11008 x 4096, one buffer -> two, before the leaner update: r = 32 0.141 -> 0.124 ms, 256 0.149 -> 0.131,
-        // 448 0.152 -> 0.148, 512 0.154 -> 0.160.
+        // epilogue buffer per warp.  bf16 G and X in single terms: a second buffer, paid for with an A slot and N
+        // slots; the update is bound by bytes in flight until the products take as long.  Pairs, which keep
+        // three of six N slots, below rank 512: 11008 x 4096, one buffer -> two, before the leaner update: r = 32 0.141 ->
+        // 0.124 ms, 256 0.149 -> 0.131, 448 0.152 -> 0.148, 512 0.154 -> 0.160.  Single CTAs (widths that are no multiple
+        // of 128), which keep one of three (twice as large), up to rank 192: eight 4104 x 4104 r = 16 0.394 -> 0.378, 192
+        // 0.402 -> 0.402, 208 0.401 -> 0.456, 400 0.433 -> 0.643; 24 of 2712 x 1000 r = 192 0.210 -> 0.199, 256 0.213 ->
+        // 0.227, 400 0.227 -> 0.313.
         g.a_slots = (a_terms == 1) ? 4 : 2;
-        if (XG == 3 && a_terms == 1 && g.k_blocks < 8) { g.a_slots = 3; g.epi_bufs = 2; }
+        if (XG == 3 && a_terms == 1 && g.k_blocks < (pair ? 8 : 4)) { g.a_slots = 3; g.epi_bufs = 2; }
     }
     if (NMODE == tc::N_IMG_MN) {
         if (pair) {

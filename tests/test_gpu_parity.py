@@ -167,6 +167,14 @@ def test_fused_pass_buffer_edges(shape):
     one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR, passes={2: 1, 3: 1})
 
 
+# widths that are no multiple of 128: two epilogue buffers up to rank 192, one above
+@pytest.mark.parametrize("shape", [(2200, 2056, 192), (2200, 2056, 208)])
+def test_fused_pass_buffers_at_ragged_widths(shape):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, BF16, BF16, seed=m + n + r)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR, passes={2: 1, 3: 1})
+
+
 @pytest.mark.parametrize("shape", [(384, 640, 64), (1000, 264, 128), (136, 2056, 32), (640, 384, 272)])
 @pytest.mark.parametrize("mode", MODES)
 @pytest.mark.parametrize("m_scale", [0.3, 3e-4, 300.0])
