@@ -2039,18 +2039,20 @@ inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const
         finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, ts.colsq, prof::S_K3, st);
 }
 
-// Columns per tile of a product between images (`copies`: matrices times depth chunks; lower: tiles that touch the lower
-// triangle).  256 columns, in CTA pairs where the rank allows, do the least work; 128 where all such
-// tiles run at once on multiprocessors that the wide ones leave idle.  An entry is summed in the same order either way.
+// Columns per tile of a product between images (`copies`: matrices times depth chunks).  256 columns, in CTA pairs
+// where the rank allows, do the least work; 128 where all such tiles run at once on multiprocessors that the wide ones
+// leave idle.  A Gram product's tiles above the diagonal count: they are skipped, but the tiles of a launch are dealt
+// out in order, so a launch of more tiles than multiprocessors gives some of those two real ones.  (Counted without:
+// ten 14336 x 1024 matrices at r = 512, Gram products of a step 0.658 -> 0.940 ms, twelve 2048 x 2048 0.245 -> 0.300; six
+// 4096 x 4096 at r = 192 0.167 -> 0.188.)  An entry is summed in the same order either way.
 // Measured, 256 -> 128 columns: one 4096 x 4096 matrix at r = 256, Gram products of a step 0.170 -> 0.152 ms, applies 0.110 ->
 // 0.090; 4096 x 3584 at r = 512 0.238 -> 0.203 and 0.118 -> 0.095; 28 matrices 1000 wide at r = 272 0.911 -> 0.727 and
 // 0.487 -> 0.469.  (64 columns: another 5 % at r = 256, but 0.304 -> 0.357 ms for the Gram products of 11008 x 4096 at r = 1024.)
-inline int image_bn(int r, int64_t out_rows, int64_t copies, bool lower) {
+inline int image_bn(int r, int64_t out_rows, int64_t copies) {
     const int wide = std::min(r, 256);
     if (wide <= 128) return wide;
     const int64_t rows = (out_rows + tc::BM - 1) / tc::BM, cols = (r + 127) / 128;
-    const int64_t tiles = lower ? rows * (rows + 1) / 2 : rows * cols;
-    return tiles * copies <= SPLIT_SMS ? 128 : wide;
+    return rows * cols * copies <= SPLIT_SMS ? 128 : wide;
 }
 
 // Depth split of the Gram product.  The Gram matrix is one output tile at small ranks and ten at r = 1024,
@@ -2078,15 +2080,23 @@ inline int gram_chunks(int r, int64_t rows) {
     const int per = (kb + want - 1) / want;
     return (kb + per - 1) / per;             // every chunk non-empty
 }
-// Partial matrices in memory of a Gram product in a call of `matrices`.  Above r = 256 the line is where the
-// undivided tiles fill the device (there the partial matrices would be megabytes each), and there are none
-// when the workspace is to be `lean`.  Measured, the Gram
-// products of a step: one 11008 x 4096 matrix at r = 1024 0.64 -> 0.35 ms, one 4096 x 3584 matrix at r = 512 0.36 -> 0.26.
+// Partial matrices in memory of a Gram product in a call of `matrices`.  Above r = 256 the line is where chunks as tiles of
+// their own take fewer depth blocks one after the other than undivided tiles, with six more for starting and storing a
+// chunk (tiles above the diagonal hold a place too, see image_bn); none in calls of more than two waves of tiles, where
+// the partial matrices would be megabytes for each of many matrices, and none when the workspace is to be `lean`.
+// Measured, the Gram products of a step, undivided and in chunks: one 11008 x 4096 matrix at r = 1024 0.64 and 0.35 ms,
+// one 4096 x 3584 at r = 512 0.36 and 0.26; n x 1024 at r = 512: 4096, 8 matrices 0.276 and 0.213, 12 0.277 and 0.320, 20
+// 0.453 and 0.416; 8192, 9 0.430 and 0.324, 12 0.422 and 0.416, 16 0.434 and 0.484, 20 0.745 and 0.588, 28 0.768 and
+// 0.766; 14336, 12 0.636 and 0.554, 14 0.648 and 0.628, 16 0.660 and 0.689.  r = 384 (single CTAs): 4096, 12 0.295 and
+// 0.215, 20 0.300 and 0.337, 28 0.501 and 0.451; 8192, 16 0.345 and 0.415; 14336, 16 0.526 and 0.510.
 inline int gram_ksplit(int r, int64_t rows, int matrices, bool lean) {
     if (r <= 256) return gram_chunks(r, rows);
     if (lean) return 1;
-    const int room = r % 256 ? SPLIT_SMS : SPLIT_SMS / 2;
-    return (int64_t)matrices * gram_tiles(r) <= room ? gram_chunks(r, rows) : 1;
+    const int room = r % 256 ? SPLIT_SMS : SPLIT_SMS / 2, high = r % 256 ? 128 : 256, wide = std::min(r, 256);
+    const int64_t tiles = (int64_t)matrices * ((r + high - 1) / high) * ((r + wide - 1) / wide);
+    const int chunks = gram_chunks(r, rows), kb = (int)((rows + tc::BK - 1) / tc::BK);
+    auto waves = [&](int64_t t) { return (t + room - 1) / room; };
+    return tiles <= 2 * room && waves(tiles * chunks) * ((kb + chunks - 1) / chunks + 6) < waves(tiles) * kb ? chunks : 1;
 }
 
 // dst <- sum of the `ksplit` partial results at `part` (4 * total4 floats each, one after the
@@ -2114,7 +2124,7 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
                         int only_shift_bit, cudaStream_t st) {
     const int chunks = gram_chunks(r, rows);
     tc::GemmArgs g{};
-    g.Mrows = r; g.Ncols = r; g.Kdim = (int32_t)rows; g.BN = image_bn(r, r, (int64_t)b.count * (ksplit > 1 ? chunks : 1), true);
+    g.Mrows = r; g.Ncols = r; g.Kdim = (int32_t)rows; g.BN = image_bn(r, r, (int64_t)b.count * (ksplit > 1 ? chunks : 1));
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = src; g.n2 = no_img(); g.lower_only = 1;
     g.out.normal = dest_none(); g.out.normal.f32 = ksplit > 1 ? part : gram; g.out.normal.has_f32 = 1;
     g.out.shifted = g.out.normal; g.out.ld = r;
@@ -2138,7 +2148,7 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
 inline void tensor_apply(int r, int passes, const Batch& b, const TensorScratch& ts, ImgRef src, int64_t rows,
                          tc::OutSpec out, bool unit, cudaStream_t st) {
     tc::GemmArgs g{};
-    g.Mrows = (int32_t)rows; g.Ncols = r; g.Kdim = r; g.BN = image_bn(r, rows, b.count, false);
+    g.Mrows = (int32_t)rows; g.Ncols = r; g.Kdim = r; g.BN = image_bn(r, rows, b.count);
     g.passes = passes; g.passes2 = 1; g.a = src; g.n1 = ts.linv; g.n2 = no_img(); g.tri = 1;
     g.colsq_off = ts.colsq;
     g.cscale_off = unit ? ts.fscale : -1;
