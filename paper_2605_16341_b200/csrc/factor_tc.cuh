@@ -395,6 +395,9 @@ __device__ __forceinline__ float ct_diag_scale(const float (&v)[8], const uint4&
     return s;
 }
 
+// (Two CTAs per multiprocessor leave 80 registers a thread, and the panels of the diagonal blocks want more: ptxas
+// reports 620 bytes of spill stores and 492 of loads, 764 and 616 in the MULTI form.  Not tried: one CTA per
+// multiprocessor where the call has no more.)
 template <bool MULTI>
 __global__ void __launch_bounds__(CT_THREADS, 2)
 factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {

@@ -1425,7 +1425,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         // 80 registers that 22 warps leave a thread, and a load whose register is spilled is waited for at
         // once: what else lives in the loop is two pointers and one offset, and only one chunk is split
         // at a time.  Before, with indexes per chunk, two tiles of either type and both chunks split
-        // together, 88 bytes were spilled with bf16 gradients and 292 with fp32.  With the issuer above, one 11008 x 4096
+        // together, 88 bytes were spilled with bf16 gradients and 292 with fp32; 0 to 24 are now, over all roles.  With the issuer above, one 11008 x 4096
         // matrix, first and second product: r = 32 0.111 -> 0.092 and 0.100 -> 0.063 ms, r = 128 0.134 -> 0.106 and
         // 0.126 -> 0.088; fp32 gradients, r = 32 0.184 -> 0.097 and 0.102 -> 0.068; six layers of 2048-wide matrices,
         // r = 512 0.979 -> 0.869 and 1.145 -> 1.047.
