@@ -29,7 +29,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     float* sD = reinterpret_cast<float*>(smem + CT_OFF_D);
     __shared__ float red[FS_THREADS / 32];
     __shared__ float s_up[2];                 // scales of a tiny matrix (see ct_rsqrt)
-    __shared__ float s_min[2], s_max[2];      // pivots, by the half of their diagonal block
+    __shared__ float s_min, s_max;            // smallest and largest pivot
 
     const MatWork& w = batch.w[blockIdx.x];
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
@@ -96,7 +96,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
         const float shift = attempt ? a.shift_rel * trace : 0.f;
         const float pad = A[0] + shift;         // diagonal of the padding: the first pivot (see factor_tc.cuh)
-        if (tid < 2) { s_min[tid] = 3.0e38f; s_max[tid] = 0.f; }
+        if (tid == 0) { s_min = 3.0e38f; s_max = 0.f; }
         for (int k = 0; k < nb; ++k) {
             const int k0 = k * CT_NB, nbk = min(CT_NB, r - k0);
             // diagonal block
@@ -116,16 +116,13 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             __syncthreads();
             if (warp < CT_DIAG_WARPS) {
                 float mn, mx;
-                ct_diag_block<64>(sD, smem + CT_OFF_D, nbk, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
-                if (lane == 0 && (warp == 0 || (warp == 3 && nbk > 32))) {
-                    s_min[warp / 3] = mx <= 3.0e38f ? fminf(s_min[warp / 3], mn) : -1.f;
-                    s_max[warp / 3] = fmaxf(s_max[warp / 3], mx);
-                }
+                ct_diag_block(sD, reinterpret_cast<float*>(smem + CT_OFF_D + CT_DG_BLK), nbk, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                if (tid == 0) { s_min = mx <= 3.0e38f ? fminf(s_min, mn) : -1.f; s_max = fmaxf(s_max, mx); }
             }
             __syncthreads();
             for (int q = tid; q < CT_NB * CT_NB; q += FS_THREADS) {
                 const int i = q / CT_NB, j = q % CT_NB;
-                const float v = sD[max(i, j) * CT_LDD + min(i, j)] * s_up[1];
+                const float v = sD[min(i, j) * CT_LDD + max(i, j)] * s_up[1];
                 if (i < nbk && j < nbk) W[(int64_t)(k0 + i) * r + k0 + j] = v;
                 Xs[i * SIMT_LD + j] = (i <= j && j < nbk) ? v : 0.f;         // X_k(j, i)
             }
@@ -162,7 +159,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             }
             __syncthreads();
         }
-        const float mn = fminf(s_min[0], s_min[1]), mx = fmaxf(s_max[0], s_max[1]);
+        const float mn = s_min, mx = s_max;
         const bool fail = !(mn > 0.f);
         const bool ill = (a.pass == 1) && (sqrtf(mx) > a.cond_limit * sqrtf(mn));
         if (!fail && !(ill && attempt == 0)) {

@@ -43,20 +43,17 @@ constexpr int CT_NB = 64;                     // block width, tile rows
 constexpr int CT_TERM = CT_NB * 128;          // one bf16 term of a 64 x 64 tile: 64 image rows of 128 bytes
 constexpr int CT_TILE = 2 * CT_TERM;
 constexpr int CT_LDD = 68;                    // diagonal block, fp32 (rows 16-byte aligned, conflict-free by row)
-constexpr int CT_LDT = 68;                    // transposed factor columns: 32 x 64 (the second half's in place of L11's)
 constexpr int CT_LDS = 65;                    // transposing buffer of the first-order inverse
 // dynamic shared memory: two stages of an A tile and a B tile, then the diagonal block's work area
 constexpr int CT_OFF_D = 4 * CT_TILE;
-constexpr int CT_DG_LT = CT_NB * CT_LDD * 4;                   // work area of a diagonal block: the block itself first
-constexpr int CT_DG_BLK = CT_DG_LT + 32 * CT_LDT * 4;
-constexpr int CT_DG_S = CT_DG_BLK + 64 * 4;
-constexpr int CT_DG_BYTES = CT_DG_S + 32 * 32 * 4;
+constexpr int CT_DG_BLK = CT_NB * CT_LDD * 4;                  // work area of a diagonal block: the block itself, a panel's 8 x 8 block
+constexpr int CT_DG_BYTES = CT_DG_BLK + 64 * 4;
 constexpr int CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;              // the block of the odd columns (the even ones': CT_OFF_D)
 constexpr int CT_SMEM_BYTES = CT_OFF_D2 + CT_NB * CT_LDD * 4 + 1024;     // + alignment of the tiles
 static_assert(2 * (CT_SMEM_BYTES + 2048) <= 228 * 1024, "two CTAs per multiprocessor");
 static_assert(3 * CT_NB * CT_LDS * 4 <= 4 * CT_TILE, "three transposing buffers fit the operand stages");
 constexpr int CT_MAX_BLOCKS = 64;             // r <= 4096
-constexpr int CT_STAT_FLOATS = 5 * CT_MAX_BLOCKS;   // per block: smallest and largest pivot of its halves, row-sum bound
+constexpr int CT_STAT_FLOATS = 3 * CT_MAX_BLOCKS;   // per block: smallest and largest pivot, row-sum bound
 constexpr float CT_THIRD_PASS_LIMIT = 0.02f; // bound on |Gram - I|_2 of the second pass above which a third follows
 constexpr float CT_SERIES_LIMIT = 1.4e-3f;   // bound on |Gram - I|_2 below which L^{-1} = I - Phi(E) is used
 
@@ -66,8 +63,8 @@ __device__ __forceinline__ void ct_bar_sync(int id, int threads) {
 __device__ __forceinline__ void ct_bar_arrive(int id, int threads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-// named barriers (0: the whole CTA); CT_BAR_XT: two, by the parity of the column; CT_BAR_HAND: four, by the panel
-constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_X = 4, CT_BAR_XT = 5, CT_BAR_HAND = 7, CT_BAR_JOIN = 11;
+// named barriers (0: the whole CTA); CT_BAR_XT: two, by the parity of the column
+constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_X = 4, CT_BAR_XT = 5, CT_BAR_HAND = 7;
 
 __device__ __forceinline__ void ct_cp16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
@@ -164,24 +161,22 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 
 // ---- diagonal blocks (fp32, four warps) ----------------------------------------------------------
 // sD (64 x 64 block, ld CT_LDD, beyond nbk a diagonal of the matrix's first pivot; row by row the lower part
-// counts) -> X, the inverse of its Cholesky factor L, in the lower part of sD, and the rows of X^T = L^{-T} as they
-// are found: out(row, chunk, z) gets the entries 8 chunk .. + 7 of a row.
+// counts) -> X^T = L^{-T}, L its Cholesky factor, in the upper part of sD; out(row, chunk, z) gets the entries
+// 8 chunk .. + 7 of every row as they are found (zeros left of the diagonal).
 //
 // As in the large, [D; I] L^{-T} = [L; L^{-T}]: rows of the block and of the identity go through the same
-// elimination, a row per lane.  The columns are taken in panels of eight, whose 8 x 8 diagonal block every
-// lane factors for itself from shared memory (a chain of eight reciprocal square roots and 16 products, no shuffle
-// in it); then the lane solves its own eight entries and the panel's columns of L go to the others through LT
-// (LT[j][i] = L(i, j)).  What bounds it is this chain, so everything else runs beside it: only the next
-// panel's columns are updated at once, the others while the next panel is being factored, and what is not needed for the
-// next panel by a warp that follows behind:
-//   first half (columns 0 .. 31)        second half
-//   warp 0  L11                         rows 0 .. 31 of L^{-T} beyond column 32
-//   warp 1  L21                         their sums  -X11^T L21^T, ahead
-//   warp 2  rows 0 .. 31 of L^{-T}      rows 32 .. 63 of L^{-T}
-//   warp 3  D22 - L21 L21^T, behind     L22
-// Measured alone, cycles for 64 columns: 11200 with all updates in the chain, 9300 so.  (Two 32-column
-// factorisations by one warp with the columns passed by shuffle, then triangular solves and the update
-// one after the other: 16 thousand.)
+// elimination, in panels of eight columns.  Row i of the block is done with its own panel, and row i of the identity begins
+// there: 64 row slots in place, a thread each.  Two warps form the chain: every lane factors the panel's 8 x 8 diagonal
+// block for itself (eight reciprocal square roots one after the other, no shuffle), solves its row's eight
+// entries and brings the next panel's columns of its row up to date.  Two warps follow with the columns behind those, and
+// with the output.
+// What bounds it is the chain and, no less, the instruction cache: a CTA of a cluster comes here once or twice in a
+// factorisation, so the code is fetched as it is run.  Hence one loop over the panels, and one over the columns, of
+// some 600 instructions together.  (Straight-line halves of 32 columns with every lane's row in registers: 9300 cycles alone
+// and warm, but 23000 in the kernel and 42000 for the first block.)  Step, that form -> this, with the Gram entries
+// of the next diagonal block fetched before the wait for the inverse: 4096 x 4096 r = 256 0.483 -> 0.423 ms, column shard 4096 x
+// 3584 r = 512 0.845 -> 0.775, 11008 x 4096 r = 1024 1.885 -> 1.811, one-kernel QR 520 x 384 r = 64 0.1095 -> 0.1011, fp32
+// engine 1023 x 777 r = 40 0.244 -> 0.229.
 // Pivots are normal numbers here: the form of rsqrt that takes subnormal ones costs the chain three more
 // dependent instructions per column.  A Gram matrix so small that its pivots may be subnormal (squared column
 // norms of the factor below 2^-60) comes into sD times CT_TINY_UP, and `unit`, the root of that, in place of the
@@ -196,8 +191,16 @@ __device__ __forceinline__ float ct_rsqrt(float x) {
     asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-// the lane's row entries a[0 .. 7] -> its entries z of [L; L^{-T}]; blk: the panel's 8 x 8 diagonal block
-__device__ __forceinline__ void ct_panel8(const float* blk, const float* a, float (&z)[8], float& dmin, float& dmax) {
+__device__ __forceinline__ void ct_ld8(float (&v)[8], const float* p) {
+    const float4 x = *reinterpret_cast<const float4*>(p), y = *reinterpret_cast<const float4*>(p + 4);
+    v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w; v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+}
+__device__ __forceinline__ void ct_st8(float* p, const float (&v)[8]) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+    *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+}
+// the lane's row entries z -> its entries of [L; L^{-T}]; blk: the panel's 8 x 8 diagonal block
+__device__ __forceinline__ void ct_panel8(const float* blk, float (&z)[8], float& dmin, float& dmax) {
     float b[8][8];
 #pragma unroll
     for (int i = 0; i < 8; ++i)
@@ -206,8 +209,6 @@ __device__ __forceinline__ void ct_panel8(const float* blk, const float* a, floa
             const float4 v = *reinterpret_cast<const float4*>(blk + i * 8 + c);
             b[i][c] = v.x; b[i][c + 1] = v.y; b[i][c + 2] = v.z; b[i][c + 3] = v.w;
         }
-#pragma unroll
-    for (int j = 0; j < 8; ++j) z[j] = a[j];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
         const float d = b[j][j], inv = ct_rsqrt(d);
@@ -226,159 +227,68 @@ __device__ __forceinline__ void ct_panel8(const float* blk, const float* a, floa
             for (int c = j + 1; c <= i; ++c) b[i][c] = fmaf(-b[i][j], b[c][j], b[i][c]);
     }
 }
-// a[0 .. 4 n4) -= sum_j z_j LT[j][c0 ..]
-template <int N4>
-__device__ __forceinline__ void ct_rank8(float* a, const float (&z)[8], const float* LT, int c0) {
+// a[0 .. 3] -= sum_j z_j L(c .. c + 3, j), the rows of L eight entries each, CT_LDD apart
+__device__ __forceinline__ void ct_rank8(float* a, const float (&z)[8], const float* L) {
 #pragma unroll
-    for (int c = 0; c < 4 * N4; c += 4) {
+    for (int c = 0; c < 4; ++c) {
+        float l[8];
+        ct_ld8(l, L + c * CT_LDD);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-            const float4 l = *reinterpret_cast<const float4*>(LT + j * CT_LDT + c0 + c);
-            a[c] = fmaf(-z[j], l.x, a[c]); a[c + 1] = fmaf(-z[j], l.y, a[c + 1]);
-            a[c + 2] = fmaf(-z[j], l.z, a[c + 2]); a[c + 3] = fmaf(-z[j], l.w, a[c + 3]);
-        }
+        for (int j = 0; j < 8; ++j) a[c] = fmaf(-z[j], l[j], a[c]);
     }
 }
-// `rest`: CT_DG_BYTES of shared memory whose first part may be sD itself.  dmin, dmax: smallest (-1: breakdown)
-// and largest pivot, in the lanes of warp 0 (one half) or warp 3 (two).  unit: 1, or what ct_rsqrt says.
-// COLS: at most so many columns (16, 32 or 64).
-template <int COLS, class Out>
-__device__ __forceinline__ void ct_diag_block(float* sD, unsigned char* rest, int nbk, float unit, int dw, int lane, float& dmin, float& dmax, Out out) {
-    float* LT = reinterpret_cast<float*>(rest + CT_DG_LT);
-    float* blk = reinterpret_cast<float*>(rest + CT_DG_BLK);
-    float* sS = reinterpret_cast<float*>(rest + CT_DG_S);
-    constexpr int NA = COLS < 32 ? COLS : 32;
-    const bool two = COLS > 32 && nbk > 32;
-    // cur: the lane's entries of the panel at hand, a: of the columns behind it (the first ones)
-    float a[NA], cur[8], z[8];
+// `blk`: 64 floats of shared memory.  dmin, dmax: smallest (-1: breakdown) and largest pivot, in every lane of warps 0
+// and 1.  unit: 1, or what ct_rsqrt says.  Called by four warps (dw).
+template <class Out>
+__device__ __forceinline__ void ct_diag_block(float* sD, float* blk, int nbk, float unit, int dw, int lane, float& dmin, float& dmax, Out out) {
+    const int np = (nbk + 7) / 8, row = (dw & 1) * 32 + lane, own = row / 8;
+    float* sR = sD + row * CT_LDD;
     dmin = 3.0e38f; dmax = 0.f;
-    {
-        // this lane's row: of D11, D21, the identity, D22
-        const float* src = sD + (lane + (dw == 1 || dw == 3 ? 32 : 0)) * CT_LDD + (dw == 3 ? 32 : 0);
-#pragma unroll
-        for (int c = 0; c < NA; c += 4) {
-            float4 v = make_float4(lane == c ? unit : 0.f, lane == c + 1 ? unit : 0.f, lane == c + 2 ? unit : 0.f, lane == c + 3 ? unit : 0.f);
-            if (dw != 2 && (dw == 0 || two)) v = *reinterpret_cast<const float4*>(src + c);
-            a[c] = v.x; a[c + 1] = v.y; a[c + 2] = v.z; a[c + 3] = v.w;
-        }
-    }
-    auto shift = [&]() {            // the first eight of a become the panel at hand
-#pragma unroll
-        for (int c = 0; c < 8; ++c) cur[c] = a[c];
-#pragma unroll
-        for (int c = 0; c < NA - 8; ++c) a[c] = a[8 + c];
-    };
-    auto put_blk = [&](int p) {     // rows 8 p .. + 7 of the warp that factors
-        if (lane / 8 == p) {
-            *reinterpret_cast<float4*>(blk + (lane % 8) * 8) = make_float4(cur[0], cur[1], cur[2], cur[3]);
-            *reinterpret_cast<float4*>(blk + (lane % 8) * 8 + 4) = make_float4(cur[4], cur[5], cur[6], cur[7]);
-        }
-    };
-    // One panel of the warps in step (w: the one that factors): cur -> z, and the update of the panel before (zp) in
-    // the columns beyond this panel; then store(z), and the next panel's columns.
-    auto panel = [&](int p, int np, bool factors, auto store) {
-        float zp[8];
-#pragma unroll
-        for (int j = 0; j < 8; ++j) zp[j] = z[j];
-        ct_panel8(blk, cur, z, dmin, dmax);
-        if (NA > 16 && (p == 1 || p == 2)) {
-            const float* Lp = LT + (p - 1) * 8 * CT_LDT;
-            ct_rank8<2>(a, zp, Lp, 8 * (p + 1));
-            if (p == 1) ct_rank8<2>(a + NA / 4, zp, Lp, 8 * (p + 2));
-        }
-        store();
-        ct_bar_sync(CT_BAR_DIAG, 96);
-        if (p + 1 < np) {
-            shift();
-            ct_rank8<2>(cur, z, LT + p * 8 * CT_LDT, 8 * (p + 1));
-            if (factors) put_blk(p + 1);
-        }
-    };
-    const int np = two ? 4 : (nbk + 7) / 8;
-    if (dw < 3) {
-        shift();
-        if (dw == 0) put_blk(0);
+    if (dw < 2) {
+        float z[8];
+        ct_ld8(z, sR);
+        if (own == 0) ct_st8(blk + row * 8, z);
+        ct_bar_sync(CT_BAR_DIAG, 64);
 #pragma unroll 1
         for (int p = 0; p < np; ++p) {
-            ct_bar_sync(CT_BAR_DIAG, 96);
-            panel(p, np, dw == 0, [&]() {
-                if (dw < 2) {
+            if (own == p) {                 // the identity's row begins
 #pragma unroll
-                    for (int j = 0; j < 8; ++j) LT[(8 * p + j) * CT_LDT + 32 * dw + lane] = z[j];
-                    if (dw == 1 && two) ct_bar_arrive(CT_BAR_HAND + p, 64);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) sD[(8 * p + j) * CT_LDD + lane] = z[j];
-                }
-            });
-            if (dw == 2) out(lane, p, z);
-        }
-    } else if constexpr (COLS > 32) {
-        if (two) {
-#pragma unroll 1
-        for (int p = 0; p < 4; ++p) {
-            const float* L = LT + p * 8 * CT_LDT;
-            ct_bar_sync(CT_BAR_HAND + p, 64);
-#pragma unroll
-            for (int j = 0; j < 8; ++j) z[j] = L[j * CT_LDT + 32 + lane];
-            ct_rank8<8>(a, z, L, 32);
-        }
-        }
-    }
-    if constexpr (COLS > 32) {
-    if (!two) return;
-    ct_bar_sync(CT_BAR_JOIN, 128);
-    // second half; LT's first 32 columns hold L22 from here on
-    if (dw == 1) {
-        // the lane's row of X11^T times L21^T, eight columns after the other
-#pragma unroll
-        for (int j = 0; j < 32; ++j) a[j] = sD[j * CT_LDD + lane];
-#pragma unroll 1
-        for (int p = 0; p < 4; ++p) {
-            float t[8] = {};
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                const float4 u = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 32 + 8 * p);
-                const float4 v = *reinterpret_cast<const float4*>(LT + j * CT_LDT + 36 + 8 * p);
-                t[0] = fmaf(a[j], u.x, t[0]); t[1] = fmaf(a[j], u.y, t[1]); t[2] = fmaf(a[j], u.z, t[2]); t[3] = fmaf(a[j], u.w, t[3]);
-                t[4] = fmaf(a[j], v.x, t[4]); t[5] = fmaf(a[j], v.y, t[5]); t[6] = fmaf(a[j], v.z, t[6]); t[7] = fmaf(a[j], v.w, t[7]);
+                for (int c = 0; c < 8; ++c) z[c] = row % 8 == c ? unit : 0.f;
             }
+            ct_panel8(blk, z, dmin, dmax);
+            ct_st8(sR + 8 * p, z);
+            ct_bar_sync(CT_BAR_HAND, 128);
+            if (p + 1 < np) {
+                float a[8] = {};
+                if (own != p) ct_ld8(a, sR + 8 * (p + 1));
+                const float* L = sD + 8 * (p + 1) * CT_LDD + 8 * p;
+                ct_rank8(a, z, L);
+                ct_rank8(a + 4, z, L + 4 * CT_LDD);
+                if (own == p + 1) ct_st8(blk + (row % 8) * 8, a);
 #pragma unroll
-            for (int c = 0; c < 8; ++c) sS[(8 * p + c) * 32 + lane] = t[c];
-            ct_bar_arrive(CT_BAR_HAND + p, 64);
-        }
-        return;
-    }
-    if (dw == 3) { dmin = 3.0e38f; dmax = 0.f; }
-    else {
-#pragma unroll
-        for (int c = 0; c < 32; ++c) a[c] = dw == 2 && lane == c ? unit : 0.f;
-    }
-    shift();
-    if (dw == 3) put_blk(0);
-    const float mn0 = dmin, mx0 = dmax;
-#pragma unroll 1
-    for (int p = 0; p < 4; ++p) {
-        ct_bar_sync(CT_BAR_DIAG, 96);
-        if (dw == 0) {
-            ct_bar_sync(CT_BAR_HAND + p, 64);
-#pragma unroll
-            for (int c = 0; c < 8; ++c) cur[c] -= sS[(8 * p + c) * 32 + lane];
-        }
-        panel(p, 4, dw == 3, [&]() {
-            if (dw == 3) {
-#pragma unroll
-                for (int j = 0; j < 8; ++j) LT[(8 * p + j) * CT_LDT + lane] = z[j];
-            } else {
-                float* dst = sD + (32 + 8 * p) * CT_LDD + (dw == 2 ? 32 : 0) + lane;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) dst[j * CT_LDD] = z[j];
+                for (int c = 0; c < 8; ++c) z[c] = a[c];
+                ct_bar_sync(CT_BAR_DIAG, 64);
             }
-        });
-        if (dw == 2) out(32 + lane, 4 + p, z);
-        else if (dw == 0) out(lane, 4 + p, z);
-    }
-    if (dw == 0) { dmin = mn0; dmax = mx0; }        // (what it reports is the first half)
+        }
+    } else {
+#pragma unroll 1
+        for (int p = 0; p < np; ++p) {
+            ct_bar_sync(CT_BAR_HAND, 128);
+            float z[8];
+            ct_ld8(z, sR + 8 * p);
+#pragma unroll 1
+            for (int c = 8 * (p + 2); c < 8 * np; c += 4) {
+                const float4 v = own == p ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(sR + c);
+                float a[4] = {v.x, v.y, v.z, v.w};
+                ct_rank8(a, z, sD + c * CT_LDD + 8 * p);
+                *reinterpret_cast<float4*>(sR + c) = make_float4(a[0], a[1], a[2], a[3]);
+            }
+            if (own > p) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) z[c] = 0.f;
+            }
+            out(row, p, z);
+        }
     }
 }
 
@@ -395,9 +305,8 @@ __device__ __forceinline__ float ct_diag_scale(const float (&v)[8], const uint4&
     return s;
 }
 
-// (Two CTAs per multiprocessor leave 80 registers a thread, and the panels of the diagonal blocks want more: ptxas
-// reports 620 bytes of spill stores and 492 of loads, 764 and 616 in the MULTI form.  Not tried: one CTA per
-// multiprocessor where the call has no more.)
+// (Two CTAs per multiprocessor leave 80 registers a thread: ptxas reports 20 bytes of spill stores and 60 of loads,
+// 104 and 96 in the MULTI form.)
 template <bool MULTI>
 __global__ void __launch_bounds__(CT_THREADS, 2)
 factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
@@ -546,13 +455,13 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     mx = fmaxf(mx, s <= 3.0e38f ? s : 3.3e38f);
                 }
                 for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                if (lane == 0) gstat[4 * CT_MAX_BLOCKS + t] = mx;
+                if (lane == 0) gstat[2 * CT_MAX_BLOCKS + t] = mx;
             }
             __syncthreads();
         }
         phase_sync();
         float mx = 0.f;
-        for (int t = 0; t < nb; ++t) mx = fmaxf(mx, __ldcg(gstat + 4 * CT_MAX_BLOCKS + t));
+        for (int t = 0; t < nb; ++t) mx = fmaxf(mx, __ldcg(gstat + 2 * CT_MAX_BLOCKS + t));
         // Second pass with Q1 far from orthonormal (cond(Y)^2 u was not small): its result will
         // not be orthonormal to working accuracy either, so ask for the third pass.
         if (a.pass == 2 && !(mx <= CT_THIRD_PASS_LIMIT) && tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
@@ -660,8 +569,8 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                 acc[nf][2 * h + 1] = v.y - acc[nf][2 * h + 1];
             }
     };
-    // Z[t, k] = acc X_k^T -> its image; leaves the tile in the A slot of stage ^ 1
-    auto panel = [&](float (&acc)[4][4], int t, int k) {
+    // Z[t, k] = acc X_k^T, left in the A slot of stage ^ 1
+    auto panel = [&](float (&acc)[4][4], int k) {
         load_tile(b_slot(stage), x_tile(k, k));
         ct_cp_commit();
         ct_store_tile(a_slot(stage), acc, warp, lane);
@@ -671,6 +580,9 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         ct_tile_mma_nt(o, a_slot(stage), b_slot(stage), warp, lane);
         ct_store_tile(a_slot(stage ^ 1), o, warp, lane);
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
+    };
+    // ... and from there to its image
+    auto panel_out = [&](int t, int k) {
         unsigned char* dst = t < k ? x_tile(t, k) : l_tile(t, k);
         const unsigned char* src = smem + (size_t)(stage ^ 1) * 2 * CT_TILE;
 #pragma unroll
@@ -680,10 +592,9 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
             *reinterpret_cast<uint4*>(dst + term + q) = *reinterpret_cast<const uint4*>(src + CT_TERM + q);
         }
     };
-    // sD <- diagonal block k: Gram - accd, the diagonal itself from gdiag (+ shift); beyond r the matrix's first pivot on
-    // the diagonal, which changes neither the smallest nor the largest (a one would: it is not of the matrix's scale)
-    auto write_diag = [&](const float (&accd)[4][4], int k, float shift) {
-        float* sD = diag_buf(k);
+    // d <- diagonal block k of the Gram matrix less d, the diagonal itself from gdiag (+ shift); beyond r the matrix's first
+    // pivot on the diagonal, which changes neither the smallest nor the largest (a one would: it is not of the matrix's scale)
+    auto diag_base = [&](float (&d)[4][4], int k, float shift) {
         const float pad = __ldcg(gdiag) + shift;
 #pragma unroll
         for (int nf = 0; nf < 4; ++nf)
@@ -692,9 +603,20 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                 const int il = mrow + 8 * (e / 2), jl = mcol + nf * 8 + (e % 2);
                 const int i = k * CT_NB + il, j = k * CT_NB + jl;
                 float v = il == jl ? pad : 0.f;
-                if (i < r && j < r) v = (il == jl ? __ldcg(gdiag + i) + shift : A[(int64_t)i * r + j]) - accd[nf][e];
-                sD[il * CT_LDD + jl] = trace < CT_TINY_TRACE ? v * CT_TINY_UP : v;         // see ct_rsqrt
+                if (i < r && j < r) v = (il == jl ? __ldcg(gdiag + i) + shift : A[(int64_t)i * r + j]) - d[nf][e];
+                d[nf][e] = v;
             }
+    };
+    // the work area of diagonal block k <- d - z
+    auto diag_store = [&](const float (&d)[4][4], const float (&z)[4][4], int k) {
+        float* sD = diag_buf(k);
+        const float up = trace < CT_TINY_TRACE ? CT_TINY_UP : 1.f;         // see ct_rsqrt
+#pragma unroll
+        for (int nf = 0; nf < 4; ++nf)
+#pragma unroll
+            for (int h = 0; h < 2; ++h)
+                *reinterpret_cast<float2*>(sD + (mrow + 8 * h) * CT_LDD + mcol + nf * 8) =
+                    make_float2((d[nf][2 * h] - z[nf][2 * h]) * up, (d[nf][2 * h + 1] - z[nf][2 * h + 1]) * up);
     };
 
     bool ok = false;
@@ -704,7 +626,9 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         if (mma_role) {
             if (crank == 0) {
                 const float none[4][4] = {};
-                write_diag(none, 0, shift);
+                float d[4][4] = {};
+                diag_base(d, 0, shift);
+                diag_store(d, none, 0);
                 ct_bar_arrive(CT_BAR_READY, CT_THREADS);
             }
             for (int k = 0; k < nb; ++k) {
@@ -719,23 +643,24 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                     if (t > k) prefetch_gram(t, k);
                     sum_products(acc, accd, t, k, next);
                     finish_sum(acc, t, k);
+                    if (next) diag_base(accd, k + 1, shift);
                 }
                 // X_k is in memory
                 if (MULTI) cluster_sync_all();
                 else ct_bar_sync(CT_BAR_X, CT_THREADS);
                 if (first) {
-                    panel(acc, t, k);
+                    panel(acc, k);
                     if (next) {
+                        // the chain goes on before anything else
                         const uint32_t z = a_slot(stage ^ 1);
-                        ct_tile_mma(accd, z, z, warp, lane);
-                        write_diag(accd, k + 1, shift);
+                        float dz[4][4] = {};
+                        ct_tile_mma(dz, z, z, warp, lane);
+                        diag_store(accd, dz, k + 1);
                         ct_bar_arrive(CT_BAR_READY, CT_THREADS);
-                        t = crank;
-                        seek();
-                    } else {
-                        t += nshare;
-                        seek();
                     }
+                    panel_out(t, k);
+                    t = next ? crank : t + nshare;
+                    seek();
                     for (; t < nb;) {
                         if (t > k) prefetch_gram(t, k);
 #pragma unroll
@@ -744,7 +669,8 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                             for (int e = 0; e < 4; ++e) acc[nf][e] = 0.f;
                         sum_products(acc, accd, t, k, false);
                         finish_sum(acc, t, k);
-                        panel(acc, t, k);
+                        panel(acc, k);
+                        panel_out(t, k);
                         t += nshare;
                         seek();
                     }
@@ -775,18 +701,14 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                         *reinterpret_cast<uint4*>(xt + o) = t0;
                         *reinterpret_cast<uint4*>(xt + term + o) = t1;
                     };
-                    if (dw == 1) {
-                        const float zero[8] = {};
-#pragma unroll
-                        for (int ch = 0; ch < 4; ++ch) out(32 + lane, ch, zero);
-                    }
                     float mn, mx;
-                    ct_diag_block<64>(diag_buf(k), smem + CT_OFF_D, nbk, trace < CT_TINY_TRACE ? CT_TINY_UP_ROOT : 1.f, dw, lane, mn, mx, out);
-                    // statistics: squared diagonal entries of L; two halves: warp 0's first, warp 3's second
-                    if (lane == 0 && (dw == 0 || (dw == 3 && nbk > 32))) {
+                    ct_diag_block(diag_buf(k), reinterpret_cast<float*>(smem + CT_OFF_D + CT_DG_BLK), nbk,
+                                  trace < CT_TINY_TRACE ? CT_TINY_UP_ROOT : 1.f, dw, lane, mn, mx, out);
+                    // statistics: squared diagonal entries of L
+                    if (lane == 0 && dw == 0) {
                         if (!(mx <= 3.0e38f)) mn = -1.f;
-                        gstat[(dw ? CT_MAX_BLOCKS : 0) + k] = mn;
-                        gstat[(dw ? 3 : 2) * CT_MAX_BLOCKS + k] = mx;
+                        gstat[k] = mn;
+                        gstat[CT_MAX_BLOCKS + k] = mx;
                     }
                 }
                 if (MULTI) {
@@ -805,13 +727,10 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         bool fail = false;
         float mn = 3.0e38f, mx = 0.f;
         for (int k = 0; k < nb; ++k) {
-            const int halves = r - k * CT_NB > 32 ? 2 : 1;
-            for (int h = 0; h < halves; ++h) {
-                const float lo = __ldcg(gstat + h * CT_MAX_BLOCKS + k);
-                if (!(lo > 0.f)) fail = true;
-                mn = fminf(mn, lo);
-                mx = fmaxf(mx, __ldcg(gstat + (2 + h) * CT_MAX_BLOCKS + k));
-            }
+            const float lo = __ldcg(gstat + k);
+            if (!(lo > 0.f)) fail = true;
+            mn = fminf(mn, lo);
+            mx = fmaxf(mx, __ldcg(gstat + CT_MAX_BLOCKS + k));
         }
         const bool ill = (a.pass == 1) && (sqrtf(mx) > a.cond_limit * sqrtf(mn));
         if (!fail && !(ill && attempt == 0)) {

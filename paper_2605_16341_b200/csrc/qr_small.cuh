@@ -102,7 +102,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
     float* part = sD;
     float* G = reinterpret_cast<float*>(smem + CT_DG_BYTES);     // Gram matrix, then L^{-T}
     float* Y = G + R * R;                            // this CTA's rows
-    __shared__ float s_min[2], s_max[2], s_bound;
+    __shared__ float s_min, s_max, s_bound;
     static_assert(GROUPS * R * R * 4 <= CT_DG_BYTES, "partial Gram matrices fit the diagonal block's area");
 
     grid_dependency();
@@ -428,14 +428,11 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     if (tiny) scale_block(CT_TINY_UP);
                     if (warp < CT_DIAG_WARPS) {
                         float mn, mx;
-                        ct_diag_block<R>(sD, smem, r, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
-                        if (lane == 0 && (warp == 0 || (warp == 3 && r > 32))) {
-                            s_min[warp / 3] = mx <= 3.0e38f ? mn : -1.f;
-                            s_max[warp / 3] = mx;
-                        }
+                        ct_diag_block(sD, reinterpret_cast<float*>(smem + CT_DG_BLK), r, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
+                        if (tid == 0) { s_min = mx <= 3.0e38f ? mn : -1.f; s_max = mx; }
                     }
                     __syncthreads();
-                    const float mn = r > 32 ? fminf(s_min[0], s_min[1]) : s_min[0], mx = r > 32 ? fmaxf(s_max[0], s_max[1]) : s_max[0];
+                    const float mn = s_min, mx = s_max;
                     const bool fail = !(mn > 0.f);
                     const bool ill = pass == 1 && sqrtf(mx) > a.cond_limit * sqrtf(mn);
                     if (!fail && !(ill && attempt == 0)) ok = true;
@@ -449,7 +446,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                 if (tiny) scale_block(CT_TINY_UP_ROOT);
                 for (int q = tid; q < R * R; q += QS_THREADS) {
                     const int k = q / R, j = q % R;
-                    G[q] = (k <= j && j < r) ? sD[j * CT_LDD + k] : 0.f;
+                    G[q] = (k <= j && j < r) ? sD[k * CT_LDD + j] : 0.f;
                 }
             }
             __syncthreads();
