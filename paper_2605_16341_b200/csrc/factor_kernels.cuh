@@ -18,7 +18,8 @@ struct CholArgs {
     // into its fp32 accumulator, which biases long sums of squares low; the off-diagonal sums have
     // no such bias.)
     Sel colsq;
-    int32_t use_colsq, pad;
+    int32_t use_colsq;
+    int32_t ahead;       // launches overlap: run the code of the diagonal blocks once while the kernel before is still at work
     // tensor engine: split image of L^{-T} (the result there, operand of the apply product; the image of L has the
     // same geometry and lies at MatWork::aux1), the Gram diagonal (fp32 [r]), the statistics of the
     // diagonal blocks, and later passes: L^{-1}(j, j) over the value that its two image terms hold (fp32 [r], then

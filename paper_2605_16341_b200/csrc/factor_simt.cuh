@@ -18,7 +18,8 @@ namespace od {
 
 constexpr int FS_THREADS = 256;
 constexpr int FS_OFF_X = 4 * SIMT_KC * SIMT_LD * 4;      // X_k transposed, after the two operand stages
-static_assert(FS_OFF_X + CT_NB * SIMT_LD * 4 <= CT_OFF_D, "operand stages and X_k before the diagonal block's area");
+constexpr int FS_OFF_D = FS_OFF_X + CT_NB * SIMT_LD * 4;     // the diagonal block's area
+constexpr int FS_SMEM_BYTES = FS_OFF_D + CT_DG_BYTES;
 
 __global__ void __launch_bounds__(FS_THREADS, 2)
 factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
@@ -26,7 +27,7 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
     SimtStage* As = reinterpret_cast<SimtStage*>(smem);
     SimtStage* Bs = As + 2;
     float* Xs = reinterpret_cast<float*>(smem + FS_OFF_X);
-    float* sD = reinterpret_cast<float*>(smem + CT_OFF_D);
+    float* sD = reinterpret_cast<float*>(smem + FS_OFF_D);
     __shared__ float red[FS_THREADS / 32];
     __shared__ float s_up[2];                 // scales of a tiny matrix (see ct_rsqrt)
     __shared__ float s_min, s_max;            // smallest and largest pivot
@@ -115,9 +116,8 @@ factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
             }
             __syncthreads();
             if (warp < CT_DIAG_WARPS) {
-                float mn, mx;
-                ct_diag_block(sD, reinterpret_cast<float*>(smem + CT_OFF_D + CT_DG_BLK), nbk, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
-                if (tid == 0) { s_min = mx <= 3.0e38f ? fminf(s_min, mn) : -1.f; s_max = fmaxf(s_max, mx); }
+                const float2 mm = ct_diag_block(FS_OFF_D, FS_OFF_D + CT_DG_BLK, nbk, 1.f, warp, lane, nullptr, 0, nullptr);
+                if (tid == 0) { s_min = mm.y <= 3.0e38f ? fminf(s_min, mm.x) : -1.f; s_max = fmaxf(s_max, mm.y); }
             }
             __syncthreads();
             for (int q = tid; q < CT_NB * CT_NB; q += FS_THREADS) {

@@ -1,5 +1,5 @@
 // r x r factor kernel of the tensor-core engine: Cholesky factor of the Gram matrix and its explicit
-// inverse, one CTA per matrix or one matrix per thread-block cluster (MULTI).
+// inverse, one matrix per thread-block cluster (of one CTA in calls with many matrices).
 //
 // Z L^T = [Gram; I] has the solution Z = [L; L^{-T}]: appending the identity below the Gram matrix
 // turns the inverse into more rows of the factorisation.  Both are therefore ONE left-looking
@@ -10,24 +10,25 @@
 // (common.cuh), i.e. in the two bf16 terms that the products read anyway; the image of L^{-T} is the
 // operand of the apply product, so nothing is converted afterwards.  Tile products run on the
 // warp-level tensor path (mma.sync m16n8k16, hi*hi + hi*lo + lo*hi: about 2^-16), operand tiles of
-// 64 x 64 come in by cp.async one step ahead.
+// 64 x 64 come in by cp.async three steps ahead.
 //
 // What bounds it: the chain of r / 64 diagonal blocks.  Four extra warps per CTA factor and invert a
-// 64 x 64 block in fp32 (below) while the eight product warps do the S sums of
-// the same block column, which do not depend on it; the tile below the diagonal goes first, together
-// with the next diagonal block's own sum, so that the chain never waits for the rest.  64-wide
-// blocks instead of 32: half the barriers.
-// Measured, factor stage of a step (six launches, ms), before (32-wide blocks, fp32 tiles split at every
-// use, a pairwise inversion afterwards) -> now: one matrix r = 256 0.74 -> 0.21, r = 512
-// 1.47 -> 0.32, r = 1024 3.68 -> 0.68; 56 matrices at r = 512 2.7 -> 0.7, 154 of them 5.0 -> 1.5.
+// 64 x 64 block in fp32 (below) while the eight product warps do the S sums of the same block column, which do not
+// depend on it.  The tile below the diagonal goes first, and the next diagonal block's own sum is kept up column by
+// column, so that the chain (block 10000 cycles, barrier 1000, panel 2400, next block's last product 1300)
+// never waits for the rest.  One CTA per multiprocessor: 161 registers a thread without spills and four operand stages (two
+// CTAs with 80 registers and two stages: 25000 cycles a block column at r = 1024, where a sum of 15 tiles took
+// longer than the chain).  Step, before all this -> now: 4096 x 4096 r = 256 0.423 -> 0.412 ms, column shard 4096 x 3584 r = 512
+// 0.775 -> 0.730, 11008 x 4096 r = 1024 1.811 -> 1.687, 28 matrices 1000 wide at r = 272 1.65 -> 1.61; the 1.1B and 8B
+// groups (one CTA per matrix) as before.
 //
 // The later passes of a CholeskyQR see a Gram matrix I + E with E tiny; when a rigorous bound on
 // |E|_2 is small enough, L^{-1} = I - Phi(E) (first order) replaces the factorisation.
 //
-// MULTI form: the row tiles are dealt out over the CTAs of the cluster (tile t to CTA t mod size); the
+// The row tiles are dealt out over the CTAs of the cluster (tile t to CTA t mod size); the
 // matrix stays in global memory (L2), phases are separated by release/acquire cluster barriers, and
-// what another CTA may have written is read past L1.  Per tile the arithmetic and its order are
-// those of the single-CTA form: a matrix gets the same bits in either.  Decisions that steer control
+// what another CTA may have written is read past L1.  Per tile the arithmetic and its order do not depend on the size of
+// the cluster: a matrix gets the same bits with any.  Decisions that steer control
 // flow are taken from values that every CTA reads from memory after a barrier.
 #pragma once
 #include "common.cuh"
@@ -44,14 +45,14 @@ constexpr int CT_TERM = CT_NB * 128;          // one bf16 term of a 64 x 64 tile
 constexpr int CT_TILE = 2 * CT_TERM;
 constexpr int CT_LDD = 68;                    // diagonal block, fp32 (rows 16-byte aligned, conflict-free by row)
 constexpr int CT_LDS = 65;                    // transposing buffer of the first-order inverse
-// dynamic shared memory: two stages of an A tile and a B tile, then the diagonal block's work area
-constexpr int CT_OFF_D = 4 * CT_TILE;
+// dynamic shared memory: the operand stages, then the diagonal block's work area
+constexpr int CT_STAGES = 4;                  // operand stages, an A tile and a B tile each (a power of two)
+constexpr int CT_OFF_D = CT_STAGES * 2 * CT_TILE;
 constexpr int CT_DG_BLK = CT_NB * CT_LDD * 4;                  // work area of a diagonal block: the block itself, a panel's 8 x 8 block
 constexpr int CT_DG_BYTES = CT_DG_BLK + 64 * 4;
 constexpr int CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;              // the block of the odd columns (the even ones': CT_OFF_D)
 constexpr int CT_SMEM_BYTES = CT_OFF_D2 + CT_NB * CT_LDD * 4 + 1024;     // + alignment of the tiles
-static_assert(2 * (CT_SMEM_BYTES + 2048) <= 228 * 1024, "two CTAs per multiprocessor");
-static_assert(3 * CT_NB * CT_LDS * 4 <= 4 * CT_TILE, "three transposing buffers fit the operand stages");
+static_assert(6 * CT_NB * CT_LDS * 4 <= CT_OFF_D, "six transposing buffers fit the operand stages");
 constexpr int CT_MAX_BLOCKS = 64;             // r <= 4096
 constexpr int CT_STAT_FLOATS = 3 * CT_MAX_BLOCKS;   // per block: smallest and largest pivot, row-sum bound
 constexpr float CT_THIRD_PASS_LIMIT = 0.02f; // bound on |Gram - I|_2 of the second pass above which a third follows
@@ -70,7 +71,8 @@ __device__ __forceinline__ void ct_cp16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
 }
 __device__ __forceinline__ void ct_cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void ct_cp_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void ct_cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void ct_prefetch(const void* p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
 
 __device__ __forceinline__ void mma_bf16_16x8x16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -161,8 +163,8 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 
 // ---- diagonal blocks (fp32, four warps) ----------------------------------------------------------
 // sD (64 x 64 block, ld CT_LDD, beyond nbk a diagonal of the matrix's first pivot; row by row the lower part
-// counts) -> X^T = L^{-T}, L its Cholesky factor, in the upper part of sD; out(row, chunk, z) gets the entries
-// 8 chunk .. + 7 of every row as they are found (zeros left of the diagonal).
+// counts) -> X^T = L^{-T}, L its Cholesky factor, in the upper part of sD and, with xt, as the two terms (`term` bytes
+// apart) of an image tile, row chunk by row chunk as the entries are found.
 //
 // As in the large, [D; I] L^{-T} = [L; L^{-T}]: rows of the block and of the identity go through the same
 // elimination, in panels of eight columns.  Row i of the block is done with its own panel, and row i of the identity begins
@@ -172,7 +174,7 @@ __device__ __forceinline__ void ct_store_tile(uint32_t tile, const float (&v)[4]
 // with the output.
 // What bounds it is the chain and, no less, the instruction cache: a CTA of a cluster comes here once or twice in a
 // factorisation, so the code is fetched as it is run.  Hence one loop over the panels, and one over the columns, of
-// some 600 instructions together.  (Straight-line halves of 32 columns with every lane's row in registers: 9300 cycles alone
+// some 600 instructions together, and the trial run ahead of time in factor_kernel.  (Straight-line halves of 32 columns with every lane's row in registers: 9300 cycles alone
 // and warm, but 23000 in the kernel and 42000 for the first block.)  Step, that form -> this, with the Gram entries
 // of the next diagonal block fetched before the wait for the inverse: 4096 x 4096 r = 256 0.483 -> 0.423 ms, column shard 4096 x
 // 3584 r = 512 0.845 -> 0.775, 11008 x 4096 r = 1024 1.885 -> 1.811, one-kernel QR 520 x 384 r = 64 0.1095 -> 0.1011, fp32
@@ -237,13 +239,30 @@ __device__ __forceinline__ void ct_rank8(float* a, const float (&z)[8], const fl
         for (int j = 0; j < 8; ++j) a[c] = fmaf(-z[j], l[j], a[c]);
     }
 }
-// `blk`: 64 floats of shared memory.  dmin, dmax: smallest (-1: breakdown) and largest pivot, in every lane of warps 0
-// and 1.  unit: 1, or what ct_rsqrt says.  Called by four warps (dw).
-template <class Out>
-__device__ __forceinline__ void ct_diag_block(float* sD, float* blk, int nbk, float unit, int dw, int lane, float& dmin, float& dmax, Out out) {
+// v[e] over the value that its two bf16 terms hold
+__device__ __forceinline__ float ct_diag_scale(const float (&v)[8], const uint4& t0, const uint4& t1, int e) {
+    const uint32_t h[4] = {t0.x, t0.y, t0.z, t0.w}, l[4] = {t1.x, t1.y, t1.z, t1.w};
+    float s = 1.f;
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if (i == e) {
+            const uint32_t hp = h[i / 2], lp = l[i / 2];
+            s = v[i] / ((i & 1) ? bf16hi_to_f32(hp) + bf16hi_to_f32(lp) : bf16lo_to_f32(hp) + bf16lo_to_f32(lp));
+        }
+    return s;
+}
+
+// d_off, blk_off: byte offsets of sD and of 64 more floats in dynamic shared memory.  gscale: corrections of the rounded
+// diagonal, or null.  Returns the smallest (-1: breakdown) and the largest pivot in every lane of warps 0 and 1.  unit: 1,
+// or what ct_rsqrt says.  Called by four warps (dw).  (Not inlined, 16500 cycles a block in place of 13000.)
+__device__ __forceinline__ float2 ct_diag_block(uint32_t d_off, uint32_t blk_off, int nbk, float unit, int dw, int lane,
+                                             unsigned char* xt, int64_t term, float* gscale) {
+    extern __shared__ __align__(16) unsigned char ct_dyn_smem[];
+    float* sD = reinterpret_cast<float*>(ct_dyn_smem + d_off);
+    float* blk = reinterpret_cast<float*>(ct_dyn_smem + blk_off);
     const int np = (nbk + 7) / 8, row = (dw & 1) * 32 + lane, own = row / 8;
     float* sR = sD + row * CT_LDD;
-    dmin = 3.0e38f; dmax = 0.f;
+    float dmin = 3.0e38f, dmax = 0.f;
     if (dw < 2) {
         float z[8];
         ct_ld8(z, sR);
@@ -277,42 +296,32 @@ __device__ __forceinline__ void ct_diag_block(float* sD, float* blk, int nbk, fl
             float z[8];
             ct_ld8(z, sR + 8 * p);
 #pragma unroll 1
-            for (int c = 8 * (p + 2); c < 8 * np; c += 4) {
-                const float4 v = own == p ? make_float4(0.f, 0.f, 0.f, 0.f) : *reinterpret_cast<const float4*>(sR + c);
-                float a[4] = {v.x, v.y, v.z, v.w};
+            for (int c = 8 * (p + 2); c < 8 * np; c += 8) {
+                float a[8] = {};
+                if (own != p) ct_ld8(a, sR + c);
                 ct_rank8(a, z, sD + c * CT_LDD + 8 * p);
-                *reinterpret_cast<float4*>(sR + c) = make_float4(a[0], a[1], a[2], a[3]);
+                ct_rank8(a + 4, z, sD + (c + 4) * CT_LDD + 8 * p);
+                ct_st8(sR + c, a);
             }
-            if (own > p) {
+            if (!xt) continue;
+            // (beyond nbk the elimination has left the padding's part)
 #pragma unroll
-                for (int c = 0; c < 8; ++c) z[c] = 0.f;
-            }
-            out(row, p, z);
+            for (int c = 0; c < 8; ++c) z[c] = own <= p && row < nbk && 8 * p + c < nbk ? z[c] : 0.f;
+            uint4 t0, t1;
+            split8(z, t0, t1);
+            if (gscale && own == p && row < nbk) gscale[row] = ct_diag_scale(z, t0, t1, row % 8);
+            const int o = row * 128 + img_chunk_offset(row, p);
+            *reinterpret_cast<uint4*>(xt + o) = t0;
+            *reinterpret_cast<uint4*>(xt + term + o) = t1;
         }
     }
+    return make_float2(dmin, dmax);
 }
 
-// v[e] over the value that its two bf16 terms hold
-__device__ __forceinline__ float ct_diag_scale(const float (&v)[8], const uint4& t0, const uint4& t1, int e) {
-    const uint32_t h[4] = {t0.x, t0.y, t0.z, t0.w}, l[4] = {t1.x, t1.y, t1.z, t1.w};
-    float s = 1.f;
-#pragma unroll
-    for (int i = 0; i < 8; ++i)
-        if (i == e) {
-            const uint32_t hp = h[i / 2], lp = l[i / 2];
-            s = v[i] / ((i & 1) ? bf16hi_to_f32(hp) + bf16hi_to_f32(lp) : bf16lo_to_f32(hp) + bf16lo_to_f32(lp));
-        }
-    return s;
-}
-
-// (Two CTAs per multiprocessor leave 80 registers a thread: ptxas reports 20 bytes of spill stores and 60 of loads,
-// 104 and 96 in the MULTI form.)
-template <bool MULTI>
-__global__ void __launch_bounds__(CT_THREADS, 2)
+__global__ void __launch_bounds__(CT_THREADS, 1)
 factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
-    extern __shared__ unsigned char smem_raw[];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float red[CT_THREADS / 32];
-    __shared__ float s_row[64];
     __shared__ int s_status;
     unsigned char* smem = smem_raw;
     {
@@ -320,27 +329,16 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         smem += ((raw + 1023u) & ~1023u) - raw;
     }
     const uint32_t smem0 = static_cast<uint32_t>(__cvta_generic_to_shared(smem));
-    auto diag_buf = [&](int k) { return reinterpret_cast<float*>(smem + ((k & 1) ? CT_OFF_D2 : CT_OFF_D)); };
-    float* s_part = reinterpret_cast<float*>(smem);       // partial column sums, before the operand stages are in use
+    float* s_part = reinterpret_cast<float*>(smem);       // partial sums, before the operand stages are in use
 
-    // MULTI: the csize CTAs of a cluster (ranks 0 .. csize-1) share matrix blockIdx.x / csize
-    const int crank = MULTI ? (int)(blockIdx.x % (unsigned)csize) : 0;
-    const int nshare = MULTI ? csize : 1;
-    const MatWork& w = batch.w[MULTI ? blockIdx.x / (unsigned)csize : blockIdx.x];
+    // the csize CTAs of a cluster (ranks 0 .. csize-1) share matrix blockIdx.x / csize
+    const int crank = (int)(blockIdx.x % (unsigned)csize);
+    const MatWork& w = batch.w[blockIdx.x / (unsigned)csize];
     const int tid = threadIdx.x, lane = tid % 32, warp = tid / 32;
     const int r = a.r;
     const int nb = (r + CT_NB - 1) / CT_NB;
     const int shift_bit = a.which ? ST_SHIFT_R : ST_SHIFT_L;
-    auto phase_sync = [&]() { if (MULTI) cluster_sync_all(); else __syncthreads(); };
-
-    grid_dependency();
-    if (tid == 0) s_status = *w.status;
-    __syncthreads();
-    // every CTA of the cluster has read the status word before any of them may change it
-    if (MULTI) cluster_sync_all();
-    const int st0 = s_status;
-    if (st0 & ST_FAILED) return;
-    if (a.pass == 3 && !(st0 & shift_bit)) return;
+    const bool mma_role = warp < CT_MMA_WARPS;
 
     const float* __restrict__ A = pick(w, a.gram);     // Gram matrix: never written here
     unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
@@ -351,47 +349,64 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     unsigned char* limg = scr + (int64_t)w.aux1 * 1024;
     auto l_tile = [&](int t, int c) { return limg + ((int64_t)c * a.img.rows_pad + (int64_t)t * CT_NB) * 128; };
     auto x_tile = [&](int t, int c) { return scr + a.img.off + ((int64_t)c * a.img.rows_pad + (int64_t)t * CT_NB) * 128; };
-
-    // ---- Gram diagonal (from the fp32 column sums of squares), by row tile --------------------
-    // Eight interleaved partial sums per column, added in order: the order depends on the number of
-    // partials only.
-    if (a.use_colsq) {
-        const float* cs = pick(w, a.colsq);
-        const int nparts = w.aux0;
-        const int grp = tid / 128, g = (tid % 128) / 16, q4 = (tid % 16) * 4;     // three tiles at a time
-        for (int t0 = crank; t0 < nb; t0 += 3 * nshare) {
-            const int t = t0 + grp * nshare, col = t * CT_NB + q4;
-            float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (col < r) {
-#pragma unroll 8
-                for (int kb = g; kb < nparts; kb += 8) {
-                    const float4 v = *reinterpret_cast<const float4*>(cs + (int64_t)kb * r + col);
-                    d.x += v.x; d.y += v.y; d.z += v.z; d.w += v.w;
-                }
-            }
-            *reinterpret_cast<float4*>(s_part + (grp * 8 + g) * 64 + q4) = d;
-            __syncthreads();
-            const int c = tid % 128, i = t * CT_NB + c;
-            if (c < 64 && i < r) {
-                float sum = 0.f;
-                for (int q = 0; q < 8; ++q) sum += s_part[(grp * 8 + q) * 64 + c];
-                gdiag[i] = sum;
-                if (a.cnorm_off >= 0) reinterpret_cast<float*>(w.scratch + a.cnorm_off)[i] = sum;
-            }
-            __syncthreads();
-        }
-    } else {
-        for (int t = crank; t < nb; t += nshare)
-            if (tid < 64 && t * CT_NB + tid < r) {
-                const int i = t * CT_NB + tid;
-                const float d = A[(int64_t)i * r + i];
-                gdiag[i] = d;
-                if (a.cnorm_off >= 0) reinterpret_cast<float*>(w.scratch + a.cnorm_off)[i] = d;
-            }
-    }
-    phase_sync();
     float trace = 0.f;
-    {
+
+    // All that comes before the factorisation.  False: there is nothing (more) to do.
+    auto prepare = [&]() -> bool {
+        if (tid == 0) s_status = *w.status;
+        __syncthreads();
+        // every CTA of the cluster has read the status word before any of them may change it
+        cluster_sync_all();
+        const int st0 = s_status;
+        if (st0 & ST_FAILED) return false;
+        if (a.pass == 3 && !(st0 & shift_bit)) return false;
+
+        // ---- Gram diagonal (from the fp32 column sums of squares), by row tile --------------------
+        // 24 interleaved partial sums per column, added in order: the order depends on the number of
+        // partials only.  Loads go out eight at a time, whatever the remainder (one matrix of 11008 rows, r = 1024, with
+        // a loop for the rest and a third of the threads per tile: 13300 cycles).
+        if (a.use_colsq) {
+            const float* cs = pick(w, a.colsq);
+            const int nparts = w.aux0;
+            const int g = tid / 16, q4 = (tid % 16) * 4;
+            for (int t = crank; t < nb; t += csize) {
+                const int col = t * CT_NB + q4;
+                float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (col < r) {
+#pragma unroll 1
+                    for (int kb = g; kb < nparts; kb += 8 * (CT_THREADS / 16)) {
+                        float4 v[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const int k = kb + e * (CT_THREADS / 16);
+                            v[e] = k < nparts ? *reinterpret_cast<const float4*>(cs + (int64_t)k * r + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) { d.x += v[e].x; d.y += v[e].y; d.z += v[e].z; d.w += v[e].w; }
+                    }
+                }
+                *reinterpret_cast<float4*>(s_part + g * 64 + q4) = d;
+                __syncthreads();
+                const int i = t * CT_NB + tid;
+                if (tid < 64 && i < r) {
+                    float sum = 0.f;
+#pragma unroll
+                    for (int q = 0; q < CT_THREADS / 16; ++q) sum += s_part[q * 64 + tid];
+                    gdiag[i] = sum;
+                    if (a.cnorm_off >= 0) reinterpret_cast<float*>(w.scratch + a.cnorm_off)[i] = sum;
+                }
+                __syncthreads();
+            }
+        } else {
+            for (int t = crank; t < nb; t += csize)
+                if (tid < 64 && t * CT_NB + tid < r) {
+                    const int i = t * CT_NB + tid;
+                    const float d = A[(int64_t)i * r + i];
+                    gdiag[i] = d;
+                    if (a.cnorm_off >= 0) reinterpret_cast<float*>(w.scratch + a.cnorm_off)[i] = d;
+                }
+        }
+        cluster_sync_all();
         for (int i = tid; i < r; i += CT_THREADS) trace += __ldcg(gdiag + i);
         for (int o = 16; o; o >>= 1) trace += __shfl_xor_sync(0xffffffffu, trace, o);
         if (lane == 0) red[warp] = trace;
@@ -399,59 +414,77 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         trace = 0.f;
         for (int i = 0; i < CT_THREADS / 32; ++i) trace += red[i];
         __syncthreads();
-    }
-    // (the same sum in the same order in every CTA of a cluster: all of them take this exit or none)
-    if (!(fabsf(trace) <= 3.0e38f)) {   // Inf or NaN
-        if (tid == 0 && crank == 0) atomicOr(w.status, ST_NONFINITE);
-        return;
-    }
-
-    // Tiles of the L^{-T} image below its diagonal that the apply product reads as zeros: those inside the
-    // same 256-column block; and a last diagonal tile that is written in part
-    for (int t = crank; t < nb; t += nshare)
-        for (int c = t & ~3; c < t + (t * CT_NB + CT_NB > r ? 1 : 0); ++c) {
-            unsigned char* dst = x_tile(t, c);
-            for (int q = tid; q < 1024; q += CT_THREADS)
-                *reinterpret_cast<uint4*>(dst + (q >= 512 ? term : 0) + (q & 511) * 16) = make_uint4(0u, 0u, 0u, 0u);
+        // (the same sum in the same order in every CTA of a cluster: all of them take this exit or none)
+        if (!(fabsf(trace) <= 3.0e38f)) {   // Inf or NaN
+            if (tid == 0 && crank == 0) atomicOr(w.status, ST_NONFINITE);
+            return false;
         }
 
-    // ---- later passes of the QR: the Gram matrix is I + E with E small ------------------------
-    // L = I + X with X + X^T + X X^T = E, so L^{-1} = I - Phi(E) + O(|E|^2), Phi = strict lower part
-    // plus half the diagonal.  |E|_2 <= max row sum of |E| (E is symmetric); when that bound is
-    // below CT_SERIES_LIMIT the dropped terms are below 2e-6 and the factorisation is skipped.
-    if (a.pass >= 2) {
-        for (int t = crank; t < nb; t += nshare) {
-            const int i0 = t * CT_NB;
-            // left of the diagonal: a row per warp
-            for (int i = i0 + warp; i < min(r, i0 + CT_NB); i += CT_THREADS / 32) {
+        // Tiles of the L^{-T} image below its diagonal that the apply product reads as zeros: those inside the
+        // same 256-column block; and a last diagonal tile that is written in part
+        for (int t = crank; t < nb; t += csize)
+            for (int c = t & ~3; c < t + (t * CT_NB + CT_NB > r ? 1 : 0); ++c) {
+                unsigned char* dst = x_tile(t, c);
+                for (int q = tid; q < 1024; q += CT_THREADS)
+                    *reinterpret_cast<uint4*>(dst + (q >= 512 ? term : 0) + (q & 511) * 16) = make_uint4(0u, 0u, 0u, 0u);
+            }
+        if (a.pass < 2) return true;
+
+        // ---- later passes of the QR: the Gram matrix is I + E with E small ------------------------
+        // L = I + X with X + X^T + X X^T = E, so L^{-1} = I - Phi(E) + O(|E|^2), Phi = strict lower part
+        // plus half the diagonal.  |E|_2 <= max row sum of |E| (E is symmetric); when that bound is
+        // below CT_SERIES_LIMIT the dropped terms are below 2e-6 and the factorisation is skipped.
+        for (int t = crank; t < nb; t += csize) {
+            const int i0 = t * CT_NB, g = tid / 16, j4 = (tid % 16) * 4;
+            float* s_row = s_part + 24 * 64;
+            // left of the diagonal: 24 rows at a time, 16 threads along each, four loads under way
+            for (int i = i0 + g; i < i0 + CT_NB; i += 24) {
                 float s = 0.f;
-                for (int j = lane * 4; j < i; j += 128) {
-                    const float4 v = *reinterpret_cast<const float4*>(A + (int64_t)i * r + j);
-                    s += fabsf(v.x) + (j + 1 < i ? fabsf(v.y) : 0.f) + (j + 2 < i ? fabsf(v.z) : 0.f) + (j + 3 < i ? fabsf(v.w) : 0.f);
-                }
-                for (int o = 16; o; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                if (lane == 0) s_row[i - i0] = s;
+                if (i < r)
+#pragma unroll 1
+                    for (int j0 = j4; j0 < i; j0 += 256) {
+                        float4 v[4];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            v[e] = j0 + 64 * e < i ? *reinterpret_cast<const float4*>(A + (int64_t)i * r + j0 + 64 * e) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            const int j = j0 + 64 * e;
+                            s += (j < i ? fabsf(v[e].x) : 0.f) + (j + 1 < i ? fabsf(v[e].y) : 0.f) + (j + 2 < i ? fabsf(v[e].z) : 0.f) +
+                                 (j + 3 < i ? fabsf(v[e].w) : 0.f);
+                        }
+                    }
+                const unsigned mask = 0xffffu << (lane & 16);
+                for (int o = 8; o; o >>= 1) s += __shfl_xor_sync(mask, s, o);
+                if (tid % 16 == 0) s_row[i - i0] = s;
             }
             // below the diagonal (the mirror of the row's right part): 24 row groups x 64 columns
             {
-                const int g = tid / 16, j = i0 + (tid % 16) * 4;
+                const int j = i0 + j4;
                 float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (j < r) {
-#pragma unroll 4
-                    for (int i = i0 + g; i < r; i += 24) {
-                        const float4 v = *reinterpret_cast<const float4*>(A + (int64_t)i * r + j);
-                        s.x += i > j ? fabsf(v.x) : 0.f; s.y += i > j + 1 ? fabsf(v.y) : 0.f;
-                        s.z += i > j + 2 ? fabsf(v.z) : 0.f; s.w += i > j + 3 ? fabsf(v.w) : 0.f;
+                if (j < r)
+#pragma unroll 1
+                    for (int ib = i0 + g; ib < r; ib += 24 * 8) {
+                        float4 v[8];
+#pragma unroll
+                        for (int e = 0; e < 8; ++e)
+                            v[e] = ib + 24 * e < r ? *reinterpret_cast<const float4*>(A + (int64_t)(ib + 24 * e) * r + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
+                            const int i = ib + 24 * e;
+                            s.x += i > j ? fabsf(v[e].x) : 0.f; s.y += i > j + 1 ? fabsf(v[e].y) : 0.f;
+                            s.z += i > j + 2 ? fabsf(v[e].z) : 0.f; s.w += i > j + 3 ? fabsf(v[e].w) : 0.f;
+                        }
                     }
-                }
-                *reinterpret_cast<float4*>(s_part + g * 64 + (tid % 16) * 4) = s;
+                *reinterpret_cast<float4*>(s_part + g * 64 + j4) = s;
             }
             __syncthreads();
             if (warp == 0) {
                 float mx = 0.f;
                 for (int q = lane; q < 64 && i0 + q < r; q += 32) {
                     float s = fabsf(__ldcg(gdiag + i0 + q) - 1.f) + s_row[q];
-                    for (int g = 0; g < 24; ++g) s += s_part[g * 64 + q];
+#pragma unroll
+                    for (int e = 0; e < 24; ++e) s += s_part[e * 64 + q];
                     mx = fmaxf(mx, s <= 3.0e38f ? s : 3.3e38f);
                 }
                 for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
@@ -459,7 +492,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
             }
             __syncthreads();
         }
-        phase_sync();
+        cluster_sync_all();
         float mx = 0.f;
         for (int t = 0; t < nb; ++t) mx = fmaxf(mx, __ldcg(gstat + 2 * CT_MAX_BLOCKS + t));
         // Second pass with Q1 far from orthonormal (cond(Y)^2 u was not small): its result will
@@ -467,62 +500,66 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
         if (a.pass == 2 && !(mx <= CT_THIRD_PASS_LIMIT) && tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
         // (a diagonal this close to one is held by its two terms to 2^-20: no correction)
         if (tid == 0 && crank == 0) gscale[r] = mx <= CT_SERIES_LIMIT ? 0.f : 1.f;
-        if (mx <= CT_SERIES_LIMIT) {
-            // Image tiles (ta, tb), tb >= ta, of L^{-T}: entry (row, col) = -E(col, row) right of the
-            // diagonal.  Three groups of four warps, each with a transposing buffer of its own.
-            const int grp = tid / 128, gt = tid % 128;
-            float* buf = reinterpret_cast<float*>(smem) + grp * CT_NB * CT_LDS;
-            const int pairs = nb * (nb + 1) / 2;
-            for (int q0 = crank * 3; q0 < pairs; q0 += 3 * nshare) {
-                int tb = 0, q = q0 + grp;
-                const bool on = q < pairs;
-                while (on && q > tb) { q -= tb + 1; ++tb; }
-                const int ta = q;
-                if (on) {
+        if (!(mx <= CT_SERIES_LIMIT)) return true;
+        // Image tiles (ta, tb), tb >= ta, of L^{-T}: entry (row, col) = -E(col, row) right of the
+        // diagonal.  Three groups of four warps, each with two transposing buffers of its own and the next tile's entries
+        // under way while it writes one.
+        const int grp = tid / 128, gt = tid % 128;
+        float* bufs = reinterpret_cast<float*>(smem) + grp * 2 * CT_NB * CT_LDS;
+        const int pairs = nb * (nb + 1) / 2, step = 3 * csize;
+        int ta = 0, tb = 0;
+        float4 v[8];
+        auto fetch = [&](int q) {                // tile q of the list, if there is one
+            tb = 0;
+            while (q > tb) { q -= tb + 1; ++tb; }
+            ta = q;
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
-                        const int i = gt / 16 + 8 * e, j = (gt % 16) * 4;
-                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (tb * CT_NB + i < r && ta * CT_NB + j < r)
-                            v = *reinterpret_cast<const float4*>(A + (int64_t)(tb * CT_NB + i) * r + ta * CT_NB + j);
-                        buf[i * CT_LDS + j] = v.x; buf[i * CT_LDS + j + 1] = v.y;
-                        buf[i * CT_LDS + j + 2] = v.z; buf[i * CT_LDS + j + 3] = v.w;
-                    }
-                }
-                __syncthreads();
-                if (on) {
-                    unsigned char* dst = x_tile(ta, tb);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const int row = gt / 8 + 16 * e, ch = gt % 8;
-                        const int gr = ta * CT_NB + row, gc = tb * CT_NB + ch * 8;
-                        float v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = gc + i > gr ? -buf[(ch * 8 + i) * CT_LDS + row] : 0.f;
-                        if (gr >= gc && gr < gc + 8 && gr < r) {
-                            const float dg = 0.5f * (3.f - __ldcg(gdiag + gr));
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) v[i] = gc + i == gr ? dg : v[i];
-                        }
-                        uint4 t0, t1;
-                        split8(v, t0, t1);
-                        const int o = row * 128 + img_chunk_offset(row, ch);
-                        *reinterpret_cast<uint4*>(dst + o) = t0;
-                        *reinterpret_cast<uint4*>(dst + term + o) = t1;
-                    }
-                }
-                __syncthreads();
+            for (int e = 0; e < 8; ++e) {
+                const int i = tb * CT_NB + gt / 16 + 8 * e, j = ta * CT_NB + (gt % 16) * 4;
+                v[e] = i < r && j < r ? *reinterpret_cast<const float4*>(A + (int64_t)i * r + j) : make_float4(0.f, 0.f, 0.f, 0.f);
             }
-            return;
+        };
+        int q = crank * 3 + grp, b = 0;
+        if (q < pairs) fetch(q);
+        for (; q < pairs; q += step, b ^= 1) {
+            float* buf = bufs + b * CT_NB * CT_LDS;
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                float* o = buf + (gt / 16 + 8 * e) * CT_LDS + (gt % 16) * 4;
+                o[0] = v[e].x; o[1] = v[e].y; o[2] = v[e].z; o[3] = v[e].w;
+            }
+            const int ca = ta, cb = tb;
+            ct_bar_sync(CT_BAR_MMA + grp, 128);
+            if (q + step < pairs) fetch(q + step);
+            unsigned char* dst = x_tile(ca, cb);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int row = gt / 8 + 16 * e, ch = gt % 8;
+                const int gr = ca * CT_NB + row, gc = cb * CT_NB + ch * 8;
+                float x[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) x[i] = gc + i > gr ? -buf[(ch * 8 + i) * CT_LDS + row] : 0.f;
+                if (gr >= gc && gr < gc + 8 && gr < r) {
+                    const float dg = 0.5f * (3.f - __ldcg(gdiag + gr));
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) x[i] = gc + i == gr ? dg : x[i];
+                }
+                uint4 t0, t1;
+                split8(x, t0, t1);
+                const int o = row * 128 + img_chunk_offset(row, ch);
+                *reinterpret_cast<uint4*>(dst + o) = t0;
+                *reinterpret_cast<uint4*>(dst + term + o) = t1;
+            }
         }
-    }
+        return false;
+    };
 
     // ---- factorisation and inverse ------------------------------------------------------------
-    const bool mma_role = warp < CT_MMA_WARPS;
     const int mrow = (warp % 4) * 16 + lane / 4, mcol = (warp / 4) * 32 + (lane % 4) * 2;     // first element of acc
+    const uint32_t dyn0 = static_cast<uint32_t>(smem - smem_raw);
+    auto diag_off = [&](int k) { return dyn0 + ((k & 1) ? CT_OFF_D2 : CT_OFF_D); };
     int stage = 0;                     // operand stage that the next load goes to
-    auto a_slot = [&](int s) { return smem0 + (uint32_t)s * 2 * CT_TILE; };
-    auto b_slot = [&](int s) { return smem0 + (uint32_t)s * 2 * CT_TILE + CT_TILE; };
+    auto slot = [&](int s) { return (s & (CT_STAGES - 1)) * 2 * CT_TILE; };      // A tile, then B tile
     auto load_tile = [&](uint32_t dst, const unsigned char* src) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -531,22 +568,28 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
             ct_cp16(dst + CT_TERM + q, src + term + q);
         }
     };
-    // acc += sum_{c in [c0, k)} Z[t, c] L[k, c]^T; with `next` also accd += sum Z[t, c] Z[t, c]^T
-    auto sum_products = [&](float (&acc)[4][4], float (&accd)[4][4], int t, int k, bool next) {
+    // acc += sum_{c < k} Z[t, c] L[k, c]^T, accd += sum_{d0 <= c < k} Z[t, c] Z[t, c]^T
+    auto sum_products = [&](float (&acc)[4][4], float (&accd)[4][4], int t, int k, int d0) {
         const int c0 = t < k ? t : 0;
         auto load = [&](int c, int s) {
-            load_tile(a_slot(s), t < k ? x_tile(t, c) : l_tile(t, c));
-            load_tile(b_slot(s), l_tile(k, c));
+            if (c < k) {
+                load_tile(smem0 + slot(s), t < k ? x_tile(t, c) : l_tile(t, c));
+                load_tile(smem0 + slot(s) + CT_TILE, l_tile(k, c));
+            }
             ct_cp_commit();
         };
-        if (c0 < k) load(c0, stage);
+        if (c0 >= k) return;
+#pragma unroll
+        for (int e = 0; e < CT_STAGES - 1; ++e) load(c0 + e, stage + e);
+#pragma unroll 1
         for (int c = c0; c < k; ++c) {
-            ct_cp_wait_all();
+            ct_cp_wait<CT_STAGES - 2>();
             ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
-            if (c + 1 < k) load(c + 1, stage ^ 1);
-            ct_tile_mma(acc, a_slot(stage), b_slot(stage), warp, lane);
-            if (next) ct_tile_mma(accd, a_slot(stage), a_slot(stage), warp, lane);
-            stage ^= 1;
+            load(c + CT_STAGES - 1, stage + CT_STAGES - 1);
+            const uint32_t at = smem0 + slot(stage);
+            ct_tile_mma(acc, at, at + CT_TILE, warp, lane);
+            if (c >= d0) ct_tile_mma(accd, at, at, warp, lane);
+            ++stage;
         }
     };
     auto prefetch_gram = [&](int t, int k) {
@@ -569,22 +612,23 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                 acc[nf][2 * h + 1] = v.y - acc[nf][2 * h + 1];
             }
     };
-    // Z[t, k] = acc X_k^T, left in the A slot of stage ^ 1
+    // Z[t, k] = acc X_k^T, left in the A slot of the stage that is loaded last
     auto panel = [&](float (&acc)[4][4], int k) {
-        load_tile(b_slot(stage), x_tile(k, k));
+        const uint32_t at = smem0 + slot(stage);
+        load_tile(at + CT_TILE, x_tile(k, k));
         ct_cp_commit();
-        ct_store_tile(a_slot(stage), acc, warp, lane);
-        ct_cp_wait_all();
+        ct_store_tile(at, acc, warp, lane);
+        ct_cp_wait<0>();
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
         float o[4][4] = {};
-        ct_tile_mma_nt(o, a_slot(stage), b_slot(stage), warp, lane);
-        ct_store_tile(a_slot(stage ^ 1), o, warp, lane);
+        ct_tile_mma_nt(o, at, at + CT_TILE, warp, lane);
+        ct_store_tile(smem0 + slot(stage + CT_STAGES - 1), o, warp, lane);
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
     };
     // ... and from there to its image
     auto panel_out = [&](int t, int k) {
         unsigned char* dst = t < k ? x_tile(t, k) : l_tile(t, k);
-        const unsigned char* src = smem + (size_t)(stage ^ 1) * 2 * CT_TILE;
+        const unsigned char* src = smem + slot(stage + CT_STAGES - 1);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int q = (tid + CT_MMA_THREADS * e) * 16;
@@ -609,7 +653,7 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     };
     // the work area of diagonal block k <- d - z
     auto diag_store = [&](const float (&d)[4][4], const float (&z)[4][4], int k) {
-        float* sD = diag_buf(k);
+        float* sD = reinterpret_cast<float*>(smem_raw + diag_off(k));
         const float up = trace < CT_TINY_TRACE ? CT_TINY_UP : 1.f;         // see ct_rsqrt
 #pragma unroll
         for (int nf = 0; nf < 4; ++nf)
@@ -618,126 +662,123 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
                 *reinterpret_cast<float2*>(sD + (mrow + 8 * h) * CT_LDD + mcol + nf * 8) =
                     make_float2((d[nf][2 * h] - z[nf][2 * h]) * up, (d[nf][2 * h + 1] - z[nf][2 * h + 1]) * up);
     };
+    auto clear = [&](float (&d)[4][4]) {
+#pragma unroll
+        for (int nf = 0; nf < 4; ++nf)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) d[nf][e] = 0.f;
+    };
 
+    grid_dependency_launch();
     bool ok = false;
-    const int max_attempts = (a.pass == 1) ? 2 : 1;
-    for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
-        const float shift = attempt ? a.shift_rel * trace : 0.f;
-        if (mma_role) {
-            if (crank == 0) {
-                const float none[4][4] = {};
-                float d[4][4] = {};
-                diag_base(d, 0, shift);
-                diag_store(d, none, 0);
-                ct_bar_arrive(CT_BAR_READY, CT_THREADS);
-            }
-            for (int k = 0; k < nb; ++k) {
-                const bool next = k + 1 < nb && (k + 1) % nshare == crank;      // this CTA has the next diagonal block
-                // own tiles of this block column, the one below the diagonal first
-                int t = next ? k + 1 : crank;
-                auto seek = [&]() { while (t < nb && (t == k || (next && t == k + 1))) t += nshare; };
-                if (!next) seek();
-                float acc[4][4] = {}, accd[4][4] = {};
-                const bool first = t < nb;
-                if (first) {
-                    if (t > k) prefetch_gram(t, k);
-                    sum_products(acc, accd, t, k, next);
-                    finish_sum(acc, t, k);
-                    if (next) diag_base(accd, k + 1, shift);
+    // Where launches overlap, the diagonal warps first run a block of three panels on whatever shared memory holds, while
+    // the kernel before is still at work: their code then is in the instruction cache (a block in the chain of one matrix:
+    // 19000 cycles the first and 13000 the others, 10000 either way so).
+#pragma unroll 1
+    for (int dry = a.ahead ? 1 : 0; dry >= 0; --dry) {
+        if (dry && mma_role) continue;
+        if (!dry) {
+            grid_dependency_wait();
+            if (!prepare()) return;
+        }
+        const int max_attempts = (a.pass == 1 && !dry) ? 2 : 1;
+        for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
+            const float shift = attempt ? a.shift_rel * trace : 0.f;
+            if (mma_role) {
+                // The next diagonal block of this CTA, dt: its sum is kept up with column by column, as the tiles of its
+                // row are found (columns below dc are in accd), so that it does not lengthen the column that it is wanted in.
+                float accd[4][4] = {};
+                int dt = crank ? crank : csize, dc = 0;
+                if (crank == 0) {
+                    const float none[4][4] = {};
+                    diag_base(accd, 0, shift);
+                    diag_store(accd, none, 0);
+                    ct_bar_arrive(CT_BAR_READY, CT_THREADS);
+                    clear(accd);
                 }
-                // X_k is in memory
-                if (MULTI) cluster_sync_all();
-                else ct_bar_sync(CT_BAR_X, CT_THREADS);
-                if (first) {
-                    panel(acc, k);
-                    if (next) {
-                        // the chain goes on before anything else
-                        const uint32_t z = a_slot(stage ^ 1);
-                        float dz[4][4] = {};
-                        ct_tile_mma(dz, z, z, warp, lane);
-                        diag_store(accd, dz, k + 1);
-                        ct_bar_arrive(CT_BAR_READY, CT_THREADS);
-                    }
-                    panel_out(t, k);
-                    t = next ? crank : t + nshare;
-                    seek();
-                    for (; t < nb;) {
-                        if (t > k) prefetch_gram(t, k);
-#pragma unroll
-                        for (int nf = 0; nf < 4; ++nf)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) acc[nf][e] = 0.f;
-                        sum_products(acc, accd, t, k, false);
-                        finish_sum(acc, t, k);
-                        panel(acc, k);
-                        panel_out(t, k);
-                        t += nshare;
-                        seek();
-                    }
+                for (int k = 0; k < nb; ++k) {
+                    const bool next = k + 1 < nb && dt == k + 1;
+                    // own tiles of this block column, the one below the diagonal first
+                    int t = next ? k + 1 : crank;
+                    auto seek = [&]() { while (t < nb && (t == k || (next && t == k + 1))) t += csize; };
+                    if (!next) seek();
+                    bool first = true;
+                    do {
+                        float acc[4][4] = {};
+                        const bool on = t < nb, lead = first && next;
+                        if (on) {
+                            if (t > k) prefetch_gram(t, k);
+                            sum_products(acc, accd, t, k, t == dt ? dc : k);
+                            finish_sum(acc, t, k);
+                            if (lead) diag_base(accd, k + 1, shift);
+                        }
+                        if (first) cluster_sync_all();                  // X_k is in memory
+                        if (on) {
+                            panel(acc, k);
+                            const uint32_t z = smem0 + slot(stage + CT_STAGES - 1);
+                            if (lead) {
+                                // the chain goes on before anything else
+                                float dz[4][4] = {};
+                                ct_tile_mma(dz, z, z, warp, lane);
+                                diag_store(accd, dz, k + 1);
+                                ct_bar_arrive(CT_BAR_READY, CT_THREADS);
+                                clear(accd);
+                                dt += csize; dc = 0;
+                            } else if (t == dt) {
+                                ct_tile_mma(accd, z, z, warp, lane);
+                                dc = k + 1;
+                            }
+                            panel_out(t, k);
+                            t = lead ? crank : t + csize;
+                            seek();
+                        }
+                        first = false;
+                    } while (t < nb);
+                    cluster_sync_all();                                 // block column k is in memory
                 }
-                // block column k is in memory
-                if (MULTI) cluster_sync_all();
-                else ct_bar_sync(CT_BAR_XT + (k & 1), CT_THREADS);
-            }
-        } else {
-            // The four diagonal warps.  Block k + 1 is started as soon as the product warps have its sum, while they go
-            // on with block column k: what they owe the barriers of column k is an arrival, not a wait.
-            const int dw = warp - CT_MMA_WARPS;
-            for (int k = 0; k < nb; ++k) {
-                const bool mine = k % nshare == crank;
-                const int nbk = min(CT_NB, r - k * CT_NB);
-                if (mine) {
-                    ct_bar_sync(CT_BAR_READY, CT_THREADS);
-                    // X_k^T goes to the diagonal tile of the L^{-T} image, chunk by chunk, while it is being found
-                    unsigned char* xt = x_tile(k, k);
-                    auto out = [&](int row, int ch, const float (&z)[8]) {
-                        float v[8];
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) v[i] = row < nbk && ch * 8 + i < nbk ? z[i] : 0.f;
-                        uint4 t0, t1;
-                        split8(v, t0, t1);
-                        if (a.pass >= 2 && row / 8 == ch && row < nbk) gscale[k * CT_NB + row] = ct_diag_scale(v, t0, t1, row % 8);
-                        const int o = row * 128 + img_chunk_offset(row, ch);
-                        *reinterpret_cast<uint4*>(xt + o) = t0;
-                        *reinterpret_cast<uint4*>(xt + term + o) = t1;
-                    };
-                    float mn, mx;
-                    ct_diag_block(diag_buf(k), reinterpret_cast<float*>(smem + CT_OFF_D + CT_DG_BLK), nbk,
-                                  trace < CT_TINY_TRACE ? CT_TINY_UP_ROOT : 1.f, dw, lane, mn, mx, out);
-                    // statistics: squared diagonal entries of L
-                    if (lane == 0 && dw == 0) {
-                        if (!(mx <= 3.0e38f)) mn = -1.f;
-                        gstat[k] = mn;
-                        gstat[CT_MAX_BLOCKS + k] = mx;
+            } else {
+                // The four diagonal warps.  Block k + 1 is started as soon as the product warps have its sum, while they go
+                // on with block column k: what they owe the barriers of column k is an arrival, not a wait.
+                const int dw = warp - CT_MMA_WARPS;
+                for (int k = 0; k < nb; ++k) {
+                    if (dry || k % csize == crank) {
+                        const int nbk = dry ? 24 : min(CT_NB, r - k * CT_NB);
+                        if (!dry) ct_bar_sync(CT_BAR_READY, CT_THREADS);
+                        // X_k^T goes to the diagonal tile of the L^{-T} image while it is being found
+                        const float2 mm = ct_diag_block(diag_off(k), dyn0 + CT_OFF_D + CT_DG_BLK, nbk,
+                                                        trace < CT_TINY_TRACE ? CT_TINY_UP_ROOT : 1.f, dw, lane, dry ? smem : x_tile(k, k),
+                                                        dry ? CT_TERM : term, a.pass >= 2 ? gscale + k * CT_NB : nullptr);
+                        if (dry) break;
+                        // statistics: squared diagonal entries of L
+                        if (lane == 0 && dw == 0) {
+                            gstat[k] = mm.y <= 3.0e38f ? mm.x : -1.f;
+                            gstat[CT_MAX_BLOCKS + k] = mm.y;
+                        }
                     }
-                }
-                if (MULTI) {
                     if (k) cluster_wait();                  // (the arrival of the column before)
                     cluster_sync_all();
-                } else {
-                    ct_bar_arrive(CT_BAR_X, CT_THREADS);
+                    cluster_arrive();
                 }
-                if (MULTI) cluster_arrive();
-                else ct_bar_arrive(CT_BAR_XT + (k & 1), CT_THREADS);
+                if (dry) break;
+                cluster_wait();
             }
-            if (MULTI) cluster_wait();
-        }
-        __syncthreads();
-        // every CTA reads the same statistics and takes the same branch
-        bool fail = false;
-        float mn = 3.0e38f, mx = 0.f;
-        for (int k = 0; k < nb; ++k) {
-            const float lo = __ldcg(gstat + k);
-            if (!(lo > 0.f)) fail = true;
-            mn = fminf(mn, lo);
-            mx = fmaxf(mx, __ldcg(gstat + CT_MAX_BLOCKS + k));
-        }
-        const bool ill = (a.pass == 1) && (sqrtf(mx) > a.cond_limit * sqrtf(mn));
-        if (!fail && !(ill && attempt == 0)) {
-            ok = true;
-        } else if (attempt == 0 && a.pass == 1) {
-            if (tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
-            phase_sync();                          // all have read the statistics before they are written again
+            __syncthreads();
+            // every CTA reads the same statistics and takes the same branch
+            bool fail = false;
+            float mn = 3.0e38f, mx = 0.f;
+            for (int k = 0; k < nb; ++k) {
+                const float lo = __ldcg(gstat + k);
+                if (!(lo > 0.f)) fail = true;
+                mn = fminf(mn, lo);
+                mx = fmaxf(mx, __ldcg(gstat + CT_MAX_BLOCKS + k));
+            }
+            const bool ill = (a.pass == 1) && (sqrtf(mx) > a.cond_limit * sqrtf(mn));
+            if (!fail && !(ill && attempt == 0)) {
+                ok = true;
+            } else if (attempt == 0 && a.pass == 1) {
+                if (tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
+                cluster_sync_all();                        // all have read the statistics before they are written again
+            }
         }
     }
     if (!ok && tid == 0 && crank == 0) atomicOr(w.status, ST_RANKDEF);

@@ -222,11 +222,9 @@ int ensure_attributes() {
     if (dev < 0 || dev >= kMaxDevices) return ORTHDION_ERR_CUDA;
     std::lock_guard<std::mutex> lock(mu);
     if (state[dev]) return state[dev] > 0 ? 0 : ORTHDION_ERR_CUDA;
-    cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
+    cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM_BYTES);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
+        e = cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(qr_small_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
     if (e == cudaSuccess)
@@ -234,7 +232,7 @@ int ensure_attributes() {
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(qr_small_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
     if (e == cudaSuccess) {
-        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<true>, CT_THREADS, CT_SMEM_BYTES);
+        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel, CT_THREADS, CT_SMEM_BYTES);
         g_qr_cluster_max[dev] = (signed char)std::min({largest_cluster(qr_small_kernel<16>, QS_THREADS, QS_SMEM_LIMIT),
                                                        largest_cluster(qr_small_kernel<32>, QS_THREADS, QS_SMEM_LIMIT),
                                                        largest_cluster(qr_small_kernel<64>, QS_THREADS, QS_SMEM_LIMIT)});
@@ -333,6 +331,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
         CholArgs ca{};
         ca.gram = sel(W_SCRATCH, lead.sc.gram); ca.work = sel(W_SCRATCH, lead.sc.linv);
         ca.r = r; ca.which = which; ca.pass = pass; ca.shift_rel = kShiftRel;
+        ca.ahead = lead.tensor() && pass == 1 && overlap_launches();
         ca.cond_limit = lead.tensor() ? kCondLimitTensor : kCondLimit;
         ca.colsq = sel(W_SCRATCH, 0); ca.use_colsq = 0; ca.img = no_img(); ca.cnorm_off = -1;
         if (lead.tensor()) {
@@ -345,19 +344,18 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
         auto flush = [&]() {
             if (!merged->count) return;
             if (lead.tensor()) {
-                // Fewer matrices than the device has room for CTAs (two per multiprocessor): share
-                // each matrix among the CTAs of a cluster, up to one per 64-row tile (16 only
-                // where the device can place such a cluster).
-                // (counted over the whole grouped call: with more matrices than that, the other
-                // launch batches keep the rest of the device busy on their own streams.)
+                // Fewer matrices than the device has multiprocessors (one CTA each): share each matrix among the CTAs of
+                // a cluster, up to one per 64-row tile (16 only where the device can place such a cluster).
+                // (Counted over the whole grouped call: with more matrices than that, the other launch batches keep
+                // the rest of the device busy on their own streams; counted by batch, the 1.1B and 8B groups run
+                // as before.  Twice as many CTAs, in two waves: 28 matrices at r = 272 1.61 -> 1.75 ms a step.)
                 int csize = 1;
-                const int room = 2 * sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
+                const int room = sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
                 while (csize < cluster_max(g_factor_cluster_max) && csize < tiles &&
                        std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
-                launch(csize == 1 ? factor_kernel<false> : factor_kernel<true>, dim3((unsigned)(merged->count * csize)), CT_THREADS,
-                       CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
+                launch(factor_kernel, dim3((unsigned)(merged->count * csize)), CT_THREADS, CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
             } else {
-                launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, CT_SMEM_BYTES, 1, prof::S_CHOL, st, *merged, ca);
+                launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, FS_SMEM_BYTES, 1, prof::S_CHOL, st, *merged, ca);
             }
             merged->count = 0;
         };

@@ -427,9 +427,8 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                     __syncthreads();
                     if (tiny) scale_block(CT_TINY_UP);
                     if (warp < CT_DIAG_WARPS) {
-                        float mn, mx;
-                        ct_diag_block(sD, reinterpret_cast<float*>(smem + CT_DG_BLK), r, 1.f, warp, lane, mn, mx, [](int, int, const float (&)[8]) {});
-                        if (tid == 0) { s_min = mx <= 3.0e38f ? mn : -1.f; s_max = mx; }
+                        const float2 mm = ct_diag_block(0, CT_DG_BLK, r, 1.f, warp, lane, nullptr, 0, nullptr);
+                        if (tid == 0) { s_min = mm.y <= 3.0e38f ? mm.x : -1.f; s_max = mm.y; }
                     }
                     __syncthreads();
                     const float mn = s_min, mx = s_max;
