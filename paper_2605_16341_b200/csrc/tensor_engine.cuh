@@ -38,8 +38,8 @@ constexpr int A_RING_BYTES = 4 * A_TERM_BYTES;   // two slots of two terms, or f
 constexpr int MAX_A_SLOTS = 4;
 constexpr int MAX_N_SLOTS = 6;
 constexpr int NUM_XF_WARPS = 16;             // transform warps of the kernels that form B = M + G
-constexpr int STAGING_BYTES_PER_WARP = 8192; // epilogue staging: one 32 x 64 fp32 block (or M, G, X slabs) per warp
-constexpr int BUF_STAGING_BYTES = 4096;      // the same for the products with B: one 32 x 32 fp32 block per warp
+constexpr int STAGING_BYTES_PER_WARP = 8192; // epilogue staging of the fused pass: M, G, X slabs per warp
+constexpr int STORE_STAGING_BYTES = 4096;      // of all products: one 32 x 32 fp32 block per warp
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // about two seconds
 
@@ -53,7 +53,7 @@ __host__ __device__ constexpr bool a_is_buf(int amode) { return amode == A_BUF_R
 // have sixteen transform warps already, and the image-to-image products of the QR do better with
 // the 32 KB of staging that four more warps would take spent on a third A slot (they are bound by
 // the latency of their operand tiles: measured apply 10.3 -> 9.4 ms, Gram 8.85 -> 8.5 ms).
-__host__ __device__ constexpr int epi_warps(int amode, int epi) { (void)amode; return epi == EPI_K5 ? 8 : 4; }
+__host__ __device__ constexpr int epi_warps(int amode, int epi) { return epi == EPI_K5 || !a_is_buf(amode) ? 8 : 4; }
 __host__ __device__ constexpr int gemm_threads(int amode, int epi) {
     return 32 * (2 + epi_warps(amode, epi) + (a_is_buf(amode) ? NUM_XF_WARPS : 0));
 }
@@ -522,7 +522,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     unsigned char* a_ring = smem;
     unsigned char* n_ring = smem + g.a_slots * g.a_slot_bytes;
     unsigned char* staging = n_ring + (size_t)g.n_slots * g.n_piece_bytes;
-    unsigned char* tail = staging + NE * (A_BUF ? BUF_STAGING_BYTES : g.epi_bufs * STAGING_BYTES_PER_WARP);
+    unsigned char* tail = staging + NE * (EPI == EPI_STORE ? STORE_STAGING_BYTES : g.epi_bufs * STAGING_BYTES_PER_WARP);
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
     const uint32_t a_full0 = smem_u32(bars), a_empty0 = a_full0 + 8 * MAX_A_SLOTS;
     const uint32_t n_full0 = a_empty0 + 8 * MAX_A_SLOTS, n_empty0 = n_full0 + 8 * MAX_N_SLOTS;
@@ -531,7 +531,6 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
     const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
-    StatusCache scache;
 
     // Pairs: the "full" barriers of the operand rings and the "empty" barriers of the accumulators
     // that are used are the leader's; they count the arrivals of both CTAs.
@@ -565,6 +564,9 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     }
     tc_fence_before();
     grid_dependency_wait();
+    // (most often the matrix of the first tile: on its way while the CTA gathers)
+    StatusCache scache;
+    scache.b = 0; scache.st = *batch.w[0].status;
     __syncthreads();
     if (PAIR) cluster_sync_all();       // the peer's barriers are initialised before anything reaches them
     tc_fence_after();
@@ -871,8 +873,6 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         if (scale_on) cscale = f;
                     }
                 }
-                if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
-                tc_fence_after();
                 const int stw = scache.st;
                 const Dest& d = (g.out.shift_bit && (stw & g.out.shift_bit)) ? g.out.shifted : g.out.normal;
                 const uint32_t taddr = tmem_base + acc * acc_stride + ((uint32_t)(quarter * 32) << 16);
@@ -880,28 +880,37 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
                 // (a run of tiles with chunks of their own: image and column squares when the sum is complete)
                 const bool whole = !(A_BUF && RUN) || c.chunk == g.run - 1;
+                const bool add = !A_BUF && RUN && g.run > 1 && c.chunk > 0;      // Gram product: to what this very thread has stored
                 const bool to_img = d.img.off >= 0 && whole;
                 float* csq = d.colsq && whole ? reinterpret_cast<float*>(w.scratch + g.colsq_off) +
                                            (int64_t)(c.mt * 4 + quarter) * g.Ncols : nullptr;
-                if constexpr (A_BUF) {
                 // 32 columns at a time: this warp's 32 x 32 block goes through a 4 KB staging buffer so that
                 // global stores run along rows: 8 lines per instruction where one row per lane took 32.  Tiles
                 // of 512 columns leave no second accumulator, and the tensor core waits for this (19 % of the first
                 // product and 33 % of the second at r = 512, before).  First and second product: six layers of
                 // 2048-wide matrices, r = 192 0.772 -> 0.699 and 0.768 -> 0.700 ms, r = 512 0.873 -> 0.870 and 1.044 -> 0.933; 24 layers of 768-wide ones, r = 192 0.407 -> 0.385 and 0.472 -> 0.417.
-                unsigned char* stg = staging + (warp - 2) * BUF_STAGING_BYTES;
+                // One rolled loop for all products: in launches of a tile or two its code is fetched as it is run.
+                unsigned char* stg = staging + (warp - 2) * STORE_STAGING_BYTES;
                 const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
                 // (pairs: the CTA whose rows lie beyond the matrix stores nothing)
                 const bool has_rows = !PAIR || (int64_t)c.mt * BM < g.Mrows;
                 const int bn64 = !has_rows ? 0 : (to_img ? (c.bn + 63) / 64 * 64 : c.bn);
                 // (the last tile of a run may have fewer chunks than the others)
-                const int tile_chunks = RUN && c.chunk > 0 ? (c.kb_end - c.kb_begin + g.kb_per_chunk - 1) / g.kb_per_chunk : g.acc_chunks;
+                const int tile_chunks = !A_BUF ? 1 : RUN && c.chunk > 0 ? (c.kb_end - c.kb_begin + g.kb_per_chunk - 1) / g.kb_per_chunk : g.acc_chunks;
                 const int srow = lane / 4, sch = lane % 4;      // stores: 8 rows x 4 chunks of 8 columns per step
-                for (int cc = 0; cc < bn64; cc += 32) {
+                // Image products: before the first tile's accumulator is there, one trial run of the loop that stores nothing (its
+                // code then is in the instruction cache).
+                const int cc0 = (warp - 2) / 4 * 32;
+                bool live = A_BUF || t != tile0;
+                if (live) {
+                    if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
+                    tc_fence_after();
+                }
+                for (int cc = cc0; cc < bn64; cc += 8 * NE) {
                     uint32_t v[2][16];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        if (cc + 16 * h < c.bn) {
+                        if (cc + 16 * h < c.bn && live) {
                             tmem_ld16(taddr + cc + 16 * h, v[h]);
                         } else {
 #pragma unroll
@@ -909,7 +918,19 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                         }
                     }
                     tmem_ld_wait();
-                    if (RUN && c.chunk > 0 && gi0 + lane < g.Mrows) {
+                    if (!A_BUF && cscale) {
+#pragma unroll
+                        for (int i = 0; i < 32; i += 4) {
+                            if (cc + i < c.bn) {
+                                const float4 f = *reinterpret_cast<const float4*>(cscale + c.n0 + cc + i);
+                                const float fe[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    v[i / 16][i % 16 + e] = __float_as_uint(__uint_as_float(v[i / 16][i % 16 + e]) * fe[e]);
+                            }
+                        }
+                    }
+                    if (A_BUF && RUN && c.chunk > 0 && gi0 + lane < g.Mrows) {
                         // the sum so far of this lane's row, stored by this warp
                         const float* o = C + (gi0 + lane) * g.out.ld + c.n0 + cc;
 #pragma unroll
@@ -946,186 +967,92 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     __syncwarp();
                     const int gj = c.n0 + cc;
                     if (csq) {
-                        // column sums of squares over the 32 rows of this warp: fold 32 values over the five
-                        // lane bits, after which every lane has the sum of one column
-                        float s[32];
+                        // column sums of squares over the 32 rows of this warp
+                        float sum;
+                        if constexpr (A_BUF) {
+                            // in registers (22 warps leave none for addresses): fold 32 values over the five lane bits, after
+                            // which every lane has the sum of one column
+                            float s[32];
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) { const float x = __uint_as_float(v[i / 16][i % 16]); s[i] = __fmul_rn(x, x); }
+                            for (int i = 0; i < 32; ++i) { const float x = __uint_as_float(v[i / 16][i % 16]); s[i] = __fmul_rn(x, x); }
 #pragma unroll
-                        for (int half = 16; half >= 1; half >>= 1) {
-                            const bool up = (lane & half) != 0;
+                            for (int half = 16; half >= 1; half >>= 1) {
+                                const bool up = (lane & half) != 0;
 #pragma unroll
-                            for (int i = 0; i < 16; ++i) {
-                                if (i < half) {
-                                    const float send = up ? s[i] : s[i + half];
-                                    const float keep = up ? s[i + half] : s[i];
-                                    s[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                                for (int i = 0; i < 16; ++i) {
+                                    if (i < half) {
+                                        const float send = up ? s[i] : s[i + half];
+                                        const float keep = up ? s[i + half] : s[i];
+                                        s[i] = keep + __shfl_xor_sync(0xffffffffu, send, half);
+                                    }
                                 }
                             }
+                            sum = s[0];
+                        } else {
+                            // a column per lane, in less code
+                            float q[4] = {};
+#pragma unroll 2
+                            for (int i = 0; i < 32; i += 4)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    const float x = *reinterpret_cast<const float*>(stg + (i + e) * 128 + img_chunk_offset(i + e, lane / 4) + lane % 4 * 4);
+                                    q[e] = fmaf(x, x, q[e]);
+                                }
+                            sum = (q[0] + q[1]) + (q[2] + q[3]);
                         }
-                        if (cc + lane < c.bn) csq[gj + lane] = s[0];
+                        if (cc + lane < c.bn && live) csq[gj + lane] = sum;
                     }
                     // (the image has 128 rows per tile, the fp32 result only those of the matrix)
-                    const int rows = (int)min((int64_t)32, g.Mrows - gi0) - srow;
+                    const int rows = live ? (int)min((int64_t)32, g.Mrows - gi0) - srow : 0;
                     const bool col_in = cc + sch * 8 < c.bn;
                     float* Cp = C + (gi0 + srow) * g.out.ld + gj + sch * 8;
                     unsigned char* ip = scr + (to_img ? img_row_offset(d.img, 0, gj / 64, gi0 + srow) : 0) +
                                         img_chunk_offset(srow, gj % 64 / 8 + sch);
                     const int64_t plane_bytes = (int64_t)d.img.panels * d.img.rows_pad * 128;
+                    // (all loads first: one behind a store that may alias it would wait for the store)
+                    float4 old[4][2];
+                    if (add) {
+#pragma unroll
+                        for (int it = 0; it < 4; ++it) {
+                            const bool in = it * 8 < rows && col_in;
+                            old[it][0] = in ? *reinterpret_cast<const float4*>(Cp + it * 8 * g.out.ld) : make_float4(0.f, 0.f, 0.f, 0.f);
+                            old[it][1] = in ? *reinterpret_cast<const float4*>(Cp + it * 8 * g.out.ld + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                    }
 #pragma unroll
                     for (int it = 0; it < 4; ++it) {
                         const unsigned char* sp = stg + (it * 8 + srow) * 128;
-                        const float4 x = *reinterpret_cast<const float4*>(sp + img_chunk_offset(srow, 2 * sch));
-                        const float4 y = *reinterpret_cast<const float4*>(sp + img_chunk_offset(srow, 2 * sch + 1));
+                        float4 x = *reinterpret_cast<const float4*>(sp + img_chunk_offset(srow, 2 * sch));
+                        float4 y = *reinterpret_cast<const float4*>(sp + img_chunk_offset(srow, 2 * sch + 1));
+                        if (add) {
+                            x = make_float4(old[it][0].x + x.x, old[it][0].y + x.y, old[it][0].z + x.z, old[it][0].w + x.w);
+                            y = make_float4(old[it][1].x + y.x, old[it][1].y + y.y, old[it][1].z + y.z, old[it][1].w + y.w);
+                        }
                         if (C && it * 8 < rows && col_in) {
                             *reinterpret_cast<float4*>(Cp + it * 8 * g.out.ld) = x;
                             *reinterpret_cast<float4*>(Cp + it * 8 * g.out.ld + 4) = y;
                         }
                         if (to_img) {
+                            const bool st = A_BUF || live;
                             const float f[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
                             uint4 t0, t1;
                             split8(f, t0, t1);
-                            *reinterpret_cast<uint4*>(ip + it * 1024) = t0;
-                            *reinterpret_cast<uint4*>(ip + plane_bytes + it * 1024) = t1;
-                            if (d.img.planes == 3) *reinterpret_cast<uint4*>(ip + 2 * plane_bytes + it * 1024) = half8(f, 1.f);
+                            if (st) *reinterpret_cast<uint4*>(ip + it * 1024) = t0;
+                            if (st) *reinterpret_cast<uint4*>(ip + plane_bytes + it * 1024) = t1;
+                            if (d.img.planes == 3 && st) *reinterpret_cast<uint4*>(ip + 2 * plane_bytes + it * 1024) = half8(f, 1.f);
                         }
                     }
                     __syncwarp();
-                }
-                } else {
-                // 64 columns at a time: this warp's 32 x 64 block goes through an 8 KB staging
-                // buffer so that global stores run along rows.  A plane's block is 32 image rows of
-                // 128 bytes, byte for byte what the image holds, so it leaves as one 4 KB run.
-                unsigned char* stg = staging + (warp - 2) * STAGING_BYTES_PER_WARP;
-                const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
-                const bool has_rows = !PAIR || (int64_t)c.mt * BM < g.Mrows;
-                const int groups = has_rows ? (c.bn + 63) / 64 : 0;
-                for (int cg = (warp - 2) / 4; cg < groups; cg += NE / 4) {
-                    const int valid = min(64, c.bn - cg * 64);          // multiple of 16
-                    const int gj0 = c.n0 + cg * 64;
-                    float f[64];
-#pragma unroll
-                    for (int q4 = 0; q4 < 4; ++q4) {
-                        uint32_t v[16];
-                        if (q4 * 16 < valid) {
-                            tmem_ld16(taddr + cg * 64 + q4 * 16, v);
-                            tmem_ld_wait();
-                        } else {
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) v[i] = 0u;
-                        }
-#pragma unroll
-                        for (int i = 0; i < 16; ++i) f[q4 * 16 + i] = __uint_as_float(v[i]);
-                        if (cscale && q4 * 16 < valid) {
-#pragma unroll
-                            for (int i = 0; i < 16; i += 4) {
-                                const float4 cv = *reinterpret_cast<const float4*>(cscale + gj0 + q4 * 16 + i);
-                                f[q4 * 16 + i] *= cv.x; f[q4 * 16 + i + 1] *= cv.y;
-                                f[q4 * 16 + i + 2] *= cv.z; f[q4 * 16 + i + 3] *= cv.w;
-                            }
-                        }
-                        if (csq && q4 * 16 < valid) {
-                            // column sums of squares over the 32 rows of this warp: fold 16 values
-                            // over the lane bits 4..1, then add the two lanes that hold the same column
-                            float s[16];
-#pragma unroll
-                            for (int i = 0; i < 16; ++i) { const float x = f[q4 * 16 + i]; s[i] = x * x; }
-#pragma unroll
-                            for (int half = 8, bit = 16; half >= 1; half >>= 1, bit >>= 1) {
-                                const bool up = (lane & bit) != 0;
-#pragma unroll
-                                for (int i = 0; i < 8; ++i) {
-                                    if (i < half) {
-                                        const float send = up ? s[i] : s[i + half];
-                                        const float keep = up ? s[i + half] : s[i];
-                                        s[i] = keep + __shfl_xor_sync(0xffffffffu, send, bit);
-                                    }
-                                }
-                            }
-                            s[0] += __shfl_xor_sync(0xffffffffu, s[0], 1);
-                            const int col = ((lane >> 4) & 1) * 8 + ((lane >> 3) & 1) * 4 + ((lane >> 2) & 1) * 2 + ((lane >> 1) & 1);
-                            if (!(lane & 1)) csq[gj0 + q4 * 16 + col] = s[0];
-                        }
-                    }
-                    if (C) {
-                        // fp32 block: 32 rows x 256 bytes, 16-byte chunks swizzled by (row & 7)
-                        const bool add = RUN && g.run > 1 && c.chunk > 0;
-#pragma unroll
-                        for (int ch = 0; ch < 16; ++ch)
-                            *reinterpret_cast<float4*>(stg + lane * 256 + ((ch ^ (lane & 7)) << 4)) =
-                                make_float4(f[4 * ch], f[4 * ch + 1], f[4 * ch + 2], f[4 * ch + 3]);
-                        __syncwarp();
-                        if (add) {
-                            // the sum so far, stored by this very thread; all loads first (a load behind a store that
-                            // may alias it would wait for the store)
-                            float4 o[16];
-#pragma unroll
-                            for (int it = 0; it < 16; ++it) {
-                                const int r = it * 2 + lane / 16, ch = lane % 16;
-                                o[it] = make_float4(0.f, 0.f, 0.f, 0.f);
-                                if (gi0 + r < g.Mrows && ch * 4 < valid)
-                                    o[it] = *reinterpret_cast<const float4*>(C + (gi0 + r) * g.out.ld + gj0 + ch * 4);
-                            }
-#pragma unroll
-                            for (int it = 0; it < 16; ++it) {
-                                const int r = it * 2 + lane / 16, ch = lane % 16;
-                                const float4 x = *reinterpret_cast<const float4*>(stg + r * 256 + ((ch ^ (r & 7)) << 4));
-                                if (gi0 + r < g.Mrows && ch * 4 < valid)
-                                    *reinterpret_cast<float4*>(C + (gi0 + r) * g.out.ld + gj0 + ch * 4) =
-                                        make_float4(o[it].x + x.x, o[it].y + x.y, o[it].z + x.z, o[it].w + x.w);
-                            }
-                        } else {
-#pragma unroll
-                        for (int it = 0; it < 16; ++it) {
-                            const int r = it * 2 + lane / 16, ch = lane % 16;
-                            const float4 x = *reinterpret_cast<const float4*>(stg + r * 256 + ((ch ^ (r & 7)) << 4));
-                            if (gi0 + r < g.Mrows && ch * 4 < valid)
-                                *reinterpret_cast<float4*>(C + (gi0 + r) * g.out.ld + gj0 + ch * 4) = x;
-                        }
-                        }
-                        __syncwarp();
-                    }
-                    if (to_img) {
-                        // the two bf16 planes together (4 KB each in the staging buffer), then the fp16 plane
-                        const int panel = gj0 / 64;
-#pragma unroll
-                        for (int ch = 0; ch < 8; ++ch) {
-                            const float fv[8] = {f[8 * ch], f[8 * ch + 1], f[8 * ch + 2], f[8 * ch + 3],
-                                                 f[8 * ch + 4], f[8 * ch + 5], f[8 * ch + 6], f[8 * ch + 7]};
-                            uint4 t0, t1;
-                            split8(fv, t0, t1);
-                            const int o = lane * 128 + img_chunk_offset(lane, ch);
-                            *reinterpret_cast<uint4*>(stg + o) = t0;
-                            *reinterpret_cast<uint4*>(stg + 4096 + o) = t1;
-                        }
-                        __syncwarp();
-                        unsigned char* dst0 = scr + img_row_offset(d.img, 0, panel, gi0);
-                        unsigned char* dst1 = scr + img_row_offset(d.img, 1, panel, gi0);
-#pragma unroll
-                        for (int it = 0; it < 8; ++it) {
-                            *reinterpret_cast<uint4*>(dst0 + it * 512 + lane * 16) =
-                                *reinterpret_cast<const uint4*>(stg + it * 512 + lane * 16);
-                            *reinterpret_cast<uint4*>(dst1 + it * 512 + lane * 16) =
-                                *reinterpret_cast<const uint4*>(stg + 4096 + it * 512 + lane * 16);
-                        }
-                        __syncwarp();
-                        if (d.img.planes == 3) {
-#pragma unroll
-                            for (int ch = 0; ch < 8; ++ch) {
-                                const float fv[8] = {f[8 * ch], f[8 * ch + 1], f[8 * ch + 2], f[8 * ch + 3],
-                                                     f[8 * ch + 4], f[8 * ch + 5], f[8 * ch + 6], f[8 * ch + 7]};
-                                *reinterpret_cast<uint4*>(stg + lane * 128 + img_chunk_offset(lane, ch)) = half8(fv, 1.f);
-                            }
-                            __syncwarp();
-                            unsigned char* dst2 = scr + img_row_offset(d.img, 2, panel, gi0);
-#pragma unroll
-                            for (int it = 0; it < 8; ++it)
-                                *reinterpret_cast<uint4*>(dst2 + it * 512 + lane * 16) =
-                                    *reinterpret_cast<const uint4*>(stg + it * 512 + lane * 16);
-                            __syncwarp();
-                        }
+                    if (!live) {
+                        if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
+                        tc_fence_after();
+                        live = true;
+                        cc = cc0 - 8 * NE;
                     }
                 }
+                if (!ok) break;
+                if (!live) {        // (no columns here: the accumulator is only handed on)
+                    if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) { ok = false; break; }
                 }
                 tc_fence_before();
                 __syncwarp();
@@ -1798,13 +1725,13 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
         // ring: r = 512 0.858 -> 0.917.)
         max_n_slots = 3;
         g.a_slots = 3;
-        if (3 * (size_t)g.a_slot_bytes + 3 * (size_t)g.n_piece_bytes + 4 * tc::BUF_STAGING_BYTES + 2304 > 196 * 1024) g.a_slots = 2;
+        if (3 * (size_t)g.a_slot_bytes + 3 * (size_t)g.n_piece_bytes + 4 * tc::STORE_STAGING_BYTES + 2304 > 196 * 1024) g.a_slots = 2;
     }
     // (the fused pass on other types than bf16 loads M, G and X into registers: the same line.  bf16 X and fp32 G, 4096 x 4096
     // r = 128 0.079 -> 0.066 ms, r = 512 0.088 -> 0.075; fp32 X fits one slot either way)
     if (EPI == tc::EPI_K5 && XG != 3) max_n_slots = 2;
     const size_t fixed = (size_t)g.a_slots * g.a_slot_bytes +
-                         (size_t)tc::epi_warps(AMODE, EPI) * (tc::a_is_buf(AMODE) ? tc::BUF_STAGING_BYTES : g.epi_bufs * tc::STAGING_BYTES_PER_WARP) +
+                         (size_t)tc::epi_warps(AMODE, EPI) * (EPI == tc::EPI_STORE ? tc::STORE_STAGING_BYTES : g.epi_bufs * tc::STAGING_BYTES_PER_WARP) +
                          256 + 1024;
     g.n_slots = (int)std::min<size_t>(max_n_slots, (tc::SMEM_LIMIT - fixed) / (size_t)g.n_piece_bytes);
     // more than half of an SM's shared memory: one CTA per SM, whatever its tensor-memory share
@@ -1931,8 +1858,9 @@ struct FinishArgs {
     Sel dst, part;
     int64_t rows;
     int32_t r, ksplit;
-    ImgRef img;
+    ImgRef img;                 // its geometry decides the launch
     int64_t colsq_off;
+    int32_t to_img;
 };
 __global__ void __launch_bounds__(256)
 finish_split_kernel(const __grid_constant__ Batch batch, FinishArgs a) {
