@@ -29,13 +29,10 @@ struct CholArgs {
     int64_t cnorm_off;   // >= 0: also leave the Gram diagonal (squared column norms) there, fp32 [r]
 };
 
-// ---- ColNorm (Alg. 1, normalisation step, Dion branch): Q[:,j] = R[:,j] / ||R[:,j]||_2 ----------------------
+// ---- ColNorm of the SIMT engine (Alg. 1, normalisation step, Dion branch): Q[:,j] = R[:,j] / ||R[:,j]||_2 ---
 // One CTA per 32 columns: 32 x 32 threads, lanes along columns (coalesced rows).
-// part: 0 = the whole operation; 1 = only the squared column norms of the rows at hand, left at
-// cnorm_off (a column-sharded matrix sums them over the shards before it scales); 2 = only the
-// scaling, with the squared norms taken from cnorm_off.
 __global__ void __launch_bounds__(1024)
-colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t cnorm_off, int part_sel) {
+colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
@@ -44,26 +41,57 @@ colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t cn
     const int lane = threadIdx.x % 32, ry = threadIdx.x / 32;
     const int j = blockIdx.x * 32 + lane;
     float s = 0.f;
-    if (j < r && part_sel != 2)
+    if (j < r)
         for (int64_t i = ry; i < n; i += 32) { float v = w.R[i * r + j]; s = fmaf(v, v, s); }
     part[ry][lane] = s;
     __syncthreads();
     if (ry == 0) {
         float t = 0.f;
-        if (part_sel == 2) {
-            if (j < r) t = reinterpret_cast<const float*>(w.scratch + cnorm_off)[j];
-        } else {
-            for (int k = 0; k < 32; ++k) t += part[k][lane];
-            if (cnorm_off >= 0 && j < r) reinterpret_cast<float*>(w.scratch + cnorm_off)[j] = t;
-        }
+        for (int k = 0; k < 32; ++k) t += part[k][lane];
         float nrm = sqrtf(t);
-        if (j < r && !(nrm > 0.f) && part_sel != 1) atomicOr(w.status, ST_ZEROCOL);
+        if (j < r && !(nrm > 0.f)) atomicOr(w.status, ST_ZEROCOL);
         inv[lane] = (nrm > 0.f) ? 1.f / nrm : 0.f;
     }
     __syncthreads();
-    if (j < r && part_sel != 1) {
+    if (j < r) {
         const float sc = inv[lane];
         for (int64_t i = ry; i < n; i += 32) w.Q[i * r + j] = w.R[i * r + j] * sc;
+    }
+}
+
+// ---- squared column norms -----------------------------------------------------------------------
+// dst[j * stride] <- sum over the blocks of the column sums of squares that a product kernel has left per 32 rows
+// (colsq[block * r + j]).  stride 1: the squared column norms; r + 1: the diagonal of a Gram matrix (fp32 sums: the tensor
+// core's truncating accumulation would bias it low), so that a sum of it over shards carries the exact diagonal along.
+// One CTA per 64 columns: 16 interleaved sums per column, eight loads of each under way (latency is all there is: a serial
+// loop took 11.5 us for 3584 rows at r = 512).
+__global__ void __launch_bounds__(256)
+colsum_kernel(const __grid_constant__ Batch batch, int64_t colsq_off, int blocks, int r, Sel dst, int64_t stride) {
+    grid_dependency();
+    const MatWork& w = batch.w[blockIdx.z];
+    if (*w.status & ST_FAILED) return;
+    __shared__ float part[16][64];
+    const float* cs = reinterpret_cast<const float*>(w.scratch + colsq_off);
+    const int g = threadIdx.x / 16, q4 = threadIdx.x % 16 * 4, col = blockIdx.x * 64 + q4;
+    float4 d = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (col < r)
+#pragma unroll 1
+        for (int kb = g; kb < blocks; kb += 128) {
+            float4 v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                v[e] = kb + 16 * e < blocks ? *reinterpret_cast<const float4*>(cs + (int64_t)(kb + 16 * e) * r + col) : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) { d.x += v[e].x; d.y += v[e].y; d.z += v[e].z; d.w += v[e].w; }
+        }
+    *reinterpret_cast<float4*>(&part[g][q4]) = d;
+    __syncthreads();
+    const int j = blockIdx.x * 64 + threadIdx.x;
+    if (threadIdx.x < 64 && j < r) {
+        float sum = 0.f;
+#pragma unroll
+        for (int k = 0; k < 16; ++k) sum += part[k][threadIdx.x];
+        pick(w, dst)[j * stride] = sum;
     }
 }
 
@@ -85,22 +113,6 @@ colsq_blocks_kernel(const __grid_constant__ Batch batch, Sel src, int64_t rows, 
     for (int k = 0; k < 32; ++k)
         if (i0 + k < rows) { const float v = S[(i0 + k) * r + j]; s = fmaf(v, v, s); }
     out[(int64_t)blockIdx.x * r + j] = s;
-}
-
-// Gram diagonal <- sum of the per-block column sums of squares (fp32 sums: the tensor core's
-// truncating accumulation would bias the diagonal low), so that a reduction of the r x r matrix
-// over the shards carries the exact diagonal along.
-__global__ void __launch_bounds__(256)
-gram_diag_kernel(const __grid_constant__ Batch batch, Sel gram, int r, int64_t colsq_off, int blocks) {
-    grid_dependency();
-    const MatWork& w = batch.w[blockIdx.z];
-    if (*w.status & ST_FAILED) return;
-    const int j = blockIdx.x * 256 + threadIdx.x;
-    if (j >= r) return;
-    const float* cs = reinterpret_cast<const float*>(w.scratch + colsq_off);
-    float d = 0.f;
-    for (int b = 0; b < blocks; ++b) d += cs[(int64_t)b * r + j];
-    pick(w, gram)[(int64_t)j * r + j] = d;
 }
 
 __global__ void init_status_kernel(const __grid_constant__ Batch batch) {

@@ -72,6 +72,11 @@ bool fused_fp16(const orthdion_plan* p) {
     return p->engine == ORTHDION_ENGINE_TENSOR && p->passes[2] == 1 && p->passes[3] == 1;
 }
 
+// Image planes of Q that a step reads: the fused pass's, and for the diagnostics the bf16 terms.
+int q_planes(const orthdion_plan* p) { return (fused_fp16(p) ? 4 : 3) | (p->diag ? 3 : 0); }
+// Whether R's bf16 terms are read: by the right QR, or by the fused pass.
+bool right_image(const orthdion_plan* p) { return p->mode == ORTHDION_MODE_ORTH || !fused_fp16(p); }
+
 // matrices: of the whole call.  lean: no partial results in memory beyond those that a product cannot do without.
 // The same chunks are then added up in tensor memory or tile by tile: the same bits, longer launches for a few
 // matrices.  A lean layout never needs more than the plan's images and fixed slots.
@@ -418,7 +423,7 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
     a.dst = sel(which ? W_Q : W_P);
     if (which) {
         // the fused pass reads R and Q (the diagnostics Q's bf16 terms)
-        a.img = ts.q; a.img_planes = (fp16 ? 4 : 3) | (p->diag ? 3 : 0);
+        a.img = ts.q; a.img_planes = q_planes(p);
         a.copy_r = splits > 1; a.r_dst = slot; a.r_img = ts.r; a.r_planes = fp16 ? 4 : 3; a.rscale_off = ts.rscale;
     } else {
         a.img = ts.p; a.img_planes = fp16 ? 7 : 3;
@@ -558,7 +563,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const orthdion_plan* p = c.p;
         const int gb = p->g_dtype == ORTHDION_DTYPE_BF16;
         if (c.tensor()) tensor_k3(p->m, p->n, p->r, gb, p->passes[0], *c.b, c.sc.ts, sel(W_SCRATCH, c.sc.gram_part), st,
-                                  small_qr(p, p->n) ? OUT_F32 : OUT_IMAGE);
+                                  small_qr(p, p->n) ? OUT_F32 : right_image(p) ? OUT_IMAGE : OUT_NORM);
         else launch_simt(*c.b, p->n, p->r, p->m, RdBuffer{p->n, gb, 1}, RdPlain{sP, 1, p->r},
                          SimtOut{sR, sR, 0, 0, p->r, 0, 0}, prof::S_K3, st);
     }
@@ -571,9 +576,13 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
             small_qr_stage(c, 1, c.sc.ts.r_parts, call_matrices, st);
             continue;
         }
-        launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b, p->n,
-               p->r, c.tensor() ? c.sc.ts.cnorm : (int64_t)-1, 0);
-        if (c.tensor()) launch_pack(*c.b, sQ, p->n, p->r, c.sc.ts.q, st);
+        if (c.tensor()) {
+            launch_colsum(*c.b, c.sc.ts, p->n, p->r, sel(W_SCRATCH, c.sc.ts.cnorm), 1, prof::S_COLNORM, st);
+            launch_pack_right(*c.b, p->n, p->r, c.sc.ts, fused_fp16(p), q_planes(p), st);
+        } else {
+            launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b,
+                   p->n, p->r);
+        }
     }
     // Alg. 1, update and error-feedback steps:  M <- a B - b P R^T ;  X <- c X - d P Q^T
     for (ClassRun& c : cls) {
@@ -582,7 +591,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const float cc = 1.f - p->eta * p->wd, dd = p->eta * p->scale;
         if (c.tensor()) {
             const int fp16 = fused_fp16(p) ? 1 : 0;
-            if (fp16 && !small_qr(p, p->n)) launch_pack_half(*c.b, p->n, p->r, c.sc.ts, st);
+            if (fp16 && !small_qr(p, p->n) && p->mode == ORTHDION_MODE_ORTH) launch_pack_right(*c.b, p->n, p->r, c.sc.ts, true, 0, st);
             tensor_k5(p->m, p->n, p->r, gb, xb, p->passes[2], p->passes[3], fp16, p->ef_a, p->ef_b, cc, dd, *c.b,
                       c.sc.ts, st);
         } else {
@@ -867,8 +876,7 @@ void shard_gram(ShardRun& sr, const ImgRef& src, int64_t rows, cudaStream_t st) 
     const orthdion_plan* p = sr.c.p;
     const Sel gram = sel(W_SCRATCH, sr.c.sc.gram);
     tensor_gram(p->r, p->passes[1], sr.batch, src, rows, gram, sel(W_SCRATCH, sr.c.sc.gram_part), sr.c.sc.ts.gram_parts_n, 0, st);
-    launch(gram_diag_kernel, dim3((unsigned)((p->r + 255) / 256)), 256, 0, 1, prof::S_MISC, st, sr.batch, gram, p->r, sr.c.sc.ts.colsq,
-           (int)(4 * ((rows + 127) / 128)));
+    launch_colsum(sr.batch, sr.c.sc.ts, rows, p->r, gram, p->r + 1, prof::S_MISC, st);
 }
 
 void shard_fused_pass(ShardRun& sr, cudaStream_t st) {
@@ -876,7 +884,7 @@ void shard_fused_pass(ShardRun& sr, cudaStream_t st) {
     const int gb = p->g_dtype == ORTHDION_DTYPE_BF16, xb = p->x_dtype == ORTHDION_DTYPE_BF16;
     const float cc = 1.f - p->eta * p->wd, dd = p->eta * p->scale;
     const int fp16 = fused_fp16(p) ? 1 : 0;
-    if (fp16) launch_pack_half(sr.batch, p->n, p->r, sr.c.sc.ts, st);
+    if (fp16 && p->mode == ORTHDION_MODE_ORTH) launch_pack_right(sr.batch, p->n, p->r, sr.c.sc.ts, true, 0, st);
     tensor_k5(p->m, p->n, p->r, gb, xb, p->passes[2], p->passes[3], fp16, p->ef_a, p->ef_b, cc, dd, sr.batch,
               sr.c.sc.ts, st);
 }
@@ -911,11 +919,12 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
                    st, sr->batch, sel(W_P), p->m, r, ts.colsq);
         }
         qr_stage(cls, only, 0, merged, 1, st, true);
-        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st, OUT_IMAGE);
+        tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st,
+                  right_image(p) ? OUT_IMAGE : OUT_NORM);
         if (orth) {
             shard_gram(*sr, ts.r, p->n, st);
         } else {
-            launch(colnorm_kernel, dim3((unsigned)((r + 31) / 32)), 1024, 0, 1, prof::S_COLNORM, st, sr->batch, p->n, r, ts.cnorm, 1);
+            launch_colsum(sr->batch, ts, p->n, r, sel(W_SCRATCH, ts.cnorm), 1, prof::S_COLNORM, st);
         }
     } else if (phase == 2 && orth) {
         chol_stage(cls, only, 1, 1, merged, 1, st, true);
@@ -925,8 +934,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
         tensor_apply(r, p->passes[1], sr->batch, ts, ts.r, p->n, out, false, st);
         shard_gram(*sr, img_view(ts.w1, p->n), p->n, st);
     } else if (phase == 2) {
-        launch(colnorm_kernel, dim3((unsigned)((r + 31) / 32)), 1024, 0, 1, prof::S_COLNORM, st, sr->batch, p->n, r, ts.cnorm, 2);
-        launch_pack(sr->batch, sel(W_Q), p->n, r, ts.q, st);
+        launch_pack_right(sr->batch, p->n, r, ts, fused_fp16(p), q_planes(p), st);
         shard_fused_pass(*sr, st);
     } else {
         chol_stage(cls, only, 1, 2, merged, 1, st, true);

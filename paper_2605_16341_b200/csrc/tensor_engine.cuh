@@ -369,63 +369,87 @@ pack_kernel(const __grid_constant__ Batch batch, PackArgs a) {
         const int o = rho * 128 + img_chunk_offset(rho, c);
         *reinterpret_cast<uint4*>(out0 + o) = t0;
         *reinterpret_cast<uint4*>(out1 + o) = t1;
-        if (a.dst.planes == 3)
-            *reinterpret_cast<uint4*>(reinterpret_cast<unsigned char*>(w.scratch) +
-                                      img_row_offset(a.dst, 2, panel, (int64_t)rb * 128) + o) = half8(v, 1.f);
     }
 }
 
-// fp16 plane of R for the single-pass fused feedback/update product.  R is scaled by the power of
-// two that brings its largest column norm to about 2^10 (no entry can then overflow fp16, and
-// typical entries stay far from the subnormal range); the inverse scale is left at `rscale_off`
-// for the epilogue.  cnorm holds the squared column norms of R (written by the Cholesky of the
-// right QR, or by ColNorm).  One CTA per (panel, 128-row block), 256 threads.
-struct PackHalfArgs {
+// Power of two that brings the largest of `cols` squared column norms (cn) to a norm of about 2^10, for the fp16 plane of R
+// in the single-pass fused feedback/update product (no entry can then overflow fp16, and typical entries stay far from the
+// subnormal range); its inverse is left at *inverse, if there is such a place.  Called by 256 threads.
+__device__ __forceinline__ float half_scale(const float* cn, int cols, float* inverse) {
+    __shared__ float red[8];
+    float mx = 0.f;
+    for (int j = threadIdx.x; j < cols; j += 256) mx = fmaxf(mx, cn[j]);
+    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = mx;
+    __syncthreads();
+    mx = red[0];
+#pragma unroll
+    for (int i = 1; i < 8; ++i) mx = fmaxf(mx, red[i]);
+    int e = 0;
+    const float nrm = sqrtf(mx);
+    if (nrm > 0.f && nrm <= 3.0e38f) frexpf(nrm, &e);      // nrm = f * 2^e, 0.5 <= f < 1
+    if (inverse && threadIdx.x == 0) *inverse = ldexpf(1.f, e - 10);
+    return ldexpf(1.f, 10 - e);
+}
+
+// The fp16 plane of R; with `normalise` also column-normalised Dion's Q = R / column norms, fp32 and image planes, in the
+// same pass over R (before: a normalisation that read R twice with one CTA per 32 columns, a pack of Q and one of R; the
+// stages of a 1.1B model at r = 128 0.50 -> 0.24 ms, its step 7.23 -> 6.92; one 4096 x 4096 matrix at r = 256 0.314 -> 0.283).  cnorm holds the squared column norms of R.  One CTA
+// per (panel, 128-row block), 256 threads.
+struct PackRightArgs {
     int32_t rows, cols;
-    ImgRef dst;
+    ImgRef r_img, q_img;
+    int32_t r_half;           // write R's fp16 plane
+    int32_t normalise;        // bit mask of Q's image planes (1 | 2 bf16 terms, 4 fp16), 0: Q is not asked for
     int64_t cnorm_off, rscale_off;
 };
 
 __global__ void __launch_bounds__(256)
-pack_half_kernel(const __grid_constant__ Batch batch, PackHalfArgs a) {
+pack_right_kernel(const __grid_constant__ Batch batch, PackRightArgs a) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
-    __shared__ float red[8];
-    __shared__ float s_scale;
-    const float* cn = reinterpret_cast<const float*>(w.scratch + a.cnorm_off);
-    float mx = 0.f;
-    for (int j = threadIdx.x; j < a.cols; j += 256) mx = fmaxf(mx, cn[j]);
-    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (threadIdx.x % 32 == 0) red[threadIdx.x / 32] = mx;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int i = 1; i < 8; ++i) mx = fmaxf(mx, red[i]);
-        int e = 0;
-        const float nrm = sqrtf(mx);
-        if (nrm > 0.f && nrm <= 3.0e38f) frexpf(nrm, &e);      // nrm = f * 2^e, 0.5 <= f < 1
-        const float scale = ldexpf(1.f, 10 - e);
-        s_scale = scale;
-        if (blockIdx.x == 0 && blockIdx.y == 0)
-            *reinterpret_cast<float*>(w.scratch + a.rscale_off) = ldexpf(1.f, e - 10);
-    }
-    __syncthreads();
-    const float scale = s_scale;
     const int panel = blockIdx.x, rb = blockIdx.y;
-    unsigned char* out = reinterpret_cast<unsigned char*>(w.scratch) + img_row_offset(a.dst, 2, panel, (int64_t)rb * 128);
+    const float* cn = reinterpret_cast<const float*>(w.scratch + a.cnorm_off);
+    float scale = 1.f;
+    if (a.r_half) scale = half_scale(cn, a.cols, panel == 0 && rb == 0 ? reinterpret_cast<float*>(w.scratch + a.rscale_off) : nullptr);
+    unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
+    const int c = threadIdx.x % 8;
+    const int64_t gk = (int64_t)panel * 64 + c * 8;
+    float inv[8] = {};
+    if (a.normalise && gk < a.cols) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float nrm = sqrtf(cn[gk + i]);
+            if (!(nrm > 0.f) && rb == 0 && threadIdx.x < 8) atomicOr(w.status, ST_ZEROCOL);
+            inv[i] = nrm > 0.f ? 1.f / nrm : 0.f;
+        }
+    }
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
-        const int q = threadIdx.x + 256 * e;
-        const int rho = q / 8, c = q % 8;
-        const int64_t gr = (int64_t)rb * 128 + rho, gk = (int64_t)panel * 64 + c * 8;
-        float v[8];
-        if (gr < a.rows && gk < a.cols) {
-            load8(w.R, gr * a.cols + gk, 0, v);
-        } else {
+        const int rho = threadIdx.x / 8 + 32 * e;
+        const int64_t gr = (int64_t)rb * 128 + rho;
+        const int o = img_chunk_offset(rho, c);
+        float v[8] = {};
+        const bool in = gr < a.rows && gk < a.cols;
+        if (in) load8(w.R, gr * a.cols + gk, 0, v);
+        if (a.r_half) *reinterpret_cast<uint4*>(scr + img_row_offset(a.r_img, 2, panel, gr) + o) = half8(v, scale);
+        if (a.normalise) {
 #pragma unroll
-            for (int i = 0; i < 8; ++i) v[i] = 0.f;
+            for (int i = 0; i < 8; ++i) v[i] *= inv[i];
+            if (in) {
+                float4* q = reinterpret_cast<float4*>(w.Q + gr * a.cols + gk);
+                q[0] = make_float4(v[0], v[1], v[2], v[3]);
+                q[1] = make_float4(v[4], v[5], v[6], v[7]);
+            }
+            if (a.normalise & 3) {
+                uint4 t0, t1;
+                split8(v, t0, t1);
+                *reinterpret_cast<uint4*>(scr + img_row_offset(a.q_img, 0, panel, gr) + o) = t0;
+                *reinterpret_cast<uint4*>(scr + img_row_offset(a.q_img, 1, panel, gr) + o) = t1;
+            }
+            if (a.normalise & 4) *reinterpret_cast<uint4*>(scr + img_row_offset(a.q_img, 2, panel, gr) + o) = half8(v, 1.f);
         }
-        *reinterpret_cast<uint4*>(out + rho * 128 + img_chunk_offset(rho, c)) = half8(v, scale);
     }
 }
 
@@ -889,7 +913,8 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 // of 512 columns leave no second accumulator, and the tensor core waits for this (19 % of the first
                 // product and 33 % of the second at r = 512, before).  First and second product: six layers of
                 // 2048-wide matrices, r = 192 0.772 -> 0.699 and 0.768 -> 0.700 ms, r = 512 0.873 -> 0.870 and 1.044 -> 0.933; 24 layers of 768-wide ones, r = 192 0.407 -> 0.385 and 0.472 -> 0.417.
-                // One rolled loop for all products: in launches of a tile or two its code is fetched as it is run.
+                // One rolled loop for all products: in launches of a tile or two its code is fetched as it is run.  (Image products in
+                // unrolled blocks of 64 columns on four warps: 12000 of the 21000 cycles of a one-tile apply.)
                 unsigned char* stg = staging + (warp - 2) * STORE_STAGING_BYTES;
                 const int64_t gi0 = (int64_t)c.mt * BM + quarter * 32;
                 // (pairs: the CTA whose rows lie beyond the matrix stores nothing)
@@ -1637,11 +1662,18 @@ inline cudaError_t tensor_engine_set_attributes() {
     return cudaSuccess;
 }
 
-inline void launch_pack_half(const Batch& b, int64_t rows, int64_t cols, const TensorScratch& ts, cudaStream_t st) {
-    tc::PackHalfArgs a{};
-    a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.dst = ts.r; a.cnorm_off = ts.cnorm; a.rscale_off = ts.rscale;
+// half: R's fp16 plane; normalise: image planes of Q = R / column norms (0: Q comes from elsewhere)
+inline void launch_pack_right(const Batch& b, int64_t rows, int64_t cols, const TensorScratch& ts, bool half, int normalise, cudaStream_t st) {
+    tc::PackRightArgs a{};
+    a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.r_img = ts.r; a.q_img = ts.q; a.r_half = half ? 1 : 0; a.normalise = normalise;
+    a.cnorm_off = ts.cnorm; a.rscale_off = ts.rscale;
     dim3 grid((unsigned)ts.r.panels, (unsigned)(ts.r.rows_pad / 128), (unsigned)b.count);
-    launch(tc::pack_half_kernel, grid, 256, 0, 1, prof::S_PACK, st, b, a);
+    launch(tc::pack_right_kernel, grid, 256, 0, 1, normalise ? prof::S_COLNORM : prof::S_PACK, st, b, a);
+}
+// the column squares of `rows` rows, added up
+inline void launch_colsum(const Batch& b, const TensorScratch& ts, int64_t rows, int r, Sel dst, int64_t stride, int stage, cudaStream_t st) {
+    launch(colsum_kernel, dim3((unsigned)((r + 63) / 64), 1, (unsigned)b.count), 256, 0, 1, stage, st, b, ts.colsq,
+           (int)(4 * ((rows + 127) / 128)), r, dst, stride);
 }
 
 inline void launch_pack(const Batch& b, Sel src, int64_t rows, int64_t cols, ImgRef dst, cudaStream_t st, bool init = false) {
@@ -1887,12 +1919,14 @@ finish_split_kernel(const __grid_constant__ Batch batch, FinishArgs a) {
         D[0] = make_float4(v[0], v[1], v[2], v[3]);
         D[1] = make_float4(v[4], v[5], v[6], v[7]);
     }
-    uint4 t0, t1;
-    split8(v, t0, t1);
-    unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
-    const int o = img_chunk_offset(rho, c);
-    *reinterpret_cast<uint4*>(scr + img_row_offset(a.img, 0, panel, row) + o) = t0;
-    *reinterpret_cast<uint4*>(scr + img_row_offset(a.img, 1, panel, row) + o) = t1;
+    if (a.to_img) {
+        uint4 t0, t1;
+        split8(v, t0, t1);
+        unsigned char* scr = reinterpret_cast<unsigned char*>(w.scratch);
+        const int o = img_chunk_offset(rho, c);
+        *reinterpret_cast<uint4*>(scr + img_row_offset(a.img, 0, panel, row) + o) = t0;
+        *reinterpret_cast<uint4*>(scr + img_row_offset(a.img, 1, panel, row) + o) = t1;
+    }
 #pragma unroll
     for (int i = 0; i < 8; ++i) sq[rho][c * 8 + i] = __fmul_rn(v[i], v[i]);
     __syncthreads();
@@ -1908,10 +1942,10 @@ finish_split_kernel(const __grid_constant__ Batch batch, FinishArgs a) {
         reinterpret_cast<float*>(w.scratch + a.colsq_off)[(int64_t)blockIdx.y * a.r + panel * 64 + threadIdx.x] = s[0];
     }
 }
-inline void finish_split_product(const Batch& b, Sel dst, Sel part, int64_t rows, int r, int ksplit, ImgRef img,
+inline void finish_split_product(const Batch& b, Sel dst, Sel part, int64_t rows, int r, int ksplit, ImgRef img, bool to_img,
                                  int64_t colsq_off, int stage, cudaStream_t st) {
     FinishArgs a{};
-    a.dst = dst; a.part = part; a.rows = rows; a.r = r; a.ksplit = ksplit; a.img = img; a.colsq_off = colsq_off;
+    a.dst = dst; a.part = part; a.rows = rows; a.r = r; a.ksplit = ksplit; a.img = img; a.colsq_off = colsq_off; a.to_img = to_img ? 1 : 0;
     launch(finish_split_kernel, dim3((unsigned)img.panels, (unsigned)(img.rows_pad / 32), (unsigned)b.count), 256, 0, 1, stage, st, b, a);
 }
 
@@ -1919,7 +1953,8 @@ inline void finish_split_product(const Batch& b, Sel dst, Sel part, int64_t rows
 enum ProductOut : int {
     OUT_IMAGE = 0,     // operand image and column squares (and the fp32 R slot)
     OUT_F32 = 1,       // fp32 slot, or partial results of a depth split, for the small-rank QR kernel
-    OUT_SUM = 2        // fp32 slot only: one shard of the columns, to be summed over the shards
+    OUT_SUM = 2,       // fp32 slot only: one shard of the columns, to be summed over the shards
+    OUT_NORM = 3       // fp32 slot and column squares, for the column normalisation
 };
 // Y = (M + G) Q_prev  -> image w0 (+ column squares)              (Alg. 1, buffer and left-factor steps)
 // First kernel of a step: its packing of Q_prev also clears the status words.
@@ -1942,7 +1977,7 @@ inline void tensor_k1(int64_t m, int64_t n, int r, int g_bf16, int passes, const
     else launch_gemm<tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_K1, st);
     // (a sum in parts goes through the fp32 P slot, which holds nothing yet at this point of a step)
     if (ksplit > 1 && kind == OUT_IMAGE)
-        finish_split_product(b, Sel{W_P, 0, 0}, part, m, r, ksplit, img_view(ts.w0, m), ts.colsq, prof::S_K1, st);
+        finish_split_product(b, Sel{W_P, 0, 0}, part, m, r, ksplit, img_view(ts.w0, m), true, ts.colsq, prof::S_K1, st);
 }
 
 // R = (M + G)^T P  -> fp32 R slot, image r (+ column squares)     (Alg. 1, right-factor step)
@@ -1958,13 +1993,14 @@ inline void tensor_k3(int64_t m, int64_t n, int r, int g_bf16, int passes, const
     if (ksplit > 1) { g.out.normal.f32 = part; g.split_stride = n * r; }
     else {
         g.out.normal.f32 = Sel{W_R, 0, 0};
-        if (kind == OUT_IMAGE) { g.out.normal.img = ts.r; g.out.normal.colsq = 1; }
+        if (kind == OUT_IMAGE) g.out.normal.img = ts.r;
+        if (kind != OUT_F32) g.out.normal.colsq = 1;
     }
     g.out.shifted = g.out.normal; g.out.ld = r;
     if (g_bf16) launch_gemm<tc::A_BUF_COL, tc::N_IMG_MN, tc::EPI_STORE, 1>(b, g, prof::S_K3, st);
     else launch_gemm<tc::A_BUF_COL, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_K3, st);
-    if (ksplit > 1 && kind == OUT_IMAGE)
-        finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, ts.colsq, prof::S_K3, st);
+    if (ksplit > 1 && kind != OUT_F32)
+        finish_split_product(b, Sel{W_R, 0, 0}, part, n, r, ksplit, ts.r, kind == OUT_IMAGE, ts.colsq, prof::S_K3, st);
 }
 
 // Columns per tile of a product between images (`copies`: matrices times depth chunks).  256 columns, in CTA pairs
@@ -2086,7 +2122,7 @@ inline void tensor_apply(int r, int passes, const Batch& b, const TensorScratch&
 
 // M <- a (M + G) - b P R^T ;  X <- c X - d P Q^T                  (Alg. 1, update and error-feedback steps)
 // fp16 = 1: both products run as one fp16 pass from the fp16 planes of P, R, Q (R's plane must
-// have been written by launch_pack_half).
+// have been written by launch_pack_right).
 inline void tensor_k5(int64_t m, int64_t n, int r, int g_bf16, int x_bf16, int passes_m, int passes_x, int fp16,
                       float ef_a, float ef_b, float wc, float wd, const Batch& b, const TensorScratch& ts,
                       cudaStream_t st) {
