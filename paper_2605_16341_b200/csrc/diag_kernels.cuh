@@ -160,8 +160,8 @@ __device__ __forceinline__ float diag_block_sum(float v, float* red) {
     __syncthreads();                       // red may still be read from the previous call
     if (lane == 0) red[warp] = v;
     __syncthreads();
-    float t = 0.f;
-    for (int k = 0; k < DIAG_THREADS / 32; ++k) t += red[k];
+    float t = red[lane];
+    for (int o = 16; o; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
     return t;
 }
 
@@ -239,9 +239,17 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
     }
     ent = diag_block_sum(ent, red);
 
-    // mirror the lower triangle
-    for (int i = warp; i < r; i += DIAG_THREADS / 32)
-        for (int j = i + 1 + lane; j < r; j += 32) g[(int64_t)i * r + j] = g[(int64_t)j * r + i];
+    // mirror the lower triangle: rows of it are read, a warp takes every 32nd; eight loads go out before the stores that may
+    // alias them
+    for (int j = warp; j < r; j += DIAG_THREADS / 32)
+        for (int i0 = lane; i0 < j; i0 += 256) {
+            float x[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) x[e] = i0 + 32 * e < j ? g[(int64_t)j * r + i0 + 32 * e] : 0.f;
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (i0 + 32 * e < j) g[(int64_t)(i0 + 32 * e) * r + j] = x[e];
+        }
     for (int j = tid; j < r; j += DIAG_THREADS) g[(int64_t)j * r + j] = qsq[j];
     float nrm2 = 0.f;
     for (int j = tid; j < r; j += DIAG_THREADS) {
@@ -259,20 +267,37 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
     bool done = false;
     while (!done) {
         // y = G v - beta_j v_prev ;  alpha = <y, v>
-        for (int i = warp; i < r; i += DIAG_THREADS / 32) {
-            const float* row = g + (int64_t)i * r;
-            float acc = 0.f;
-            if (r % 4 == 0) {
+        if (r % 4 == 0) {
+            // four rows of a warp side by side: what bounds the product is the latency of its loads from L2
+            for (int i0 = warp; i0 < r; i0 += 4 * (DIAG_THREADS / 32)) {
+                float acc[4] = {};
                 for (int j = lane * 4; j < r; j += 128) {
-                    const float4 gv = *reinterpret_cast<const float4*>(row + j);
                     const float4 vv = *reinterpret_cast<const float4*>(v + j);
-                    acc = fmaf(gv.x, vv.x, fmaf(gv.y, vv.y, fmaf(gv.z, vv.z, fmaf(gv.w, vv.w, acc))));
+                    float4 gv[4];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int i = i0 + e * (DIAG_THREADS / 32);
+                        gv[e] = i < r ? *reinterpret_cast<const float4*>(g + (int64_t)i * r + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e)
+                        acc[e] = fmaf(gv[e].x, vv.x, fmaf(gv[e].y, vv.y, fmaf(gv[e].z, vv.z, fmaf(gv[e].w, vv.w, acc[e]))));
                 }
-            } else {
-                for (int j = lane; j < r; j += 32) acc = fmaf(row[j], v[j], acc);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    for (int o = 16; o; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+                    const int i = i0 + e * (DIAG_THREADS / 32);
+                    if (lane == 0 && i < r) y[i] = acc[e] - beta_j * vp[i];
+                }
             }
-            for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-            if (lane == 0) y[i] = acc - beta_j * vp[i];
+        } else {
+            for (int i = warp; i < r; i += DIAG_THREADS / 32) {
+                const float* row = g + (int64_t)i * r;
+                float acc = 0.f;
+                for (int j = lane; j < r; j += 32) acc = fmaf(row[j], v[j], acc);
+                for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0) y[i] = acc - beta_j * vp[i];
+            }
         }
         __syncthreads();
         float a = 0.f;
