@@ -38,8 +38,9 @@ constexpr int A_RING_BYTES = 4 * A_TERM_BYTES;   // two slots of two terms, or f
 constexpr int MAX_A_SLOTS = 4;
 constexpr int MAX_N_SLOTS = 6;
 constexpr int NUM_XF_WARPS = 16;             // transform warps of the kernels that form B = M + G
-constexpr int STAGING_BYTES_PER_WARP = 8192; // epilogue staging of the fused pass: M, G, X slabs per warp
-constexpr int STORE_STAGING_BYTES = 4096;      // of all products: one 32 x 32 fp32 block per warp
+constexpr int STORE_STAGING_BYTES = 4096;    // epilogue staging of the products: one 32 x 32 fp32 block per warp
+// ... of the fused pass: 32 x 32 slabs of M, G and X per warp (xg bit 0: G is bf16, bit 1: X is)
+__host__ __device__ constexpr int slab_bytes(int xg) { return 4096 + ((xg & 1) ? 2048 : 4096) + ((xg & 2) ? 2048 : 4096); }
 constexpr int SMEM_LIMIT = 227 * 1024;
 constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // about two seconds
 
@@ -80,6 +81,7 @@ struct GemmArgs {
     int32_t passes, passes2;                 // 1 or 3; passes2: second product of the fused pass
     int32_t ks;                              // N_IMG_MN: depth of one N-side piece (16, 32 or 64)
     int32_t n_slots, n_piece_bytes;          // N ring
+    int32_t n_split;                         // fused pass: the R piece and the Q piece of a depth block in slots of their own
     int32_t acc_bufs;                        // accumulator buffers in tensor memory (1 or 2)
     int32_t tmem_cols;                       // allocation (power of two >= 32)
     int32_t fp16;                            // single-pass fp16 products from plane 2 of the images
@@ -464,6 +466,8 @@ struct StatusCache { int b = -1; int st = 0; };
 // Pair launches (g.pair): a scheduled row tile is 256 rows, CTA `rank` of the pair owns its
 // rows 128 * rank .. ; c.mt stays the 128-row tile index (it may lie one past the last tile when
 // the number of tiles is odd: that CTA multiplies zeros and stores nothing).
+template <bool V> struct BoolConst { static constexpr bool value = V; };
+
 template <int EPI>
 __device__ __forceinline__ TileCoord decode_tile(const Batch& batch, const GemmArgs& g, int t, StatusCache& sc,
                                                  int rank) {
@@ -512,13 +516,6 @@ __device__ __forceinline__ int mn_pieces(const GemmArgs& g, int kb) {
 //        EPI_K5     M <- a (M+G) - b D1,  X <- c X - d D2     (Alg. 1, update and error-feedback steps), D1 = P R^T, D2 = P Q^T
 // XG     bit 0: G is bf16, bit 1: X is bf16
 // ------------------------------------------------------------------------------------------
-template <int XG>
-struct K5Pre {      // M, G, X of one 32 x 32 slab: 8 steps of (4 rows x 32 columns) per warp
-    float4 m[8];
-    uint32_t g[8][(XG & 1) ? 2 : 4];
-    uint32_t x[8][(XG & 2) ? 2 : 4];
-};
-
 // RUN    the tiles come in runs (GemmArgs::run): the Gram product, and products with B that have more chunks than
 //        accumulators.  (Instantiations of their own for the latter: the test for a run alone cost the other
 //        products with B up to 1 % of a step, in registers that the transform warps then lack.)
@@ -546,7 +543,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     unsigned char* a_ring = smem;
     unsigned char* n_ring = smem + g.a_slots * g.a_slot_bytes;
     unsigned char* staging = n_ring + (size_t)g.n_slots * g.n_piece_bytes;
-    unsigned char* tail = staging + NE * (EPI == EPI_STORE ? STORE_STAGING_BYTES : g.epi_bufs * STAGING_BYTES_PER_WARP);
+    unsigned char* tail = staging + NE * (EPI == EPI_STORE ? STORE_STAGING_BYTES : g.epi_bufs * slab_bytes(XG));
     uint64_t* bars = reinterpret_cast<uint64_t*>(tail);
     const uint32_t a_full0 = smem_u32(bars), a_empty0 = a_full0 + 8 * MAX_A_SLOTS;
     const uint32_t n_full0 = a_empty0 + 8 * MAX_A_SLOTS, n_empty0 = n_full0 + 8 * MAX_N_SLOTS;
@@ -629,7 +626,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     at = next(at); akb = -1;
                 }
             };
-            auto n_pieces = [&](int kb) { return NMODE == N_IMG_MN ? mn_pieces(g, kb) : (nc.bn + 127) / 128; };
+            auto n_pieces = [&](int kb) { return NMODE == N_IMG_MN ? mn_pieces(g, kb) : g.n_split ? 2 : 1; };
             auto n_seek = [&]() {           // make (nt_, nkb, npc) valid or finish
                 while (!n_done) {
                     if (nt_ >= g.total_tiles) { n_done = true; break; }
@@ -676,17 +673,19 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                                 tma_load_box_pair(dst + blk * blk_bytes, &g.map_n1, nkb * BK + npc * g.ks,
                                                   nc.n0 / 64 + blk * 4 + crank * 2, plane, nc.b, fb);
                         } else {
-                            tma_load_box_pair(dst, crank == 0 ? &g.map_n1 : &g.map_n2, nc.n0 + npc * 128, nkb, plane,
-                                              nc.b, fb);
+                            tma_load_box_pair(dst, crank == 0 ? &g.map_n1 : &g.map_n2, nc.n0, nkb, plane, nc.b, fb);
                         }
                     } else {
-                        mbar_arrive_expect_tx(fb, (uint32_t)g.n_piece_bytes);
                         if (NMODE == N_IMG_MN) {
+                            mbar_arrive_expect_tx(fb, (uint32_t)g.n_piece_bytes);
                             tma_load_box(dst, &g.map_n1, nkb * BK + npc * g.ks, nc.n0 / 64, plane, nc.b, fb);
+                        } else if (g.n_split) {
+                            mbar_arrive_expect_tx(fb, (uint32_t)((npc == 0 ? n1_terms : g.passes2 == 3 ? 2 : 1) * A_TERM_BYTES));
+                            tma_load_box(dst, npc == 0 ? &g.map_n1 : &g.map_n2, nc.n0, nkb, plane, nc.b, fb);
                         } else {
-                            tma_load_box(dst, &g.map_n1, nc.n0 + npc * 128, nkb, plane, nc.b, fb);
-                            if (EPI == EPI_K5)
-                                tma_load_box(dst + n1_terms * A_TERM_BYTES, &g.map_n2, nc.n0 + npc * 128, nkb, plane, nc.b, fb);
+                            mbar_arrive_expect_tx(fb, (uint32_t)g.n_piece_bytes);
+                            tma_load_box(dst, &g.map_n1, nc.n0, nkb, plane, nc.b, fb);
+                            tma_load_box(dst + n1_terms * A_TERM_BYTES, &g.map_n2, nc.n0, nkb, plane, nc.b, fb);
                         }
                     }
                     if (++ns == g.n_slots) { ns = 0; nph ^= 1; }
@@ -796,7 +795,8 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         int acc = 0; uint32_t acc_phase = 0;
         bool ok = true;
         // descriptor high parts (layout, strides) and address units of 16 bytes
-        const uint64_t op_hi = smem_desc(0, 16, 1024);
+        const uint64_t op_desc = smem_desc(0, 16, 1024);
+        const uint32_t op_lo = (uint32_t)op_desc, op_hi = (uint32_t)(op_desc >> 32);
         const uint32_t slice16 = 32u >> 4;               // one 16-deep slice of either operand
         const uint32_t a_ring16 = smem_u32(a_ring) >> 4, n_ring16 = smem_u32(n_ring) >> 4;
         const uint32_t a_slot16 = (uint32_t)g.a_slot_bytes >> 4, n_slot16 = (uint32_t)g.n_piece_bytes >> 4;
@@ -809,57 +809,55 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
             const uint32_t dacc = tmem_base + acc * acc_stride;
             for (int kb = c.kb_begin; kb < c.kb_end && ok; ++kb) {
                 if (!mbar_wait(a_full0 + 8 * as, aph, abort_flag)) { ok = false; break; }
-                const int chunks = (c.bn + 127) / 128;
                 const int nsl = min(4, (g.Kdim - kb * BK + 15) / 16);
-                for (int ch = 0; ch < chunks && ok; ++ch) {
+                // N of the instruction must be a multiple of 16: round a ragged last tile up
+                // (rows beyond the matrix are zero in the images; those columns of D are never stored)
+                const uint32_t ncols = (uint32_t)((c.bn + 15) / 16 * 16);
+                const uint32_t accum = kb > c.kb_begin ? 1u : 0u;
+                for (int pc = 0; pc < (g.n_split ? 2 : 1) && ok; ++pc) {
                     if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
                     if (lane == 0) {
-                        const uint32_t sa = smem_u32(a_ring + as * g.a_slot_bytes);
-                        const uint32_t sn = smem_u32(n_ring + (size_t)ns * g.n_piece_bytes);
-                        // N of the instruction must be a multiple of 16: round a ragged last chunk up
-                        // (rows beyond the matrix are zero in the images; those columns of D are never stored)
-                        const uint32_t ncols = (uint32_t)((min(128, c.bn - ch * 128) + 15) / 16 * 16);
-                        const uint32_t idesc = instr_desc(ncols, 0u, 0u, fmt, MROWS);
-                        // Fused pass with single-term operands: the R piece and the Q piece lie back
-                        // to back in the slot (256 rows of one K-major tile) and their accumulators in
-                        // adjacent columns, so one N = 256 instruction serves both products and reads
-                        // the P slice from shared memory once.
-                        const bool both = g.passes == 1 && g.passes2 == 1 && ncols == 128 && g.BN == 128;
-                        const uint32_t idesc2 = instr_desc(256u, 0u, 0u, fmt, MROWS);
-                        if (both) {
-                            // one instruction per 16-deep slice; descriptors advanced by additions so
-                            // that the issuing thread spends a handful of operations per instruction
-                            uint64_t a0 = op_hi + (a_ring16 + as * a_slot16);
-                            uint64_t b0 = op_hi + (n_ring16 + ns * n_slot16);
-                            const uint32_t d1 = dacc + ch * 128;
-                            umma_any<PAIR>(d1, a0, b0, idesc2, kb > c.kb_begin ? 1u : 0u);
-                            for (int j = 1; j < nsl; ++j) {
-                                a0 += slice16; b0 += slice16;
-                                umma_any<PAIR>(d1, a0, b0, idesc2, 1u);
+                        const uint32_t a0 = (uint32_t)op_lo + a_ring16 + as * a_slot16, b0 = (uint32_t)op_lo + n_ring16 + ns * n_slot16;
+                        if (g.passes == 1 && g.passes2 == 1) {
+                            // Single-term operands: the R piece and the Q piece lie back
+                            // to back in the slot (256 rows of one K-major tile) and their accumulators in
+                            // adjacent columns, so one N = 256 instruction serves both products and reads
+                            // the P slice from shared memory once (two of them on a ragged last tile).
+                            if (ncols == 128) {
+                                const uint32_t idesc = instr_desc(256u, 0u, 0u, fmt, MROWS);
+                                for (int j = 0; j < nsl; ++j)
+                                    umma_slices<PAIR, 1, false>(dacc, a0 + j * slice16, op_hi, b0 + j * slice16, op_hi, 0, 0, 0, 0, idesc, j ? 1u : accum);
+                            } else {
+                                const uint32_t idesc = instr_desc(ncols, 0u, 0u, fmt, MROWS);
+                                for (int j = 0; j < nsl; ++j) {
+                                    umma_slices<PAIR, 1, false>(dacc, a0 + j * slice16, op_hi, b0 + j * slice16, op_hi, 0, 0, 0, 0, idesc, j ? 1u : accum);
+                                    umma_slices<PAIR, 1, false>(dacc + g.BN, a0 + j * slice16, op_hi, b0 + (A_TERM_BYTES >> 4) + j * slice16, op_hi, 0, 0, 0, 0,
+                                                                idesc, j ? 1u : accum);
+                                }
                             }
-                        }
-                        // (In the general form below the descriptors are rebuilt per instruction on
-                        // purpose: its N = 128 instructions ran best when not issued back to back.)
-                        for (int j = 0; j < nsl && !both; ++j) {
-                            const uint64_t a0 = smem_desc(sa + j * 32, 16, 1024);
-                            const uint64_t a1 = smem_desc(sa + A_TERM_BYTES + j * 32, 16, 1024);
-                            const uint64_t b0 = smem_desc(sn + j * 32, 16, 1024);
-                            const uint64_t b1 = smem_desc(sn + A_TERM_BYTES + j * 32, 16, 1024);
-                            const uint32_t accum = (kb > c.kb_begin || j > 0) ? 1u : 0u;
-                            const uint32_t d1 = dacc + ch * 128;
-                            umma_any<PAIR>(d1, a0, b0, idesc, accum);
-                            if (g.passes == 3) {
-                                umma_any<PAIR>(d1, a0, b1, idesc, 1u);
-                                umma_any<PAIR>(d1, a1, b0, idesc, 1u);
-                            }
-                            const uint32_t s2 = sn + n1_terms * A_TERM_BYTES;
-                            const uint64_t c0 = smem_desc(s2 + j * 32, 16, 1024);
-                            const uint64_t c1 = smem_desc(s2 + A_TERM_BYTES + j * 32, 16, 1024);
-                            const uint32_t d2 = dacc + g.BN;
-                            umma_any<PAIR>(d2, a0, c0, idesc, accum);
-                            if (g.passes2 == 3) {
-                                umma_any<PAIR>(d2, a0, c1, idesc, 1u);
-                                umma_any<PAIR>(d2, a1, c0, idesc, 1u);
+                        } else {
+                            // (never a pair) split terms: the slot holds those of R and Q, or of one of them.  In straight lines: the
+                            // issuer bounds this form (28 matrices 2048 wide at r = 256 with three passes for M, step with descriptors
+                            // rebuilt in a loop over products 2.04, now 1.95 ms).
+                            const uint32_t idesc = instr_desc(ncols, 0u, 0u, fmt, MROWS);
+                            constexpr uint32_t term = A_TERM_BYTES >> 4;
+                            auto product = [&](uint32_t d, uint32_t b, bool three) {
+                                if (nsl == 4) {
+                                    if (three) umma_slices<PAIR, 4, true>(d, a0, op_hi, b, op_hi, slice16, slice16, term, term, idesc, accum);
+                                    else umma_slices<PAIR, 4, false>(d, a0, op_hi, b, op_hi, slice16, slice16, 0, 0, idesc, accum);
+                                    return;
+                                }
+                                for (int j = 0; j < nsl; ++j) {
+                                    const uint32_t aj = a0 + j * slice16, bj = b + j * slice16, acc_j = j ? 1u : accum;
+                                    if (three) umma_slices<PAIR, 1, true>(d, aj, op_hi, bj, op_hi, 0, 0, term, term, idesc, acc_j);
+                                    else umma_slices<PAIR, 1, false>(d, aj, op_hi, bj, op_hi, 0, 0, 0, 0, idesc, acc_j);
+                                }
+                            };
+                            if (!g.n_split) {
+                                product(dacc, b0, g.passes == 3);
+                                product(dacc + g.BN, b0 + n1_terms * term, g.passes2 == 3);
+                            } else {
+                                product(dacc + pc * g.BN, b0, (pc ? g.passes2 : g.passes) == 3);
                             }
                         }
                         commit_any<PAIR>(n_empty0 + 8 * ns);
@@ -1090,198 +1088,69 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
             // accumulator slabs go through a swizzled staging block so that global accesses run
             // along rows (8 lanes x 16 bytes per row).
             const int half = (warp - 2) / 4;
-            if constexpr (XG == 3) {
-                // bf16 G and X.  The 32 x 32 slabs of M, G, X come in by asynchronous copies
-                // (cp.async, no registers) into a per-warp buffer, one or two slabs ahead; each
-                // lane then updates its own row in place (accumulators stay in the layout tensor
-                // memory gives: one row per lane), and the buffer goes out along rows.
-                //   buffer: M 32 x 128 B | G 32 x 64 B | X 32 x 64 B, 16-byte chunks swizzled so that
-                //   both the row-per-lane and the 8-(or 4-)lanes-per-row accesses avoid bank conflicts
-                const int nbuf = g.epi_bufs;
-                unsigned char* bufs = staging + (size_t)(warp - 2) * nbuf * STAGING_BYTES_PER_WARP;
-                const int mrow = lane / 8, mch = lane % 8;      // M: 4 rows x 8 chunks per step
-                const int hrow = lane / 4, hch = lane % 4;      // G, X: 8 rows x 4 chunks per step
-                auto m_off = [](int r, int ch) { return r * 128 + ((ch ^ (r & 7)) << 4); };
-                auto h_off = [](int r, int ch) { return r * 64 + ((ch ^ ((r >> 1) & 3)) << 4); };
-                // the same for this lane's chunk of step `it` (rows 4 it + mrow and 8 it + hrow)
-                const int m_off0 = m_off(mrow, mch), h_off0 = h_off(hrow, hch);
-                auto m_step = [&](int it) { return (m_off0 ^ ((it & 1) << 6)) + it * 512; };
-                auto h_step = [&](int it) { return h_off0 + it * 512; };
-                // The slabs of this warp in order: (tile, 0), (tile, 1), (next tile, 0), ...  A warp has little time
-                // per slab (14 KB, 8 warps: at the rate of the memory about 4800 cycles), and most of what it executed
-                // was addresses: a tile is decoded once now, rows are reached by additions.  11008 x 4096 at
-                // r = 32 / 256 0.123 / 0.132 -> 0.118 / 0.122 ms, six layers of 2048-wide matrices 0.840 / 0.866 -> 0.798 / 0.792.
-                struct Slab { int t, slab, b, i0, j0; };
-                auto advance = [&](Slab& s) {
-                    if (s.slab == 0) { s.slab = 1; s.j0 += 32; return; }
-                    for (s.t += tstride; s.t < g.total_tiles; s.t += tstride) {
-                        const TileCoord c = decode_tile<EPI>(batch, g, s.t, scache, crank);
-                        if (!c.active) continue;
-                        s.slab = 0; s.b = c.b; s.i0 = c.mt * BM + quarter * 32; s.j0 = c.n0 + half * 64;
-                        return;
-                    }
-                };
-                const int64_t ld = g.ld;
-                auto issue = [&](const Slab& s, unsigned char* buf) {
-                    const MatWork& w = batch.w[s.b];
-                    const uint32_t sb = smem_u32(buf);
-                    const float* Mp = w.M + (s.i0 + mrow) * ld + s.j0 + mch * 4;
-                    const int mleft = s.j0 + mch * 4 < g.Ncols ? g.Mrows - s.i0 - mrow : 0;
-#pragma unroll
-                    for (int it = 0; it < 8; ++it)
-                        if (it * 4 < mleft) cp_async16(sb + m_step(it), Mp + it * 4 * ld);
-                    const int64_t hidx = (s.i0 + hrow) * ld + s.j0 + hch * 8;
-                    const __nv_bfloat16* Gp = reinterpret_cast<const __nv_bfloat16*>(w.G) + hidx;
-                    const __nv_bfloat16* Xp = reinterpret_cast<const __nv_bfloat16*>(w.X) + hidx;
-                    const int hleft = s.j0 + hch * 8 < g.Ncols ? g.Mrows - s.i0 - hrow : 0;
-#pragma unroll
-                    for (int it = 0; it < 4; ++it)
-                        if (it * 8 < hleft) {
-                            cp_async16(sb + 4096 + h_step(it), Gp + it * 8 * ld);
-                            cp_async16(sb + 6144 + h_step(it), Xp + it * 8 * ld);
-                        }
-                    cp_async_commit();
-                };
-                auto process = [&](const Slab& s, unsigned char* buf) -> bool {
-                    const MatWork& w = batch.w[s.b];
-                    const int slab = s.slab;
-                    const float efb = g.fp16 ? g.ef_b * *reinterpret_cast<const float*>(w.scratch + g.rscale_off) : g.ef_b;
-                    if (slab == 0) {
-                        if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) return false;
-                        tc_fence_after();
-                    }
-                    const uint32_t taddr = tmem_base + acc * acc_stride + ((uint32_t)(quarter * 32) << 16) +
-                                           (uint32_t)(half * 64 + slab * 32);
-#pragma unroll
-                    for (int hh = 0; hh < 2; ++hh) {
-                        uint32_t va[16], vc[16];
-                        tmem_ld16(taddr + hh * 16, va);
-                        tmem_ld16(taddr + g.BN + hh * 16, vc);
-                        tmem_ld_wait();
-                        uint4 gq[2], xq[2];
-#pragma unroll
-                        for (int k = 0; k < 2; ++k) {
-                            gq[k] = *reinterpret_cast<const uint4*>(buf + 4096 + h_off(lane, hh * 2 + k));
-                            xq[k] = *reinterpret_cast<const uint4*>(buf + 6144 + h_off(lane, hh * 2 + k));
-                        }
-                        const uint32_t gw[8] = {gq[0].x, gq[0].y, gq[0].z, gq[0].w, gq[1].x, gq[1].y, gq[1].z, gq[1].w};
-                        const uint32_t xw[8] = {xq[0].x, xq[0].y, xq[0].z, xq[0].w, xq[1].x, xq[1].y, xq[1].z, xq[1].w};
-                        uint32_t xo[8];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            float4* mp = reinterpret_cast<float4*>(buf + m_off(lane, hh * 4 + k));
-                            const float4 mv = *mp;
-                            const float mvv[4] = {mv.x, mv.y, mv.z, mv.w};
-                            float mo[4], xf[4];
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int i = 4 * k + e;
-                                const uint32_t gp = gw[i / 2], xp = xw[i / 2];
-                                const float gval = (i & 1) ? bf16hi_to_f32(gp) : bf16lo_to_f32(gp);
-                                const float xval = (i & 1) ? bf16hi_to_f32(xp) : bf16lo_to_f32(xp);
-                                const float bval = mvv[e] + gval;
-                                mo[e] = g.ef_a * bval - efb * __uint_as_float(va[i]);
-                                xf[e] = g.wc * xval - g.wd * __uint_as_float(vc[i]);
-                            }
-                            *mp = make_float4(mo[0], mo[1], mo[2], mo[3]);
-                            xo[2 * k] = pack_bf16x2(xf[0], xf[1]);
-                            xo[2 * k + 1] = pack_bf16x2(xf[2], xf[3]);
-                        }
-#pragma unroll
-                        for (int k = 0; k < 2; ++k)
-                            *reinterpret_cast<uint4*>(buf + 6144 + h_off(lane, hh * 2 + k)) =
-                                make_uint4(xo[4 * k], xo[4 * k + 1], xo[4 * k + 2], xo[4 * k + 3]);
-                    }
-                    if (slab == 1) {
-                        // the accumulators of this tile are in registers / shared memory now
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) { if (PAIR) mbar_arrive_remote(tempty_ld + 8 * acc); else mbar_arrive(tempty0 + 8 * acc); }
-                        if (++acc == g.acc_bufs) { acc = 0; acc_phase ^= 1; }
-                    }
-                    __syncwarp();
-                    float* Mp = w.M + (s.i0 + mrow) * ld + s.j0 + mch * 4;
-                    const int mleft = s.j0 + mch * 4 < g.Ncols ? g.Mrows - s.i0 - mrow : 0;
-#pragma unroll
-                    for (int it = 0; it < 8; ++it)
-                        if (it * 4 < mleft)
-                            *reinterpret_cast<float4*>(Mp + it * 4 * ld) = *reinterpret_cast<const float4*>(buf + m_step(it));
-                    __nv_bfloat16* Xp = reinterpret_cast<__nv_bfloat16*>(w.X) + (s.i0 + hrow) * ld + s.j0 + hch * 8;
-                    const int hleft = s.j0 + hch * 8 < g.Ncols ? g.Mrows - s.i0 - hrow : 0;
-#pragma unroll
-                    for (int it = 0; it < 4; ++it)
-                        if (it * 8 < hleft)
-                            *reinterpret_cast<uint4*>(Xp + it * 8 * ld) = *reinterpret_cast<const uint4*>(buf + 6144 + h_step(it));
-                    __syncwarp();
-                    return true;
-                };
-                Slab cur{tile0 - tstride, 1, 0, 0, 0};
-                int ib = 0;
-                advance(cur);
-                if (cur.t < g.total_tiles) issue(cur, bufs);
-                while (cur.t < g.total_tiles) {
-                    Slab nxt = cur;
-                    advance(nxt);
-                    if (nbuf == 2) {
-                        if (nxt.t < g.total_tiles) issue(nxt, bufs + (ib ^ 1) * STAGING_BYTES_PER_WARP);
-                        else cp_async_commit();
-                        cp_async_wait<1>();
-                    } else {
-                        cp_async_wait<0>();
-                    }
-                    __syncwarp();
-                    if (!process(cur, bufs + ib * STAGING_BYTES_PER_WARP)) break;
-                    if (nbuf == 2) ib ^= 1;
-                    else if (nxt.t < g.total_tiles) issue(nxt, bufs);
-                    cur = nxt;
-                }
-                cp_async_wait<0>();
-            } else {
-            auto next_tile = [&](int t) {
-                for (t += tstride; t < g.total_tiles; t += tstride)
-                    if (decode_tile<EPI>(batch, g, t, scache, crank).active) return t;
-                return g.total_tiles;
-            };
-            // the slabs of this warp in order: (tile, 0), (tile, 1), (next tile, 0), ...
-            auto advance = [&](int& t, int& slab) {
-                if (++slab == 2) { slab = 0; t = next_tile(t); }
-            };
-            unsigned char* S1 = staging + (warp - 2) * STAGING_BYTES_PER_WARP;
-            unsigned char* S2 = S1 + 4096;
-            const int rl = lane / 8, cq = lane % 8;      // row within a step, 4-column group
-
-            auto fetch = [&](K5Pre<XG>& p, int t, int slab) {
-                const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
-                const MatWork& w = batch.w[c.b];
-                const int64_t gj = (int64_t)c.n0 + half * 64 + slab * 32 + cq * 4;
-#pragma unroll
-                for (int it = 0; it < 8; ++it) {
-                    const int64_t gi = (int64_t)c.mt * BM + quarter * 32 + it * 4 + rl;
-                    if (gi < g.Mrows && gj < g.Ncols) {
-                        const int64_t idx = gi * g.ld + gj;
-                        p.m[it] = *reinterpret_cast<const float4*>(w.M + idx);
-                        if constexpr (G_BF16) {
-                            const uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(w.G) + idx);
-                            p.g[it][0] = u.x; p.g[it][1] = u.y;
-                        } else {
-                            const uint4 u = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(w.G) + idx);
-                            p.g[it][0] = u.x; p.g[it][1] = u.y; p.g[it][2] = u.z; p.g[it][3] = u.w;
-                        }
-                        if constexpr (X_BF16) {
-                            const uint2 u = *reinterpret_cast<const uint2*>(reinterpret_cast<const __nv_bfloat16*>(w.X) + idx);
-                            p.x[it][0] = u.x; p.x[it][1] = u.y;
-                        } else {
-                            const uint4 u = *reinterpret_cast<const uint4*>(reinterpret_cast<const float*>(w.X) + idx);
-                            p.x[it][0] = u.x; p.x[it][1] = u.y; p.x[it][2] = u.z; p.x[it][3] = u.w;
-                        }
-                    }
+            // The 32 x 32 slabs of M, G, X come in by asynchronous copies (cp.async, no registers) into a per-warp buffer,
+            // one or two slabs ahead; each
+            // lane then updates its own row in place (accumulators stay in the layout tensor
+            // memory gives: one row per lane), and the buffer goes out along rows.
+            //   buffer: M | G | X, rows of 128 bytes (fp32) or 64 (bf16), 16-byte chunks swizzled so that
+            //   both the row-per-lane and the 8-(or 4-)lanes-per-row accesses avoid bank conflicts
+            // (fp32 G or X were fetched into registers, when the slab before was done, and a depth block's operands had one
+            // slot.  Step before -> now: 28 matrices 2048 wide, Dion, fp32 X and G, r = 64 1.83 -> 1.50 ms, fp32 X r = 256 2.32 -> 2.19; one
+            // 4096 x 4096 matrix r = 128, fp32 X and G 0.399 -> 0.364, fp32 G 0.386 -> 0.359.)
+            constexpr int SLAB = slab_bytes(XG), G_AT = 4096, X_AT = G_AT + (G_BF16 ? 2048 : 4096);
+            const int nbuf = g.epi_bufs;
+            unsigned char* bufs = staging + (size_t)(warp - 2) * nbuf * SLAB;
+            const int mrow = lane / 8, mch = lane % 8;      // fp32: 4 rows x 8 chunks per step
+            const int hrow = lane / 4, hch = lane % 4;      // bf16: 8 rows x 4 chunks per step
+            auto m_off = [](int r, int ch) { return r * 128 + ((ch ^ (r & 7)) << 4); };
+            auto h_off = [](int r, int ch) { return r * 64 + ((ch ^ ((r >> 1) & 3)) << 4); };
+            // the same for this lane's chunk of step `it` (rows 4 it + mrow and 8 it + hrow)
+            const int m_off0 = m_off(mrow, mch), h_off0 = h_off(hrow, hch);
+            auto m_step = [&](int it) { return (m_off0 ^ ((it & 1) << 6)) + it * 512; };
+            auto h_step = [&](int it) { return h_off0 + it * 512; };
+            // The slabs of this warp in order: (tile, 0), (tile, 1), (next tile, 0), ...  A warp has little time
+            // per slab (14 KB, 8 warps: at the rate of the memory about 4800 cycles), and most of what it executed
+            // was addresses: a tile is decoded once now, rows are reached by additions.  11008 x 4096 at
+            // r = 32 / 256 0.123 / 0.132 -> 0.118 / 0.122 ms, six layers of 2048-wide matrices 0.840 / 0.866 -> 0.798 / 0.792.
+            struct Slab { int t, slab, b, i0, j0; };
+            auto advance = [&](Slab& s) {
+                if (s.slab == 0) { s.slab = 1; s.j0 += 32; return; }
+                for (s.t += tstride; s.t < g.total_tiles; s.t += tstride) {
+                    const TileCoord c = decode_tile<EPI>(batch, g, s.t, scache, crank);
+                    if (!c.active) continue;
+                    s.slab = 0; s.b = c.b; s.i0 = c.mt * BM + quarter * 32; s.j0 = c.n0 + half * 64;
+                    return;
                 }
             };
-
-            // one slab: accumulators -> staging -> row-wise update of M and X
-            auto process = [&](const K5Pre<XG>& cur, int t, int slab) -> bool {
-                const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
-                const MatWork& w = batch.w[c.b];
+            const int64_t ld = g.ld;
+            // rows of the slab from this lane's first one on, if its columns are inside
+            auto m_left = [&](const Slab& s) { return s.j0 + mch * 4 < g.Ncols ? g.Mrows - s.i0 - mrow : 0; };
+            auto h_left = [&](const Slab& s) { return s.j0 + hch * 8 < g.Ncols ? g.Mrows - s.i0 - hrow : 0; };
+            auto issue = [&](const Slab& s, unsigned char* buf) {
+                const MatWork& w = batch.w[s.b];
+                const uint32_t sb = smem_u32(buf);
+                const int64_t midx = (s.i0 + mrow) * ld + s.j0 + mch * 4, hidx = (s.i0 + hrow) * ld + s.j0 + hch * 8;
+                const int mleft = m_left(s), hleft = h_left(s);
+                auto copy32 = [&](int at, const void* base) {
+                    const float* p = reinterpret_cast<const float*>(base) + midx;
+#pragma unroll
+                    for (int it = 0; it < 8; ++it)
+                        if (it * 4 < mleft) cp_async16(sb + at + m_step(it), p + it * 4 * ld);
+                };
+                auto copy16 = [&](int at, const void* base) {
+                    const __nv_bfloat16* p = reinterpret_cast<const __nv_bfloat16*>(base) + hidx;
+#pragma unroll
+                    for (int it = 0; it < 4; ++it)
+                        if (it * 8 < hleft) cp_async16(sb + at + h_step(it), p + it * 8 * ld);
+                };
+                copy32(0, w.M);
+                if constexpr (G_BF16) copy16(G_AT, w.G); else copy32(G_AT, w.G);
+                if constexpr (X_BF16) copy16(X_AT, w.X); else copy32(X_AT, w.X);
+                cp_async_commit();
+            };
+            auto process = [&](const Slab& s, unsigned char* buf) -> bool {
+                const MatWork& w = batch.w[s.b];
+                const int slab = s.slab;
                 const float efb = g.fp16 ? g.ef_b * *reinterpret_cast<const float*>(w.scratch + g.rscale_off) : g.ef_b;
                 if (slab == 0) {
                     if (!mbar_wait(tfull0 + 8 * acc, acc_phase, abort_flag)) return false;
@@ -1289,86 +1158,103 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 }
                 const uint32_t taddr = tmem_base + acc * acc_stride + ((uint32_t)(quarter * 32) << 16) +
                                        (uint32_t)(half * 64 + slab * 32);
-                {
-                    uint32_t va[16], vb[16], vc[16], vd[16];
-                    tmem_ld16(taddr, va);
-                    tmem_ld16(taddr + 16, vb);
-                    tmem_ld16(taddr + g.BN, vc);
-                    tmem_ld16(taddr + g.BN + 16, vd);
+#pragma unroll
+                for (int hh = 0; hh < 2; ++hh) {
+                    uint32_t va[16], vc[16];
+                    tmem_ld16(taddr + hh * 16, va);
+                    tmem_ld16(taddr + g.BN + hh * 16, vc);
                     tmem_ld_wait();
+                    // eight columns of this lane's row, from the slab at `at`
+                    auto read8 = [&](auto bf16, int at, int k, float (&f)[8]) {
+                        if constexpr (decltype(bf16)::value) {
+                            const uint4 u = *reinterpret_cast<const uint4*>(buf + at + h_off(lane, hh * 2 + k));
+                            const uint32_t p[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
-                    for (int ch = 0; ch < 4; ++ch) {
-                        const int o0 = lane * 128 + img_chunk_offset(lane, ch);
-                        const int o1 = lane * 128 + img_chunk_offset(lane, ch + 4);
-                        *reinterpret_cast<uint4*>(S1 + o0) = make_uint4(va[4 * ch], va[4 * ch + 1], va[4 * ch + 2], va[4 * ch + 3]);
-                        *reinterpret_cast<uint4*>(S1 + o1) = make_uint4(vb[4 * ch], vb[4 * ch + 1], vb[4 * ch + 2], vb[4 * ch + 3]);
-                        *reinterpret_cast<uint4*>(S2 + o0) = make_uint4(vc[4 * ch], vc[4 * ch + 1], vc[4 * ch + 2], vc[4 * ch + 3]);
-                        *reinterpret_cast<uint4*>(S2 + o1) = make_uint4(vd[4 * ch], vd[4 * ch + 1], vd[4 * ch + 2], vd[4 * ch + 3]);
-                    }
-                }
-                __syncwarp();
-                const int64_t gj = (int64_t)c.n0 + half * 64 + slab * 32 + cq * 4;
-#pragma unroll
-                for (int it = 0; it < 8; ++it) {
-                    const int r = it * 4 + rl;
-                    const int64_t gi = (int64_t)c.mt * BM + quarter * 32 + r;
-                    const int o = r * 128 + img_chunk_offset(r, cq);
-                    const float4 d1 = *reinterpret_cast<const float4*>(S1 + o);
-                    const float4 d2 = *reinterpret_cast<const float4*>(S2 + o);
-                    if (gi < g.Mrows && gj < g.Ncols) {
-                        const int64_t idx = gi * g.ld + gj;
-                        float gv[4], xv[4];
-                        if constexpr (G_BF16) {
-                            gv[0] = bf16lo_to_f32(cur.g[it][0]); gv[1] = bf16hi_to_f32(cur.g[it][0]);
-                            gv[2] = bf16lo_to_f32(cur.g[it][1]); gv[3] = bf16hi_to_f32(cur.g[it][1]);
+                            for (int i = 0; i < 4; ++i) { f[2 * i] = bf16lo_to_f32(p[i]); f[2 * i + 1] = bf16hi_to_f32(p[i]); }
                         } else {
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) gv[e] = __uint_as_float(cur.g[it][e]);
+                            for (int i = 0; i < 2; ++i) {
+                                const float4 u = *reinterpret_cast<const float4*>(buf + at + m_off(lane, hh * 4 + 2 * k + i));
+                                f[4 * i] = u.x; f[4 * i + 1] = u.y; f[4 * i + 2] = u.z; f[4 * i + 3] = u.w;
+                            }
                         }
-                        if constexpr (X_BF16) {
-                            xv[0] = bf16lo_to_f32(cur.x[it][0]); xv[1] = bf16hi_to_f32(cur.x[it][0]);
-                            xv[2] = bf16lo_to_f32(cur.x[it][1]); xv[3] = bf16hi_to_f32(cur.x[it][1]);
-                        } else {
+                    };
+                    auto write8 = [&](int at, int k, const float (&f)[8]) {
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) xv[e] = __uint_as_float(cur.x[it][e]);
-                        }
-                        const float mv[4] = {cur.m[it].x, cur.m[it].y, cur.m[it].z, cur.m[it].w};
-                        const float a1[4] = {d1.x, d1.y, d1.z, d1.w};
-                        const float a2[4] = {d2.x, d2.y, d2.z, d2.w};
-                        float mo[4], xo[4];
+                        for (int i = 0; i < 2; ++i)
+                            *reinterpret_cast<float4*>(buf + at + m_off(lane, hh * 4 + 2 * k + i)) =
+                                make_float4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
+                    };
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
+                    for (int k = 0; k < 2; ++k) {
+                        float mv[8], gv[8], xv[8];
+                        read8(BoolConst<false>(), 0, k, mv);
+                        read8(BoolConst<G_BF16>(), G_AT, k, gv);
+                        read8(BoolConst<X_BF16>(), X_AT, k, xv);
+#pragma unroll
+                        for (int e = 0; e < 8; ++e) {
                             const float bval = mv[e] + gv[e];
-                            mo[e] = g.ef_a * bval - efb * a1[e];
-                            xo[e] = g.wc * xv[e] - g.wd * a2[e];
+                            mv[e] = g.ef_a * bval - efb * __uint_as_float(va[8 * k + e]);
+                            xv[e] = g.wc * xv[e] - g.wd * __uint_as_float(vc[8 * k + e]);
                         }
-                        *reinterpret_cast<float4*>(w.M + idx) = make_float4(mo[0], mo[1], mo[2], mo[3]);
-                        if constexpr (X_BF16) {
-                            *reinterpret_cast<uint2*>(reinterpret_cast<__nv_bfloat16*>(w.X) + idx) =
-                                make_uint2(pack_bf16x2(xo[0], xo[1]), pack_bf16x2(xo[2], xo[3]));
-                        } else {
-                            *reinterpret_cast<float4*>(reinterpret_cast<float*>(w.X) + idx) =
-                                make_float4(xo[0], xo[1], xo[2], xo[3]);
-                        }
+                        write8(0, k, mv);
+                        if constexpr (X_BF16)
+                            *reinterpret_cast<uint4*>(buf + X_AT + h_off(lane, hh * 2 + k)) =
+                                make_uint4(pack_bf16x2(xv[0], xv[1]), pack_bf16x2(xv[2], xv[3]), pack_bf16x2(xv[4], xv[5]), pack_bf16x2(xv[6], xv[7]));
+                        else
+                            write8(X_AT, k, xv);
                     }
                 }
-                __syncwarp();
                 if (slab == 1) {
+                    // the accumulators of this tile are in registers / shared memory now
                     tc_fence_before();
                     __syncwarp();
                     if (lane == 0) { if (PAIR) mbar_arrive_remote(tempty_ld + 8 * acc); else mbar_arrive(tempty0 + 8 * acc); }
                     if (++acc == g.acc_bufs) { acc = 0; acc_phase ^= 1; }
                 }
+                __syncwarp();
+                const int64_t midx = (s.i0 + mrow) * ld + s.j0 + mch * 4, hidx = (s.i0 + hrow) * ld + s.j0 + hch * 8;
+                const int mleft = m_left(s), hleft = h_left(s);
+                auto store32 = [&](float* p, int at) {
+#pragma unroll
+                    for (int it = 0; it < 8; ++it)
+                        if (it * 4 < mleft)
+                            *reinterpret_cast<float4*>(p + it * 4 * ld) = *reinterpret_cast<const float4*>(buf + at + m_step(it));
+                };
+                store32(w.M + midx, 0);
+                if constexpr (X_BF16) {
+                    __nv_bfloat16* Xp = reinterpret_cast<__nv_bfloat16*>(w.X) + hidx;
+#pragma unroll
+                    for (int it = 0; it < 4; ++it)
+                        if (it * 8 < hleft)
+                            *reinterpret_cast<uint4*>(Xp + it * 8 * ld) = *reinterpret_cast<const uint4*>(buf + X_AT + h_step(it));
+                } else {
+                    store32(reinterpret_cast<float*>(w.X) + midx, X_AT);
+                }
+                __syncwarp();
                 return true;
             };
-            int t = next_tile(tile0 - tstride), slab = 0;
-            K5Pre<XG> pa;
-            while (t < g.total_tiles) {
-                fetch(pa, t, slab);
-                if (!process(pa, t, slab)) break;
-                advance(t, slab);
+            Slab cur{tile0 - tstride, 1, 0, 0, 0};
+            int ib = 0;
+            advance(cur);
+            if (cur.t < g.total_tiles) issue(cur, bufs);
+            while (cur.t < g.total_tiles) {
+                Slab nxt = cur;
+                advance(nxt);
+                if (nbuf == 2) {
+                    if (nxt.t < g.total_tiles) issue(nxt, bufs + (ib ^ 1) * SLAB);
+                    else cp_async_commit();
+                    cp_async_wait<1>();
+                } else {
+                    cp_async_wait<0>();
+                }
+                __syncwarp();
+                if (!process(cur, bufs + ib * SLAB)) break;
+                if (nbuf == 2) ib ^= 1;
+                else if (nxt.t < g.total_tiles) issue(nxt, bufs);
+                cur = nxt;
             }
-            }
+            cp_async_wait<0>();
         }
     } else if (A_BUF) {
         // ---------------- transform warps: A tile of B = M + G (Alg. 1, buffer step) ----------------
@@ -1739,7 +1625,13 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
         }
     } else {
         g.ks = 64;
-        g.n_piece_bytes = (n1_terms + (EPI == tc::EPI_K5 ? n2_terms : 0)) * tc::A_TERM_BYTES;
+        // The R and Q pieces of a depth block in one slot, or in slots of their own where not even two such slots fit (one:
+        // nothing is under way while the products run).  bf16 X and G with three passes for M only, two slots of 48 KB ->
+        // three of 32: 28 matrices 2048 wide at r = 256 1.93 -> 1.97 ms.
+        g.n_piece_bytes = (n1_terms + n2_terms) * tc::A_TERM_BYTES;
+        const int room = tc::SMEM_LIMIT - g.a_slots * g.a_slot_bytes - 8 * g.epi_bufs * tc::slab_bytes(XG) - 256 - 1024;
+        g.n_split = n1_terms + n2_terms > 2 && room < 2 * g.n_piece_bytes;
+        if (g.n_split) g.n_piece_bytes = 2 * tc::A_TERM_BYTES;
         if (pair) g.n_piece_bytes = tc::A_TERM_BYTES;    // the R piece (leader) or the Q piece (peer)
     }
     const int accw = (EPI == tc::EPI_K5) ? 2 * g.BN : g.acc_chunks * g.BN;
@@ -1759,11 +1651,8 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
         g.a_slots = 3;
         if (3 * (size_t)g.a_slot_bytes + 3 * (size_t)g.n_piece_bytes + 4 * tc::STORE_STAGING_BYTES + 2304 > 196 * 1024) g.a_slots = 2;
     }
-    // (the fused pass on other types than bf16 loads M, G and X into registers: the same line.  bf16 X and fp32 G, 4096 x 4096
-    // r = 128 0.079 -> 0.066 ms, r = 512 0.088 -> 0.075; fp32 X fits one slot either way)
-    if (EPI == tc::EPI_K5 && XG != 3) max_n_slots = 2;
     const size_t fixed = (size_t)g.a_slots * g.a_slot_bytes +
-                         (size_t)tc::epi_warps(AMODE, EPI) * (EPI == tc::EPI_STORE ? tc::STORE_STAGING_BYTES : g.epi_bufs * tc::STAGING_BYTES_PER_WARP) +
+                         (size_t)tc::epi_warps(AMODE, EPI) * (EPI == tc::EPI_STORE ? tc::STORE_STAGING_BYTES : g.epi_bufs * tc::slab_bytes(XG)) +
                          256 + 1024;
     g.n_slots = (int)std::min<size_t>(max_n_slots, (tc::SMEM_LIMIT - fixed) / (size_t)g.n_piece_bytes);
     // more than half of an SM's shared memory: one CTA per SM, whatever its tensor-memory share
