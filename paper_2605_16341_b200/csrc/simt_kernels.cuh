@@ -15,21 +15,40 @@
 
 namespace od {
 
-// ---- operand readers: value of the logical operand at (row i, depth k) ----------------------
+// ---- operand readers: values of the logical operand at (row i, depth k) ----------------------
+// fetch() sends eight loads out and waits for none; value() is what comes of them.  (With the sum of M and G formed element
+// by element as they were read, a 32-deep step of B Q_prev took 9500 cycles, one load after the other.)
 struct RdPlain {            // fp32 matrix with arbitrary strides: elem(i,k) = p[i*rs + k*cs]
     Sel sel; int64_t rs, cs;
+    struct Raw { float v[8]; };
     __device__ __forceinline__ bool depth_contiguous() const { return cs == 1; }
-    __device__ __forceinline__ float operator()(const MatWork& w, int64_t i, int64_t k) const {
-        return pick(w, sel)[i * rs + k * cs];
+    __device__ __forceinline__ void fetch(const MatWork& w, const int64_t (&i)[8], const int64_t (&k)[8], const bool (&in)[8], Raw& r) const {
+        const float* p = pick(w, sel);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) r.v[e] = in[e] ? p[i[e] * rs + k[e] * cs] : 0.f;
     }
+    __device__ __forceinline__ float value(const Raw& r, int e) const { return r.v[e]; }
 };
 struct RdBuffer {           // B = M + G formed on the fly (Alg. 1, buffer step); trans: elem(i,k)=B[k][i]
     int64_t ld; int32_t g_bf16; int32_t trans;
+    struct Raw { float m[8]; uint32_t g[8]; };
     __device__ __forceinline__ bool depth_contiguous() const { return !trans; }
-    __device__ __forceinline__ float operator()(const MatWork& w, int64_t i, int64_t k) const {
-        const int64_t idx = trans ? (k * ld + i) : (i * ld + k);
-        return w.M[idx] + load_elem(w.G, idx, g_bf16);
+    __device__ __forceinline__ void fetch(const MatWork& w, const int64_t (&i)[8], const int64_t (&k)[8], const bool (&in)[8], Raw& r) const {
+        int64_t idx[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            idx[e] = trans ? k[e] * ld + i[e] : i[e] * ld + k[e];
+            r.m[e] = in[e] ? w.M[idx[e]] : 0.f;
+        }
+        if (g_bf16) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) r.g[e] = in[e] ? (uint32_t)reinterpret_cast<const uint16_t*>(w.G)[idx[e]] << 16 : 0u;
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) r.g[e] = in[e] ? reinterpret_cast<const uint32_t*>(w.G)[idx[e]] : 0u;
+        }
     }
+    __device__ __forceinline__ float value(const Raw& r, int e) const { return r.m[e] + __uint_as_float(r.g[e]); }
 };
 
 struct SimtOut {            // C[i*ld + j] = acc ; destination may depend on the shift flag
@@ -64,23 +83,27 @@ __device__ __forceinline__ void simt_pos(bool depth_fast, int e, int& ii, int& k
 }
 template <class RD>
 __device__ __forceinline__ void simt_load(const RD& rd, const MatWork& w, int64_t i0, int64_t k0, int64_t rows, int64_t kend,
-                                          float (&v)[8]) {
+                                          typename RD::Raw& raw) {
     const bool fast = rd.depth_contiguous();
+    int64_t i[8], k[8];
+    bool in[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         int ii, kk;
         simt_pos(fast, e, ii, kk);
-        v[e] = (i0 + ii < rows && k0 + kk < kend) ? rd(w, i0 + ii, k0 + kk) : 0.f;
+        i[e] = i0 + ii; k[e] = k0 + kk;
+        in[e] = i[e] < rows && k[e] < kend;
     }
+    rd.fetch(w, i, k, in, raw);
 }
 template <class RD>
-__device__ __forceinline__ void simt_store(const RD& rd, SimtStage& s, const float (&v)[8]) {
+__device__ __forceinline__ void simt_store(const RD& rd, SimtStage& s, const typename RD::Raw& raw) {
     const bool fast = rd.depth_contiguous();
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
         int ii, kk;
         simt_pos(fast, e, ii, kk);
-        s[kk][ii] = v[e];
+        s[kk][ii] = rd.value(raw, e);
     }
 }
 __device__ __forceinline__ void simt_fma(float (&acc)[4][4], const SimtStage& a, const SimtStage& b, int ty, int tx) {
@@ -115,7 +138,8 @@ simt_gemm_kernel(const __grid_constant__ Batch batch, int64_t Md, int64_t Nd, in
     const int64_t per = (Kd + (int64_t)parts * SIMT_KC - 1) / ((int64_t)parts * SIMT_KC) * SIMT_KC;
     const int64_t kbeg = rank * per, kend = min(Kd, kbeg + per);
     float acc[4][4] = {};
-    float va[8], vb[8];
+    typename RA::Raw va;
+    typename RB::Raw vb;
     if (kbeg < kend) {
         simt_load(ra, w, i0, kbeg, Md, kend, va);
         simt_load(rb, w, j0, kbeg, Nd, kend, vb);
@@ -177,13 +201,17 @@ simt_update_kernel(const __grid_constant__ Batch batch, int64_t m, int64_t n, in
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
-    __shared__ SimtStage Ps, Rs, Qs;
+    // the operand steps, then the two products by rows (65 floats apart: both ways without bank conflicts)
+    __shared__ __align__(16) float buf[2 * 64 * 65];
+    static_assert(3 * SIMT_KC * SIMT_LD <= 2 * 64 * 65, "three operand steps fit");
+    SimtStage* st = reinterpret_cast<SimtStage*>(buf);
+    SimtStage &Ps = st[0], &Rs = st[1], &Qs = st[2];
     const int tid = threadIdx.x;
     const int tx = tid % 16, ty = tid / 16;
     const int64_t i0 = (int64_t)blockIdx.y * 64, j0 = (int64_t)blockIdx.x * 64;
     const RdPlain rp{Sel{W_P, 0, 0}, r, 1}, rr{Sel{W_R, 0, 0}, r, 1}, rq{Sel{W_Q, 0, 0}, r, 1};
     float accm[4][4] = {}, accx[4][4] = {};
-    float vp[8], vr[8], vq[8];
+    RdPlain::Raw vp, vr, vq;
     simt_load(rp, w, i0, 0, m, r, vp);
     simt_load(rr, w, j0, 0, n, r, vr);
     simt_load(rq, w, j0, 0, n, r, vq);
@@ -201,26 +229,49 @@ simt_update_kernel(const __grid_constant__ Batch batch, int64_t m, int64_t n, in
         simt_fma(accx, Ps, Qs, ty, tx);
         __syncthreads();
     }
+    float *dm = buf, *dx = buf + 64 * 65;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        // all reads of a row first: a load behind a store that may alias it would wait for the store
-        const int64_t gi = i0 + ty * 4 + e;
-        float bv[4], xv[4];
+    for (int e = 0; e < 4; ++e)
 #pragma unroll
         for (int f = 0; f < 4; ++f) {
-            const int64_t gj = j0 + tx * 4 + f, idx = gi * n + gj;
-            const bool in = gi < m && gj < n;
-            bv[f] = in ? w.M[idx] + load_elem(w.G, idx, g_bf16) : 0.f;
-            xv[f] = in ? load_elem(w.X, idx, x_bf16) : 0.f;
+            dm[(ty * 4 + e) * 65 + tx * 4 + f] = accm[e][f];
+            dx[(ty * 4 + e) * 65 + tx * 4 + f] = accx[e][f];
         }
+    __syncthreads();
+    // rows of the tile, lanes along them; eight elements of M, G and X under way (read where they were wanted, one after the
+    // other, this took most of 20 us for 1023 x 777)
+#pragma unroll 1
+    for (int h = 0; h < 2; ++h) {
+        float mv[8];
+        uint32_t gv[8], xv[8];
+        int64_t idx[8];
+        bool in[8];
 #pragma unroll
-        for (int f = 0; f < 4; ++f) {
-            const int64_t gj = j0 + tx * 4 + f, idx = gi * n + gj;
-            if (gi >= m || gj >= n) continue;
-            w.M[idx] = a * bv[f] - b * accm[e][f];
-            const float x = c * xv[f] - d * accx[e][f];
-            if (x_bf16) reinterpret_cast<__nv_bfloat16*>(w.X)[idx] = __float2bfloat16_rn(x);
-            else reinterpret_cast<float*>(w.X)[idx] = x;
+        for (int e = 0; e < 8; ++e) {
+            const int64_t gi = i0 + h * 32 + e * 4 + tid / 64, gj = j0 + tid % 64;
+            in[e] = gi < m && gj < n;
+            idx[e] = gi * n + gj;
+            mv[e] = in[e] ? w.M[idx[e]] : 0.f;
+        }
+        auto raw = [&](const void* p, int bf16, uint32_t (&v)[8]) {
+            if (bf16) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = in[e] ? (uint32_t)reinterpret_cast<const uint16_t*>(p)[idx[e]] << 16 : 0u;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = in[e] ? reinterpret_cast<const uint32_t*>(p)[idx[e]] : 0u;
+            }
+        };
+        raw(w.G, g_bf16, gv);
+        raw(w.X, x_bf16, xv);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int q = (h * 32 + e * 4 + tid / 64) * 65 + tid % 64;
+            if (!in[e]) continue;
+            w.M[idx[e]] = a * (mv[e] + __uint_as_float(gv[e])) - b * dm[q];
+            const float x = c * __uint_as_float(xv[e]) - d * dx[q];
+            if (x_bf16) reinterpret_cast<__nv_bfloat16*>(w.X)[idx[e]] = __float2bfloat16_rn(x);
+            else reinterpret_cast<float*>(w.X)[idx[e]] = x;
         }
     }
 }
