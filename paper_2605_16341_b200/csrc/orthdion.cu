@@ -219,6 +219,10 @@ int largest_cluster(K* kernel, int threads, size_t smem) {
     return 8;
 }
 
+// by rank (16, 32, 64) and threads (256, 512)
+void (*const kQrSmall[6])(Batch, QrSmallArgs) = {qr_small_kernel<16, 256>, qr_small_kernel<16, 512>, qr_small_kernel<32, 256>,
+                                                 qr_small_kernel<32, 512>, qr_small_kernel<64, 256>, qr_small_kernel<64, 512>};
+
 int ensure_attributes() {
     static std::mutex mu;
     static signed char state[kMaxDevices] = {};   // 0 unknown, 1 ok, -1 failed
@@ -230,17 +234,14 @@ int ensure_attributes() {
     cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM_BYTES);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(qr_small_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(qr_small_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(qr_small_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
+    g_qr_cluster_max[dev] = 16;
+    for (int k = 0; k < 6 && e == cudaSuccess; ++k) {
+        e = cudaFuncSetAttribute(kQrSmall[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
+        if (e == cudaSuccess)
+            g_qr_cluster_max[dev] = (signed char)std::min<int>(g_qr_cluster_max[dev], largest_cluster(kQrSmall[k], k % 2 ? 512 : 256, QS_SMEM_LIMIT));
+    }
     if (e == cudaSuccess) {
         g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel, CT_THREADS, CT_SMEM_BYTES);
-        g_qr_cluster_max[dev] = (signed char)std::min({largest_cluster(qr_small_kernel<16>, QS_THREADS, QS_SMEM_LIMIT),
-                                                       largest_cluster(qr_small_kernel<32>, QS_THREADS, QS_SMEM_LIMIT),
-                                                       largest_cluster(qr_small_kernel<64>, QS_THREADS, QS_SMEM_LIMIT)});
     }
     if (e == cudaSuccess) e = tensor_engine_set_attributes();
     if (e != cudaSuccess) {
@@ -383,7 +384,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
 
 // Whether the factor with `rows` rows is orthonormalised by the one-kernel QR (ranks up to 64).
 bool small_qr(const orthdion_plan* p, int64_t rows) {
-    return p->engine == ORTHDION_ENGINE_TENSOR && qs_fits(rows, p->r, cluster_max(g_qr_cluster_max));
+    return qs_fits(rows, p->r, cluster_max(g_qr_cluster_max), p->engine != ORTHDION_ENGINE_TENSOR);
 }
 
 // Whether the launches of a call's one chain overlap (programmatic dependent launch).  Not with several
@@ -415,23 +416,26 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
     a.src = splits > 1 ? sel(W_SCRATCH, c.sc.gram_part) : slot;
     a.splits = splits; a.split_stride = (int64_t)a.rows * p->r;
     const int cmax = cluster_max(g_qr_cluster_max), parts = qs_parts(a.rows, p->r, cmax);
-    a.csize = qs_ctas(a.rows, p->r, cmax, call_matrices, 2 * sm_count());
+    const int threads = qs_threads(a.rows, p->r, cmax, !c.tensor());
+    a.csize = qs_ctas(a.rows, p->r, cmax, call_matrices, 512 / threads * sm_count(), threads);
     a.parts_per_cta = parts / a.csize;
     a.rows_per_part = qs_rows_per_part(a.rows, parts);
     a.colnorm = which && p->mode == ORTHDION_MODE_COLNORM;
     a.shift_rel = kShiftRel; a.cond_limit = kCondLimit;      // fp32 arithmetic
     a.dst = sel(which ? W_Q : W_P);
-    if (which) {
+    if (!c.tensor()) {
+        a.img = a.r_img = no_img();        // the fp32 engine has no images
+    } else if (which) {
         // the fused pass reads R and Q (the diagnostics Q's bf16 terms)
         a.img = ts.q; a.img_planes = q_planes(p);
         a.copy_r = splits > 1; a.r_dst = slot; a.r_img = ts.r; a.r_planes = fp16 ? 4 : 3; a.rscale_off = ts.rscale;
     } else {
         a.img = ts.p; a.img_planes = fp16 ? 7 : 3;
     }
-    const size_t smem = (size_t)qs_smem((int64_t)a.rows_per_part * a.parts_per_cta, p->r);
+    const size_t smem = (size_t)qs_smem((int64_t)a.rows_per_part * a.parts_per_cta, p->r, threads);
     const int width = qs_width(p->r);
-    launch(width == 16 ? qr_small_kernel<16> : (width == 32 ? qr_small_kernel<32> : qr_small_kernel<64>),
-           dim3((unsigned)(c.b->count * a.csize)), QS_THREADS, smem, a.csize, prof::S_QR, st, *c.b, a);
+    launch(kQrSmall[(width == 16 ? 0 : width == 32 ? 2 : 4) + (threads == 512)], dim3((unsigned)(c.b->count * a.csize)), threads, smem, a.csize,
+           prof::S_QR, st, *c.b, a);
 }
 
 // ---- tall-skinny QR of every class in `which_cls` (CholeskyQR2; third pass when flagged) --------
@@ -445,7 +449,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
     for (int ci : wanted) {
         ClassRun& c = cls[ci];
         const int64_t rows = which ? c.p->n : c.p->m;
-        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed ? 1 : (which ? c.sc.ts.r_parts : c.sc.ts.y_parts), call_matrices, st);
+        if (small_qr(c.p, rows)) small_qr_stage(c, which, summed || !c.tensor() ? 1 : (which ? c.sc.ts.r_parts : c.sc.ts.y_parts), call_matrices, st);
         else which_cls.push_back(ci);
     }
     if (which_cls.empty()) return;
@@ -573,7 +577,7 @@ void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_
         const orthdion_plan* p = c.p;
         if (p->mode == ORTHDION_MODE_ORTH) continue;
         if (small_qr(p, p->n)) {
-            small_qr_stage(c, 1, c.sc.ts.r_parts, call_matrices, st);
+            small_qr_stage(c, 1, c.tensor() ? c.sc.ts.r_parts : 1, call_matrices, st);
             continue;
         }
         if (c.tensor()) {

@@ -1,4 +1,4 @@
-// QR of a tall-skinny factor at rank <= 64 in ONE kernel (tensor engine): one matrix per cluster, its rows
+// QR of a tall-skinny factor at rank <= 64 in ONE kernel (both engines): one matrix per cluster, its rows
 // dealt out over the CTAs and kept in shared memory.
 //
 //   load the rows (adding up the partial results of a depth-split product)
@@ -22,7 +22,6 @@
 
 namespace od {
 
-constexpr int QS_THREADS = 256;
 constexpr int QS_MAX_RANK = 64;
 constexpr int QS_MAX_ROWS_64 = 640;
 constexpr int QS_SMEM_LIMIT = 227 * 1024 - 256;      // less the static variables
@@ -47,7 +46,9 @@ struct QrSmallArgs {
 
 inline int qs_width(int r) { return r <= 16 ? 16 : (r <= 32 ? 32 : 64); }
 inline int qs_row_bytes(int r) { return 4 * (r <= 16 ? 20 : (r <= 32 ? 32 : 68)); }
-inline int qs_fixed(int r) { return CT_DG_BYTES + qs_width(r) * qs_width(r) * 4; }
+// partial Gram matrices of the thread groups, or a diagonal block
+__host__ __device__ constexpr int qs_part_bytes(int threads) { return 64 * threads > CT_DG_BYTES ? 64 * threads : CT_DG_BYTES; }
+inline int qs_fixed(int r, int threads) { return qs_part_bytes(threads) + qs_width(r) * qs_width(r) * 4; }
 
 // Parts of a factor: 4096 row entries each (64 rows at r = 64, 256 at r = 16) while that gives at most max_ctas.
 inline int qs_parts(int64_t rows, int r, int max_ctas) {
@@ -57,24 +58,32 @@ inline int qs_parts(int64_t rows, int r, int max_ctas) {
     return c;
 }
 inline int qs_rows_per_part(int64_t rows, int parts) { return (int)((rows + parts * 32 - 1) / (parts * 32) * 32); }
-inline int64_t qs_smem(int64_t rows_per_cta, int r) { return rows_per_cta * qs_row_bytes(r) + qs_fixed(r); }
+// Threads of a CTA, by the plan only (they decide how a Gram matrix is summed): 512, one CTA per multiprocessor, for parts
+// of 256 rows and more and for the fp32 engine above rank 32; else 256 and two.  Step with 256 and with 512 threads: 11008 x 4096 r = 32, Dion
+// 0.324 and 0.315 ms, 14336 x 4096 r = 16 0.365 and 0.361; 360 x 360 r = 32 0.0629 and 0.0640; 1023 x 777 r = 40, fp32 engine, 0.103 and
+// 0.099; 24 layers 640 wide at r = 64 1.21 and 1.28.
+inline int qs_threads(int64_t rows, int r, int max_ctas, bool fp32_engine) {
+    return r > 32 ? (fp32_engine ? 512 : 256) : (qs_rows_per_part(rows, qs_parts(rows, r, max_ctas)) >= 256 ? 512 : 256);
+}
+inline int64_t qs_smem(int64_t rows_per_cta, int r, int threads) { return rows_per_cta * qs_row_bytes(r) + qs_fixed(r, threads); }
 // Whether the kernel takes a rows x r factor.  From r = 33 up only short ones: the fp32 products and the repeated
 // factorisations cost a call with many matrices more than the separate tensor-core kernels do, and the choice cannot
 // depend on the call (a matrix gets the same bits alone and in a group).  Step with separate kernels and with this one
 // at r = 64: 512 x 512 one 0.204 and 0.106 ms, 72 of them 0.383 and 0.321; 640 x 640 one 0.214 and 0.101, 24 0.285 and
 // 0.189, 72 0.491 and 0.547; 768 x 768 one 0.220 and 0.100, 24 0.331 and 0.207, 72 0.556 and 0.612; 24 layers of a
 // 768-wide model (168 matrices) 1.39 and 1.61; 4096 x 4096 one 0.336 and 0.263.
-inline bool qs_fits(int64_t rows, int r, int max_ctas) {
-    if (r > QS_MAX_RANK || (r > 32 && rows > QS_MAX_ROWS_64)) return false;
+// The fp32 engine's separate kernels have no such side: it takes whatever shared memory holds.
+inline bool qs_fits(int64_t rows, int r, int max_ctas, bool fp32_engine) {
+    if (r > QS_MAX_RANK || (r > 32 && rows > QS_MAX_ROWS_64 && !fp32_engine)) return false;
     const int c = qs_parts(rows, r, max_ctas);
-    return qs_smem(qs_rows_per_part(rows, c), r) <= QS_SMEM_LIMIT;
+    return qs_smem(qs_rows_per_part(rows, c), r, qs_threads(rows, r, max_ctas, fp32_engine)) <= QS_SMEM_LIMIT;
 }
 // CTAs per matrix in a call of `matrices` on a device with room for `room` CTAs.
-inline int qs_ctas(int64_t rows, int r, int max_ctas, int matrices, int room) {
+inline int qs_ctas(int64_t rows, int r, int max_ctas, int matrices, int room, int threads) {
     const int parts = qs_parts(rows, r, max_ctas), per = qs_rows_per_part(rows, parts);
     const int max_run = r > 32 ? 4 : 16;            // (tree levels held in registers)
     int c = parts;
-    while (c > 1 && (int64_t)matrices * c > room && parts / c < max_run && qs_smem((int64_t)per * (2 * parts / c), r) <= QS_SMEM_LIMIT)
+    while (c > 1 && (int64_t)matrices * c > room && parts / c < max_run && qs_smem((int64_t)per * (2 * parts / c), r, threads) <= QS_SMEM_LIMIT)
         c /= 2;
     return c;
 }
@@ -88,22 +97,22 @@ __device__ __forceinline__ void qs_st_remote4(uint32_t addr, const float4& v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
-template <int R>
-__global__ void __launch_bounds__(QS_THREADS, 2)
+template <int R, int QS_THREADS>
+__global__ void __launch_bounds__(QS_THREADS, 512 / QS_THREADS)
 qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrSmallArgs a) {
     constexpr int LD = R == 32 ? 32 : R + 4;         // row stride: no bank conflicts in either product
     constexpr int TX = R / 4;                        // threads along the columns of a 4 x 4-blocked product
     constexpr int GROUPS = QS_THREADS / (TX * TX);   // Gram product: thread groups that share the rows
     constexpr int RT = QS_THREADS / TX * 4;          // apply product: rows of a step
-    constexpr int ENT = R == 64 ? 4 : 1;             // Gram entries (in fours) per thread
+    constexpr int ENT = R * R / 4 > QS_THREADS ? R * R / 4 / QS_THREADS : 1;             // Gram entries (in fours) per thread
     constexpr int LEVELS = R == 64 ? 3 : 5;
     extern __shared__ __align__(16) unsigned char smem[];
     float* sD = reinterpret_cast<float*>(smem);      // diagonal block's area; partial Gram matrices before it
     float* part = sD;
-    float* G = reinterpret_cast<float*>(smem + CT_DG_BYTES);     // Gram matrix, then L^{-T}
+    float* G = reinterpret_cast<float*>(smem + qs_part_bytes(QS_THREADS));     // Gram matrix, then L^{-T}
     float* Y = G + R * R;                            // this CTA's rows
     __shared__ float s_min, s_max, s_bound;
-    static_assert(GROUPS * R * R * 4 <= CT_DG_BYTES, "partial Gram matrices fit the diagonal block's area");
+    static_assert(GROUPS * R * R * 4 <= qs_part_bytes(QS_THREADS), "partial Gram matrices fit the diagonal block's area");
 
     grid_dependency();
     const int C = a.csize, crank = (int)(blockIdx.x % (unsigned)C);
@@ -124,19 +133,39 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
         const float* S = pick(w, a.src) + (int64_t)row0 * r;
         float* Rd = a.copy_r ? pick(w, a.r_dst) + (int64_t)row0 * r : nullptr;
         const int total = nrows * (R / 4);
-#pragma unroll 4
-        for (int q = tid; q < total; q += QS_THREADS) {
-            const int i = q / (R / 4), c = q % (R / 4);
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c < r4) {
-                v = *reinterpret_cast<const float4*>(S + i * r + c * 4);
-                for (int p = 1; p < a.splits; ++p) {
-                    const float4 u = *reinterpret_cast<const float4*>(S + p * a.split_stride + i * r + c * 4);
-                    v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+        if (r % 4) {                // (fp32 engine)
+            for (int q = tid; q < nrows * R; q += QS_THREADS) Y[q / R * LD + q % R] = q % R < r ? S[q / R * r + q % R] : 0.f;
+        } else {
+            // four chunks of four columns, two partial results of each under way (one after the other, 11008 rows at r = 32
+            // in five parts took 40 us)
+            for (int q0 = tid; q0 < total; q0 += 4 * QS_THREADS) {
+                float4 v[4];
+#pragma unroll 1
+                for (int p = 0; p < a.splits; p += 2) {
+                    float4 u[4][2];
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        const int q = q0 + e * QS_THREADS, i = q / (R / 4), c = q % (R / 4);
+                        const bool in = q < total && c < r4;
+                        const float* s = S + p * a.split_stride + i * r + c * 4;
+                        u[e][0] = in ? *reinterpret_cast<const float4*>(s) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        u[e][1] = in && p + 1 < a.splits ? *reinterpret_cast<const float4*>(s + a.split_stride) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) {
+                        if (p == 0) v[e] = u[e][0];
+                        else { v[e].x += u[e][0].x; v[e].y += u[e][0].y; v[e].z += u[e][0].z; v[e].w += u[e][0].w; }
+                        v[e].x += u[e][1].x; v[e].y += u[e][1].y; v[e].z += u[e][1].z; v[e].w += u[e][1].w;
+                    }
                 }
-                if (Rd) *reinterpret_cast<float4*>(Rd + i * r + c * 4) = v;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int q = q0 + e * QS_THREADS, i = q / (R / 4), c = q % (R / 4);
+                    if (q >= total) continue;
+                    if (Rd && c < r4) *reinterpret_cast<float4*>(Rd + i * r + c * 4) = v[e];
+                    *reinterpret_cast<float4*>(Y + i * LD + c * 4) = v[e];
+                }
             }
-            *reinterpret_cast<float4*>(Y + i * LD + c * 4) = v;
         }
     }
     __syncthreads();
@@ -236,21 +265,22 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
     auto apply = [&]() {
         if constexpr (R == 64) {
             // L^{-T} is upper triangular: column c needs the first c + 1 entries of a row only.  Warp w takes the
-            // columns 4 w .. and 60 - 4 w .. (17 depth steps of four together, for every warp), a lane four rows.
-            const int ca = 4 * warp, cb = 60 - 4 * warp;
-            for (int i0 = 0; i0 < nrows; i0 += 128) {
-                float xa[4][4] = {}, xb[4][4] = {};
+            // columns 4 w .. and 60 - 4 w .. (17 depth steps of four together, for every warp; w of each eight), a lane two rows.
+            const int ca = 4 * (warp % 8), cb = 60 - ca;
+            constexpr int NR = 4 * 256 / QS_THREADS;            // rows of a lane
+            for (int i0 = 32 * NR * (warp / 8); i0 - 32 * NR * (warp / 8) < nrows; i0 += 128) {
+                float xa[NR][4] = {}, xb[NR][4] = {};
                 const float* yr = Y + (i0 + lane) * LD;
-                auto step = [&](float (&acc)[4][4], int k0, int col) {
-                    float4 x[4];
+                auto step = [&](float (&acc)[NR][4], int k0, int col) {
+                    float4 x[NR];
 #pragma unroll
-                    for (int e = 0; e < 4; ++e)
+                    for (int e = 0; e < NR; ++e)
                         x[e] = i0 + lane + 32 * e < nrows ? *reinterpret_cast<const float4*>(yr + 32 * e * LD + k0) : make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
                     for (int kk = 0; kk < 4; ++kk) {
                         const float4 b = *reinterpret_cast<const float4*>(G + (k0 + kk) * R + col);
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) {
+                        for (int e = 0; e < NR; ++e) {
                             const float xv = kk == 0 ? x[e].x : (kk == 1 ? x[e].y : (kk == 2 ? x[e].z : x[e].w));
                             acc[e][0] = fmaf(xv, b.x, acc[e][0]); acc[e][1] = fmaf(xv, b.y, acc[e][1]);
                             acc[e][2] = fmaf(xv, b.z, acc[e][2]); acc[e][3] = fmaf(xv, b.w, acc[e][3]);
@@ -263,7 +293,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
                 for (int k0 = 0; k0 <= cb; k0 += 4) step(xb, k0, cb);
                 __syncthreads();
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
+                for (int e = 0; e < NR; ++e)
                     if (i0 + lane + 32 * e < nrows) {
                         float* o = Y + (i0 + lane + 32 * e) * LD;
                         *reinterpret_cast<float4*>(o + ca) = make_float4(xa[e][0], xa[e][1], xa[e][2], xa[e][3]);
@@ -331,139 +361,144 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
         }
     };
 
-    gram();
-
-    // R's images for the fused pass (the fp16 plane scaled by the power of two that brings the largest
-    // column norm to about 2^10)
-    if (a.r_planes) {
-        float scale = 1.f;
-        if (a.r_planes & 4) {
-            float mx = 0.f;
-            for (int j = 0; j < r; ++j) mx = fmaxf(mx, G[j * R + j]);
-            int e = 0;
-            const float nrm = sqrtf(mx);
-            if (nrm > 0.f && nrm <= 3.0e38f) frexpf(nrm, &e);      // nrm = f * 2^e, 0.5 <= f < 1
-            scale = ldexpf(1.f, 10 - e);
-            if (crank == 0 && tid == 0) *reinterpret_cast<float*>(w.scratch + a.rscale_off) = ldexpf(1.f, e - 10);
-        }
-        write_image(a.r_img, a.r_planes, scale);
-        __syncthreads();
-    }
-
-    if (a.colnorm) {
-        float inv = 0.f;
-        if (tid < r) {
-            const float nrm = sqrtf(G[tid * R + tid]);
-            if (!(nrm > 0.f) && crank == 0) atomicOr(w.status, ST_ZEROCOL);
-            inv = nrm > 0.f ? 1.f / nrm : 0.f;
-        }
-        __syncthreads();
-        if (tid < R) G[tid] = inv;
-        __syncthreads();
-        for (int q = tid; q < nrows * R; q += QS_THREADS) Y[q / R * LD + q % R] *= G[q % R];
-        __syncthreads();
-    } else {
-        float trace = 0.f;
-        for (int j = 0; j < r; ++j) trace += G[j * R + j];
-        if (!(fabsf(trace) <= 3.0e38f)) {   // Inf or NaN
-            if (tid == 0 && crank == 0) atomicOr(w.status, ST_NONFINITE);
-            return;
-        }
-        bool third = false;
-        for (int pass = 1; pass <= 3; ++pass) {
-            if (pass > 1) gram();
-            bool series = false;
-            if (pass > 1) {
-                // |G - I|_2 <= largest absolute row sum (see factor_tc.cuh: first-order inverse, third pass)
-                constexpr int HS = QS_THREADS / R;      // threads per row
-                {
-                    const int i = tid % R, h = tid / R;
-                    float s = 0.f;
-#pragma unroll
-                    for (int j = h * (R / HS); j < (h + 1) * (R / HS); ++j)
-                        s += j < r && i < r ? fabsf(G[j * R + i] - (i == j ? 1.f : 0.f)) : 0.f;
-                    part[tid] = s;
-                }
-                __syncthreads();
-                if (warp == 0) {
+    // (one place for the Gram product: its code is fetched as it is run, and again from the cache)
+    bool third = false;
+    float trace = 0.f;
+    for (int pass = 1; pass <= 3; ++pass) {
+        gram();
+        if (pass == 1) {
+            // R's images for the fused pass (the fp16 plane scaled by the power of two that brings the largest
+            // column norm to about 2^10)
+            if (a.r_planes) {
+                float scale = 1.f;
+                if (a.r_planes & 4) {
                     float mx = 0.f;
-                    for (int i = lane; i < R; i += 32) {
-                        float s = 0.f;
-#pragma unroll
-                        for (int h = 0; h < HS; ++h) s += part[h * R + i];
-                        mx = fmaxf(mx, s <= 3.0e38f ? s : 3.3e38f);
-                    }
-                    for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-                    if (lane == 0) s_bound = mx;
+                    for (int j = 0; j < r; ++j) mx = fmaxf(mx, G[j * R + j]);
+                    int e = 0;
+                    const float nrm = sqrtf(mx);
+                    if (nrm > 0.f && nrm <= 3.0e38f) frexpf(nrm, &e);      // nrm = f * 2^e, 0.5 <= f < 1
+                    scale = ldexpf(1.f, 10 - e);
+                    if (crank == 0 && tid == 0) *reinterpret_cast<float*>(w.scratch + a.rscale_off) = ldexpf(1.f, e - 10);
                 }
-                __syncthreads();
-                if (pass == 2 && !(s_bound <= CT_THIRD_PASS_LIMIT)) third = true;
-                series = s_bound <= CT_SERIES_LIMIT;
+                write_image(a.r_img, a.r_planes, scale);
                 __syncthreads();
             }
-            if (series) {
-                for (int q = tid; q < R * R; q += QS_THREADS) {
-                    const int k = q / R, j = q % R;
-                    const float v = G[q];
-                    G[q] = k < j ? -v : (k == j ? 0.5f * (3.f - v) : 0.f);
+            if (a.colnorm) {
+                float inv = 0.f;
+                if (tid < r) {
+                    const float nrm = sqrtf(G[tid * R + tid]);
+                    if (!(nrm > 0.f) && crank == 0) atomicOr(w.status, ST_ZEROCOL);
+                    inv = nrm > 0.f ? 1.f / nrm : 0.f;
                 }
-            } else {
-                const bool tiny = pass == 1 && trace < CT_TINY_TRACE;          // see ct_rsqrt
-                auto scale_block = [&](float f) {
-                    for (int q = tid; q < R * R; q += QS_THREADS) sD[q / R * CT_LDD + q % R] *= f;
-                    __syncthreads();
-                };
-                bool ok = false;
-                for (int attempt = 0; attempt < (pass == 1 ? 2 : 1) && !ok; ++attempt) {
-                    const float shift = attempt ? a.shift_rel * trace : 0.f;
-                    const float pad = G[0] + shift;      // diagonal of the padding: the first pivot (see factor_tc.cuh)
-                    constexpr int DN = R <= 32 ? 32 : 64;
-                    for (int q = tid; q < DN * DN; q += QS_THREADS) {
-                        const int i = q / DN, j = q % DN;
-                        float v = i == j ? pad : 0.f;
-                        if (i < r && j < r) v = G[i * R + j] + (i == j ? shift : 0.f);
-                        sD[i * CT_LDD + j] = v;
-                    }
-                    __syncthreads();
-                    if (tiny) scale_block(CT_TINY_UP);
-                    if (warp < CT_DIAG_WARPS) {
-                        const float2 mm = ct_diag_block(0, CT_DG_BLK, r, 1.f, warp, lane, nullptr, 0, nullptr);
-                        if (tid == 0) { s_min = mm.y <= 3.0e38f ? mm.x : -1.f; s_max = mm.y; }
-                    }
-                    __syncthreads();
-                    const float mn = s_min, mx = s_max;
-                    const bool fail = !(mn > 0.f);
-                    const bool ill = pass == 1 && sqrtf(mx) > a.cond_limit * sqrtf(mn);
-                    if (!fail && !(ill && attempt == 0)) ok = true;
-                    else if (attempt == 0 && pass == 1) third = true;
-                    __syncthreads();
+                __syncthreads();
+                if (tid < R) G[tid] = inv;
+                __syncthreads();
+                for (int q = tid; q < nrows * R; q += QS_THREADS) Y[q / R * LD + q % R] *= G[q % R];
+                __syncthreads();
+                break;
+            }
+            for (int j = 0; j < r; ++j) trace += G[j * R + j];
+            if (!(fabsf(trace) <= 3.0e38f)) {   // Inf or NaN
+                if (tid == 0 && crank == 0) atomicOr(w.status, ST_NONFINITE);
+                return;
+            }
+        }
+        bool series = false;
+        if (pass > 1) {
+            // |G - I|_2 <= largest absolute row sum (see factor_tc.cuh: first-order inverse, third pass)
+            constexpr int HS = QS_THREADS / R < R ? QS_THREADS / R : R;      // threads per row
+            {
+                const int i = tid % R, h = tid / R;
+                float s = 0.f;
+#pragma unroll
+                for (int jj = 0; jj < R / HS; ++jj) {
+                    const int j = min(h, HS - 1) * (R / HS) + jj;
+                    s += j < r && i < r ? fabsf(G[j * R + i] - (i == j ? 1.f : 0.f)) : 0.f;
                 }
-                if (!ok) {
-                    if (tid == 0 && crank == 0) atomicOr(w.status, ST_RANKDEF | (third ? shift_bit : 0));
-                    return;
-                }
-                if (tiny) scale_block(CT_TINY_UP_ROOT);
-                for (int q = tid; q < R * R; q += QS_THREADS) {
-                    const int k = q / R, j = q % R;
-                    G[q] = (k <= j && j < r) ? sD[k * CT_LDD + j] : 0.f;
-                }
+                if (h < HS) part[tid] = s;
             }
             __syncthreads();
-            apply();
-            if (pass == 2 && !third) break;
+            if (warp == 0) {
+                float mx = 0.f;
+                for (int i = lane; i < R; i += 32) {
+                    float s = 0.f;
+#pragma unroll
+                    for (int h = 0; h < HS; ++h) s += part[h * R + i];
+                    mx = fmaxf(mx, s <= 3.0e38f ? s : 3.3e38f);
+                }
+                for (int o = 16; o; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                if (lane == 0) s_bound = mx;
+            }
+            __syncthreads();
+            if (pass == 2 && !(s_bound <= CT_THIRD_PASS_LIMIT)) third = true;
+            series = s_bound <= CT_SERIES_LIMIT;
+            __syncthreads();
         }
-        if (third && tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
+        if (series) {
+            for (int q = tid; q < R * R; q += QS_THREADS) {
+                const int k = q / R, j = q % R;
+                const float v = G[q];
+                G[q] = k < j ? -v : (k == j ? 0.5f * (3.f - v) : 0.f);
+            }
+        } else {
+            const bool tiny = pass == 1 && trace < CT_TINY_TRACE;          // see ct_rsqrt
+            auto scale_block = [&](float f) {
+                for (int q = tid; q < R * R; q += QS_THREADS) sD[q / R * CT_LDD + q % R] *= f;
+                __syncthreads();
+            };
+            bool ok = false;
+            for (int attempt = 0; attempt < (pass == 1 ? 2 : 1) && !ok; ++attempt) {
+                const float shift = attempt ? a.shift_rel * trace : 0.f;
+                const float pad = G[0] + shift;      // diagonal of the padding: the first pivot (see factor_tc.cuh)
+                constexpr int DN = R <= 32 ? 32 : 64;
+                for (int q = tid; q < DN * DN; q += QS_THREADS) {
+                    const int i = q / DN, j = q % DN;
+                    float v = i == j ? pad : 0.f;
+                    if (i < r && j < r) v = G[i * R + j] + (i == j ? shift : 0.f);
+                    sD[i * CT_LDD + j] = v;
+                }
+                __syncthreads();
+                if (tiny) scale_block(CT_TINY_UP);
+                if (warp < CT_DIAG_WARPS) {
+                    const float2 mm = ct_diag_block(0, CT_DG_BLK, r, 1.f, warp, lane, nullptr, 0, nullptr);
+                    if (tid == 0) { s_min = mm.y <= 3.0e38f ? mm.x : -1.f; s_max = mm.y; }
+                }
+                __syncthreads();
+                const float mn = s_min, mx = s_max;
+                const bool fail = !(mn > 0.f);
+                const bool ill = pass == 1 && sqrtf(mx) > a.cond_limit * sqrtf(mn);
+                if (!fail && !(ill && attempt == 0)) ok = true;
+                else if (attempt == 0 && pass == 1) third = true;
+                __syncthreads();
+            }
+            if (!ok) {
+                if (tid == 0 && crank == 0) atomicOr(w.status, ST_RANKDEF | (third ? shift_bit : 0));
+                return;
+            }
+            if (tiny) scale_block(CT_TINY_UP_ROOT);
+            for (int q = tid; q < R * R; q += QS_THREADS) {
+                const int k = q / R, j = q % R;
+                G[q] = (k <= j && j < r) ? sD[k * CT_LDD + j] : 0.f;
+            }
+        }
+        __syncthreads();
+        apply();
+        if (pass == 2 && !third) break;
     }
+    if (third && tid == 0 && crank == 0) atomicOr(w.status, shift_bit);
 
     // ---- the factor and its image ----
     {
         float* D = pick(w, a.dst) + (int64_t)row0 * r;
-        for (int q = tid; q < nrows * r4; q += QS_THREADS) {
-            const int i = q / r4, c = q % r4;
-            *reinterpret_cast<float4*>(D + i * r + c * 4) = *reinterpret_cast<const float4*>(Y + i * LD + c * 4);
-        }
+        if (r % 4)
+            for (int q = tid; q < nrows * r; q += QS_THREADS) D[q] = Y[q / r * LD + q % r];
+        else
+            for (int q = tid; q < nrows * r4; q += QS_THREADS) {
+                const int i = q / r4, c = q % r4;
+                *reinterpret_cast<float4*>(D + i * r + c * 4) = *reinterpret_cast<const float4*>(Y + i * LD + c * 4);
+            }
     }
-    write_image(a.img, a.img_planes, 1.f);
+    if (a.img_planes) write_image(a.img, a.img_planes, 1.f);
 }
 
 }  // namespace od

@@ -1696,8 +1696,12 @@ inline int64_t product_depth(int64_t tiles, int chunks, int kb) {
     const int64_t waves = (tiles * chunks + SPLIT_SMS - 1) / SPLIT_SMS;
     return waves * ((kb + chunks - 1) / chunks + 2);
 }
-// ... and what writing and adding up the partial results costs in the same unit (about a microsecond).
-inline int64_t partial_cost(int64_t tiles, int chunks, int r) { return 4 + tiles * chunks * r / 6000; }
+// Whether the one-kernel QR takes the result (nearly: its limit by shared memory needs the device) and adds the partial
+// results up as it loads them.
+inline bool summed_by_qr(int r, int64_t out_rows) { return r <= 32 || (r <= QS_MAX_RANK && out_rows <= QS_MAX_ROWS_64); }
+// ... and what writing and adding up the partial results costs in the same unit (about a microsecond): a launch, but for
+// the one-kernel QR.
+inline int64_t partial_cost(int64_t tiles, int chunks, int r, bool by_qr) { return (by_qr ? 1 : 4) + tiles * chunks * r / 6000; }
 
 // Depth split of the two products with the buffer.  With one matrix (or a few) in a call and a
 // small rank, the output has too few row tiles for the device, or one wave and a bit (a 4096-wide factor 32, an
@@ -1724,8 +1728,9 @@ inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
         const int64_t tiles = (out_rows + tc::BM - 1) / tc::BM;
         int64_t best = product_depth(tiles, 1, kb);
         int fast = 1;
-        for (int v = 2; v <= std::min(r <= 64 ? 8 : 4, kb / 4); ++v) {
-            const int64_t cost = product_depth(tiles, v, kb) + partial_cost(tiles, v, r);
+        const bool by_qr = summed_by_qr(r, out_rows);
+        for (int v = 2; v <= std::min(r <= 64 ? 8 : 4, kb / (by_qr ? 2 : 4)); ++v) {
+            const int64_t cost = product_depth(tiles, v, kb) + partial_cost(tiles, v, r, by_qr);
             if (cost < best) { best = cost; fast = v; }
         }
         want = std::max(want, fast);
@@ -1744,7 +1749,7 @@ inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices, b
     if (lean) return 1;
     const int64_t tiles = matrices * ((out_rows + tc::BM - 1) / tc::BM);
     const int kb = (int)((depth + tc::BK - 1) / tc::BK);
-    return product_depth(tiles, chunks, kb) + partial_cost(tiles, chunks, r) < product_depth(tiles, 1, kb) ? chunks : 1;
+    return product_depth(tiles, chunks, kb) + partial_cost(tiles, chunks, r, summed_by_qr(r, out_rows)) < product_depth(tiles, 1, kb) ? chunks : 1;
 }
 
 // The chunks of a product with B in `parts` tiles of their own, or in as few tiles as tensor memory allows.
