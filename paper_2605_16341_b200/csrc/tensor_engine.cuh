@@ -78,6 +78,7 @@ struct GemmArgs {
     int32_t m_tiles, n_tiles, k_blocks, total_tiles;
     int32_t tri;                             // N-side is lower triangular (apply): skip depth beyond the tile
     int32_t lower_only;                      // symmetric result (Gram): skip tiles above the diagonal
+    int32_t one_operand;                     // ... whose tiles on the diagonal have the same columns on either side
     int32_t passes, passes2;                 // 1 or 3; passes2: second product of the fused pass
     int32_t ks;                              // N_IMG_MN: depth of one N-side piece (16, 32 or 64)
     int32_t n_slots, n_piece_bytes;          // N ring
@@ -458,7 +459,7 @@ pack_right_kernel(const __grid_constant__ Batch batch, PackRightArgs a) {
 // ------------------------------------------------------------------------------------------
 // Tile bookkeeping shared by all roles of the GEMM kernel
 // ------------------------------------------------------------------------------------------
-struct TileCoord { int b, mt, nt, n0, bn, kb_begin, kb_end, chunk; bool active; };
+struct TileCoord { int b, mt, nt, n0, bn, kb_begin, kb_end, chunk; bool active, self; };    // self: the A tiles are the N side as well
 // Each role remembers the status word of the matrix it is working on (nothing changes it while
 // the kernel runs), so that only the first tile of a matrix pays for the global load.
 struct StatusCache { int b = -1; int st = 0; };
@@ -490,6 +491,7 @@ __device__ __forceinline__ TileCoord decode_tile(const Batch& batch, const GemmA
     const int st = sc.st;
     c.active = !(st & ST_FAILED);
     if (EPI != EPI_K5 && g.out.only_if_shifted && !(st & g.out.shift_bit)) c.active = false;
+    c.self = g.one_operand && c.n0 == (g.pair ? 2 * mts : mts) * BM;
     if (g.lower_only && c.n0 > (g.pair ? 2 * mts + 1 : c.mt) * BM + BM - 1) c.active = false;
     if (c.kb_begin >= c.kb_end) c.active = false;
     return c;
@@ -534,6 +536,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         else return (t + 1) % g.run ? t + 1 : t + 1 + (tstride - 1) * g.run;
     };
     constexpr bool A_MN = (AMODE == A_IMG_MN || AMODE == A_BUF_COL);
+    constexpr bool SYM = AMODE == A_IMG_MN;          // Gram product
     constexpr bool G_BF16 = (XG & 1) != 0;
     constexpr bool X_BF16 = (XG & 2) != 0;
 
@@ -631,7 +634,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                 while (!n_done) {
                     if (nt_ >= g.total_tiles) { n_done = true; break; }
                     if (nkb < 0) { nc = decode_tile<EPI>(batch, g, nt_, scache, crank); nkb = nc.kb_begin; npc = 0; }
-                    if (!nc.active || nkb >= nc.kb_end) { nt_ = next(nt_); nkb = -1; npc = 0; continue; }
+                    if (!nc.active || (SYM && nc.self) || nkb >= nc.kb_end) { nt_ = next(nt_); nkb = -1; npc = 0; continue; }
                     if (npc >= n_pieces(nkb)) { ++nkb; npc = 0; continue; }
                     break;
                 }
@@ -744,6 +747,22 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                     if (chunk_left-- == 0) { chunk_left = g.kb_per_chunk - 1; d += (uint32_t)g.BN; accum = 0; }
                     if (!mbar_wait(a_full0 + 8 * as, aph, abort_flag)) { ok = false; break; }
                     uint32_t a = a_base + as * a_slot;
+                    if (SYM && c.self) {
+                        // The A tile, in the layout that a 64-deep piece of its columns has on the N side: a third to all of the
+                        // Gram tiles' operands from L2 saved (Gram products of a step, 1.1B model r = 512 2.75 -> 2.42 ms, 8B stage
+                        // 2.50 -> 2.19; one 11008 x 4096 matrix r = 128, step 507 -> 497 us).
+                        const int depth = min(BK, kdim - kb * BK);
+                        if (three && depth == 64) {
+                            umma_slices<PAIR, 4, true>(d, a, a_hi, a, a_hi, a_step, a_step, a_term, a_term, idesc_last, accum);
+                        } else {
+                            for (int j = 0; j * 16 < depth; ++j) {
+                                const uint32_t acc_j = j > 0 ? 1u : accum, aj = a + j * a_step;
+                                if (three) umma_slices<PAIR, 1, true>(d, aj, a_hi, aj, a_hi, 0, 0, a_term, a_term, idesc_last, acc_j);
+                                else umma_slices<PAIR, 1, false>(d, aj, a_hi, aj, a_hi, 0, 0, 0, 0, idesc_last, acc_j);
+                            }
+                        }
+                        accum = 1;
+                    } else
                     for (int left = min(BK, kdim - kb * BK); left > 0; left -= ks) {
                         if (!mbar_wait(n_full0 + 8 * ns, nph, abort_flag)) { ok = false; break; }
                         uint32_t b = b_base + ns * b_slot, dc = d;
@@ -1594,6 +1613,7 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     g.ksplit = (g.chunks + g.acc_chunks - 1) / g.acc_chunks;
     g.run = g.run ? g.ksplit : 1;
     g.total_tiles = b.count * g.m_tiles * g.n_tiles * g.ksplit;
+    g.one_operand = AMODE == tc::A_IMG_MN && g.BN <= (pair ? 256 : 128);
     const int n1_terms = g.passes == 3 ? 2 : 1, n2_terms = g.passes2 == 3 ? 2 : 1;
     const int bn64 = (g.BN + 63) / 64 * 64;
     const int a_terms = (tc::a_is_buf(AMODE) || g.passes == 3 || (EPI == tc::EPI_K5 && g.passes2 == 3)) ? 2 : 1;
