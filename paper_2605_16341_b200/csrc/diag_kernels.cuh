@@ -19,6 +19,7 @@ constexpr int DIAG_RESULTS = 8;     // floats copied out per matrix
 constexpr int DIAG_STRIDE = 16;     // floats reserved per matrix: results, then two double accumulators
 constexpr int DIAG_THREADS = 1024;
 constexpr int DIAG_MAX_ITERS = 96;
+constexpr size_t DIAG_SMEM_LIMIT = 208 * 1024;      // rows of the matrix, beside the vectors
 
 enum DiagSlot : int { DG_NU = 0, DG_ERANK, DG_TR_T2, DG_NORM_R, DG_NORM_M, DG_NORM_G, DG_NORM_B, DG_ITERS };
 
@@ -195,8 +196,8 @@ __device__ float diag_tridiag_max(const float* alpha, const float* beta, int k, 
     return 0.5f * (lo + hi);
 }
 
-// One CTA per matrix: finishes the diagnostics.  `gram` holds Q^T Q (at least its lower
-// triangle; it is mirrored in place first).  Its diagonal is replaced by the column squares of Q
+// One cluster per matrix: finishes the diagnostics.  `gram` holds Q^T Q (at least its lower
+// triangle).  Its diagonal is replaced by the column squares of Q
 // summed in fp32 registers: the tensor-core accumulation rounds towards zero, which lowers a sum
 // of n positive terms by about 5e-9 n (relative), visible in nu of an orthonormal Q at n ~ 10^4;
 // the off-diagonal entries keep that bias (it enters nu only through nu^2 - 1).  nu^2 is the largest eigenvalue of Q^T Q: Lanczos
@@ -204,24 +205,43 @@ __device__ float diag_tridiag_max(const float* alpha, const float* beta, int k, 
 // used, which converges regardless), the top Ritz value taken every fourth step and the iteration
 // stopped once it has moved by less than 1e-6 (relative), the Krylov space is exhausted, or
 // DIAG_MAX_ITERS products are done.
+//
+// What bounds it: a product with the r x r matrix per iteration, 64 bytes a cycle when one multiprocessor fetches it from L2.
+// The rows are dealt out over the cluster and stay in its shared memory (SMEM) up to rank 648; the product's entries
+// go to every CTA, which then takes the same steps: one cluster barrier per iteration.  The number of CTAs follows from
+// the rank, so that a matrix gets the same bits in any call.
+// Step with diagnostics, one CTA a matrix -> this: 4096 x 4096, Dion, r = 512 1.34 -> 0.87 ms, r = 1024 3.32 -> 1.40; 28 matrices
+// 1000 wide at r = 272 1.45 -> 1.40, 112 of a 1.1B model at r = 512 11.6 either way.
+inline int diag_cluster(int r) { return r <= 128 ? 1 : r <= 256 ? 2 : r <= 416 ? 4 : 8; }
+inline size_t diag_smem(int r) {
+    const size_t bytes = (size_t)((r + diag_cluster(r) - 1) / diag_cluster(r)) * ((r + 3) / 4 * 4) * 4;
+    return bytes <= DIAG_SMEM_LIMIT ? bytes : 0;                  // 0: the rows are read from memory
+}
+
+template <bool SMEM>
 __global__ void __launch_bounds__(DIAG_THREADS)
 diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, int64_t stats_off, int mask,
-                  float ef_a, float ef_b, DiagBase d) {
+                  float ef_a, float ef_b, DiagBase d, int csize) {
     grid_dependency();
-    const MatWork& w = batch.w[blockIdx.x];
+    const int crank = (int)(blockIdx.x % (unsigned)csize);
+    const MatWork& w = batch.w[blockIdx.x / (unsigned)csize];
     float* out = diag_record(w, d);
     const int tid = threadIdx.x, warp = tid / 32, lane = tid % 32;
     if (*w.status & ST_FAILED) {                 // the step left the state untouched
-        if (tid < DIAG_RESULTS) out[tid] = __int_as_float(0x7fc00000);
+        if (tid < DIAG_RESULTS && crank == 0) out[tid] = __int_as_float(0x7fc00000);
         return;
     }
-    __shared__ __align__(16) float vp[1024], v[1024], y[1024];
+    extern __shared__ __align__(16) float rows_smem[];
+    __shared__ __align__(16) float vp[1024], v[1024], y2[2][1024];
     __shared__ float red[DIAG_THREADS / 32];
     __shared__ float alpha[DIAG_MAX_ITERS], beta[DIAG_MAX_ITERS + 1], theta_sh;
     float* g = reinterpret_cast<float*>(w.scratch + gram_off);
     const float* colsq = reinterpret_cast<const float*>(w.scratch + stats_off);
     const float* rq = colsq + r;
     const float* qsq = colsq + 2 * r;
+    const int per = (r + csize - 1) / csize, r0 = crank * per, r1 = min(r, r0 + per);     // this CTA's rows
+    const int ld = SMEM ? (r + 3) / 4 * 4 : r;
+    float* G = SMEM ? rows_smem - (int64_t)r0 * ld : g;           // row i at G + i ld
 
     // column norms of R: entropy of their distribution, ||R||_F, <R, Q>
     float s_sum = 0.f, sq_sum = 0.f, rq_sum = 0.f;
@@ -239,18 +259,37 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
     }
     ent = diag_block_sum(ent, red);
 
-    // mirror the lower triangle: rows of it are read, a warp takes every 32nd; eight loads go out before the stores that may
-    // alias them
-    for (int j = warp; j < r; j += DIAG_THREADS / 32)
-        for (int i0 = lane; i0 < j; i0 += 256) {
-            float x[8];
+    // the CTA's rows: left of the diagonal as they stand, right of it from the rows below.  Loads go out together, before the
+    // stores that may alias them
+    if constexpr (SMEM) {
+        for (int i = r0 + warp; i < r1; i += DIAG_THREADS / 32)
+            for (int j0 = lane; j0 < i; j0 += 256) {
+                float x[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) x[e] = i0 + 32 * e < j ? g[(int64_t)j * r + i0 + 32 * e] : 0.f;
+                for (int e = 0; e < 8; ++e) x[e] = j0 + 32 * e < i ? g[(int64_t)i * r + j0 + 32 * e] : 0.f;
 #pragma unroll
-            for (int e = 0; e < 8; ++e)
-                if (i0 + 32 * e < j) g[(int64_t)(i0 + 32 * e) * r + j] = x[e];
+                for (int e = 0; e < 8; ++e)
+                    if (j0 + 32 * e < i) G[(int64_t)i * ld + j0 + 32 * e] = x[e];
+            }
+        for (int i = r0 + tid; i < r1; i += DIAG_THREADS)
+            for (int j = r; j < ld; ++j) G[(int64_t)i * ld + j] = 0.f;
+    }
+    for (int jb = r0 + 1 + warp; jb < r; jb += 4 * (DIAG_THREADS / 32))
+        for (int i = r0 + lane; i < r1; i += 32) {
+            float x[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = jb + e * (DIAG_THREADS / 32);
+                x[e] = j < r && i < j ? g[(int64_t)j * r + i] : 0.f;
+            }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int j = jb + e * (DIAG_THREADS / 32);
+                if (j < r && i < j) G[(int64_t)i * ld + j] = x[e];
+            }
         }
-    for (int j = tid; j < r; j += DIAG_THREADS) g[(int64_t)j * r + j] = qsq[j];
+    for (int i = r0 + tid; i < r1; i += DIAG_THREADS) G[(int64_t)i * ld + i] = qsq[i];
+    float* y = y2[0];
     float nrm2 = 0.f;
     for (int j = tid; j < r; j += DIAG_THREADS) {
         uint32_t h = (uint32_t)j * 2654435761u + 12345u;
@@ -259,17 +298,23 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
         y[j] = s0; nrm2 += s0 * s0;
     }
     nrm2 = diag_block_sum(nrm2, red);
-    for (int j = tid; j < r; j += DIAG_THREADS) { v[j] = y[j] * rsqrtf(nrm2); vp[j] = 0.f; }
-    __syncthreads();
+    for (int j = tid; j < 1024; j += DIAG_THREADS) { v[j] = j < r ? y[j] * rsqrtf(nrm2) : 0.f; vp[j] = 0.f; }
+    cluster_sync_all();
 
     float lambda = 0.f, beta_j = 0.f;
     int it = 0;
     bool done = false;
     while (!done) {
         // y = G v - beta_j v_prev ;  alpha = <y, v>
-        if (r % 4 == 0) {
-            // four rows of a warp side by side: what bounds the product is the latency of its loads from L2
-            for (int i0 = warp; i0 < r; i0 += 4 * (DIAG_THREADS / 32)) {
+        y = y2[it & 1];
+        const uint32_t y_addr = static_cast<uint32_t>(__cvta_generic_to_shared(y));
+        auto give = [&](int i, float acc) {          // entry i of y, to every CTA of the cluster
+            const float t = acc - beta_j * vp[i];
+            if (lane < csize) asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(map_to_rank(y_addr + i * 4, lane)), "f"(t) : "memory");
+        };
+        if (SMEM || r % 4 == 0) {
+            // four rows of a warp side by side: what bounds the product is the latency of its loads
+            for (int i0 = r0 + warp; i0 < r1; i0 += 4 * (DIAG_THREADS / 32)) {
                 float acc[4] = {};
                 for (int j = lane * 4; j < r; j += 128) {
                     const float4 vv = *reinterpret_cast<const float4*>(v + j);
@@ -277,7 +322,7 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
 #pragma unroll
                     for (int e = 0; e < 4; ++e) {
                         const int i = i0 + e * (DIAG_THREADS / 32);
-                        gv[e] = i < r ? *reinterpret_cast<const float4*>(g + (int64_t)i * r + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        gv[e] = i < r1 ? *reinterpret_cast<const float4*>(G + (int64_t)i * ld + j) : make_float4(0.f, 0.f, 0.f, 0.f);
                     }
 #pragma unroll
                     for (int e = 0; e < 4; ++e)
@@ -287,19 +332,19 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
                 for (int e = 0; e < 4; ++e) {
                     for (int o = 16; o; o >>= 1) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
                     const int i = i0 + e * (DIAG_THREADS / 32);
-                    if (lane == 0 && i < r) y[i] = acc[e] - beta_j * vp[i];
+                    if (i < r1) give(i, acc[e]);
                 }
             }
         } else {
-            for (int i = warp; i < r; i += DIAG_THREADS / 32) {
-                const float* row = g + (int64_t)i * r;
+            for (int i = r0 + warp; i < r1; i += DIAG_THREADS / 32) {
+                const float* row = G + (int64_t)i * ld;
                 float acc = 0.f;
                 for (int j = lane; j < r; j += 32) acc = fmaf(row[j], v[j], acc);
                 for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                if (lane == 0) y[i] = acc - beta_j * vp[i];
+                give(i, acc);
             }
         }
-        __syncthreads();
+        cluster_sync_all();
         float a = 0.f;
         for (int j = tid; j < r; j += DIAG_THREADS) a += y[j] * v[j];
         a = diag_block_sum(a, red);
@@ -330,7 +375,7 @@ diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, 
             __syncthreads();
         }
     }
-    if (tid == 0) {
+    if (tid == 0 && crank == 0) {
         out[DG_NU] = sqrtf(fmaxf(lambda, 0.f));
         out[DG_ERANK] = expf(ent);
         out[DG_TR_T2] = rq_sum;

@@ -241,8 +241,9 @@ int ensure_attributes() {
             g_qr_cluster_max[dev] = (signed char)std::min<int>(g_qr_cluster_max[dev], largest_cluster(kQrSmall[k], k % 2 ? 512 : 256, QS_SMEM_LIMIT));
     }
     if (e == cudaSuccess) {
-        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel, CT_THREADS, CT_SMEM_BYTES);
+        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<Batch>, CT_THREADS, CT_SMEM_BYTES);
     }
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(diag_final_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM_LIMIT);
     if (e == cudaSuccess) e = tensor_engine_set_attributes();
     if (e != cudaSuccess) {
         std::fprintf(stderr, "orthdion: kernel attribute setup failed on device %d: %s\n", dev, cudaGetErrorString(e));
@@ -538,8 +539,10 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
                   (unsigned)b.count);
         launch(diag_frob_kernel, grid, 256, 0, 1, prof::S_DIAG, st, b, elems, (int)(p->g_dtype == ORTHDION_DTYPE_BF16), db);
     }
-    launch(diag_final_kernel, dim3((unsigned)b.count), DIAG_THREADS, 0, 1, prof::S_DIAG, st, b, r, c.sc.gram, stats_off, p->diag, p->ef_a,
-           p->ef_b, db);
+    const int csize = diag_cluster(r);
+    const size_t smem = diag_smem(r);
+    launch(smem ? diag_final_kernel<true> : diag_final_kernel<false>, dim3((unsigned)(b.count * csize)), DIAG_THREADS, smem, csize, prof::S_DIAG, st,
+           b, r, c.sc.gram, stats_off, p->diag, p->ef_a, p->ef_b, db, csize);
 }
 
 // One step of every class of a group, stage by stage.
