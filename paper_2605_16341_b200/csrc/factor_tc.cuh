@@ -670,17 +670,18 @@ factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
     };
 
     grid_dependency_launch();
-    bool ok = false;
-    // Where launches overlap, the diagonal warps first run a block of three panels on whatever shared memory holds, while
-    // the kernel before is still at work: their code then is in the instruction cache (a block in the chain of one matrix:
-    // 19000 cycles the first and 13000 the others, 10000 either way so).
+    bool ok = false, prepared = false;
+    // The diagonal warps first run a block of three panels on whatever shared memory holds, while the kernel before is still
+    // at work (where launches overlap) or while the first CTA of the cluster has the first block: their code then is in
+    // the instruction cache (a block in the chain of one matrix: 19000 cycles the first and 13000 the others, 10000 either way so).
 #pragma unroll 1
-    for (int dry = a.ahead ? 1 : 0; dry >= 0; --dry) {
-        if (dry && mma_role) continue;
-        if (!dry) {
+    for (int dry = a.pass == 1 && (a.ahead || crank) ? 1 : 0; dry >= 0; --dry) {
+        if (!prepared && !(dry && a.ahead)) {
             grid_dependency_wait();
             if (!prepare()) return;
+            prepared = true;
         }
+        if (dry && mma_role) continue;
         const int max_attempts = (a.pass == 1 && !dry) ? 2 : 1;
         for (int attempt = 0; attempt < max_attempts && !ok; ++attempt) {
             const float shift = attempt ? a.shift_rel * trace : 0.f;
