@@ -318,8 +318,9 @@ __device__ __forceinline__ float2 ct_diag_block(uint32_t d_off, uint32_t blk_off
     return make_float2(dmin, dmax);
 }
 
+template <class BATCH>
 __global__ void __launch_bounds__(CT_THREADS, 1)
-factor_kernel(const __grid_constant__ Batch batch, CholArgs a, int csize) {
+factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float red[CT_THREADS / 32];
     __shared__ int s_status;

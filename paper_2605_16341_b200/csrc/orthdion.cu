@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <memory>
 #include <mutex>
 #include <vector>
 
@@ -233,7 +234,9 @@ int ensure_attributes() {
     if (state[dev]) return state[dev] > 0 ? 0 : ORTHDION_ERR_CUDA;
     cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM_BYTES);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
+        e = cudaFuncSetAttribute(factor_kernel<Batch>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(factor_kernel<MergedBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
     g_qr_cluster_max[dev] = 16;
     for (int k = 0; k < 6 && e == cudaSuccess; ++k) {
         e = cudaFuncSetAttribute(kQrSmall[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
@@ -325,11 +328,19 @@ struct ClassRun {
     bool tensor() const { return p->engine == ORTHDION_ENGINE_TENSOR; }
 };
 
+// (of at most MAXB matrices)
+Batch narrow(const MergedBatch& m) {
+    Batch b;
+    b.count = m.count; b.pad = 0; b.scratch_stride = m.scratch_stride;
+    std::copy(m.w, m.w + m.count, b.w);
+    return b;
+}
+
 // Cholesky + inverse of every class's Gram matrix: classes of equal (r, engine) share launches.
 // diag_from_gram: take the diagonal from the Gram matrix itself instead of the column-square
 // partials of the producing kernel (column-sharded matrices: the reduced Gram matrix carries it).
 void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, int which, int pass,
-                Batch* merged, int call_matrices, cudaStream_t st, bool diag_from_gram = false) {
+                MergedBatch* merged, int call_matrices, cudaStream_t st, bool diag_from_gram = false) {
     std::vector<char> done(which_cls.size(), 0);
     for (size_t i = 0; i < which_cls.size(); ++i) {
         if (done[i]) continue;
@@ -360,9 +371,11 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 const int room = sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
                 while (csize < cluster_max(g_factor_cluster_max) && csize < tiles &&
                        std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
-                launch(factor_kernel, dim3((unsigned)(merged->count * csize)), CT_THREADS, CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
+                const dim3 grid((unsigned)(merged->count * csize));
+                if (merged->count > MAXB) launch(factor_kernel<MergedBatch>, grid, CT_THREADS, CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
+                else launch(factor_kernel<Batch>, grid, CT_THREADS, CT_SMEM_BYTES, csize, prof::S_CHOL, st, narrow(*merged), ca, csize);
             } else {
-                launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, FS_SMEM_BYTES, 1, prof::S_CHOL, st, *merged, ca);
+                launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, FS_SMEM_BYTES, 1, prof::S_CHOL, st, narrow(*merged), ca);
             }
             merged->count = 0;
         };
@@ -376,7 +389,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 w = c.b->w[k];
                 w.aux0 = (int32_t)(4 * ((rows + 127) / 128));
                 w.aux1 = c.tensor() ? (int32_t)(c.sc.ts.q.off / 1024) : 0;
-                if (merged->count == MAXB) flush();
+                if (merged->count == (lead.tensor() ? MAXB_MERGED : MAXB)) flush();
             }
         }
         flush();
@@ -443,7 +456,7 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
 // which = 0: P = orth(Y) (Alg. 1, left-factor step), which = 1: Q = orth(R) (Alg. 1, normalisation step).
 // Tensor engine: the input is an image (w0 holds Y, image r holds R), or what small_qr_stage reads; SIMT
 // engine: fp32 slots.  summed: the fp32 slot holds the input even where the product is split by depth.
-void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int which, Batch* merged,
+void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int which, MergedBatch* merged,
               int call_matrices, cudaStream_t st, bool summed = false) {
     const int shift_bit = which ? ST_SHIFT_R : ST_SHIFT_L;
     std::vector<int> which_cls;
@@ -546,7 +559,7 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
 }
 
 // One step of every class of a group, stage by stage.
-void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_matrices, cudaStream_t st) {
+void run_group(std::vector<ClassRun>& cls, MergedBatch* merged, DiagBase db, int call_matrices, cudaStream_t st) {
     const Sel sP = sel(W_P), sR = sel(W_R), sQ = sel(W_Q);
     std::vector<int> all, orth;
     for (size_t i = 0; i < cls.size(); ++i) {
@@ -764,8 +777,9 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     char* ws = reinterpret_cast<char*>(workspace);
-    std::vector<Batch> pool(bt.batches.size() + 1);
-    Batch* merged = &pool[bt.batches.size()];
+    std::vector<Batch> pool(bt.batches.size());
+    const std::unique_ptr<MergedBatch> merged_batch(new MergedBatch);
+    MergedBatch* merged = merged_batch.get();
     int rc = ORTHDION_OK;
     for (const auto& grp : bt.groups) {
         std::vector<ClassRun> cls;
@@ -913,7 +927,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     const int r = p->r;
     std::vector<ClassRun> cls(1, sr->c);
     const std::vector<int> only(1, 0);
-    Batch* merged = new Batch();
+    MergedBatch* merged = new MergedBatch;
     engine_error() = 0;
     overlap_launches() = overlap_pays(&h, 1);
     if (phase == 0) {
