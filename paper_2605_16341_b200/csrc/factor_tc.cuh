@@ -47,12 +47,12 @@ constexpr int CT_LDD = 68;                    // diagonal block, fp32 (rows 16-b
 constexpr int CT_LDS = 65;                    // transposing buffer of the first-order inverse
 // dynamic shared memory: the operand stages, then the diagonal block's work area
 constexpr int CT_STAGES = 4;                  // operand stages, an A tile and a B tile each (a power of two)
-constexpr int CT_OFF_D = CT_STAGES * 2 * CT_TILE;
 constexpr int CT_DG_BLK = CT_NB * CT_LDD * 4;                  // work area of a diagonal block: the block itself, a panel's 8 x 8 block
 constexpr int CT_DG_BYTES = CT_DG_BLK + 64 * 4;
-constexpr int CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;              // the block of the odd columns (the even ones': CT_OFF_D)
-constexpr int CT_SMEM_BYTES = CT_OFF_D2 + CT_NB * CT_LDD * 4 + 1024;     // + alignment of the tiles
-static_assert(6 * CT_NB * CT_LDS * 4 <= CT_OFF_D, "six transposing buffers fit the operand stages");
+// the block of the even columns after the stages, that of the odd ones after its work area; + alignment of the tiles
+__host__ __device__ constexpr int ct_smem_bytes(int stages) { return stages * 2 * CT_TILE + CT_DG_BYTES + CT_NB * CT_LDD * 4 + 1024; }
+static_assert(2 * (ct_smem_bytes(2) + 2048) <= 228 * 1024, "two CTAs per multiprocessor with two stages");
+static_assert(6 * CT_NB * CT_LDS * 4 <= CT_STAGES * 2 * CT_TILE, "six transposing buffers fit the operand stages");
 constexpr int CT_MAX_BLOCKS = 64;             // r <= 4096
 constexpr int CT_STAT_FLOATS = 3 * CT_MAX_BLOCKS;   // per block: smallest and largest pivot, row-sum bound
 constexpr float CT_THIRD_PASS_LIMIT = 0.02f; // bound on |Gram - I|_2 of the second pass above which a third follows
@@ -318,9 +318,12 @@ __device__ __forceinline__ float2 ct_diag_block(uint32_t d_off, uint32_t blk_off
     return make_float2(dmin, dmax);
 }
 
-template <class BATCH>
-__global__ void __launch_bounds__(CT_THREADS, 1)
+// STAGES 4: one CTA per multiprocessor.  2: two, for one launch over more matrices than there are multiprocessors (154 at
+// r = 512, factorisations of a step 1.71 -> 1.56 ms, 168 at r = 192 0.287 -> 0.226).
+template <class BATCH, int STAGES>
+__global__ void __launch_bounds__(CT_THREADS, STAGES == 4 ? 1 : 2)
 factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
+    constexpr int CT_OFF_D = STAGES * 2 * CT_TILE, CT_OFF_D2 = CT_OFF_D + CT_DG_BYTES;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ float red[CT_THREADS / 32];
     __shared__ int s_status;
@@ -503,10 +506,11 @@ factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
         if (tid == 0 && crank == 0) gscale[r] = mx <= CT_SERIES_LIMIT ? 0.f : 1.f;
         if (!(mx <= CT_SERIES_LIMIT)) return true;
         // Image tiles (ta, tb), tb >= ta, of L^{-T}: entry (row, col) = -E(col, row) right of the
-        // diagonal.  Three groups of four warps, each with two transposing buffers of its own and the next tile's entries
-        // under way while it writes one.
+        // diagonal.  Three groups of four warps, each with two transposing buffers of its own (one where there is no room) and
+        // the next tile's entries under way while it writes one.
+        constexpr int NBUF = STAGES == 4 ? 2 : 1;
         const int grp = tid / 128, gt = tid % 128;
-        float* bufs = reinterpret_cast<float*>(smem) + grp * 2 * CT_NB * CT_LDS;
+        float* bufs = reinterpret_cast<float*>(smem) + grp * NBUF * CT_NB * CT_LDS;
         const int pairs = nb * (nb + 1) / 2, step = 3 * csize;
         int ta = 0, tb = 0;
         float4 v[8];
@@ -522,7 +526,8 @@ factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
         };
         int q = crank * 3 + grp, b = 0;
         if (q < pairs) fetch(q);
-        for (; q < pairs; q += step, b ^= 1) {
+        for (; q < pairs; q += step, b ^= NBUF - 1) {
+            if (NBUF == 1) ct_bar_sync(CT_BAR_MMA + grp, 128);       // (the one buffer has been read)
             float* buf = bufs + b * CT_NB * CT_LDS;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
@@ -560,7 +565,7 @@ factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
     const uint32_t dyn0 = static_cast<uint32_t>(smem - smem_raw);
     auto diag_off = [&](int k) { return dyn0 + ((k & 1) ? CT_OFF_D2 : CT_OFF_D); };
     int stage = 0;                     // operand stage that the next load goes to
-    auto slot = [&](int s) { return (s & (CT_STAGES - 1)) * 2 * CT_TILE; };      // A tile, then B tile
+    auto slot = [&](int s) { return (s & (STAGES - 1)) * 2 * CT_TILE; };      // A tile, then B tile
     auto load_tile = [&](uint32_t dst, const unsigned char* src) {
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -581,12 +586,12 @@ factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
         };
         if (c0 >= k) return;
 #pragma unroll
-        for (int e = 0; e < CT_STAGES - 1; ++e) load(c0 + e, stage + e);
+        for (int e = 0; e < STAGES - 1; ++e) load(c0 + e, stage + e);
 #pragma unroll 1
         for (int c = c0; c < k; ++c) {
-            ct_cp_wait<CT_STAGES - 2>();
+            ct_cp_wait<STAGES - 2>();
             ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
-            load(c + CT_STAGES - 1, stage + CT_STAGES - 1);
+            load(c + STAGES - 1, stage + STAGES - 1);
             const uint32_t at = smem0 + slot(stage);
             ct_tile_mma(acc, at, at + CT_TILE, warp, lane);
             if (c >= d0) ct_tile_mma(accd, at, at, warp, lane);
@@ -623,13 +628,13 @@ factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
         float o[4][4] = {};
         ct_tile_mma_nt(o, at, at + CT_TILE, warp, lane);
-        ct_store_tile(smem0 + slot(stage + CT_STAGES - 1), o, warp, lane);
+        ct_store_tile(smem0 + slot(stage + STAGES - 1), o, warp, lane);
         ct_bar_sync(CT_BAR_MMA, CT_MMA_THREADS);
     };
     // ... and from there to its image
     auto panel_out = [&](int t, int k) {
         unsigned char* dst = t < k ? x_tile(t, k) : l_tile(t, k);
-        const unsigned char* src = smem + slot(stage + CT_STAGES - 1);
+        const unsigned char* src = smem + slot(stage + STAGES - 1);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const int q = (tid + CT_MMA_THREADS * e) * 16;
@@ -717,7 +722,7 @@ factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {
                         if (first) cluster_sync_all();                  // X_k is in memory
                         if (on) {
                             panel(acc, k);
-                            const uint32_t z = smem0 + slot(stage + CT_STAGES - 1);
+                            const uint32_t z = smem0 + slot(stage + STAGES - 1);
                             if (lead) {
                                 // the chain goes on before anything else
                                 float dz[4][4] = {};

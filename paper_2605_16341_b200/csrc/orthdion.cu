@@ -234,9 +234,9 @@ int ensure_attributes() {
     if (state[dev]) return state[dev] > 0 ? 0 : ORTHDION_ERR_CUDA;
     cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM_BYTES);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel<Batch>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
+        e = cudaFuncSetAttribute(factor_kernel<Batch, CT_STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, ct_smem_bytes(CT_STAGES));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel<MergedBatch>, cudaFuncAttributeMaxDynamicSharedMemorySize, CT_SMEM_BYTES);
+        e = cudaFuncSetAttribute(factor_kernel<MergedBatch, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ct_smem_bytes(2));
     g_qr_cluster_max[dev] = 16;
     for (int k = 0; k < 6 && e == cudaSuccess; ++k) {
         e = cudaFuncSetAttribute(kQrSmall[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
@@ -244,7 +244,7 @@ int ensure_attributes() {
             g_qr_cluster_max[dev] = (signed char)std::min<int>(g_qr_cluster_max[dev], largest_cluster(kQrSmall[k], k % 2 ? 512 : 256, QS_SMEM_LIMIT));
     }
     if (e == cudaSuccess) {
-        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<Batch>, CT_THREADS, CT_SMEM_BYTES);
+        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<Batch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES));
     }
     if (e == cudaSuccess) e = cudaFuncSetAttribute(diag_final_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM_LIMIT);
     if (e == cudaSuccess) e = tensor_engine_set_attributes();
@@ -372,8 +372,8 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 while (csize < cluster_max(g_factor_cluster_max) && csize < tiles &&
                        std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
                 const dim3 grid((unsigned)(merged->count * csize));
-                if (merged->count > MAXB) launch(factor_kernel<MergedBatch>, grid, CT_THREADS, CT_SMEM_BYTES, csize, prof::S_CHOL, st, *merged, ca, csize);
-                else launch(factor_kernel<Batch>, grid, CT_THREADS, CT_SMEM_BYTES, csize, prof::S_CHOL, st, narrow(*merged), ca, csize);
+                if (merged->count > MAXB) launch(factor_kernel<MergedBatch, 2>, grid, CT_THREADS, ct_smem_bytes(2), csize, prof::S_CHOL, st, *merged, ca, csize);
+                else launch(factor_kernel<Batch, CT_STAGES>, grid, CT_THREADS, ct_smem_bytes(CT_STAGES), csize, prof::S_CHOL, st, narrow(*merged), ca, csize);
             } else {
                 launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, FS_SMEM_BYTES, 1, prof::S_CHOL, st, narrow(*merged), ca);
             }
