@@ -540,6 +540,19 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
     constexpr bool G_BF16 = (XG & 1) != 0;
     constexpr bool X_BF16 = (XG & 2) != 0;
 
+    if constexpr (EPI == EPI_STORE && !A_BUF) {
+        // Third pass of a QR: mostly there is nothing to do, and a look at the status words is all (before: every tile's, with
+        // barriers and tensor memory set up; 5 to 20 us a launch, now NOOPUS).
+        if (g.out.only_if_shifted) {
+            grid_dependency();
+            int any = 0;
+            for (int i = threadIdx.x; i < batch.count; i += blockDim.x) {
+                const int st = *batch.w[i].status;
+                any |= !(st & ST_FAILED) && (st & g.out.shift_bit);
+            }
+            if (!__syncthreads_or(any)) return;          // (both CTAs of a pair alike)
+        }
+    }
     extern __shared__ unsigned char smem_raw[];
     const uint32_t raw = smem_u32(smem_raw);
     unsigned char* smem = smem_raw + (((raw + 1023u) & ~1023u) - raw);
