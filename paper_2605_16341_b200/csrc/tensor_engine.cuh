@@ -344,7 +344,9 @@ struct PackArgs {
 
 __global__ void __launch_bounds__(256)
 pack_kernel(const __grid_constant__ Batch batch, PackArgs a) {
-    grid_dependency();
+    // (the first product, which follows, reads M and G before it waits: it may not start while the step before is at work)
+    grid_dependency_wait();
+    grid_dependency_launch();
     const MatWork& w = batch.w[blockIdx.z];
     if (a.init) {
         if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *w.status = 0;
@@ -471,7 +473,7 @@ template <bool V> struct BoolConst { static constexpr bool value = V; };
 
 template <int EPI>
 __device__ __forceinline__ TileCoord decode_tile(const Batch& batch, const GemmArgs& g, int t, StatusCache& sc,
-                                                 int rank) {
+                                                 int rank, bool look = true) {         // look: at the status word (`active` counts)
     TileCoord c;
     const int per = g.m_tiles * g.n_tiles * g.ksplit;
     c.b = t / per;
@@ -487,7 +489,7 @@ __device__ __forceinline__ TileCoord decode_tile(const Batch& batch, const GemmA
     c.kb_end = g.k_blocks;
     if (g.tri) c.kb_end = min(g.k_blocks, (c.n0 + c.bn + BK - 1) / BK);
     if (g.ksplit > 1) { c.kb_begin = c.chunk * g.kb_per_tile; c.kb_end = min(g.k_blocks, c.kb_begin + g.kb_per_tile); }
-    if (c.b != sc.b) { sc.b = c.b; sc.st = *batch.w[c.b].status; }
+    if (look && c.b != sc.b) { sc.b = c.b; sc.st = *batch.w[c.b].status; }
     const int st = sc.st;
     c.active = !(st & ST_FAILED);
     if (EPI != EPI_K5 && g.out.only_if_shifted && !(st & g.out.shift_bit)) c.active = false;
@@ -600,13 +602,19 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         else tmem_alloc(smem_u32(tmem_slot), (uint32_t)g.tmem_cols);
     }
     tc_fence_before();
-    grid_dependency_wait();
-    // (most often the matrix of the first tile: on its way while the CTA gathers)
     StatusCache scache;
-    scache.b = 0; scache.st = *batch.w[0].status;
+    if constexpr (!A_BUF) {
+        grid_dependency_wait();
+        // (most often the matrix of the first tile: on its way while the CTA gathers)
+        scache.b = 0; scache.st = *batch.w[0].status;
+    }
     __syncthreads();
     if (PAIR) cluster_sync_all();       // the peer's barriers are initialised before anything reaches them
     tc_fence_after();
+    if constexpr (A_BUF) {
+        // (the transform warps have something to do first, see there)
+        if (warp < 2 + NE) grid_dependency_wait();
+    }
     // cluster addresses of the leader's gathering barriers (slot s: + 8 s)
     const uint32_t a_full_ld = PAIR ? map_to_rank(a_full0, 0) : a_full0;
     const uint32_t n_full_ld = PAIR ? map_to_rank(n_full0, 0) : n_full0;
@@ -1312,6 +1320,26 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
         const int xr = AMODE == A_BUF_ROW ? xt / 8 : xt / 16, xc = AMODE == A_BUF_ROW ? xt % 8 : xt % 16;
         const uint32_t dst_off = AMODE == A_BUF_ROW ? xr * 128 + img_chunk_offset(xr, xc)
                                                     : (xc / 8) * 8192 + xr * 128 + img_chunk_offset(xr, xc % 8);
+        // Where launches overlap, the first tiles of M and G are on their way to L2 while the kernel before is still at work: nothing
+        // in the chain of a step writes them before the fused pass, and the step's first kernel lets this one in only
+        // when all that came before the step is done.  (Prefetches, because registers that are loaded here live on into the
+        // loop: 20 to 60 more bytes spilled, 1 % of the large steps.)
+        if (tile0 < g.total_tiles) {
+            const TileCoord c = decode_tile<EPI>(batch, g, tile0, scache, crank, false);
+            const MatWork& w = batch.w[c.b];
+            for (int kb = c.kb_begin; kb < min(c.kb_end, c.kb_begin + 4); ++kb)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const int64_t row = AMODE == A_BUF_ROW ? (int64_t)c.mt * BM + xr + e * E_STEP : (int64_t)kb * BK + xr + e * E_STEP;
+                    const int64_t col = AMODE == A_BUF_ROW ? (int64_t)kb * BK + xc * 8 : (int64_t)c.mt * BM + xc * 8;
+                    if (row < (AMODE == A_BUF_ROW ? g.Mrows : g.Kdim) && col < (AMODE == A_BUF_ROW ? g.Kdim : g.Mrows)) {
+                        const int64_t idx = row * g.ld + col;
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(w.M + idx));
+                        asm volatile("prefetch.global.L2 [%0];" ::"l"(reinterpret_cast<const unsigned char*>(w.G) + idx * (G_BF16 ? 2 : 4)));
+                    }
+                }
+        }
+        grid_dependency_wait();
         for (int t = tile0; t < g.total_tiles && ok; t = next(t)) {
             const TileCoord c = decode_tile<EPI>(batch, g, t, scache, crank);
             if (!c.active) continue;
