@@ -78,10 +78,10 @@ int q_planes(const orthdion_plan* p) { return (fused_fp16(p) ? 4 : 3) | (p->diag
 // Whether R's bf16 terms are read: by the right QR, or by the fused pass.
 bool right_image(const orthdion_plan* p) { return p->mode == ORTHDION_MODE_ORTH || !fused_fp16(p); }
 
-// matrices: of the whole call.  lean: no partial results in memory beyond those that a product cannot do without.
+// matrices: of the whole call.  lean 1: no partial results in memory beyond those that a product cannot do without.
 // The same chunks are then added up in tensor memory or tile by tile: the same bits, longer launches for a few
-// matrices.  A lean layout never needs more than the plan's images and fixed slots.
-Scratch scratch_layout(const orthdion_plan* p, int matrices, bool lean) {
+// matrices.  lean 2: none of the Gram products' at rank 256 and below either.  (Products with B at rank 129 to 256 always have theirs.)
+Scratch scratch_layout(const orthdion_plan* p, int matrices, int lean) {
     Scratch s{};
     const size_t rr = align_up((size_t)p->r * p->r * 4, 256);
     size_t off = 0;
@@ -118,10 +118,10 @@ struct Batching {
     std::vector<std::vector<int>> groups;    // batch indices per group
     std::vector<size_t> batch_off;           // scratch offset of each batch inside its group
     size_t scratch_bytes = 0;                // max over groups
-    bool lean = false;                       // scratch without optional partial results
+    int lean = 0;                            // scratch without optional partial results (see scratch_layout)
 };
 
-Batching make_batches(const orthdion_t* hs, int32_t count, bool lean) {
+Batching make_batches(const orthdion_t* hs, int32_t count, int lean) {
     Batching out;
     out.lean = lean;
     std::vector<char> done(count, 0);
@@ -179,8 +179,8 @@ Layout make_layout(const orthdion_t* hs, int32_t count, size_t scratch_bytes) {
 // fits, else lean.  (So a workspace that was sized for more matrices, or for another rank, serves a smaller call although
 // partial results are kept for small calls only.)
 void plan_call(const orthdion_t* hs, int32_t count, size_t bytes, Batching* bt, Layout* lay) {
-    for (int lean = 0; lean < 2; ++lean) {
-        *bt = make_batches(hs, count, lean != 0);
+    for (int lean = 0; lean < 3; ++lean) {
+        *bt = make_batches(hs, count, lean);
         *lay = make_layout(hs, count, bt->scratch_bytes);
         if (lay->total <= bytes) return;
     }
@@ -745,11 +745,11 @@ size_t orthdion_workspace_bytes_grouped(const orthdion_t* hs, int32_t count) {
     if (!hs || count < 1) return 0;
     for (int i = 0; i < count; ++i)
         if (!valid(hs[i])) return 0;
-    size_t total = make_layout(hs, count, make_batches(hs, count, false).scratch_bytes).total;
+    size_t total = make_layout(hs, count, make_batches(hs, count, 0).scratch_bytes).total;
     // partial results do not take a plan out of orthdion_step_noalloc's reach
-    if (count == 1 && total > ORTHDION_NOALLOC_SCRATCH_BYTES) {
-        const size_t lean = make_layout(hs, count, make_batches(hs, count, true).scratch_bytes).total;
-        if (lean <= ORTHDION_NOALLOC_SCRATCH_BYTES) total = lean;
+    for (int lean = 1; count == 1 && lean < 3 && total > ORTHDION_NOALLOC_SCRATCH_BYTES; ++lean) {
+        const size_t less = make_layout(hs, count, make_batches(hs, count, lean).scratch_bytes).total;
+        if (less <= ORTHDION_NOALLOC_SCRATCH_BYTES) total = less;
     }
     return total;
 }
@@ -978,7 +978,7 @@ int orthdion_shard_reduce_buffer(orthdion_t h, int32_t phase, void* workspace, f
     if (phase < 0 || phase > (orth ? 2 : 1)) return ORTHDION_ERR_INVALID_ARG;
     // (none of these offsets depends on the partial results)
     Layout lay = make_layout(&h, 1, 0);
-    Scratch sc = scratch_layout(h, 1, false);
+    Scratch sc = scratch_layout(h, 1, 0);
     char* ws = reinterpret_cast<char*>(workspace);
     if (phase == 0) {
         *buffer = reinterpret_cast<float*>(ws + lay.p_off[0]);

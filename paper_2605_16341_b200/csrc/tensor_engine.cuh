@@ -544,7 +544,7 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
 
     if constexpr (EPI == EPI_STORE && !A_BUF) {
         // Third pass of a QR: mostly there is nothing to do, and a look at the status words is all (before: every tile's, with
-        // barriers and tensor memory set up; 5 to 20 us a launch, now NOOPUS).
+        // barriers and tensor memory set up; 5 to 20 us a launch, now 4 to 6 cold).
         if (g.out.only_if_shifted) {
             grid_dependency();
             int any = 0;
@@ -1804,7 +1804,7 @@ inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
 // (up to rank 128 always, when the workspace is to be `lean`).
 // Measured (before: always in memory, added up, packed and squared by three kernels): 154 matrices of a 1.1B model
 // at r = 128 9.7 -> 8.6 ms a step; one 4096 x 4096 matrix at r = 256, three kernels in one, 0.633 -> 0.609 ms.
-inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices, bool lean) {
+inline int buffer_ksplit(int r, int64_t out_rows, int64_t depth, int matrices, int lean) {
     const int chunks = buffer_chunks(r, out_rows, depth);
     if (r > 128 || chunks == 1) return chunks;
     if (lean) return 1;
@@ -1991,10 +1991,11 @@ inline int gram_tiles(int r) {               // tiles that touch the lower trian
 }
 inline int gram_chunks(int r, int64_t rows) {
     const int kb = (int)((rows + tc::BK - 1) / tc::BK);
-    // At least 8 depth blocks per chunk at r <= 256; 24 above, where the additions cost calls with many matrices
+    // At least 8 depth blocks per chunk at r <= 256, from 64 blocks on sixteen chunks (4096 x 4096, 8 chunks -> 16: r = 256 386 ->
+    // 375 us a step, r = 192 359 -> 352; four blocks a chunk everywhere: 24 layers of 768-wide matrices at r = 192 2.04 -> 2.17 ms); 24 above, where the additions cost calls with many matrices
     // some of their Gram time (1.1B model at r = 512 3.03 -> 3.15 ms of an 18 ms step; with 16 blocks 3.31) and 16
     // would give single matrices another 0.05 ms.
-    const int want = r <= 256 ? std::min(16, kb / 8) : std::min({16, kb / 24, 80 / gram_tiles(r)});
+    const int want = r <= 256 ? (kb >= 64 ? 16 : kb / 8) : std::min({16, kb / 24, 80 / gram_tiles(r)});
     if (want < 2) return 1;
     const int per = (kb + want - 1) / want;
     return (kb + per - 1) / per;             // every chunk non-empty
@@ -2008,8 +2009,8 @@ inline int gram_chunks(int r, int64_t rows) {
 // 0.453 and 0.416; 8192, 9 0.430 and 0.324, 12 0.422 and 0.416, 16 0.434 and 0.484, 20 0.745 and 0.588, 28 0.768 and
 // 0.766; 14336, 12 0.636 and 0.554, 14 0.648 and 0.628, 16 0.660 and 0.689.  r = 384 (single CTAs): 4096, 12 0.295 and
 // 0.215, 20 0.300 and 0.337, 28 0.501 and 0.451; 8192, 16 0.345 and 0.415; 14336, 16 0.526 and 0.510.
-inline int gram_ksplit(int r, int64_t rows, int matrices, bool lean) {
-    if (r <= 256) return gram_chunks(r, rows);
+inline int gram_ksplit(int r, int64_t rows, int matrices, int lean) {
+    if (r <= 256) return lean < 2 ? gram_chunks(r, rows) : 1;
     if (lean) return 1;
     const int room = r % 256 ? SPLIT_SMS : SPLIT_SMS / 2, high = r % 256 ? 128 : 256, wide = std::min(r, 256);
     const int64_t tiles = (int64_t)matrices * ((r + high - 1) / high) * ((r + wide - 1) / wide);
