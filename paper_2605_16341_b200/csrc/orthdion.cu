@@ -404,18 +404,20 @@ bool small_qr(const orthdion_plan* p, int64_t rows) {
 // Whether the launches of a call's one chain overlap (programmatic dependent launch).  Not with several
 // chains, where the waiting CTAs of one keep the others' kernels off the multiprocessors (four streams: 320M model
 // 2.50 -> 2.78 ms, 1.1B model 17.7 -> 18.2 ms), and not in large calls: CTAs that start early crowd on the
-// multiprocessors that fall free first.  Six long kernels (one-kernel QR on both sides) lose from about 4 M
-// elements on (9113 x 2488, r = 32: 0.273 -> 0.319 ms; 2000 x 2000: equal; 1000 x 1000: 0.095 -> 0.084), the
-// thirty kernels of a larger rank gain up to 67 M elements (4096 x 4096, r = 256 0.650 -> 0.614, 8192 x 8192,
-// r = 128 0.885 -> 0.837, r = 512 equal).
+// multiprocessors that fall free first.  Six kernels (one-kernel QR on both sides) gain up to 8 M elements: r = 32 without ->
+// with overlap 2500 x 2000 101 -> 90 us (fp32 107 -> 96), 4096 x 2048 113 -> 106 (fp32 128 -> 126); on the other side of
+// the line 4096 x 3072 140 -> 140 (fp32 160 -> 166), 9113 x 2488 fp32 244 -> 281.  The fp32 engine stays at 4 M (2001 x 3001,
+// r = 40 247 -> 252, r = 16 249 -> 240).  The thirty kernels of a larger rank gain up to 67 M elements (4096 x 4096, r = 256
+// 423 -> 374 us; 14336 x 8192, r = 256 and 1024 equal).
 bool overlap_pays(const orthdion_t* hs, int32_t count) {
     int64_t elements = 0;
-    bool small = true;
+    bool small = true, simt = false;
     for (int i = 0; i < count; ++i) {
         elements += hs[i]->m * hs[i]->n;
-        if (hs[i]->engine == ORTHDION_ENGINE_TENSOR && !(small_qr(hs[i], hs[i]->m) && small_qr(hs[i], hs[i]->n))) small = false;
+        if (hs[i]->engine != ORTHDION_ENGINE_TENSOR) simt = true;
+        else if (!(small_qr(hs[i], hs[i]->m) && small_qr(hs[i], hs[i]->n))) small = false;
     }
-    return elements <= (small ? (int64_t)4 << 20 : (int64_t)64 << 20);
+    return elements <= ((int64_t)(!small ? 64 : simt ? 4 : 8) << 20);
 }
 
 // QR of one class's left (which = 0) or right factor in one kernel, or the column normalisation of the right

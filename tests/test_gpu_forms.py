@@ -33,6 +33,25 @@ def test_one_kernel_qr_of_long_parts(shape, mode):
     one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_TENSOR)
 
 
+# a call of six kernels on either side of the size up to which its launches overlap
+@pytest.mark.parametrize("shape", [(4096, 2048, 32), (4104, 2048, 32)])
+def test_steps_back_to_back_at_the_largest_overlapping_size(shape):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, BF16, BF16, seed=m)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR)
+    pair = [GpuMatrix(spec, X, M, Q, mu=0.95, eta=0.01, engine=od.ENGINE_TENSOR) for _ in range(2)]
+    grad = G.cuda()
+    for gm in pair:
+        for _ in range(4):
+            od.orthdion_step(gm.h, gm.X, gm.M, grad, gm.Q, gm.ws)
+            if gm is pair[0]:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+    assert all(torch.equal(getattr(pair[0], k), getattr(pair[1], k)) for k in "XMQ")
+    for gm in pair:
+        gm.close()
+
+
 # the fused pass where the R and Q pieces have slots of their own (split terms of both, or fp32 G or X) and where they share
 # one: a single 16-deep slice, a ragged last depth block, a last tile of 8 columns
 @pytest.mark.parametrize("shape", [(300, 264, 16), (260, 392, 80), (600, 136, 128)])
