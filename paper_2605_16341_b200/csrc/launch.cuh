@@ -2,7 +2,8 @@
 // programmatic dependent launch the next kernel's CTAs are set up (barriers, tensor memory, tensor-map
 // fetches) while the current one still runs, and wait for its end and its memory before they touch
 // global memory.  Every kernel of the library therefore starts with grid_dependency_wait() in front of its first global access, and
-// lets its successor in right away.
+// lets its successor in right away.  One exception in two halves: the products with B prefetch M and G before they wait, and
+// the packing kernel in front of the first of them lets it in only after its own wait, i.e. when the step before is done.
 #pragma once
 #include <cuda_runtime.h>
 

@@ -49,11 +49,10 @@ enum NMode : int { N_IMG_K = 0, N_IMG_MN = 1 };
 enum EpiMode : int { EPI_STORE = 0, EPI_K5 = 1 };
 
 __host__ __device__ constexpr bool a_is_buf(int amode) { return amode == A_BUF_ROW || amode == A_BUF_COL; }
-// Eight epilogue warps (two per tensor-memory lane quarter, splitting the columns) for the fused
-// pass, whose epilogue is most of a tile's time.  Everywhere else four: the products that form B
-// have sixteen transform warps already, and the image-to-image products of the QR do better with
-// the 32 KB of staging that four more warps would take spent on a third A slot (they are bound by
-// the latency of their operand tiles: measured apply 10.3 -> 9.4 ms, Gram 8.85 -> 8.5 ms).
+// Eight epilogue warps (two per tensor-memory lane quarter, splitting the columns): the epilogue is most of a tile's time
+// in the fused pass, and a third of it in launches of one tile of an image product (one 4096 x 4096 matrix at r = 256, four ->
+// eight: step 406 -> 402 us; their staging is 32 KB, which leaves room for the third A slot).  Four in the products that
+// form B, which have sixteen transform warps already.
 __host__ __device__ constexpr int epi_warps(int amode, int epi) { return epi == EPI_K5 || !a_is_buf(amode) ? 8 : 4; }
 __host__ __device__ constexpr int gemm_threads(int amode, int epi) {
     return 32 * (2 + epi_warps(amode, epi) + (a_is_buf(amode) ? NUM_XF_WARPS : 0));
