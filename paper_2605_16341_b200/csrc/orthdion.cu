@@ -438,6 +438,7 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
     a.rows_per_part = qs_rows_per_part(a.rows, parts);
     a.colnorm = which && p->mode == ORTHDION_MODE_COLNORM;
     a.shift_rel = kShiftRel; a.cond_limit = kCondLimit;      // fp32 arithmetic
+    a.series_limit = c.tensor() ? CT_SERIES_LIMIT : QS_SERIES_LIMIT_F32;
     a.dst = sel(which ? W_Q : W_P);
     if (!c.tensor()) {
         a.img = a.r_img = no_img();        // the fp32 engine has no images

@@ -25,6 +25,10 @@ namespace od {
 constexpr int QS_MAX_RANK = 64;
 constexpr int QS_MAX_ROWS_64 = 640;
 constexpr int QS_SMEM_LIMIT = 227 * 1024 - 256;      // less the static variables
+// Bound on |Gram - I|_2 below which L^{-1} = I - Phi(E) is used on the fp32 engine: the dropped terms, of order |E|^2, are
+// then below 2^-26, a quarter of what rounding a 1 to fp32 loses.  (Below the tensor engine's CT_SERIES_LIMIT they reach 2e-6:
+// nothing beside products good to 2^-16, several roundings here.)
+constexpr float QS_SERIES_LIMIT_F32 = 1.22070312e-4f;      // 2^-13
 
 struct QrSmallArgs {
     Sel src;                // rows x r fp32, or `splits` partial results split_stride floats apart
@@ -33,7 +37,7 @@ struct QrSmallArgs {
     int32_t rows, r, csize, parts_per_cta, rows_per_part;
     int32_t which;          // 0: left QR (P), 1: right factor (Q)
     int32_t colnorm;        // 1: column normalisation instead of the QR
-    float shift_rel, cond_limit;
+    float shift_rel, cond_limit, series_limit;
     Sel dst;                // the factor, fp32
     ImgRef img;             // and its image
     int32_t img_planes;     // bit mask of the planes to write: 1 | 2 bf16 terms, 4 fp16
@@ -431,7 +435,7 @@ qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrS
             }
             __syncthreads();
             if (pass == 2 && !(s_bound <= CT_THIRD_PASS_LIMIT)) third = true;
-            series = s_bound <= CT_SERIES_LIMIT;
+            series = s_bound <= a.series_limit;
             __syncthreads();
         }
         if (series) {

@@ -24,6 +24,34 @@ def test_one_kernel_qr_of_the_fp32_engine(shape, mode):
     one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_SIMT)
 
 
+# Q1 of the first pass 1e-4 to 1.4e-3 away from orthonormal: two columns of Y all but parallel, 96 draws.  A first-order inverse in the second
+# pass leaves out up to 0.75 times the square of that, 1.5e-6; rounding alone stays below eight halves of a spacing at 1 (2^-24)
+@pytest.mark.parametrize("case", [(200, 100, 9, 0.012), (200, 100, 9, 0.02), (150, 304, 30, 0.012)])
+def test_fp32_engine_is_orthonormal_to_rounding(case):
+    m, n, r, eps = case
+    count = 96
+    gen = torch.Generator().manual_seed(m + n + r)
+    h = od.orthdion_create(m, n, r, 0.95, 0.01, 0.0, od.MODE_ORTH)
+    od.orthdion_set_dtypes(h, F32, F32)
+    od.orthdion_set_engine(h, od.ENGINE_SIMT)
+    G, Q = [], []
+    for _ in range(count):
+        Y = torch.randn(m, r, generator=gen)
+        Y[:, 1] = Y[:, 0] + eps * Y[:, 1]
+        Q.append(wl.random_orthonormal(n, r, gen).cuda())
+        G.append(Y.cuda() @ Q[-1].T)
+    X, M = ([torch.zeros(m, n, device="cuda") for _ in range(count)] for _ in range(2))
+    ws = poisoned_workspace(od.orthdion_workspace_bytes_grouped([h] * count))
+    od.orthdion_step_grouped(od.PointerTable([h] * count, X, M, G, Q), ws)
+    torch.cuda.synchronize()
+    worst = 0.0
+    for i in range(count):
+        for A in (od.orthdion_get_factors([h] * count, i, ws, (m, n, r))[0].double(), Q[i].double()):
+            worst = max(worst, (A.T @ A - torch.eye(r, device="cuda", dtype=torch.float64)).abs().max().item())
+    assert worst <= 8 * 2.0 ** -24
+    od.orthdion_destroy(h)
+
+
 # its 512-thread form (parts of 256 rows and more): the last size below, the first, a ragged one
 @pytest.mark.parametrize("shape", [(3584, 136, 32), (3585, 136, 32), (7700, 264, 16)])
 @pytest.mark.parametrize("mode", MODES)
