@@ -93,6 +93,7 @@ struct GemmArgs {
                                              // added up by the epilogue (products with B)
     int32_t ksplit, kb_per_tile;             // tiles of such chunks that a result tile is computed as, their depth
     int64_t split_stride;                    // blocks; stored split_stride floats apart
+    int32_t ahead;                           // depth blocks of M and G to prefetch while the kernel before is at work (0: launches do not overlap)
     int32_t run;                             // ksplit or 1: so many consecutive tiles (those of one result tile) go to the
                                              // same CTA, which adds each to what it has stored
     int64_t rscale_off;                      // fp16 fused pass: scratch offset of 1 / (scale of R's plane)
@@ -1321,12 +1322,14 @@ gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArg
                                                     : (xc / 8) * 8192 + xr * 128 + img_chunk_offset(xr, xc % 8);
         // Where launches overlap, the first tiles of M and G are on their way to L2 while the kernel before is still at work: nothing
         // in the chain of a step writes them before the fused pass, and the step's first kernel lets this one in only
-        // when all that came before the step is done.  (Prefetches, because registers that are loaded here live on into the
+        // when all that came before the step is done.  Not elsewhere: the loads that follow at once then queue behind the prefetches
+        // (six-kernel steps of 24 matrices 1024 wide at r = 32 238 us with, 235 without, 36 matrices 768 wide at r = 16 189.6 and 188.2).
+        // (Prefetches, because registers that are loaded here live on into the
         // loop: 20 to 60 more bytes spilled, 1 % of the large steps.)
         if (tile0 < g.total_tiles) {
             const TileCoord c = decode_tile<EPI>(batch, g, tile0, scache, crank, false);
             const MatWork& w = batch.w[c.b];
-            for (int kb = c.kb_begin; kb < min(c.kb_end, c.kb_begin + 4); ++kb)
+            for (int kb = c.kb_begin; kb < min(c.kb_end, c.kb_begin + g.ahead); ++kb)
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const int64_t row = AMODE == A_BUF_ROW ? (int64_t)c.mt * BM + xr + e * E_STEP : (int64_t)kb * BK + xr + e * E_STEP;
@@ -1653,6 +1656,7 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     g.ksplit = (g.chunks + g.acc_chunks - 1) / g.acc_chunks;
     g.run = g.run ? g.ksplit : 1;
     g.total_tiles = b.count * g.m_tiles * g.n_tiles * g.ksplit;
+    g.ahead = overlap_launches() ? 4 : 0;
     g.one_operand = AMODE == tc::A_IMG_MN && g.BN <= (pair ? 256 : 128);
     const int n1_terms = g.passes == 3 ? 2 : 1, n2_terms = g.passes2 == 3 ? 2 : 1;
     const int bn64 = (g.BN + 63) / 64 * 64;
