@@ -200,6 +200,10 @@ void plan_call(const orthdion_t* hs, int32_t count, size_t bytes, Batching* bt, 
 // Largest clusters of the factor kernel and of the small-rank QR kernel (16 CTAs where the device can
 // place one, else 8); written under ensure_attributes()'s lock.
 signed char g_factor_cluster_max[kMaxDevices] = {}, g_qr_cluster_max[kMaxDevices] = {};
+// Clusters of 1, 2, 4, 8 and 16 CTAs that the device runs at once, with one and with two CTAs per multiprocessor.  A cluster lies
+// within one group of multiprocessors, and the groups are of different sizes: 148 multiprocessors hold 74, 33, 15 and 7 of
+// them, or 148, 71, 33 and 14.  Written under the same lock.
+int g_clusters_at_once[kMaxDevices][2][5] = {};
 
 // Clusters of 16 CTAs are beyond the portable size: allowed per kernel, and used only where the
 // device says that it can place one.
@@ -218,6 +222,22 @@ int largest_cluster(K* kernel, int threads, size_t smem) {
     }
     (void)cudaGetLastError();
     return 8;
+}
+
+// Clusters of `size` CTAs of this kernel that run at once (by multiprocessors where the device cannot say).
+template <class K>
+int clusters_at_once(K* kernel, int threads, size_t smem, int size, int per_sm) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(per_sm * sm_count() / size * size), 1, 1); cfg.blockDim = dim3((unsigned)threads, 1, 1);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)size; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    int n = 0;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) == cudaSuccess && n >= 1) return n;
+    (void)cudaGetLastError();
+    return std::max(1, per_sm * sm_count() / size);
 }
 
 // by rank (16, 32, 64) and threads (256, 512)
@@ -245,6 +265,11 @@ int ensure_attributes() {
     }
     if (e == cudaSuccess) {
         g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<Batch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES));
+        // (one per multiprocessor: the factor kernel.  Two: the one-kernel QR with 256 threads and little memory.)
+        for (int l = 0; l < 5; ++l) {
+            g_clusters_at_once[dev][0][l] = clusters_at_once(factor_kernel<Batch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES), 1 << l, 1);
+            g_clusters_at_once[dev][1][l] = clusters_at_once(kQrSmall[2], 256, QS_SMEM_TWO, 1 << l, 2);
+        }
     }
     if (e == cudaSuccess) e = cudaFuncSetAttribute(diag_final_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM_LIMIT);
     if (e == cudaSuccess) e = tensor_engine_set_attributes();
@@ -261,6 +286,15 @@ int cluster_max(const signed char (&table)[kMaxDevices]) {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return 8;
     return table[dev] == 16 ? 16 : 8;
+}
+
+// Clusters of `size` CTAs (1 to 16, a power of two) that the current device runs at once, per_sm CTAs on a multiprocessor.
+int room_for_clusters(int size, int per_sm) {
+    int dev = -1, l = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) dev = 0;
+    while (1 << (l + 1) <= size) ++l;
+    const int n = g_clusters_at_once[dev][per_sm - 1][l];
+    return n > 0 ? n : per_sm * sm_count() / size;
 }
 
 // ---- internal streams of the grouped step ---------------------------------------------------
@@ -363,14 +397,17 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
             if (!merged->count) return;
             if (lead.tensor()) {
                 // Fewer matrices than the device has multiprocessors (one CTA each): share each matrix among the CTAs of
-                // a cluster, up to one per 64-row tile (16 only where the device can place such a cluster).
+                // a cluster, up to one per 64-row tile (16 only where the device can place such a cluster), as long as all
+                // clusters run at once.  (Counted in CTAs, the last clusters of 8 and 9 matrices at r = 1024, 16 to 18 at r = 512 and 34
+                // to 37 at r = 272 came in a second wave: step of 8 4096 x 4096 at r = 1024 4.27 -> 4.12 ms, 16 2048 wide at r = 512
+                // 1.45 -> 1.36, 37 1000 wide at r = 272 1.11 -> 1.01.)
                 // (Counted over the whole grouped call: with more matrices than that, the other launch batches keep
                 // the rest of the device busy on their own streams; counted by batch, the 1.1B and 8B groups run
-                // as before.  Twice as many CTAs, in two waves: 28 matrices at r = 272 1.61 -> 1.75 ms a step.)
+                // as before.)
                 int csize = 1;
-                const int room = sm_count(), tiles = (r + CT_NB - 1) / CT_NB;
+                const int tiles = (r + CT_NB - 1) / CT_NB;
                 while (csize < cluster_max(g_factor_cluster_max) && csize < tiles &&
-                       std::max(merged->count, call_matrices) * csize * 2 <= room) csize *= 2;
+                       std::max(merged->count, call_matrices) <= room_for_clusters(csize * 2, 1)) csize *= 2;
                 const dim3 grid((unsigned)(merged->count * csize));
                 if (merged->count > MAXB) launch(factor_kernel<MergedBatch, 2>, grid, CT_THREADS, ct_smem_bytes(2), csize, prof::S_CHOL, st, *merged, ca, csize);
                 else launch(factor_kernel<Batch, CT_STAGES>, grid, CT_THREADS, ct_smem_bytes(CT_STAGES), csize, prof::S_CHOL, st, narrow(*merged), ca, csize);
@@ -433,7 +470,7 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
     a.splits = splits; a.split_stride = (int64_t)a.rows * p->r;
     const int cmax = cluster_max(g_qr_cluster_max), parts = qs_parts(a.rows, p->r, cmax);
     const int threads = qs_threads(a.rows, p->r, cmax, !c.tensor());
-    a.csize = qs_ctas(a.rows, p->r, cmax, call_matrices, 512 / threads * sm_count(), threads);
+    a.csize = qs_ctas(a.rows, p->r, cmax, call_matrices, threads, room_for_clusters);
     a.parts_per_cta = parts / a.csize;
     a.rows_per_part = qs_rows_per_part(a.rows, parts);
     a.colnorm = which && p->mode == ORTHDION_MODE_COLNORM;

@@ -25,6 +25,7 @@ namespace od {
 constexpr int QS_MAX_RANK = 64;
 constexpr int QS_MAX_ROWS_64 = 640;
 constexpr int QS_SMEM_LIMIT = 227 * 1024 - 256;      // less the static variables
+constexpr int QS_SMEM_TWO = 228 * 1024 / 2 - 1024 - 256;     // up to here two CTAs of 256 threads share a multiprocessor
 // Bound on |Gram - I|_2 below which L^{-1} = I - Phi(E) is used on the fp32 engine: the dropped terms, of order |E|^2, are
 // then below 2^-26, a quarter of what rounding a 1 to fp32 loses.  (Below the tensor engine's CT_SERIES_LIMIT they reach 2e-6:
 // nothing beside products good to 2^-16, several roundings here.)
@@ -82,12 +83,16 @@ inline bool qs_fits(int64_t rows, int r, int max_ctas, bool fp32_engine) {
     const int c = qs_parts(rows, r, max_ctas);
     return qs_smem(qs_rows_per_part(rows, c), r, qs_threads(rows, r, max_ctas, fp32_engine)) <= QS_SMEM_LIMIT;
 }
-// CTAs per matrix in a call of `matrices` on a device with room for `room` CTAs.
-inline int qs_ctas(int64_t rows, int r, int max_ctas, int matrices, int room, int threads) {
+// CTAs per matrix in a call of `matrices`: the largest cluster of which all run at once.  room(size, per_sm): such clusters that
+// the device holds.  (Counted in CTAs, 128 of 148 multiprocessors for eight matrices in clusters of 16, of which seven
+// run at once: eight 4096 x 4096 at r = 32 104 us for both QRs, with two CTAs per multiprocessor 81.)
+template <class Room>
+inline int qs_ctas(int64_t rows, int r, int max_ctas, int matrices, int threads, Room room) {
     const int parts = qs_parts(rows, r, max_ctas), per = qs_rows_per_part(rows, parts);
     const int max_run = r > 32 ? 4 : 16;            // (tree levels held in registers)
     int c = parts;
-    while (c > 1 && (int64_t)matrices * c > room && parts / c < max_run && qs_smem((int64_t)per * (2 * parts / c), r, threads) <= QS_SMEM_LIMIT)
+    auto smem = [&](int ctas) { return qs_smem((int64_t)per * (parts / ctas), r, threads); };
+    while (c > 1 && matrices > room(c, threads == 256 && smem(c) <= QS_SMEM_TWO ? 2 : 1) && parts / c < max_run && smem(c / 2) <= QS_SMEM_LIMIT)
         c /= 2;
     return c;
 }
