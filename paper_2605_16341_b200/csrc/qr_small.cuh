@@ -63,14 +63,17 @@ inline int qs_parts(int64_t rows, int r, int max_ctas) {
     return c;
 }
 inline int qs_rows_per_part(int64_t rows, int parts) { return (int)((rows + parts * 32 - 1) / (parts * 32) * 32); }
+inline int64_t qs_smem(int64_t rows_per_cta, int r, int threads) { return rows_per_cta * qs_row_bytes(r) + qs_fixed(r, threads); }
 // Threads of a CTA, by the plan only (they decide how a Gram matrix is summed): 512, one CTA per multiprocessor, for parts
 // of 256 rows and more and for the fp32 engine above rank 32; else 256 and two.  Step with 256 and with 512 threads: 11008 x 4096 r = 32, Dion
 // 0.324 and 0.315 ms, 14336 x 4096 r = 16 0.365 and 0.361; 360 x 360 r = 32 0.0629 and 0.0640; 1023 x 777 r = 40, fp32 engine, 0.103 and
-// 0.099; 24 layers 640 wide at r = 64 1.21 and 1.28.
+// 0.099; 24 layers 640 wide at r = 64 1.21 and 1.28.  And 256 where the work area of 512 leaves the rows no room, up to 26112
+// rows at r = 32 and 41984 at r = 16: against separate kernels, 39700 x 512 r = 16 0.350 -> 0.274 ms, 41984 x 2048 0.620 -> 0.533,
+// 24320 x 512 r = 32 0.254 -> 0.239 (eight 25800 x 512 0.741 -> 0.759), 26112 x 512 r = 17 on the fp32 engine 0.868 -> 0.549.
 inline int qs_threads(int64_t rows, int r, int max_ctas, bool fp32_engine) {
-    return r > 32 ? (fp32_engine ? 512 : 256) : (qs_rows_per_part(rows, qs_parts(rows, r, max_ctas)) >= 256 ? 512 : 256);
+    const int per = qs_rows_per_part(rows, qs_parts(rows, r, max_ctas));
+    return (r > 32 ? fp32_engine : per >= 256) && qs_smem(per, r, 512) <= QS_SMEM_LIMIT ? 512 : 256;
 }
-inline int64_t qs_smem(int64_t rows_per_cta, int r, int threads) { return rows_per_cta * qs_row_bytes(r) + qs_fixed(r, threads); }
 // Whether the kernel takes a rows x r factor.  From r = 33 up only short ones: the fp32 products and the repeated
 // factorisations cost a call with many matrices more than the separate tensor-core kernels do, and the choice cannot
 // depend on the call (a matrix gets the same bits alone and in a group).  Step with separate kernels and with this one

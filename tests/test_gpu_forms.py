@@ -61,6 +61,16 @@ def test_one_kernel_qr_of_long_parts(shape, mode):
     one_step_compare(spec, X, M, G, Q, mode=mode, engine=od.ENGINE_TENSOR)
 
 
+# rows that only its 256-thread form has room for, up to the last ones: six launches still
+@pytest.mark.parametrize("shape", [(24320, 136, 32), (26112, 72, 32), (39700, 40, 16)])
+def test_one_kernel_qr_up_to_its_last_rows(shape):
+    m, n, r = shape
+    spec, X, M, G, Q = make_problem(m, n, r, BF16, F32, seed=m)
+    before = od.orthdion_launch_count()
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR)
+    assert od.orthdion_launch_count() == before + 6
+
+
 # a call of six kernels on either side of the size up to which its launches overlap
 @pytest.mark.parametrize("shape", [(4096, 2048, 32), (4104, 2048, 32)])
 def test_steps_back_to_back_at_the_largest_overlapping_size(shape):
