@@ -25,11 +25,11 @@ struct MatWork {
     int32_t aux1;       // and the scratch offset of the image of L in KB)
 };
 
-// Matrices per launch batch.  The table travels in the kernel parameters: a chain of empty kernels takes 3.7 us a launch with
+// Matrices of one launch.  The table travels in the kernel parameters: a chain of empty kernels takes 3.7 us a launch with
 // 17.6 KB of them (256 matrices), 2.3 with 4 KB, and the host 4.4 and 2.5 us.  256 -> 96: 28 matrices 1000 wide in four streams
-// 1.45 -> 1.39 ms a step, 520 x 384 r = 64 94 -> 91 us, host time of a 31-launch step 138 -> 79 us; 32: no further.  But a plan
-// with more matrices than that runs in two batches (128 of them, 1024 wide at r = 128 2.65 -> 2.73 ms): 128.
-constexpr int MAXB = 128;
+// 1.45 -> 1.39 ms a step, 520 x 384 r = 64 94 -> 91 us, host time of a 31-launch step 138 -> 79 us; 32: no further.  Hence kernels
+// with tables of two sizes, the smaller one up to 128 matrices.  (Larger classes in two launches of the
+// smaller one: 160 matrices 512 wide at r = 32 on one stream 0.393 -> 0.487 ms, 768 wide at r = 192 1.38 -> 1.64.)
 template <int CAP>
 struct BatchOf {
     int32_t count;
@@ -37,11 +37,9 @@ struct BatchOf {
     int64_t scratch_stride;   // w[k].scratch = w[0].scratch + k * scratch_stride (one class per batch)
     MatWork w[CAP];
 };
+constexpr int MAXB = 256, MAXB_SMALL = 128;
 using Batch = BatchOf<MAXB>;
-// Matrices of several classes in one launch of the factor kernel (calls that are stepped on one stream: a second launch
-// would wait for the first, a CTA per matrix: 154 matrices at r = 512 1.43 -> 1.77 ms of factorisations).
-constexpr int MAXB_MERGED = 256;
-using MergedBatch = BatchOf<MAXB_MERGED>;
+using SmallBatch = BatchOf<MAXB_SMALL>;
 
 // Where a kernel finds an fp32 matrix of one MatWork.
 enum Where : int32_t { W_Q = 0, W_P = 1, W_R = 2, W_SCRATCH = 3 };

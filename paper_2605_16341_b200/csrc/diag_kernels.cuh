@@ -29,7 +29,8 @@ __device__ __forceinline__ float* diag_record(const MatWork& w, const DiagBase& 
     return d.diag_base + (int64_t)(w.status - d.status_base) * DIAG_STRIDE;
 }
 
-__global__ void diag_init_kernel(const __grid_constant__ Batch batch, DiagBase d) {
+template <class BATCH>
+__global__ void diag_init_kernel(const __grid_constant__ BATCH batch, DiagBase d) {
     grid_dependency();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= batch.count * DIAG_STRIDE) return;
@@ -39,8 +40,9 @@ __global__ void diag_init_kernel(const __grid_constant__ Batch batch, DiagBase d
 // Column statistics of R and Q (both n x r fp32, row-major): stats[j] = sum_i R_ij^2,
 // stats[r + j] = sum_i R_ij Q_ij, stats[2r + j] = sum_i Q_ij^2.  One CTA per 32 columns, lanes
 // along columns.
+template <class BATCH>
 __global__ void __launch_bounds__(1024)
-diag_colstats_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t stats_off) {
+diag_colstats_kernel(const __grid_constant__ BATCH batch, int64_t n, int r, int64_t stats_off) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     __shared__ float part[3][32][33];
@@ -66,8 +68,9 @@ diag_colstats_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int6
 }
 
 // The same for r % 4 == 0: one CTA per 128 columns, a lane reads four adjacent columns.
+template <class BATCH>
 __global__ void __launch_bounds__(1024)
-diag_colstats4_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int64_t stats_off) {
+diag_colstats4_kernel(const __grid_constant__ BATCH batch, int64_t n, int r, int64_t stats_off) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     __shared__ __align__(16) float part[3][16][132];
@@ -108,8 +111,9 @@ diag_colstats4_kernel(const __grid_constant__ Batch batch, int64_t n, int r, int
 }
 
 // Sums of squares of M (fp32) and G over the whole matrix, accumulated in double.
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-diag_frob_kernel(const __grid_constant__ Batch batch, int64_t elems, int g_bf16, DiagBase d) {
+diag_frob_kernel(const __grid_constant__ BATCH batch, int64_t elems, int g_bf16, DiagBase d) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     const int64_t quads = elems / 4;
@@ -218,9 +222,9 @@ inline size_t diag_smem(int r) {
     return bytes <= DIAG_SMEM_LIMIT ? bytes : 0;                  // 0: the rows are read from memory
 }
 
-template <bool SMEM>
+template <class BATCH, bool SMEM>
 __global__ void __launch_bounds__(DIAG_THREADS)
-diag_final_kernel(const __grid_constant__ Batch batch, int r, int64_t gram_off, int64_t stats_off, int mask,
+diag_final_kernel(const __grid_constant__ BATCH batch, int r, int64_t gram_off, int64_t stats_off, int mask,
                   float ef_a, float ef_b, DiagBase d, int csize) {
     grid_dependency();
     const int crank = (int)(blockIdx.x % (unsigned)csize);

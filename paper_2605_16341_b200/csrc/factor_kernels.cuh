@@ -31,8 +31,9 @@ struct CholArgs {
 
 // ---- ColNorm of the SIMT engine (Alg. 1, normalisation step, Dion branch): Q[:,j] = R[:,j] / ||R[:,j]||_2 ---
 // One CTA per 32 columns: 32 x 32 threads, lanes along columns (coalesced rows).
+template <class BATCH>
 __global__ void __launch_bounds__(1024)
-colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r) {
+colnorm_kernel(const __grid_constant__ BATCH batch, int64_t n, int r) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
@@ -65,8 +66,9 @@ colnorm_kernel(const __grid_constant__ Batch batch, int64_t n, int r) {
 // core's truncating accumulation would bias it low), so that a sum of it over shards carries the exact diagonal along.
 // One CTA per 64 columns: 16 interleaved sums per column, eight loads of each under way (latency is all there is: a serial
 // loop took 11.5 us for 3584 rows at r = 512).
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-colsum_kernel(const __grid_constant__ Batch batch, int64_t colsq_off, int blocks, int r, Sel dst, int64_t stride) {
+colsum_kernel(const __grid_constant__ BATCH batch, int64_t colsq_off, int blocks, int r, Sel dst, int64_t stride) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
@@ -100,7 +102,7 @@ colsum_kernel(const __grid_constant__ Batch batch, int64_t colsq_off, int blocks
 // product kernels write next to their results: out[blk * r + j], blk < 4 * ceil(rows / 128)
 // (blocks beyond the matrix hold zeros).  One CTA per (32-row block, 256 columns).
 __global__ void __launch_bounds__(256)
-colsq_blocks_kernel(const __grid_constant__ Batch batch, Sel src, int64_t rows, int r, int64_t colsq_off) {
+colsq_blocks_kernel(const __grid_constant__ SmallBatch batch, Sel src, int64_t rows, int r, int64_t colsq_off) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
@@ -115,7 +117,8 @@ colsq_blocks_kernel(const __grid_constant__ Batch batch, Sel src, int64_t rows, 
     out[(int64_t)blockIdx.x * r + j] = s;
 }
 
-__global__ void init_status_kernel(const __grid_constant__ Batch batch) {
+template <class BATCH>
+__global__ void init_status_kernel(const __grid_constant__ BATCH batch) {
     grid_dependency();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < batch.count) *batch.w[i].status = 0;

@@ -21,8 +21,9 @@ constexpr int FS_OFF_X = 4 * SIMT_KC * SIMT_LD * 4;      // X_k transposed, afte
 constexpr int FS_OFF_D = FS_OFF_X + CT_NB * SIMT_LD * 4;     // the diagonal block's area
 constexpr int FS_SMEM_BYTES = FS_OFF_D + CT_DG_BYTES;
 
+template <class BATCH>
 __global__ void __launch_bounds__(FS_THREADS, 2)
-factor_simt_kernel(const __grid_constant__ Batch batch, CholArgs a) {
+factor_simt_kernel(const __grid_constant__ BATCH batch, CholArgs a) {
     extern __shared__ __align__(16) unsigned char smem[];
     SimtStage* As = reinterpret_cast<SimtStage*>(smem);
     SimtStage* Bs = As + 2;

@@ -7,6 +7,10 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <type_traits>
+
+#include "common.cuh"
 #include "profile.cuh"
 
 namespace od {
@@ -48,6 +52,18 @@ inline void launch(void (*kernel)(KArgs...), dim3 grid, int block, size_t smem, 
     cfg.numAttrs = (unsigned)n;
     prof::Scope scope(stage, st);
     if (cudaLaunchKernelEx(&cfg, kernel, args...) != cudaSuccess && !engine_error()) engine_error() = LAUNCH_FAILED;
+}
+
+// f(table) with the smaller table where it holds the matrices; table_t<decltype(table)>: its type.
+template <class T>
+using table_t = std::decay_t<T>;
+template <class F>
+inline void with_table(const Batch& b, F f) {
+    if (b.count > MAXB_SMALL) { f(b); return; }
+    SmallBatch s;
+    s.count = b.count; s.pad = 0; s.scratch_stride = b.scratch_stride;
+    std::copy(b.w, b.w + b.count, s.w);
+    f(s);
 }
 
 }  // namespace od

@@ -241,8 +241,9 @@ int clusters_at_once(K* kernel, int threads, size_t smem, int size, int per_sm) 
 }
 
 // by rank (16, 32, 64) and threads (256, 512)
-void (*const kQrSmall[6])(Batch, QrSmallArgs) = {qr_small_kernel<16, 256>, qr_small_kernel<16, 512>, qr_small_kernel<32, 256>,
-                                                 qr_small_kernel<32, 512>, qr_small_kernel<64, 256>, qr_small_kernel<64, 512>};
+template <class BATCH>
+void (*const kQrSmall[6])(BATCH, QrSmallArgs) = {qr_small_kernel<BATCH, 16, 256>, qr_small_kernel<BATCH, 16, 512>, qr_small_kernel<BATCH, 32, 256>,
+                                                 qr_small_kernel<BATCH, 32, 512>, qr_small_kernel<BATCH, 64, 256>, qr_small_kernel<BATCH, 64, 512>};
 
 int ensure_attributes() {
     static std::mutex mu;
@@ -252,26 +253,33 @@ int ensure_attributes() {
     if (dev < 0 || dev >= kMaxDevices) return ORTHDION_ERR_CUDA;
     std::lock_guard<std::mutex> lock(mu);
     if (state[dev]) return state[dev] > 0 ? 0 : ORTHDION_ERR_CUDA;
-    cudaError_t e = cudaFuncSetAttribute(factor_simt_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, FS_SMEM_BYTES);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel<Batch, CT_STAGES>, cudaFuncAttributeMaxDynamicSharedMemorySize, ct_smem_bytes(CT_STAGES));
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(factor_kernel<MergedBatch, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, ct_smem_bytes(2));
+    cudaError_t e = cudaSuccess;
+    auto set = [&](auto* kernel, size_t smem) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    };
+    set(factor_simt_kernel<SmallBatch>, FS_SMEM_BYTES);
+    set(factor_simt_kernel<Batch>, FS_SMEM_BYTES);
+    set(factor_kernel<SmallBatch, CT_STAGES>, ct_smem_bytes(CT_STAGES));
+    set(factor_kernel<Batch, 2>, ct_smem_bytes(2));
+    set(diag_final_kernel<SmallBatch, true>, DIAG_SMEM_LIMIT);
+    set(diag_final_kernel<Batch, true>, DIAG_SMEM_LIMIT);
     g_qr_cluster_max[dev] = 16;
-    for (int k = 0; k < 6 && e == cudaSuccess; ++k) {
-        e = cudaFuncSetAttribute(kQrSmall[k], cudaFuncAttributeMaxDynamicSharedMemorySize, QS_SMEM_LIMIT);
-        if (e == cudaSuccess)
-            g_qr_cluster_max[dev] = (signed char)std::min<int>(g_qr_cluster_max[dev], largest_cluster(kQrSmall[k], k % 2 ? 512 : 256, QS_SMEM_LIMIT));
+    for (int k = 0; k < 6; ++k) {
+        set(kQrSmall<SmallBatch>[k], QS_SMEM_LIMIT);
+        set(kQrSmall<Batch>[k], QS_SMEM_LIMIT);
+        if (e != cudaSuccess) break;
+        const int threads = k % 2 ? 512 : 256;
+        g_qr_cluster_max[dev] = (signed char)std::min<int>({g_qr_cluster_max[dev], largest_cluster(kQrSmall<SmallBatch>[k], threads, QS_SMEM_LIMIT),
+                                                            largest_cluster(kQrSmall<Batch>[k], threads, QS_SMEM_LIMIT)});
     }
     if (e == cudaSuccess) {
-        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<Batch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES));
+        g_factor_cluster_max[dev] = (signed char)largest_cluster(factor_kernel<SmallBatch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES));
         // (one per multiprocessor: the factor kernel.  Two: the one-kernel QR with 256 threads and little memory.)
         for (int l = 0; l < 5; ++l) {
-            g_clusters_at_once[dev][0][l] = clusters_at_once(factor_kernel<Batch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES), 1 << l, 1);
-            g_clusters_at_once[dev][1][l] = clusters_at_once(kQrSmall[2], 256, QS_SMEM_TWO, 1 << l, 2);
+            g_clusters_at_once[dev][0][l] = clusters_at_once(factor_kernel<SmallBatch, CT_STAGES>, CT_THREADS, ct_smem_bytes(CT_STAGES), 1 << l, 1);
+            g_clusters_at_once[dev][1][l] = clusters_at_once(kQrSmall<SmallBatch>[2], 256, QS_SMEM_TWO, 1 << l, 2);
         }
     }
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(diag_final_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)DIAG_SMEM_LIMIT);
     if (e == cudaSuccess) e = tensor_engine_set_attributes();
     if (e != cudaSuccess) {
         std::fprintf(stderr, "orthdion: kernel attribute setup failed on device %d: %s\n", dev, cudaGetErrorString(e));
@@ -337,8 +345,10 @@ DeviceLanes* device_lanes() {
 template <class RA, class RB>
 void launch_simt(const Batch& b, int64_t Md, int64_t Nd, int64_t Kd, RA ra, RB rb, SimtOut out, int stage, cudaStream_t st) {
     const int parts = simt_parts(Kd);
-    launch(simt_gemm_kernel<RA, RB>, dim3((unsigned)((Nd + 63) / 64 * parts), (unsigned)((Md + 63) / 64), (unsigned)b.count), 256, 0,
-           parts, stage, st, b, Md, Nd, Kd, parts, ra, rb, out);
+    with_table(b, [&](const auto& t) {
+        launch(simt_gemm_kernel<table_t<decltype(t)>, RA, RB>, dim3((unsigned)((Nd + 63) / 64 * parts), (unsigned)((Md + 63) / 64), (unsigned)b.count),
+               256, 0, parts, stage, st, t, Md, Nd, Kd, parts, ra, rb, out);
+    });
 }
 
 // What became of the launches since engine_error() was reset.  Clears the runtime's last error, so that a launch
@@ -362,19 +372,11 @@ struct ClassRun {
     bool tensor() const { return p->engine == ORTHDION_ENGINE_TENSOR; }
 };
 
-// (of at most MAXB matrices)
-Batch narrow(const MergedBatch& m) {
-    Batch b;
-    b.count = m.count; b.pad = 0; b.scratch_stride = m.scratch_stride;
-    std::copy(m.w, m.w + m.count, b.w);
-    return b;
-}
-
 // Cholesky + inverse of every class's Gram matrix: classes of equal (r, engine) share launches.
 // diag_from_gram: take the diagonal from the Gram matrix itself instead of the column-square
 // partials of the producing kernel (column-sharded matrices: the reduced Gram matrix carries it).
 void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, int which, int pass,
-                MergedBatch* merged, int call_matrices, cudaStream_t st, bool diag_from_gram = false) {
+                Batch* merged, int call_matrices, cudaStream_t st, bool diag_from_gram = false) {
     std::vector<char> done(which_cls.size(), 0);
     for (size_t i = 0; i < which_cls.size(); ++i) {
         if (done[i]) continue;
@@ -409,10 +411,15 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 while (csize < cluster_max(g_factor_cluster_max) && csize < tiles &&
                        std::max(merged->count, call_matrices) <= room_for_clusters(csize * 2, 1)) csize *= 2;
                 const dim3 grid((unsigned)(merged->count * csize));
-                if (merged->count > MAXB) launch(factor_kernel<MergedBatch, 2>, grid, CT_THREADS, ct_smem_bytes(2), csize, prof::S_CHOL, st, *merged, ca, csize);
-                else launch(factor_kernel<Batch, CT_STAGES>, grid, CT_THREADS, ct_smem_bytes(CT_STAGES), csize, prof::S_CHOL, st, narrow(*merged), ca, csize);
+                with_table(*merged, [&](const auto& t) {
+                    using BATCH = table_t<decltype(t)>;
+                    constexpr int stages = std::is_same<BATCH, SmallBatch>::value ? CT_STAGES : 2;
+                    launch(factor_kernel<BATCH, stages>, grid, CT_THREADS, ct_smem_bytes(stages), csize, prof::S_CHOL, st, t, ca, csize);
+                });
             } else {
-                launch(factor_simt_kernel, dim3((unsigned)merged->count), FS_THREADS, FS_SMEM_BYTES, 1, prof::S_CHOL, st, narrow(*merged), ca);
+                with_table(*merged, [&](const auto& t) {
+                    launch(factor_simt_kernel<table_t<decltype(t)>>, dim3((unsigned)merged->count), FS_THREADS, FS_SMEM_BYTES, 1, prof::S_CHOL, st, t, ca);
+                });
             }
             merged->count = 0;
         };
@@ -426,7 +433,7 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 w = c.b->w[k];
                 w.aux0 = (int32_t)(4 * ((rows + 127) / 128));
                 w.aux1 = c.tensor() ? (int32_t)(c.sc.ts.q.off / 1024) : 0;
-                if (merged->count == (lead.tensor() ? MAXB_MERGED : MAXB)) flush();
+                if (merged->count == MAXB) flush();
             }
         }
         flush();
@@ -488,15 +495,17 @@ void small_qr_stage(ClassRun& c, int which, int splits, int call_matrices, cudaS
     }
     const size_t smem = (size_t)qs_smem((int64_t)a.rows_per_part * a.parts_per_cta, p->r, threads);
     const int width = qs_width(p->r);
-    launch(kQrSmall[(width == 16 ? 0 : width == 32 ? 2 : 4) + (threads == 512)], dim3((unsigned)(c.b->count * a.csize)), threads, smem, a.csize,
-           prof::S_QR, st, *c.b, a);
+    with_table(*c.b, [&](const auto& t) {
+        launch(kQrSmall<table_t<decltype(t)>>[(width == 16 ? 0 : width == 32 ? 2 : 4) + (threads == 512)], dim3((unsigned)(c.b->count * a.csize)),
+               threads, smem, a.csize, prof::S_QR, st, t, a);
+    });
 }
 
 // ---- tall-skinny QR of every class in `which_cls` (CholeskyQR2; third pass when flagged) --------
 // which = 0: P = orth(Y) (Alg. 1, left-factor step), which = 1: Q = orth(R) (Alg. 1, normalisation step).
 // Tensor engine: the input is an image (w0 holds Y, image r holds R), or what small_qr_stage reads; SIMT
 // engine: fp32 slots.  summed: the fp32 slot holds the input even where the product is split by depth.
-void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int which, MergedBatch* merged,
+void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int which, Batch* merged,
               int call_matrices, cudaStream_t st, bool summed = false) {
     const int shift_bit = which ? ST_SHIFT_R : ST_SHIFT_L;
     std::vector<int> which_cls;
@@ -571,7 +580,9 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
     const int r = p->r;
     const Sel gram = sel(W_SCRATCH, c.sc.gram);
     const int64_t stats_off = c.sc.linv;          // 3 r floats of the (now free) inverse slot
-    launch(diag_init_kernel, dim3((unsigned)((b.count * DIAG_STRIDE + 255) / 256)), 256, 0, 1, prof::S_DIAG, st, b, db);
+    with_table(b, [&](const auto& t) {
+        launch(diag_init_kernel<table_t<decltype(t)>>, dim3((unsigned)((b.count * DIAG_STRIDE + 255) / 256)), 256, 0, 1, prof::S_DIAG, st, t, db);
+    });
     if (c.tensor()) {
         tensor_gram(r, p->passes[1], b, c.sc.ts.q, p->n, gram, sel(W_SCRATCH, c.sc.gram_part), c.sc.ts.gram_parts_n, 0, st);
     } else {
@@ -579,27 +590,32 @@ void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
         launch_simt(b, r, r, p->n, RdPlain{sQ, 1, r}, RdPlain{sQ, 1, r}, SimtOut{gram, gram, 0, 1, r, 0, 0},
                     prof::S_GRAM, st);
     }
-    if (r % 4 == 0)
-        launch(diag_colstats4_kernel, dim3((unsigned)((r + 127) / 128), 1, (unsigned)b.count), 1024, 0, 1, prof::S_DIAG, st, b, p->n, r,
-               stats_off);
-    else
-        launch(diag_colstats_kernel, dim3((unsigned)((r + 31) / 32), 1, (unsigned)b.count), 1024, 0, 1, prof::S_DIAG, st, b, p->n, r,
-               stats_off);
+    with_table(b, [&](const auto& t) {
+        using BATCH = table_t<decltype(t)>;
+        const int cols = r % 4 == 0 ? 128 : 32;
+        launch(r % 4 == 0 ? diag_colstats4_kernel<BATCH> : diag_colstats_kernel<BATCH>, dim3((unsigned)((r + cols - 1) / cols), 1, (unsigned)b.count),
+               1024, 0, 1, prof::S_DIAG, st, t, p->n, r, stats_off);
+    });
     if (p->diag & 2) {
         const int64_t elems = p->m * p->n;
         const int64_t want = (elems / 4 + 256 * 32 - 1) / (256 * 32);
         dim3 grid((unsigned)std::max<int64_t>(1, std::min<int64_t>(want, 1184 / std::max(1, b.count) + 1)), 1,
                   (unsigned)b.count);
-        launch(diag_frob_kernel, grid, 256, 0, 1, prof::S_DIAG, st, b, elems, (int)(p->g_dtype == ORTHDION_DTYPE_BF16), db);
+        with_table(b, [&](const auto& t) {
+            launch(diag_frob_kernel<table_t<decltype(t)>>, grid, 256, 0, 1, prof::S_DIAG, st, t, elems, (int)(p->g_dtype == ORTHDION_DTYPE_BF16), db);
+        });
     }
     const int csize = diag_cluster(r);
     const size_t smem = diag_smem(r);
-    launch(smem ? diag_final_kernel<true> : diag_final_kernel<false>, dim3((unsigned)(b.count * csize)), DIAG_THREADS, smem, csize, prof::S_DIAG, st,
-           b, r, c.sc.gram, stats_off, p->diag, p->ef_a, p->ef_b, db, csize);
+    with_table(b, [&](const auto& t) {
+        using BATCH = table_t<decltype(t)>;
+        launch(smem ? diag_final_kernel<BATCH, true> : diag_final_kernel<BATCH, false>, dim3((unsigned)(b.count * csize)), DIAG_THREADS, smem, csize,
+               prof::S_DIAG, st, t, r, c.sc.gram, stats_off, p->diag, p->ef_a, p->ef_b, db, csize);
+    });
 }
 
 // One step of every class of a group, stage by stage.
-void run_group(std::vector<ClassRun>& cls, MergedBatch* merged, DiagBase db, int call_matrices, cudaStream_t st) {
+void run_group(std::vector<ClassRun>& cls, Batch* merged, DiagBase db, int call_matrices, cudaStream_t st) {
     const Sel sP = sel(W_P), sR = sel(W_R), sQ = sel(W_Q);
     std::vector<int> all, orth;
     for (size_t i = 0; i < cls.size(); ++i) {
@@ -607,7 +623,10 @@ void run_group(std::vector<ClassRun>& cls, MergedBatch* merged, DiagBase db, int
         if (cls[i].p->mode == ORTHDION_MODE_ORTH) orth.push_back((int)i);
     }
     for (ClassRun& c : cls)
-        if (!c.tensor()) launch(init_status_kernel, dim3((unsigned)((c.b->count + 255) / 256)), 256, 0, 1, prof::S_MISC, st, *c.b);
+        if (!c.tensor())
+            with_table(*c.b, [&](const auto& t) {
+                launch(init_status_kernel<table_t<decltype(t)>>, dim3((unsigned)((t.count + 255) / 256)), 256, 0, 1, prof::S_MISC, st, t);
+            });
     // Alg. 1, buffer and left-factor steps:  Y = (M + G) Q_prev
     for (ClassRun& c : cls) {
         const orthdion_plan* p = c.p;
@@ -640,8 +659,10 @@ void run_group(std::vector<ClassRun>& cls, MergedBatch* merged, DiagBase db, int
             launch_colsum(*c.b, c.sc.ts, p->n, p->r, sel(W_SCRATCH, c.sc.ts.cnorm), 1, prof::S_COLNORM, st);
             launch_pack_right(*c.b, p->n, p->r, c.sc.ts, fused_fp16(p), q_planes(p), st);
         } else {
-            launch(colnorm_kernel, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)c.b->count), 1024, 0, 1, prof::S_COLNORM, st, *c.b,
-                   p->n, p->r);
+            with_table(*c.b, [&](const auto& t) {
+                launch(colnorm_kernel<table_t<decltype(t)>>, dim3((unsigned)((p->r + 31) / 32), 1, (unsigned)t.count), 1024, 0, 1, prof::S_COLNORM,
+                       st, t, p->n, p->r);
+            });
         }
     }
     // Alg. 1, update and error-feedback steps:  M <- a B - b P R^T ;  X <- c X - d P Q^T
@@ -656,7 +677,9 @@ void run_group(std::vector<ClassRun>& cls, MergedBatch* merged, DiagBase db, int
                       c.sc.ts, st);
         } else {
             dim3 grid((unsigned)((p->n + 63) / 64), (unsigned)((p->m + 63) / 64), (unsigned)c.b->count);
-            launch(simt_update_kernel, grid, 256, 0, 1, prof::S_K5, st, *c.b, p->m, p->n, p->r, p->ef_a, p->ef_b, cc, dd, gb, xb);
+            with_table(*c.b, [&](const auto& t) {
+                launch(simt_update_kernel<table_t<decltype(t)>>, grid, 256, 0, 1, prof::S_K5, st, t, p->m, p->n, p->r, p->ef_a, p->ef_b, cc, dd, gb, xb);
+            });
         }
     }
     for (ClassRun& c : cls)
@@ -817,29 +840,36 @@ int orthdion_step_grouped(const orthdion_t* hs, int32_t count, void* const* X, f
 
     cudaStream_t st = reinterpret_cast<cudaStream_t>(stream);
     char* ws = reinterpret_cast<char*>(workspace);
-    std::vector<Batch> pool(bt.batches.size());
-    const std::unique_ptr<MergedBatch> merged_batch(new MergedBatch);
-    MergedBatch* merged = merged_batch.get();
+    const std::unique_ptr<Batch[]> pool(new Batch[2 * bt.batches.size() + 1]);      // (not cleared: 18 KB each)
+    Batch *merged = &pool[2 * bt.batches.size()], *next_batch = pool.get();
     int rc = ORTHDION_OK;
     for (const auto& grp : bt.groups) {
         std::vector<ClassRun> cls;
+        // One class alone, and large: two halves on two internal streams.  Steps of 160 matrices, on one and on two: 512 wide r = 32 0.395
+        // and 0.359 ms, 768 wide r = 192 1.39 and 1.32.  (Both halves on one stream: 0.487 and 1.64.  Beside other classes: 34 layers 768 wide
+        // at r = 192 2.88 -> 2.95, 80 layers 512 wide at r = 128 2.86 -> 2.99, two classes of 160 and 140 at r = 128 1.19 -> 1.30.)
+        const bool halves = grp.size() == 1 && g_lanes.load() > 1;
         for (int bi : grp) {
             const auto& idx = bt.batches[bi];
-            ClassRun c{hs[idx[0]], &pool[bi], scratch_layout(hs[idx[0]], count, bt.lean)};
-            c.b->count = (int32_t)idx.size();
-            c.b->pad = 0;
-            c.b->scratch_stride = (int64_t)c.sc.bytes;
-            for (size_t k = 0; k < idx.size(); ++k) {
-                const int i = idx[k];
-                MatWork& w = c.b->w[k];
-                w.X = X[i]; w.M = M[i]; w.G = G[i]; w.Q = Q[i];
-                w.P = reinterpret_cast<float*>(ws + lay.p_off[i]);
-                w.R = reinterpret_cast<float*>(ws + lay.r_off[i]);
-                w.status = reinterpret_cast<int32_t*>(ws + lay.status_off) + i;
-                w.scratch = ws + lay.scratch_off + bt.batch_off[bi] + k * c.sc.bytes;
-                w.aux0 = 0; w.aux1 = 0;
+            const Scratch sc = scratch_layout(hs[idx[0]], count, bt.lean);
+            const size_t most = halves && idx.size() > MAXB_SMALL ? (idx.size() + 1) / 2 : idx.size();
+            for (size_t k0 = 0; k0 < idx.size(); k0 += most) {
+                ClassRun c{hs[idx[0]], next_batch++, sc};
+                c.b->count = (int32_t)std::min(most, idx.size() - k0);
+                c.b->pad = 0;
+                c.b->scratch_stride = (int64_t)sc.bytes;
+                for (int k = 0; k < c.b->count; ++k) {
+                    const int i = idx[k0 + k];
+                    MatWork& w = c.b->w[k];
+                    w.X = X[i]; w.M = M[i]; w.G = G[i]; w.Q = Q[i];
+                    w.P = reinterpret_cast<float*>(ws + lay.p_off[i]);
+                    w.R = reinterpret_cast<float*>(ws + lay.r_off[i]);
+                    w.status = reinterpret_cast<int32_t*>(ws + lay.status_off) + i;
+                    w.scratch = ws + lay.scratch_off + bt.batch_off[bi] + (k0 + k) * sc.bytes;
+                    w.aux0 = 0; w.aux1 = 0;
+                }
+                cls.push_back(c);
             }
-            cls.push_back(c);
         }
         engine_error() = 0;
         const DiagBase db{reinterpret_cast<const int32_t*>(ws + lay.status_off),
@@ -967,7 +997,7 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
     const int r = p->r;
     std::vector<ClassRun> cls(1, sr->c);
     const std::vector<int> only(1, 0);
-    MergedBatch* merged = new MergedBatch;
+    Batch* merged = new Batch;
     engine_error() = 0;
     overlap_launches() = overlap_pays(&h, 1);
     if (phase == 0) {
@@ -976,8 +1006,11 @@ int orthdion_shard_phase(orthdion_t h, int32_t phase, void* X, float* M, const v
         // the summed Y sits in the P slot: image and column squares, then the usual left QR
         if (!small_qr(p, p->m)) {
             launch_pack(sr->batch, sel(W_P), p->m, r, img_view(ts.w0, p->m), st);
-            launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((p->m + 127) / 128)), (unsigned)((r + 255) / 256)), 256, 0, 1, prof::S_MISC,
-                   st, sr->batch, sel(W_P), p->m, r, ts.colsq);
+            with_table(sr->batch, [&](const auto& t) {
+                if constexpr (std::is_same<table_t<decltype(t)>, SmallBatch>::value)         // (one matrix)
+                    launch(colsq_blocks_kernel, dim3((unsigned)(4 * ((p->m + 127) / 128)), (unsigned)((r + 255) / 256)), 256, 0, 1, prof::S_MISC,
+                           st, t, sel(W_P), p->m, r, ts.colsq);
+            });
         }
         qr_stage(cls, only, 0, merged, 1, st, true);
         tensor_k3(p->m, p->n, r, gb, p->passes[0], sr->batch, ts, sel(W_SCRATCH, sr->c.sc.gram_part), st,

@@ -109,9 +109,9 @@ __device__ __forceinline__ void qs_st_remote4(uint32_t addr, const float4& v) {
     asm volatile("st.shared::cluster.v4.f32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w) : "memory");
 }
 
-template <int R, int QS_THREADS>
+template <class BATCH, int R, int QS_THREADS>
 __global__ void __launch_bounds__(QS_THREADS, 512 / QS_THREADS)
-qr_small_kernel(const __grid_constant__ Batch batch, const __grid_constant__ QrSmallArgs a) {
+qr_small_kernel(const __grid_constant__ BATCH batch, const __grid_constant__ QrSmallArgs a) {
     constexpr int LD = R == 32 ? 32 : R + 4;         // row stride: no bank conflicts in either product
     constexpr int TX = R / 4;                        // threads along the columns of a 4 x 4-blocked product
     constexpr int GROUPS = QS_THREADS / (TX * TX);   // Gram product: thread groups that share the rows

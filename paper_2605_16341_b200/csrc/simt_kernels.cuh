@@ -122,9 +122,9 @@ __device__ __forceinline__ void simt_fma(float (&acc)[4][4], const SimtStage& a,
 // C(i,j) = sum_k A(i,k) * Bm(j,k): both operands are read as (row, depth).
 // 64 x 64 tile per cluster of `parts` CTAs (chunk `rank` of the depth each), 256 threads, 4 x 4
 // results per thread.
-template <class RA, class RB>
+template <class BATCH, class RA, class RB>
 __global__ void __launch_bounds__(256)
-simt_gemm_kernel(const __grid_constant__ Batch batch, int64_t Md, int64_t Nd, int64_t Kd, int parts, RA ra, RB rb, SimtOut out) {
+simt_gemm_kernel(const __grid_constant__ BATCH batch, int64_t Md, int64_t Nd, int64_t Kd, int parts, RA ra, RB rb, SimtOut out) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     const int st = *w.status;
@@ -195,8 +195,9 @@ simt_gemm_kernel(const __grid_constant__ Batch batch, int64_t Md, int64_t Nd, in
 
 // M <- a (M + G) - b P R^T,  X <- c X - d P Q^T  (Alg. 1, update and error-feedback steps): both products
 // in one pass, P read once.  64 x 64 tile per CTA.
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-simt_update_kernel(const __grid_constant__ Batch batch, int64_t m, int64_t n, int r, float a, float b, float c, float d,
+simt_update_kernel(const __grid_constant__ BATCH batch, int64_t m, int64_t n, int r, float a, float b, float c, float d,
                    int g_bf16, int x_bf16) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];

@@ -342,8 +342,9 @@ struct PackArgs {
     int32_t init, pad;      // first kernel of a step: clears the status word instead of reading it
 };
 
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-pack_kernel(const __grid_constant__ Batch batch, PackArgs a) {
+pack_kernel(const __grid_constant__ BATCH batch, PackArgs a) {
     // (the first product, which follows, reads M and G before it waits: it may not start while the step before is at work)
     grid_dependency_wait();
     grid_dependency_launch();
@@ -409,8 +410,9 @@ struct PackRightArgs {
     int64_t cnorm_off, rscale_off;
 };
 
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-pack_right_kernel(const __grid_constant__ Batch batch, PackRightArgs a) {
+pack_right_kernel(const __grid_constant__ BATCH batch, PackRightArgs a) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
@@ -471,8 +473,8 @@ struct StatusCache { int b = -1; int st = 0; };
 // the number of tiles is odd: that CTA multiplies zeros and stores nothing).
 template <bool V> struct BoolConst { static constexpr bool value = V; };
 
-template <int EPI>
-__device__ __forceinline__ TileCoord decode_tile(const Batch& batch, const GemmArgs& g, int t, StatusCache& sc,
+template <int EPI, class BATCH>
+__device__ __forceinline__ TileCoord decode_tile(const BATCH& batch, const GemmArgs& g, int t, StatusCache& sc,
                                                  int rank, bool look = true) {         // look: at the status word (`active` counts)
     TileCoord c;
     const int per = g.m_tiles * g.n_tiles * g.ksplit;
@@ -523,9 +525,9 @@ __device__ __forceinline__ int mn_pieces(const GemmArgs& g, int kb) {
 // RUN    the tiles come in runs (GemmArgs::run): the Gram product, and products with B that have more chunks than
 //        accumulators.  (Instantiations of their own for the latter: the test for a run alone cost the other
 //        products with B up to 1 % of a step, in registers that the transform warps then lack.)
-template <int AMODE, int NMODE, int EPI, int XG, bool PAIR, bool RUN>
+template <class BATCH, int AMODE, int NMODE, int EPI, int XG, bool PAIR, bool RUN>
 __global__ void __launch_bounds__(gemm_threads(AMODE, EPI), 1)
-gemm_kernel(const __grid_constant__ Batch batch, const __grid_constant__ GemmArgs g) {
+gemm_kernel(const __grid_constant__ BATCH batch, const __grid_constant__ GemmArgs g) {
     constexpr int NE = epi_warps(AMODE, EPI);
     // PAIR: launched in clusters of two; rank 0 (the leader) issues every MMA for both CTAs
     const int crank = PAIR ? (int)cluster_ctarank() : 0;
@@ -1575,19 +1577,19 @@ constexpr bool pair_capable(int nmode, int epi, int xg) {
     return nmode == tc::N_IMG_MN || (epi == tc::EPI_K5 && xg == 3);
 }
 
-template <int AMODE, int NMODE, int EPI, int XG>
+template <class BATCH, int AMODE, int NMODE, int EPI, int XG>
 inline cudaError_t set_gemm_attr() {
     constexpr bool GRAM = AMODE == tc::A_IMG_MN;
-    cudaError_t e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, GRAM>,
+    cudaError_t e = cudaFuncSetAttribute(tc::gemm_kernel<BATCH, AMODE, NMODE, EPI, XG, false, GRAM>,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
     if constexpr (pair_capable(NMODE, EPI, XG)) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true, GRAM>,
+            e = cudaFuncSetAttribute(tc::gemm_kernel<BATCH, AMODE, NMODE, EPI, XG, true, GRAM>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
     }
     if constexpr (tc::a_is_buf(AMODE)) {
         if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, true>,
+            e = cudaFuncSetAttribute(tc::gemm_kernel<BATCH, AMODE, NMODE, EPI, XG, false, true>,
                                      cudaFuncAttributeMaxDynamicSharedMemorySize, tc::SMEM_LIMIT);
     }
     return e;
@@ -1595,7 +1597,8 @@ inline cudaError_t set_gemm_attr() {
 
 inline cudaError_t tensor_engine_set_attributes() {
     cudaError_t e;
-#define OD_SET(...) if ((e = set_gemm_attr<__VA_ARGS__>()) != cudaSuccess) return e;
+#define OD_SET(...) \
+    if ((e = set_gemm_attr<SmallBatch, __VA_ARGS__>()) != cudaSuccess || (e = set_gemm_attr<Batch, __VA_ARGS__>()) != cudaSuccess) return e;
     OD_SET(tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 0)
     OD_SET(tc::A_BUF_ROW, tc::N_IMG_MN, tc::EPI_STORE, 1)
     OD_SET(tc::A_BUF_COL, tc::N_IMG_MN, tc::EPI_STORE, 0)
@@ -1616,12 +1619,16 @@ inline void launch_pack_right(const Batch& b, int64_t rows, int64_t cols, const 
     a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.r_img = ts.r; a.q_img = ts.q; a.r_half = half ? 1 : 0; a.normalise = normalise;
     a.cnorm_off = ts.cnorm; a.rscale_off = ts.rscale;
     dim3 grid((unsigned)ts.r.panels, (unsigned)(ts.r.rows_pad / 128), (unsigned)b.count);
-    launch(tc::pack_right_kernel, grid, 256, 0, 1, normalise ? prof::S_COLNORM : prof::S_PACK, st, b, a);
+    with_table(b, [&](const auto& t) {
+        launch(tc::pack_right_kernel<table_t<decltype(t)>>, grid, 256, 0, 1, normalise ? prof::S_COLNORM : prof::S_PACK, st, t, a);
+    });
 }
 // the column squares of `rows` rows, added up
 inline void launch_colsum(const Batch& b, const TensorScratch& ts, int64_t rows, int r, Sel dst, int64_t stride, int stage, cudaStream_t st) {
-    launch(colsum_kernel, dim3((unsigned)((r + 63) / 64), 1, (unsigned)b.count), 256, 0, 1, stage, st, b, ts.colsq,
-           (int)(4 * ((rows + 127) / 128)), r, dst, stride);
+    with_table(b, [&](const auto& t) {
+        launch(colsum_kernel<table_t<decltype(t)>>, dim3((unsigned)((r + 63) / 64), 1, (unsigned)b.count), 256, 0, 1, stage, st, t, ts.colsq,
+               (int)(4 * ((rows + 127) / 128)), r, dst, stride);
+    });
 }
 
 inline void launch_pack(const Batch& b, Sel src, int64_t rows, int64_t cols, ImgRef dst, cudaStream_t st, bool init = false) {
@@ -1629,7 +1636,7 @@ inline void launch_pack(const Batch& b, Sel src, int64_t rows, int64_t cols, Img
     a.init = init ? 1 : 0;
     a.src = src; a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.dst = dst;
     dim3 grid((unsigned)dst.panels, (unsigned)(dst.rows_pad / 128), (unsigned)b.count);
-    launch(tc::pack_kernel, grid, 256, 0, 1, prof::S_PACK, st, b, a);
+    with_table(b, [&](const auto& t) { launch(tc::pack_kernel<table_t<decltype(t)>>, grid, 256, 0, 1, prof::S_PACK, st, t, a); });
 }
 
 // Fills in the tiling, ring and tensor-memory fields and launches.
@@ -1728,21 +1735,24 @@ inline void launch_gemm(const Batch& b, tc::GemmArgs g, int stage, cudaStream_t 
     if (EPI == tc::EPI_K5) encode_img_map(&g.map_n2, b, g.n2, 128, 1, n2_terms);
     if (engine_error()) return;
     constexpr bool GRAM = AMODE == tc::A_IMG_MN;
-    if constexpr (pair_capable(NMODE, EPI, XG)) {
-        if (pair) {
-            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, true, GRAM>, dim3((unsigned)(2 * std::min(g.total_tiles / g.run, sm_count() / 2))),
-                   tc::gemm_threads(AMODE, EPI), smem, 2, stage, st, b, g);
-            return;
+    constexpr int threads = tc::gemm_threads(AMODE, EPI);
+    const dim3 grid((unsigned)(pair ? 2 * std::min(g.total_tiles / g.run, sm_count() / 2) : std::min(g.total_tiles / g.run, sm_count())));
+    with_table(b, [&](const auto& t) {
+        using BATCH = table_t<decltype(t)>;
+        if constexpr (pair_capable(NMODE, EPI, XG)) {
+            if (pair) {
+                launch(tc::gemm_kernel<BATCH, AMODE, NMODE, EPI, XG, true, GRAM>, grid, threads, smem, 2, stage, st, t, g);
+                return;
+            }
         }
-    }
-    const dim3 grid((unsigned)std::min(g.total_tiles / g.run, sm_count()));
-    if constexpr (tc::a_is_buf(AMODE)) {
-        if (g.run > 1) {
-            launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, true>, grid, tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
-            return;
+        if constexpr (tc::a_is_buf(AMODE)) {
+            if (g.run > 1) {
+                launch(tc::gemm_kernel<BATCH, AMODE, NMODE, EPI, XG, false, true>, grid, threads, smem, 1, stage, st, t, g);
+                return;
+            }
         }
-    }
-    launch(tc::gemm_kernel<AMODE, NMODE, EPI, XG, false, GRAM>, grid, tc::gemm_threads(AMODE, EPI), smem, 1, stage, st, b, g);
+        launch(tc::gemm_kernel<BATCH, AMODE, NMODE, EPI, XG, false, GRAM>, grid, threads, smem, 1, stage, st, t, g);
+    });
 }
 
 inline tc::Dest dest_none() {
@@ -1852,8 +1862,9 @@ struct FinishArgs {
     int64_t colsq_off;
     int32_t to_img;
 };
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-finish_split_kernel(const __grid_constant__ Batch batch, FinishArgs a) {
+finish_split_kernel(const __grid_constant__ BATCH batch, FinishArgs a) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     if (*w.status & ST_FAILED) return;
@@ -1904,7 +1915,10 @@ inline void finish_split_product(const Batch& b, Sel dst, Sel part, int64_t rows
                                  int64_t colsq_off, int stage, cudaStream_t st) {
     FinishArgs a{};
     a.dst = dst; a.part = part; a.rows = rows; a.r = r; a.ksplit = ksplit; a.img = img; a.colsq_off = colsq_off; a.to_img = to_img ? 1 : 0;
-    launch(finish_split_kernel, dim3((unsigned)img.panels, (unsigned)(img.rows_pad / 32), (unsigned)b.count), 256, 0, 1, stage, st, b, a);
+    with_table(b, [&](const auto& t) {
+        launch(finish_split_kernel<table_t<decltype(t)>>, dim3((unsigned)img.panels, (unsigned)(img.rows_pad / 32), (unsigned)b.count), 256, 0, 1,
+               stage, st, t, a);
+    });
 }
 
 // Where a product with B goes.
@@ -2024,8 +2038,9 @@ inline int gram_ksplit(int r, int64_t rows, int matrices, int lean) {
 
 // dst <- sum of the `ksplit` partial results at `part` (4 * total4 floats each, one after the
 // other), added in the order of the chunks
+template <class BATCH>
 __global__ void __launch_bounds__(256)
-gram_reduce_kernel(const __grid_constant__ Batch batch, Sel gram, Sel part, int64_t total4, int ksplit, int only_shift_bit) {
+gram_reduce_kernel(const __grid_constant__ BATCH batch, Sel gram, Sel part, int64_t total4, int ksplit, int only_shift_bit) {
     grid_dependency();
     const MatWork& w = batch.w[blockIdx.z];
     const int st = *w.status;
@@ -2059,8 +2074,10 @@ inline void tensor_gram(int r, int passes, const Batch& b, ImgRef src, int64_t r
     launch_gemm<tc::A_IMG_MN, tc::N_IMG_MN, tc::EPI_STORE, 0>(b, g, prof::S_GRAM, st);
     if (ksplit > 1) {
         const int64_t total4 = (int64_t)r * r / 4;
-        launch(gram_reduce_kernel, dim3((unsigned)((total4 + 255) / 256), 1, (unsigned)b.count), 256, 0, 1, prof::S_GRAM, st, b, gram,
-               part, total4, ksplit, only_shift_bit);
+        with_table(b, [&](const auto& t) {
+            launch(gram_reduce_kernel<table_t<decltype(t)>>, dim3((unsigned)((total4 + 255) / 256), 1, (unsigned)b.count), 256, 0, 1, prof::S_GRAM, st,
+                   t, gram, part, total4, ksplit, only_shift_bit);
+        });
     }
 }
 

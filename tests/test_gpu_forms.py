@@ -145,6 +145,33 @@ def test_merged_factorisations_of_one_stream_leave_the_same_bits(r):
         od.orthdion_destroy(h)
 
 
+# more matrices of one plan than the smaller launch table holds: no more launches, and every matrix the bits that it gets alone
+@pytest.mark.parametrize("case", [(96, 104, 32, od.MODE_ORTH, od.ENGINE_TENSOR, 0), (200, 160, 80, od.MODE_COLNORM, od.ENGINE_TENSOR, 3),
+                                  (160, 144, 96, od.MODE_ORTH, od.ENGINE_TENSOR, 1), (90, 77, 24, od.MODE_ORTH, od.ENGINE_SIMT, 1),
+                                  (110, 120, 70, od.MODE_ORTH, od.ENGINE_SIMT, 0), (110, 121, 70, od.MODE_COLNORM, od.ENGINE_SIMT, 0)])
+def test_more_matrices_than_the_smaller_launch_table(case):
+    m, n, r, mode, engine, diag = case
+    probs = [make_problem(m, n, r, F32, BF16, seed=i) for i in range(132)]
+    h = od.orthdion_create(m, n, r, 0.95, 0.01, 0.0, mode)
+    od.orthdion_set_dtypes(h, F32, BF16)
+    od.orthdion_set_engine(h, engine)
+    od.orthdion_set_diagnostics(h, diag)
+    launches = []
+    for count, lanes in ((128, 1), (132, 1), (132, 4)):
+        before = od.orthdion_launch_count()
+        X, M, Q, flags = _grouped(None, probs[:count], [h] * count, lanes)
+        launches.append(od.orthdion_launch_count() - before)
+        assert flags == [0] * count
+        for i in (0, 65, 66, 127, count - 1):
+            spec, x, mm, g, q = probs[i]
+            gm = GpuMatrix(spec, x, mm, q, mu=0.95, eta=0.01, mode=mode, engine=engine)
+            gm.step(g)
+            assert torch.equal(gm.X, X[i]) and torch.equal(gm.M, M[i]) and torch.equal(gm.Q, Q[i])
+            gm.close()
+    assert launches[1] == launches[0]
+    od.orthdion_destroy(h)
+
+
 @pytest.mark.parametrize("r", [96, 256, 272])
 def test_third_pass_of_one_matrix_among_others(r):
     """Products of a third pass look at the status words of their launch first: the one matrix that asked for the pass gets
