@@ -319,7 +319,8 @@ __device__ __forceinline__ float2 ct_diag_block(uint32_t d_off, uint32_t blk_off
 }
 
 // STAGES 4: one CTA per multiprocessor.  2: two, for one launch over more matrices than there are multiprocessors (154 at
-// r = 512, factorisations of a step 1.71 -> 1.56 ms, 168 at r = 192 0.287 -> 0.226).
+// r = 512, factorisations of a step 1.71 -> 1.56 ms, 168 at r = 192 0.287 -> 0.226).  Not below that: 140 at r = 512 0.888 with one
+// and 1.036 with two, 129 at r = 192 0.167 and 0.184, 148 at r = 272 0.316 and 0.358.
 template <class BATCH, int STAGES>
 __global__ void __launch_bounds__(CT_THREADS, STAGES == 4 ? 1 : 2)
 factor_kernel(const __grid_constant__ BATCH batch, CholArgs a, int csize) {

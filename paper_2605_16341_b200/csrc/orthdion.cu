@@ -260,6 +260,7 @@ int ensure_attributes() {
     set(factor_simt_kernel<SmallBatch>, FS_SMEM_BYTES);
     set(factor_simt_kernel<Batch>, FS_SMEM_BYTES);
     set(factor_kernel<SmallBatch, CT_STAGES>, ct_smem_bytes(CT_STAGES));
+    set(factor_kernel<Batch, CT_STAGES>, ct_smem_bytes(CT_STAGES));
     set(factor_kernel<Batch, 2>, ct_smem_bytes(2));
     set(diag_final_kernel<SmallBatch, true>, DIAG_SMEM_LIMIT);
     set(diag_final_kernel<Batch, true>, DIAG_SMEM_LIMIT);
@@ -413,8 +414,13 @@ void chol_stage(std::vector<ClassRun>& cls, const std::vector<int>& which_cls, i
                 const dim3 grid((unsigned)(merged->count * csize));
                 with_table(*merged, [&](const auto& t) {
                     using BATCH = table_t<decltype(t)>;
-                    constexpr int stages = std::is_same<BATCH, SmallBatch>::value ? CT_STAGES : 2;
-                    launch(factor_kernel<BATCH, stages>, grid, CT_THREADS, ct_smem_bytes(stages), csize, prof::S_CHOL, st, t, ca, csize);
+                    if constexpr (std::is_same<BATCH, Batch>::value) {
+                        if (t.count > sm_count()) {          // two CTAs on a multiprocessor, see factor_kernel
+                            launch(factor_kernel<BATCH, 2>, grid, CT_THREADS, ct_smem_bytes(2), csize, prof::S_CHOL, st, t, ca, csize);
+                            return;
+                        }
+                    }
+                    launch(factor_kernel<BATCH, CT_STAGES>, grid, CT_THREADS, ct_smem_bytes(CT_STAGES), csize, prof::S_CHOL, st, t, ca, csize);
                 });
             } else {
                 with_table(*merged, [&](const auto& t) {

@@ -131,9 +131,9 @@ def _grouped(specs, probs, hs, lanes):
 
 @pytest.mark.parametrize("r", [128, 272])
 def test_merged_factorisations_of_one_stream_leave_the_same_bits(r):
-    # 130 matrices of two shapes: on one stream their factorisations are one launch (two CTAs per multiprocessor), on
+    # 155 matrices of two shapes: on one stream their factorisations are one launch (two CTAs per multiprocessor), on
     # several one per shape
-    shapes = [(300, 320, r)] * 70 + [(320, 280, r)] * 60
+    shapes = [(300, 320, r)] * 80 + [(320, 280, r)] * 75
     probs = [make_problem(*s, BF16, BF16, seed=50 + i) for i, s in enumerate(shapes)]
     plans = {s: od.orthdion_create(*s, 0.95, 0.01, 0.0, od.MODE_ORTH) for s in set(shapes)}
     hs = [plans[s] for s in shapes]
