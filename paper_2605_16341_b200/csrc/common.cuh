@@ -57,11 +57,6 @@ __device__ __forceinline__ float* pick(const MatWork& w, Sel s) {
     }
 }
 
-__device__ __forceinline__ float load_elem(const void* p, int64_t idx, int is_bf16) {
-    if (is_bf16) return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(p)[idx]);
-    return reinterpret_cast<const float*>(p)[idx];
-}
-
 // ---- thread-block clusters ---------------------------------------------------------------------
 __device__ __forceinline__ void cluster_sync_all() {
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");

@@ -10,13 +10,13 @@
 // (common.cuh), i.e. in the two bf16 terms that the products read anyway; the image of L^{-T} is the
 // operand of the apply product, so nothing is converted afterwards.  Tile products run on the
 // warp-level tensor path (mma.sync m16n8k16, hi*hi + hi*lo + lo*hi: about 2^-16), operand tiles of
-// 64 x 64 come in by cp.async three steps ahead.
+// 64 x 64 come in by cp.async up to three steps ahead (one in the two-stage form).
 //
 // What bounds it: the chain of r / 64 diagonal blocks.  Four extra warps per CTA factor and invert a
 // 64 x 64 block in fp32 (below) while the eight product warps do the S sums of the same block column, which do not
 // depend on it.  The tile below the diagonal goes first, and the next diagonal block's own sum is kept up column by
 // column, so that the chain (block 10000 cycles, barrier 1000, panel 2400, next block's last product 1300)
-// never waits for the rest.  One CTA per multiprocessor: 161 registers a thread without spills and four operand stages (two
+// never waits for the rest.  One CTA per multiprocessor: 164 registers a thread without spills and four operand stages (two
 // CTAs with 80 registers and two stages: 25000 cycles a block column at r = 1024, where a sum of 15 tiles took
 // longer than the chain).  Step, before all this -> now: 4096 x 4096 r = 256 0.423 -> 0.412 ms, column shard 4096 x 3584 r = 512
 // 0.775 -> 0.730, 11008 x 4096 r = 1024 1.811 -> 1.687, 28 matrices 1000 wide at r = 272 1.65 -> 1.61; the 1.1B and 8B
@@ -64,8 +64,8 @@ __device__ __forceinline__ void ct_bar_sync(int id, int threads) {
 __device__ __forceinline__ void ct_bar_arrive(int id, int threads) {
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-// named barriers (0: the whole CTA); CT_BAR_XT: two, by the parity of the column
-constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_X = 4, CT_BAR_XT = 5, CT_BAR_HAND = 7;
+// named barriers (0: the whole CTA; CT_BAR_MMA + 1 and + 2 also serve the thread groups of the first-order inverse)
+constexpr int CT_BAR_MMA = 1, CT_BAR_DIAG = 2, CT_BAR_READY = 3, CT_BAR_HAND = 4;
 
 __device__ __forceinline__ void ct_cp16(uint32_t dst, const void* src) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");

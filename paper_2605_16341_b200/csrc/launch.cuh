@@ -2,8 +2,11 @@
 // programmatic dependent launch the next kernel's CTAs are set up (barriers, tensor memory, tensor-map
 // fetches) while the current one still runs, and wait for its end and its memory before they touch
 // global memory.  Every kernel of the library therefore starts with grid_dependency_wait() in front of its first global access, and
-// lets its successor in right away.  One exception in two halves: the products with B prefetch M and G before they wait, and
-// the packing kernel in front of the first of them lets it in only after its own wait, i.e. when the step before is done.
+// lets its successor in right away.  One exception: the products with B prefetch M and G to L2 before they wait.  That is safe whatever
+// is still at work, and only because it is a prefetch: L2 is where all kernels of the device meet, and no value gets into a register or
+// shared memory before the wait.  A load in its place would need all writers of M and G to be done, which nothing promises: the packing kernel
+// in front of a step's first product does wait before it lets that in (so that the prefetch finds what will be read), but the
+// phases of a column-sharded step begin with other kernels too.
 #pragma once
 #include <cuda_runtime.h>
 

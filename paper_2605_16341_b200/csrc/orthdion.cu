@@ -579,7 +579,7 @@ void qr_stage(std::vector<ClassRun>& cls, const std::vector<int>& wanted, int wh
 }
 
 // Diagnostics of one class, after its step: Q^T Q from the engine's Gram product, column
-// statistics of R, optionally the norms of M' and G, then one CTA per matrix for the rest.
+// statistics of R, optionally the norms of M' and G, then one cluster per matrix for the rest.
 void diag_stage(ClassRun& c, DiagBase db, cudaStream_t st) {
     const orthdion_plan* p = c.p;
     const Batch& b = *c.b;

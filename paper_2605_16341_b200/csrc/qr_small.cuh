@@ -15,6 +15,8 @@
 // The rows are cut into 1 to 16 parts by row count and rank only, the parts' Gram matrices are added as a
 // balanced binary tree, and a CTA takes one part or a run of them: a call with many matrices uses fewer CTAs
 // for each (they would all factor the same matrix again) and a matrix still gets the same bits alone and in any group.
+// The diagonal block takes all of the 128 registers and puts 4 to 15 others away meanwhile (ptxas: 16 to 58 bytes of spill stores, none
+// without the block); the batched loads of the rows spill nothing.
 // Measured, both QRs of a step with their launches (23 -> 6 per step): one 256 x 512 fp32 matrix, r = 16: step
 // 198 -> 67 us; 520 x 384, r = 64: 235 -> 115 us; 4096 x 4096, r = 32: 442 -> 240 us.
 #pragma once
@@ -80,7 +82,9 @@ inline int qs_threads(int64_t rows, int r, int max_ctas, bool fp32_engine) {
 // at r = 64: 512 x 512 one 0.204 and 0.106 ms, 72 of them 0.383 and 0.321; 640 x 640 one 0.214 and 0.101, 24 0.285 and
 // 0.189, 72 0.491 and 0.547; 768 x 768 one 0.220 and 0.100, 24 0.331 and 0.207, 72 0.556 and 0.612; 24 layers of a
 // 768-wide model (168 matrices) 1.39 and 1.61; 4096 x 4096 one 0.336 and 0.263.
-// The fp32 engine's separate kernels have no such side: it takes whatever shared memory holds.
+// The fp32 engine's separate kernels have no such side, at any number of matrices: 767 x 767 r = 40 one 0.217 and 0.091 ms, 24 0.702 and
+// 0.494, 72 1.82 and 1.39, 168 3.98 and 2.99; r = 64 24 0.722 and 0.499, 168 4.00 and 3.02; 72 of 1400 x 1100 r = 40 4.57 and 3.31.  It
+// takes whatever shared memory holds.
 inline bool qs_fits(int64_t rows, int r, int max_ctas, bool fp32_engine) {
     if (r > QS_MAX_RANK || (r > 32 && rows > QS_MAX_ROWS_64 && !fp32_engine)) return false;
     const int c = qs_parts(rows, r, max_ctas);

@@ -345,7 +345,7 @@ struct PackArgs {
 template <class BATCH>
 __global__ void __launch_bounds__(256)
 pack_kernel(const __grid_constant__ BATCH batch, PackArgs a) {
-    // (the first product, which follows, reads M and G before it waits: it may not start while the step before is at work)
+    // (the first product, which follows, prefetches M and G before it waits: not while the step before is still writing M)
     grid_dependency_wait();
     grid_dependency_launch();
     const MatWork& w = batch.w[blockIdx.z];
@@ -1322,9 +1322,8 @@ gemm_kernel(const __grid_constant__ BATCH batch, const __grid_constant__ GemmArg
         const int xr = AMODE == A_BUF_ROW ? xt / 8 : xt / 16, xc = AMODE == A_BUF_ROW ? xt % 8 : xt % 16;
         const uint32_t dst_off = AMODE == A_BUF_ROW ? xr * 128 + img_chunk_offset(xr, xc)
                                                     : (xc / 8) * 8192 + xr * 128 + img_chunk_offset(xr, xc % 8);
-        // Where launches overlap, the first tiles of M and G are on their way to L2 while the kernel before is still at work: nothing
-        // in the chain of a step writes them before the fused pass, and the step's first kernel lets this one in only
-        // when all that came before the step is done.  Not elsewhere: the loads that follow at once then queue behind the prefetches
+        // Where launches overlap, the first tiles of M and G are on their way to L2 while the kernel before is still at work (prefetches
+        // may be early, loads may not: see launch.cuh).  Not elsewhere: the loads that follow at once then queue behind the prefetches
         // (six-kernel steps of 24 matrices 1024 wide at r = 32 238 us with, 235 without, 36 matrices 768 wide at r = 16 189.6 and 188.2).
         // (Prefetches, because registers that are loaded here live on into the
         // loop: 20 to 60 more bytes spilled, 1 % of the large steps.)
@@ -1774,7 +1773,9 @@ inline int64_t product_depth(int64_t tiles, int chunks, int kb) {
 // results up as it loads them.
 inline bool summed_by_qr(int r, int64_t out_rows) { return r <= 32 || (r <= QS_MAX_RANK && out_rows <= QS_MAX_ROWS_64); }
 // ... and what writing and adding up the partial results costs in the same unit (about a microsecond): a launch, but for
-// the one-kernel QR.
+// the one-kernel QR.  (Their bytes have one price here, although one cluster of at most 16 multiprocessors loads what that
+// kernel adds up, half of its 45 us at 11008 rows and r = 32.  Steps with this rule against the one without that kernel's term, 8192 to
+// 24576 rows: 1.00 to 1.09 times as fast.)
 inline int64_t partial_cost(int64_t tiles, int chunks, int r, bool by_qr) { return (by_qr ? 1 : 4) + tiles * chunks * r / 6000; }
 
 // Depth split of the two products with the buffer.  With one matrix (or a few) in a call and a
@@ -1794,6 +1795,11 @@ inline int64_t partial_cost(int64_t tiles, int chunks, int r, bool by_qr) { retu
 // r = 64 0.091 -> 0.086; 20480 x 4096 r = 32 0.170 -> 0.127, r = 128 0.198 -> 0.176.  Against four chunks at most above
 // r = 64: one 16384 x 1024 matrix at r = 96 0.470 -> 0.426 ms a step, 2048 x 5632 r = 128 0.379 -> 0.368; in a group, where
 // the tiles of a run follow one another, six layers of a 1.1B model at r = 128 1.127 -> 1.155.
+// In front of the one-kernel QR a chunk may have two depth blocks.  Against four at least, r = 16: one 256 x 256 step
+// 57.5 -> 52.9 us, 512 x 512 68.6 -> 58.8, 768 x 768 58.9 -> 57.5; r = 32 1024 x 1024 70 -> 68; two to eight up to 576 wide mostly 3 to 17 % faster.  What it costs:
+// the count is the plan's, and four to eight equal matrices 640 to 1536 wide have tiles enough for the longer
+// chunks: 8 x 768 r = 16 76 -> 79.5, 8 x 1024 r = 32 114 -> 125.  In models of 7 to 56 matrices of such widths it comes out even (0.92 to
+// 1.05 times).
 inline int buffer_chunks(int r, int64_t out_rows, int64_t depth) {
     if (r > 256) return 1;
     const int kb = (int)((depth + tc::BK - 1) / tc::BK), pairs = (int)((out_rows + 255) / 256);
@@ -1995,8 +2001,8 @@ inline int image_bn(int r, int64_t out_rows, int64_t copies) {
 // each with a main loop over all rows of the tall matrix: the depth is cut into chunks whose results are
 // added in a fixed order.  Their number depends on the rank and the row count only, so a matrix gets the same
 // bits alone and in any group.  The chunks run as tiles of their own and leave partial matrices that a small
-// kernel adds up; above r = 256, in calls with tiles enough for the device, one CTA takes the chunks of a tile
-// one after the other and adds each to the tile it has stored (the two accumulators alternate, so
+// kernel adds up; above r = 256, in calls with tiles enough for the device, and at any rank where a workspace has no room
+// for the partial matrices, one CTA takes the chunks of a tile one after the other and adds each to the tile it has stored (the two accumulators alternate, so
 // the additions run beside the next chunk's products).
 inline int gram_tiles(int r) {               // tiles that touch the lower triangle
     const int rows = r % 256 ? 128 : 256, cols = std::min(r, 256);
