@@ -63,12 +63,13 @@ def test_one_kernel_qr_of_long_parts(shape, mode):
 
 
 # rows that only its 256-thread form has room for, up to the last ones: six launches still
-@pytest.mark.parametrize("shape", [(24320, 136, 32), (26112, 72, 32), (39700, 40, 16)])
-def test_one_kernel_qr_up_to_its_last_rows(shape):
-    m, n, r = shape
+@pytest.mark.parametrize("case", [(24320, 136, 32, od.ENGINE_TENSOR), (26112, 72, 32, od.ENGINE_TENSOR), (39700, 40, 16, od.ENGINE_TENSOR),
+                                  (11263, 71, 41, od.ENGINE_SIMT), (26111, 60, 18, od.ENGINE_SIMT)])
+def test_one_kernel_qr_up_to_its_last_rows(case):
+    m, n, r, engine = case
     spec, X, M, G, Q = make_problem(m, n, r, BF16, F32, seed=m)
     before = od.orthdion_launch_count()
-    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=od.ENGINE_TENSOR)
+    one_step_compare(spec, X, M, G, Q, mode=od.MODE_ORTH, engine=engine)
     assert od.orthdion_launch_count() == before + 6
 
 
